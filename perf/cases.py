@@ -142,61 +142,87 @@ def _config(case, n_pages, cap, batch_tokens, boundary_tokens=0, host=False):
                          max_batch_tokens=batch_tokens, max_boundary_tokens=boundary_tokens, host_staging=host)
 
 
-def prepare(case, seed):
+def _prompts(case, u, lens, fracs, g):
+    """(keys, values, tokens) of every prompt that a pass or its preparation hands over, in order: one per group that shares."""
+    at = range(0, case["requests"], case["group"]) if case["kind"] == "prefix" else range(case["requests"])
+    for i, f in zip(at, fracs):
+        yield _prompt(case, lens[i], u, f, g) + (lens[i],)
+
+
+def _start(case, seed):
+    """The generator, head directions, prompt lengths and shares of heavy hitters that a state's inputs begin with."""
     g = torch.Generator(device=DEV)
     g.manual_seed(seed)
     cpu = torch.Generator()
     cpu.manual_seed(seed)
-    kind, n_req, L, steps, page = case["kind"], case["requests"], case["layers"], case["steps"], case["page"]
     u = _unit(case, g)
     lens = _lengths(case, cpu)
-    fracs = torch.exp(torch.rand(n_req, generator=cpu, dtype=torch.float64) * math.log(40.0) + math.log(0.005)).tolist()
+    fracs = torch.exp(torch.rand(case["requests"], generator=cpu, dtype=torch.float64) * math.log(40.0) + math.log(0.005)).tolist()
+    return g, u, lens, fracs
 
+
+def _dense_inputs(case, u, g):
+    shape = (case["requests"], case["hkv"], case["hi"], case["d"])
+    heavy = torch.rand((case["requests"], 1, case["hi"], 1), generator=g, device=DEV) < 0.05
+    k, v = _keys(shape, u[0][None, :, None], heavy, g), _values(shape, g)
+    q = torch.randn((case["requests"], case["hq"], case["d"]), generator=g, device=DEV, dtype=torch.bfloat16)
+    q += (2.0 * u[0]).repeat_interleave(case["hq"] // case["hkv"], dim=0)[None]
+    return q, k, v
+
+
+def _ring(case):
+    """Decode steps of inputs that a state keeps."""
+    kind, steps = case["kind"], case["steps"]
+    if kind in ("admit", "prefix"):
+        return steps
+    row = case["requests"] * case["layers"] * (case["hq"] + 2 * case["hkv"]) * case["d"] * 2
+    return max(2, min(64 if kind == "layers" else 1024, int((2.0e8 if kind == "host" else RING_BYTES) / row)) // steps) * steps
+
+
+def _norm_weights(case, g):
+    return [1.0 + 0.1 * torch.randn(case["d"], generator=g, device=DEV) for _ in range(2)]
+
+
+def _pages(case, lens):
+    """Pages of the pool, and the most a request may have.  Decoding kinds: a few pages to spare, the first grants take
+    them and from then on a boundary compresses."""
+    kind, n_req, page = case["kind"], case["requests"], case["page"]
+    pages = [n // page + 1 for n in lens]
+    if kind == "admit":
+        return sum(pages) + 2 * n_req, case["hi"] // page + 2
+    if kind == "prefix":
+        p0 = pages[0]
+        return n_req // case["group"] * (p0 - 1) + n_req * (p0 + 2), p0 + 3
+    return sum(pages) + max(2, sum(pages) // 50), case["hi"] // page + 5
+
+
+def prepare(case, seed):
+    kind, n_req, L, steps, page = case["kind"], case["requests"], case["layers"], case["steps"], case["page"]
+    g, u, lens, fracs = _start(case, seed)
     if kind == "dense":
-        shape = (n_req, case["hkv"], case["hi"], case["d"])
-        heavy = torch.rand((n_req, 1, case["hi"], 1), generator=g, device=DEV) < 0.05
-        k, v = _keys(shape, u[0][None, :, None], heavy, g), _values(shape, g)
-        q = torch.randn((n_req, case["hq"], case["d"]), generator=g, device=DEV, dtype=torch.bfloat16)
-        q += (2.0 * u[0]).repeat_interleave(case["hq"] // case["hkv"], dim=0)[None]
+        q, k, v = _dense_inputs(case, u, g)
         return dict(case=case, q=q, k=k, v=v, lens=torch.tensor(lens, dtype=torch.int32, device=DEV),
                     out=torch.empty((n_req, case["hq"], case["d"]), dtype=torch.float32, device=DEV))
 
-    pages = [n // page + 1 for n in lens]
-    if kind == "admit":
-        n_pages, cap, batch, bound = sum(pages) + 2 * n_req, case["hi"] // page + 2, 0, 0
-    elif kind == "prefix":
-        p0 = lens[0] // page + 1
-        groups = n_req // case["group"]
-        n_pages, cap, batch, bound = groups * (p0 - 1) + n_req * (p0 + 2), p0 + 3, n_req * (p0 + 3) * page, 0
-    else:
-        # a few pages to spare: the first grants take them, from then on a boundary compresses
-        spare = max(2, sum(pages) // 50)
-        n_pages, cap = sum(pages) + spare, case["hi"] // page + 5
-        batch, bound = n_pages * page, max(cap, n_pages // 4) * page
+    n_pages, cap = _pages(case, lens)
+    batch, bound = {"admit": (0, 0), "prefix": (n_req * cap * page, 0)}.get(kind, (n_pages * page, max(cap, n_pages // 4) * page))
     pool = B.Pool(_config(case, n_pages, cap, batch, bound, host=kind == "host"))
     st = dict(case=case, pool=pool, at=0)
     act = torch.zeros((steps, n_req), dtype=torch.int32, device=DEV)
     out = torch.zeros((steps, L, n_req, case["hq"], case["d"]), dtype=torch.float32, device=DEV)
     if kind in ("admit", "prefix"):
-        # what arrives later: the prompts (one per group that shares), and the first decode steps' inputs
-        distinct = lens if kind == "admit" else lens[::case["group"]]
-        st["prompts"] = [_prompt(case, n, u, f, g) + (n,) for n, f in zip(distinct, fracs)]
-        ring = steps
+        st["prompts"] = list(_prompts(case, u, lens, fracs, g))       # what arrives later
     else:
-        for n, f in zip(lens, fracs):
-            k, v = _prompt(case, n, u, f, g)
+        for k, v, n in _prompts(case, u, lens, fracs, g):
             status, _ = pool.request_add(-1, 0, k, v, n, 0)
             assert status == B.GP_OK, status
-        row = n_req * L * (case["hq"] + 2 * case["hkv"]) * case["d"] * 2
-        ring = max(2, min(64 if kind == "layers" else 1024, int((2.0e8 if kind == "host" else RING_BYTES) / row)) // steps) * steps
-    qs, ks, vs = _step_inputs(case, n_req, ring, u, torch.tensor(fracs, device=DEV), g)
+    qs, ks, vs = _step_inputs(case, n_req, _ring(case), u, torch.tensor(fracs, device=DEV), g)
     ids = torch.arange(n_req, dtype=torch.int32, device=DEV)
     if kind == "host":
         qs, ks, vs = (list(torch.stack(x).cpu().pin_memory()) for x in (qs, ks, vs))
         ids, act, out = ids.cpu().pin_memory(), act.cpu().pin_memory(), out.cpu().pin_memory()
     if kind == "layers":
-        st["wq"] = 1.0 + 0.1 * torch.randn(case["d"], generator=g, device=DEV)
-        st["wk"] = 1.0 + 0.1 * torch.randn(case["d"], generator=g, device=DEV)
+        st["wq"], st["wk"] = _norm_weights(case, g)
         qs, ks, vs = ([list(x) for x in xs] for xs in (qs, ks, vs))          # a model hands over one layer's tensors at a time
     st.update(ids=ids, q=qs, k=ks, v=vs, out=out, act=act)
     return st
@@ -287,3 +313,104 @@ def tolerance(case):
     if case["kind"] == "dense":
         return {"rel": 8e-7, "max": 7e-6}
     return {"rel": 1.3e-5, "max": 9e-5, "differ": 0.0}
+
+
+# ---- the same in 64 bits --------------------------------------------------------------------------------------------
+def _rotate(x, pos, theta):
+    """Rotary embedding of the last dimension at a position (rotate-half pairing); theta 0: none."""
+    if theta == 0.0:
+        return x
+    half = x.shape[-1] // 2
+    ang = float(pos) * theta ** (-torch.arange(half, dtype=torch.float64, device=x.device) / half)
+    c, s = ang.cos(), ang.sin()
+    return torch.cat([x[..., :half] * c - x[..., half:] * s, x[..., half:] * c + x[..., :half] * s], dim=-1)
+
+
+def _view(q, k):
+    """Attention of a group's heads over candidate keys, each head its own softmax, averaged: [L][hkv][G][d], [L][hkv][n][d] -> [L][hkv][n]."""
+    return torch.softmax(q @ k.transpose(-1, -2) / math.sqrt(q.shape[-1]), dim=-1).mean(dim=-2)
+
+
+def _working_set(a, p=0.99):
+    """Smallest number of weights whose sum reaches p, summed over layers and heads."""
+    c = torch.cumsum(torch.sort(a, dim=-1, descending=True)[0], dim=-1)
+    return int(torch.clamp((c < p).sum(dim=-1) + 1, max=a.shape[-1]).sum())
+
+
+def _kept(s, page, k_loc):
+    """Slots that stay when `page` of the candidates go: the k' best of every page, and the best of the rest; ascending."""
+    n = s.shape[-1]
+    blocks = -(-n // page)
+    quota = min(k_loc, (n - page) // blocks)
+    padded = torch.nn.functional.pad(s, (0, blocks * page - n), value=-1.0).unflatten(-1, (blocks, page))
+    rank = torch.sort(torch.sort(padded, dim=-1, descending=True, stable=True)[1], dim=-1)[1].flatten(-2)[..., :n]
+    order = torch.sort(torch.where(rank < quota, math.inf, s), dim=-1, descending=True, stable=True)[1]
+    return torch.sort(order[..., :n - page], dim=-1)[0]
+
+
+class _Request:
+    """One request's retained keys and values (bf16, as the caller gave them) and its two query summaries in 64 bits."""
+
+    def __init__(self, case, k, v, n, page):
+        room = n + case["steps"] + page
+        self.k, self.v = (torch.zeros((case["layers"], case["hkv"], room, case["d"]), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+        self.k[:, :, :n], self.v[:, :, :n] = k.transpose(1, 2), v.transpose(1, 2)
+        self.n, self.pos, self.pages, self.short, self.long = n, n, n // page + 1, None, None
+
+
+def exact(case, seed):
+    """The outputs of a state's first pass in 64 bits.  None when that takes too long."""
+    n_req, hq, hkv, d, steps, page, theta = (case[x] for x in ("requests", "hq", "hkv", "d", "steps", "page", "rope"))
+    L, G, kind = case["layers"], hq // hkv, case["kind"]
+    g, u, lens, fracs = _start(case, seed)
+    if kind == "dense":
+        q, k, v = _dense_inputs(case, u, g)
+        out = torch.empty((n_req, hq, d), dtype=torch.float64, device=DEV)
+        for i, n in enumerate(lens):
+            z = q[i].double().view(hkv, G, d) @ k[i, :, :n].double().transpose(-1, -2) / math.sqrt(d)
+            out[i] = (torch.softmax(z, dim=-1) @ v[i, :, :n].double()).view(hq, d)
+        return out
+    if steps * sum(lens) * L * hkv * d > 4e11 or steps * n_req * L * hq * d > 1.5e9:
+        return None
+    prompts = list(_prompts(case, u, lens, fracs, g))
+    reqs = [_Request(case, *prompts[i // case["group"]], page) for i in range(n_req)]
+    del prompts
+    qs, ks, vs = _step_inputs(case, n_req, _ring(case), u, torch.tensor(fracs, device=DEV), g)
+    weights = _norm_weights(case, g) if kind == "layers" else None
+    n_pages, cap = _pages(case, lens)
+    # (a prefix pool has pages for every copy and grant of the pass)
+    free = 1 << 30 if kind == "prefix" else n_pages - sum(r.pages for r in reqs)
+    out = torch.empty((steps, L, n_req, hq, d), dtype=torch.float64, device=DEV)
+    for j in range(steps):
+        for i, r in enumerate(reqs):
+            q, k = qs[j][:, i].double(), ks[j][:, i].double()
+            if weights:
+                # normalised per head, rounded as a model rounds them, the key rotated before that
+                q, k = (x / torch.sqrt((x * x).mean(dim=-1, keepdim=True) + 1e-6) * w.double() for x, w in zip((q, k), weights))
+                q, k = q.float().bfloat16().double(), _rotate(k, r.pos, theta).float().bfloat16().double()
+            r.k[:, :, r.n], r.v[:, :, r.n] = k.bfloat16(), vs[j][:, i]
+            t, r.n, r.pos = r.pos, r.n + 1, r.pos + 1
+            kk = r.k[:, :, :r.n].double()
+            z = _rotate(q, t, theta).view(L, hkv, G, d) @ kk.transpose(-1, -2) / math.sqrt(d)
+            out[j, :, i] = (torch.softmax(z, dim=-1) @ r.v[:, :, :r.n].double()).view(L, hq, d)
+            r.short = q if r.short is None else 0.9 * r.short + (1.0 - 0.9) * q
+            r.long = q if r.long is None else 0.999 * r.long + (1.0 - 0.999) * q
+            if r.n < r.pages * page:
+                continue
+            # the capacity boundary: working sets under both summaries, then one more page, or one page of tokens evicted
+            rms = lambda x: torch.sqrt((x * x).mean(dim=-1, keepdim=True))
+            qs_, ql_ = (_rotate(rms(q) / rms(x) * x, t, theta).view(L, hkv, G, d) for x in (r.short, r.long))
+            demand = kk[:, :, :r.n - page]
+            r.wants = _working_set(_view(qs_, demand)) > _working_set(_view(ql_, demand))
+            r.score = torch.maximum(_view(qs_, kk[:, :, :r.n - 16]), _view(ql_, kk[:, :, :r.n - 16]))
+        for r in reqs:                                                      # ascending request id
+            if r.n < r.pages * page:
+                continue
+            if r.wants and r.pages < cap and free > 0:
+                r.pages, free = r.pages + 1, free - 1
+                continue
+            keep = torch.cat([_kept(r.score, page, case["k_loc"]), torch.arange(r.n - 16, r.n, device=DEV).expand(L, hkv, 16)], dim=-1)
+            r.n -= page
+            for x in (r.k, r.v):
+                x[:, :, :r.n] = torch.gather(x, 2, keep[..., None].expand(-1, -1, -1, d))
+    return out, None
