@@ -420,7 +420,7 @@ int gp_test_withhold(gp_pool* pool, int32_t what, int32_t spin_limit);
 
 /* ---- attention without any allocation ------------------------------------------------------------ */
 
-#define GP_NOALLOC_SPLITS   8      /* parts a request's tokens are split into                           */
+#define GP_NOALLOC_SPLITS   8      /* parts a request's tokens can be split into at that limit (fewer rows: more) */
 #define GP_NOALLOC_MAX_ROWS 2048   /* limit on n_req * n_q_heads                                        */
 
 /* (The paper has no counterpart of this call; it exists for deployments, not for the method.)

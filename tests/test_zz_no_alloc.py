@@ -97,3 +97,65 @@ def test_noalloc_rejects_what_does_not_fit():
     with pytest.raises(B.GpError) as e:
         B.gp_attention_noalloc(z.data_ptr(), z.data_ptr(), z.data_ptr(), z.data_ptr(), 1, 8, 2, 96, 4, z.data_ptr(), 0)
     assert e.value.status == B.GP_ERR_INVALID
+
+
+def _dense(rng, hq, hkv, d, lens, max_len, offset=0):
+    """Queries, keys and values on the device, keys and values `offset` elements past a 16-byte boundary; their values as float64."""
+    import torch
+    f = W.bf16_bits_to_f64
+    arrays = [W.f32_to_bf16_bits((2.0 * rng.standard_normal(shape)).astype(np.float32))
+              for shape in ((len(lens), hq, d), (len(lens), hkv, max_len, d), (len(lens), hkv, max_len, d))]
+    on_gpu = []
+    for i, a in enumerate(arrays):
+        flat = torch.zeros(a.size + 8, dtype=torch.int16, device="cuda")
+        part = flat[offset if i else 0:][:a.size]
+        part.copy_(torch.from_numpy(a.view(np.int16).reshape(-1)))
+        on_gpu.append(part)
+    return on_gpu, [f(a) for a in arrays]
+
+
+# Lengths at the edges of the 16- and 32-token tiles, of the warps' shares and of the splits (256 tokens of the longest
+# request); every size of a group; keys and values on and off a 16-byte boundary.  Products of bf16 numbers are exact
+# in fp32, weights keep 24 bits, and a sum of n tokens is rounded at most n / 16 / 4 + 30 times, each within 2^-24 of
+# the sum of magnitudes: under 1e-6 of the result at these lengths and widths, where values do not cancel to nothing.
+@pytest.mark.parametrize("hq,hkv,d,lens,offset", [
+    (8, 2, 64, (1, 15, 16, 17, 31, 32, 33, 0, 127, 128, 129), 0),
+    (6, 2, 64, (255, 256, 257, 513), 0),
+    (8, 8, 128, (1, 15, 16, 17, 63, 64, 65, 0, 129), 0),
+    (16, 2, 128, (1023, 1024, 1025, 3, 2000), 0),
+    (5, 1, 128, (300, 7, 0), 0),
+    (1, 1, 64, (5000,), 0),
+    (8, 2, 128, (77, 300), 1),
+    (7, 1, 64, (77, 300), 4),
+])
+def test_noalloc_attention_at_tile_and_split_edges(hq, hkv, d, lens, offset):
+    import torch
+    rng = np.random.default_rng(23)
+    max_len = max(lens) + 3
+    (q, K, V), (qf, Kf, Vf) = _dense(rng, hq, hkv, d, lens, max_len, offset)
+    lens_d = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    out = torch.full((len(lens), hq, d), float("nan"), dtype=torch.float32, device="cuda")
+    B.gp_attention_noalloc(q.data_ptr(), K.data_ptr(), V.data_ptr(), lens_d.data_ptr(), len(lens), hq, hkv, d, max_len,
+                           out.data_ptr(), 0)
+    got = out.cpu().numpy().astype(np.float64)
+    for r, n in enumerate(lens):
+        want = O.attention_decode(qf[r], Kf[r, :, :n], Vf[r, :, :n]) if n else np.zeros((hq, d))
+        assert np.linalg.norm(got[r] - want) <= 1e-6 * np.linalg.norm(want), (r, n)
+
+
+def test_noalloc_attention_with_an_infinite_value_keeps_the_other_columns():
+    import torch
+    rng = np.random.default_rng(29)
+    hq, hkv, d, n = 8, 2, 128, 100
+    (q, K, V), (qf, Kf, Vf) = _dense(rng, hq, hkv, d, (n,), n)
+    V.view(1, hkv, n, d)[0, 1, 40, 5] = 0x7f80                     # +inf
+    lens_d = torch.tensor([n], dtype=torch.int32, device="cuda")
+    out = torch.zeros((1, hq, d), dtype=torch.float32, device="cuda")
+    B.gp_attention_noalloc(q.data_ptr(), K.data_ptr(), V.data_ptr(), lens_d.data_ptr(), 1, hq, hkv, d, n, out.data_ptr(), 0)
+    got = out.cpu().numpy().astype(np.float64)[0]
+    want = O.attention_decode(qf[0], Kf[0], Vf[0])
+    want[4:, 5] = np.inf
+    # weights here are no smaller than about 2^-60, so that inf x weight is inf
+    assert np.array_equal(np.isinf(got), np.isinf(want)) and not np.isnan(got).any()
+    fin = np.isfinite(want)
+    assert np.linalg.norm(got[fin] - want[fin]) <= 1e-6 * np.linalg.norm(want[fin])
