@@ -3,10 +3,10 @@
 // exp(logit - the page's maximum logit) of every candidate key, and per 16-token page the maximum and the sum of
 // those exponentials.  The work on them, in the order of its dependences:
 //
-//   selection jobs    per unit, three independent jobs, one CTA each: per-head softmax over the candidate
-//                     set and group mean -> a^S or a^L and its working-set size K^S or K^L (Eq. 7); and,
-//                     speculatively, the b slots a compression would evict (Eq. 9, Eq. 10).  Under the
-//                     Shrink policy a fourth job lists the 2b slots a Shrink would evict (Eq. 13).
+//   selection         per unit, one CTA: per-head softmax over the candidate set and group mean -> a^S and a^L;
+//                     then, side by side on warps of their own, the working-set sizes K^S and K^L (Eq. 7) and,
+//                     speculatively, the b slots a compression would evict (Eq. 9, Eq. 10).  Under the Shrink policy
+//                     the 2b slots a Shrink would evict as well (Eq. 13).
 //   decisions         by the CTA that finishes its jobs last: Eq. 8 per request, the action (grow, compress,
 //                     shrink), the device allocator: grants first, then copy-on-write targets, each in ascending
 //                     request id.
@@ -27,401 +27,26 @@
 //   (and gp_decide_kernel)                (large pools, the layer-by-layer step; with the KV heads spread over several
 //                                         pools the decisions wait for the sums of all pools in a kernel of their own).
 //
-// Everything that decides an integer outcome is fp64.  Top-p counting and the eviction cut work on the
-// IEEE bit patterns of the (non-negative) scores: one pass into a two-level histogram (4096 fine bins under
-// 256 coarse ones) when the scores' top bits are uniform, else a radix descent, 11 bits per level; the
-// histograms live in shared memory, and the top-p mass is accumulated in 2^62 fixed point with integer
-// atomics, so the result does not depend on the order in which threads add.
+// Everything that decides an integer outcome is fp64.  Top-p counting and the eviction cut work on the IEEE bit
+// patterns of the (non-negative) scores: a radix descent, 8 bits per level from the first bit in which the unit's
+// scores differ, until the bin with the crossing point holds at most 32 scores, which one warp sorts.  The top-p mass
+// is accumulated in 2^62 fixed point with integer atomics, so the result does not depend on the order in which
+// threads add.
 #include "../../include/growpage.h"
 #include "gp_dev.cuh"
 
 namespace {
 
-constexpr int NBINS = 2048;
-constexpr int NBINS_PAD = NBINS + NBINS / 8;     // bins are stored at b + (b >> 3): a thread's 8 consecutive bins and
-#define HIDX(b) ((b) + ((b) >> 3))              // its neighbours' then fall into different banks
 constexpr double TWO62 = 4611686018427387904.0;
 constexpr int SEL_T = 256;           // threads of the selection kernel
 constexpr int SEL_NW = SEL_T / 32;
-constexpr int SEL_CAP = 6144;        // candidate tokens whose scores are staged in shared memory
+constexpr int SEL_CAP = 5120;        // candidate tokens whose scores (both views) are kept in shared memory, at most
 constexpr int CT = 256;              // threads of the compaction kernel
 constexpr int MOVE_TOK = GP_MOVE_TOK;     // source slots per compaction chunk
 constexpr int CMP_SHRINK = 1 << 30;       // flag on a compressing request's boundary index: the action is a Shrink
 
 __device__ __forceinline__ unsigned long long to_fix(double a) {
   return (unsigned long long)__double2ll_rn(a * TWO62);
-}
-
-struct PairCU { unsigned c; unsigned long long s; };
-
-// exclusive suffix sum over the block: sum of the values of threads with a higher id
-template <int BT>
-__device__ __forceinline__ PairCU block_suffix_excl(unsigned c, unsigned long long s, unsigned* wc,
-                                                    unsigned long long* wsum) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned ic = c; unsigned long long is = s;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    unsigned tc = __shfl_down_sync(0xffffffffu, ic, off);
-    unsigned long long ts = __shfl_down_sync(0xffffffffu, is, off);
-    if (lane + off < 32) { ic += tc; is += ts; }
-  }
-  if (lane == 0) { wc[warp] = ic; wsum[warp] = is; }
-  __syncthreads();
-  PairCU r; r.c = ic - c; r.s = is - s;
-  for (int w = warp + 1; w < BT / 32; ++w) { r.c += wc[w]; r.s += wsum[w]; }
-  __syncthreads();
-  return r;
-}
-// exclusive prefix count over the block
-template <int BT>
-__device__ __forceinline__ unsigned block_prefix_excl(unsigned c, unsigned* wc) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned ic = c;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    unsigned tc = __shfl_up_sync(0xffffffffu, ic, off);
-    if (lane >= off) ic += tc;
-  }
-  if (lane == 31) wc[warp] = ic;
-  __syncthreads();
-  unsigned r = ic - c;
-  for (int w = 0; w < warp; ++w) r += wc[w];
-  __syncthreads();
-  return r;
-}
-
-__device__ __constant__ int kWidths[6] = {11, 11, 11, 11, 11, 8};   // 63 bits below the sign
-
-// 64-bit add into a (low, high) pair of 32-bit shared-memory words with two native atomics; the pair is
-// exact once all adds have landed (the carry travels with the high word's add).
-__device__ __forceinline__ void add64_split(unsigned* lo, unsigned* hi, unsigned long long x) {
-  const unsigned xl = (unsigned)x, xh = (unsigned)(x >> 32);
-  const unsigned old = atomicAdd(lo, xl);
-  const unsigned carry = (old + xl) < old ? 1u : 0u;
-  if (xh + carry) atomicAdd(hi, xh + carry);
-}
-
-// Eq. 7: smallest k such that the k largest of a[0..n) sum to at least p.
-template <int BT>
-__device__ __noinline__ int top_p_count(const GpDev& p, const double* a, int n, unsigned long long p_fix, unsigned* hcnt,
-                           unsigned long long* hsum64, unsigned* wc, unsigned long long* wsum, long long* s_res) {
-  unsigned* hlo = reinterpret_cast<unsigned*>(hsum64);
-  unsigned* hhi = hlo + NBINS_PAD;
-  const int tid = threadIdx.x;
-  unsigned long long prefix = 0;
-  unsigned cnt_above = 0;
-  unsigned long long sum_above = 0;
-  int shift = 63;
-  int bin_star = 0;
-  for (int lvl = 0; lvl < 6; ++lvl) {
-    const int w = kWidths[lvl];
-    shift -= w;
-    const int nb = 1 << w;
-    for (int i = tid; i < nb + (nb >> 3); i += BT) { hcnt[i] = 0; hlo[i] = 0; hhi[i] = 0; }
-    if (tid == 0) s_res[0] = -1;
-    __syncthreads();
-    for (int i = tid; i < n; i += BT) {
-      const double v = a[i];
-      const unsigned long long key = (unsigned long long)__double_as_longlong(v);
-      if (lvl == 0 || (key >> (shift + w)) == prefix) {
-        const int bin = (int)((key >> shift) & (unsigned long long)(nb - 1));
-        atomicAdd(&hcnt[HIDX(bin)], 1u);
-        add64_split(&hlo[HIDX(bin)], &hhi[HIDX(bin)], to_fix(v));
-      }
-    }
-    __syncthreads();
-    const int per = nb / BT > 0 ? nb / BT : 1;
-    const int lo = tid * per, hi = lo + per;     // this thread's bins [lo, hi)
-    unsigned c = 0; unsigned long long s = 0;
-    if (lo < nb) for (int b = lo; b < hi; ++b) { c += hcnt[HIDX(b)]; s += ((unsigned long long)hhi[HIDX(b)] << 32) + hlo[HIDX(b)]; }
-    PairCU ex = block_suffix_excl<BT>(c, s, wc, wsum);
-    if (lo < nb) {
-      unsigned long long run_s = sum_above + ex.s;
-      unsigned run_c = cnt_above + ex.c;
-      for (int b = hi - 1; b >= lo; --b) {
-        const unsigned long long before = run_s;
-        run_s += ((unsigned long long)hhi[HIDX(b)] << 32) + hlo[HIDX(b)];
-        if (before < p_fix && run_s >= p_fix) { s_res[0] = b; s_res[1] = run_c; s_res[2] = (long long)before; }
-        run_c += hcnt[HIDX(b)];
-      }
-    }
-    __syncthreads();
-    if (s_res[0] < 0) return n;                  // rounding kept the total below p: everything
-    bin_star = (int)s_res[0];
-    cnt_above = (unsigned)s_res[1];
-    sum_above = (unsigned long long)s_res[2];
-    const unsigned cstar = hcnt[HIDX(bin_star)];
-    __syncthreads();
-    if (cstar == 1) return (int)cnt_above + 1;
-    prefix = (prefix << w) | (unsigned long long)bin_star;
-  }
-  // all bits fixed: the bin holds copies of one value
-  const unsigned c = hcnt[HIDX(bin_star)];
-  const unsigned long long f = (((unsigned long long)hhi[HIDX(bin_star)] << 32) + hlo[HIDX(bin_star)]) / c;
-  unsigned long long j = (p_fix - sum_above + f - 1) / f;
-  if (j < 1) j = 1;
-  if (j > c) j = c;
-  __syncthreads();
-  return (int)cnt_above + (int)j;
-}
-
-// ------------------------------------------------------------------------------------------------------
-// fast path: one pass fills a 4096-bin histogram and its 256-bin summary; a one-warp sort finishes
-// ------------------------------------------------------------------------------------------------------
-// Scores of a candidate set are probabilities of similar magnitude: bits 62..58 of their IEEE patterns are
-// nearly always the same (the softmax pass reports whether they are).  Then bits 57..46 (low exponent bits and
-// the top of the mantissa) order the scores finely enough that the crossing point falls into a bin with a
-// handful of members.  The 256-bin summary (bits 57..50) is scanned by the block, one bin per thread; the 16
-// fine bins under the crossing summary bin by half a warp; the members of the crossing fine bin are sorted by
-// one warp.  When the top bits differ or the bin is crowded, the callers fall back on the general radix
-// descent above.
-constexpr int FBINS = 4096;
-constexpr int FB_PAD = FBINS + FBINS / 16;       // plane stride (the general routine pads its bins)
-constexpr int CBINS = 256;                       // summary bins: 16 fine bins each, one per thread
-constexpr int FSHIFT = 46;
-static_assert(CBINS <= SEL_T, "one summary bin per thread");
-
-struct FastHist {
-  unsigned* cnt; unsigned* lo; unsigned* hi;       // [FBINS] members, and their fixed-point mass in two halves
-  unsigned* ccnt; unsigned* clo; unsigned* chi;    // [CBINS] the same per summary bin
-};
-
-__device__ __forceinline__ void fast_hist_zero(const FastHist& H, bool with_mass) {
-  const uint4 z = make_uint4(0, 0, 0, 0);
-  for (int i = threadIdx.x; i < FBINS / 4; i += SEL_T) {
-    reinterpret_cast<uint4*>(H.cnt)[i] = z;
-    if (with_mass) { reinterpret_cast<uint4*>(H.lo)[i] = z; reinterpret_cast<uint4*>(H.hi)[i] = z; }
-  }
-  if (threadIdx.x < CBINS) {
-    H.ccnt[threadIdx.x] = 0;
-    if (with_mass) { H.clo[threadIdx.x] = 0; H.chi[threadIdx.x] = 0; }
-  }
-}
-
-// sorts (v, tag) across the 32 lanes: descending v when DESC, else ascending v with larger tag first among
-// equal v
-template <bool DESC>
-__device__ __forceinline__ void warp_sort(double& v, int& tag) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, v, j);
-      const int ot = __shfl_xor_sync(0xffffffffu, tag, j);
-      // "first" = the element that belongs earlier in the final order
-      const bool mine_first = DESC ? (v > ov || (v == ov && tag < ot)) : (v < ov || (v == ov && tag > ot));
-      const bool want_first = (((lane & k) == 0) == ((lane & j) == 0));
-      if (mine_first != want_first) { v = ov; tag = ot; }
-    }
-  }
-}
-
-// Eq. 7 on the fast path (histograms already zeroed, s_res[0] = -1, *s_cnt = 0); returns -1 when the general
-// routine has to take over
-__device__ int top_p_fast(const GpDev& p, const double* a, int n, unsigned long long p_fix, const FastHist& H,
-                          unsigned* wc, unsigned long long* wsum, long long* s_res, double* list, int* s_cnt) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < n; i += SEL_T) {
-    const double v = a[i];
-    const int bin = (int)(((unsigned long long)__double_as_longlong(v) >> FSHIFT) & (FBINS - 1));
-    const unsigned long long f = to_fix(v);
-    atomicAdd(&H.cnt[bin], 1u);
-    add64_split(&H.lo[bin], &H.hi[bin], f);
-    atomicAdd(&H.ccnt[bin >> 4], 1u);
-    add64_split(&H.clo[bin >> 4], &H.chi[bin >> 4], f);
-  }
-  __syncthreads();
-  {                                               // summary level: thread t owns bin t; higher bins = larger scores
-    const unsigned c = tid < CBINS ? H.ccnt[tid] : 0u;
-    const unsigned long long m = tid < CBINS ? ((unsigned long long)H.chi[tid] << 32) + H.clo[tid] : 0ull;
-    const PairCU ex = block_suffix_excl<SEL_T>(c, m, wc, wsum);
-    if (tid < CBINS && ex.s < p_fix && ex.s + m >= p_fix) { s_res[0] = tid; s_res[1] = ex.c; s_res[2] = (long long)ex.s; }
-  }
-  __syncthreads();
-  if (s_res[0] < 0) return n;                    // rounding kept the total below p: everything
-  if (tid < 32) {                                // fine level: lane j owns the (j+1)-th highest bin of the 16
-    const int cb = (int)s_res[0];
-    const int fb = cb * 16 + 15 - (tid & 15);
-    const unsigned c = tid < 16 ? H.cnt[fb] : 0u;
-    const unsigned long long m = tid < 16 ? ((unsigned long long)H.hi[fb] << 32) + H.lo[fb] : 0ull;
-    unsigned ic = c; unsigned long long im = m;
-#pragma unroll
-    for (int off = 1; off < 16; off <<= 1) {
-      const unsigned tc = __shfl_up_sync(0xffffffffu, ic, off);
-      const unsigned long long tm = __shfl_up_sync(0xffffffffu, im, off);
-      if (tid >= off) { ic += tc; im += tm; }
-    }
-    const unsigned long long before = (unsigned long long)s_res[2] + im - m;
-    if (tid < 16 && before < p_fix && before + m >= p_fix) {
-      s_res[4] = fb; s_res[5] = s_res[1] + (long long)(ic - c); s_res[6] = (long long)before; s_res[7] = c;
-    }
-  }
-  __syncthreads();
-  const int bstar = (int)s_res[4];
-  const unsigned cnt_above = (unsigned)s_res[5];
-  const unsigned long long sum_above = (unsigned long long)s_res[6];
-  const unsigned cstar = (unsigned)s_res[7];
-  if (cstar == 1) return (int)cnt_above + 1;
-  if (cstar > 32) return -1;
-  for (int i = tid; i < n; i += SEL_T) {
-    const double v = a[i];
-    if ((int)(((unsigned long long)__double_as_longlong(v) >> FSHIFT) & (FBINS - 1)) == bstar) list[atomicAdd(s_cnt, 1)] = v;
-  }
-  __syncthreads();
-  if (tid < 32) {
-    double v = tid < (int)cstar ? list[tid] : -1.0;
-    int tag = tid;
-    warp_sort<true>(v, tag);
-    unsigned long long inc = tid < (int)cstar ? to_fix(v) : 0ull;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned long long o = __shfl_up_sync(0xffffffffu, inc, off);
-      if (tid >= off) inc += o;
-    }
-    const unsigned hit = __ballot_sync(0xffffffffu, tid < (int)cstar && sum_above + inc >= p_fix);
-    if (tid == 0) s_res[3] = (long long)cnt_above + (hit ? __ffs(hit) : (int)cstar);
-  }
-  __syncthreads();
-  return (int)s_res[3];
-}
-
-// Eq. 10 global cut on the fast path (counts already zeroed, s_res[0] = -1, s_cnt[0..1] = 0): lists the ne
-// (b, or 2b for a Shrink) evicted slots in ev[] (unsorted) and returns true, or returns false when the general routine has to take
-// over.  `a` holds Eq. 9 scores, `loc` the block-local quota bits (those slots are never evicted).
-__device__ bool evict_fast(const double* a, int nC, const unsigned* loc, const FastHist& H, unsigned* wc, long long* s_res,
-                           double* list, int* list_slot, int* s_cnt, int* ev, const unsigned ne) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < nC; i += SEL_T) {
-    if (!((loc[i >> 5] >> (i & 31)) & 1u)) {
-      const int bin = (int)(((unsigned long long)__double_as_longlong(a[i]) >> FSHIFT) & (FBINS - 1));
-      atomicAdd(&H.cnt[bin], 1u);
-      atomicAdd(&H.ccnt[bin >> 4], 1u);
-    }
-  }
-  __syncthreads();
-  {                                               // summary level, ascending: the b lowest scores go
-    const unsigned c = tid < CBINS ? H.ccnt[tid] : 0u;
-    const unsigned ex = block_prefix_excl<SEL_T>(c, wc);
-    if (tid < CBINS && ex < ne && ex + c >= ne) { s_res[0] = tid; s_res[1] = ex; }
-  }
-  __syncthreads();
-  if (s_res[0] < 0) return false;
-  if (tid < 32) {
-    const int fb = (int)s_res[0] * 16 + (tid & 15);
-    const unsigned c = tid < 16 ? H.cnt[fb] : 0u;
-    unsigned ic = c;
-#pragma unroll
-    for (int off = 1; off < 16; off <<= 1) {
-      const unsigned tc = __shfl_up_sync(0xffffffffu, ic, off);
-      if (tid >= off) ic += tc;
-    }
-    const unsigned before = (unsigned)s_res[1] + ic - c;
-    if (tid < 16 && before < ne && before + c >= ne) { s_res[4] = fb; s_res[5] = before; s_res[6] = c; }
-  }
-  __syncthreads();
-  const int bstar = (int)s_res[4];
-  const int cnt_below = (int)s_res[5], cstar = (int)s_res[6];
-  const bool exact = (cnt_below + cstar == (int)ne);
-  if (!exact && cstar > 32) return false;
-  for (int i = tid; i < nC; i += SEL_T) {
-    if (!((loc[i >> 5] >> (i & 31)) & 1u)) {
-      const int bin = (int)(((unsigned long long)__double_as_longlong(a[i]) >> FSHIFT) & (FBINS - 1));
-      if (bin < bstar || (exact && bin == bstar)) ev[atomicAdd(&s_cnt[0], 1)] = i;
-      else if (bin == bstar) { const int at = atomicAdd(&s_cnt[1], 1); list[at] = a[i]; list_slot[at] = i; }
-    }
-  }
-  __syncthreads();
-  if (!exact && tid < 32) {                      // the lowest scores of the bin, later slots first among equals
-    double v = tid < cstar ? list[tid] : INFINITY;
-    int slot = tid < cstar ? list_slot[tid] : -1;
-    warp_sort<false>(v, slot);
-    if (tid < (int)ne - cnt_below) ev[cnt_below + tid] = slot;
-  }
-  __syncthreads();
-  return true;
-}
-
-// Eq. 10 global cut, general routine (radix descent over the score bits): lists the ne evicted slots in ev[]
-__device__ __noinline__ void evict_general(const GpDev& p, const double* a, int nC, const unsigned* loc, unsigned* hcnt,
-                                           unsigned* wc, long long* s_res, int* s_i, int* ev, const unsigned ne) {
-  const int tid = threadIdx.x;
-      __syncthreads();
-    unsigned long long prefix = 0;
-  unsigned cnt_below = 0;
-  unsigned long long thr = 0;        // evict keys strictly below thr ...
-  unsigned long long tie_key = 0;    // ... and need_eq of the highest slots whose key equals tie_key
-  int need_eq = 0;
-  {
-    int shift = 63;
-    bool done = false;
-    for (int lvl = 0; lvl < 6 && !done; ++lvl) {
-      const int w = kWidths[lvl];
-      shift -= w;
-      const int nb = 1 << w;
-      for (int i = tid; i < nb + (nb >> 3); i += SEL_T) hcnt[i] = 0;
-      if (tid == 0) s_res[0] = -1;
-      __syncthreads();
-      for (int i = tid; i < nC; i += SEL_T) {
-        if (!((loc[i >> 5] >> (i & 31)) & 1u)) {
-          const unsigned long long key = (unsigned long long)__double_as_longlong(a[i]);
-          if (lvl == 0 || (key >> (shift + w)) == prefix)
-            atomicAdd(&hcnt[HIDX((int)((key >> shift) & (unsigned long long)(nb - 1)))], 1u);
-        }
-      }
-      __syncthreads();
-      const int per = nb / SEL_T > 0 ? nb / SEL_T : 1;
-      const int lo = tid * per, hi = lo + per;
-      unsigned c = 0;
-      if (lo < nb) for (int b = lo; b < hi; ++b) c += hcnt[HIDX(b)];
-      const unsigned ex = block_prefix_excl<SEL_T>(c, wc);
-      if (lo < nb) {
-        unsigned run = cnt_below + ex;
-        for (int b = lo; b < hi; ++b) {
-          const unsigned before = run;
-          run += hcnt[HIDX(b)];
-          if (before < ne && run >= ne) { s_res[0] = b; s_res[1] = before; }
-        }
-      }
-      __syncthreads();
-      if (s_res[0] < 0) {                                  // fewer than b candidates: cannot happen
-        if (tid == 0) atomicOr(p.err, GP_E_BOUNDS);
-        break;
-      }
-      const int bin_star = (int)s_res[0];
-      cnt_below = (unsigned)s_res[1];
-      const unsigned cstar = hcnt[HIDX(bin_star)];
-      __syncthreads();
-      prefix = (prefix << w) | (unsigned long long)bin_star;
-      if (cnt_below + cstar == ne) {        // the bin fits exactly: no tie to break
-        thr = (prefix + 1ull) << shift;
-        done = true;
-      }
-    }
-    if (!done) {                                           // equal scores straddle the cut
-      thr = prefix;
-      tie_key = prefix;
-      need_eq = (int)ne - (int)cnt_below;
-    }
-  }
-  for (int i = tid; i < nC; i += SEL_T) {
-    if (!((loc[i >> 5] >> (i & 31)) & 1u)) {
-      const unsigned long long key = (unsigned long long)__double_as_longlong(a[i]);
-      if (key < thr) { const int at = atomicAdd(&s_i[0], 1); if (at < (int)ne) ev[at] = i; }
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    int cntv = s_i[0];
-    for (int i = nC - 1; i >= 0 && need_eq > 0; --i) {     // rare: older (lower) slots win ties
-      if (!((loc[i >> 5] >> (i & 31)) & 1u)) {
-        const unsigned long long key = (unsigned long long)__double_as_longlong(a[i]);
-        if (key == tie_key) { if (cntv < (int)ne) ev[cntv] = i; ++cntv; --need_eq; }
-      }
-    }
-    if (cntv != (int)ne) atomicOr(p.err, GP_E_BOUNDS);
-  }
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -598,18 +223,24 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
   }
 }
 
-// one copy of the fp64 exponential in the image: the selection jobs run once per launch, so what they cost
-// is mostly the fetching of their instructions
-__device__ __noinline__ double exp_once(double x) { return exp(x); }
-// factor of a page and column when the factors' table does not fit (very large candidate sets)
-__device__ __noinline__ double factor_slow(const double* zs_entry, double M) { return exp(__ldcg(zs_entry) - M); }
-
-// L2 loads the compiler may not sink towards their first use: the selection jobs issue all loads of a phase
-// together and only then wait (a plain load is free to drift past the block barriers in between)
+// L2 loads the compiler may not sink towards their first use: the selection issues all loads of a phase together and
+// only then waits (a plain load is free to drift past the block barriers in between)
 __device__ __forceinline__ double2 ld_early2(const double* ptr) {
   double2 v;
   asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(ptr));
   return v;
+}
+// the GG values of one token and view: 8, 16, 32 or 64 contiguous bytes
+template <int GG>
+__device__ __forceinline__ void ld_early_row(const double* ptr, double* v) {
+  if (GG == 1) asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v[0]) : "l"(ptr));
+  else if (GG == 2) asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1 % GG]) : "l"(ptr));
+  else {
+#pragma unroll
+    for (int i = 0; i < GG; i += 4)
+      asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];"
+                   : "=d"(v[i]), "=d"(v[(i + 1) % GG]), "=d"(v[(i + 2) % GG]), "=d"(v[(i + 3) % GG]) : "l"(ptr + i));
+  }
 }
 
 // max or sum over the block of one value per thread, separately for each of `ncols` interleaved columns
@@ -631,323 +262,593 @@ __device__ __forceinline__ void column_reduce(double v, int ncols, double* red, 
   __syncthreads();
 }
 
-// Per-head softmax over C and the group mean (Sec. 3.2), then a^S, a^L or s = max(a^S, a^L) (Eq. 9) of every
-// candidate into a[].  The attention kernel left, per 16-token page t and column c, the page's maximum logit
-// m_tc and s_tc = sum of exp(z - m_tc), and per token x = exp(z - m_tc).  With M_c the maximum over pages and
-// f_tc = exp(m_tc - M_c):  softmax = x f_tc / Z_c,  Z_c = sum_t s_tc f_tc.  So this pass takes one exponential
-// per page and column instead of one per token and column; the factors f_tc sit in shared memory (F, f_cap
-// entries; when the candidate set has more page-columns than that, they are recomputed per token).
-// All loads of the prologue (page partials and the first batch of x) are issued together.
-template <int GG>
-__device__ __noinline__ bool job_softmax(const GpDev& p, const double* __restrict__ x, size_t view_stride,
-                                         const double* __restrict__ zs, double* __restrict__ a, int nC, int task,
-                                         double* red, double* sM, double* sZ, double* F, int f_cap) {
-  constexpr int G2 = 2 * GG;
-  constexpr int U = 4;                                   // 16-byte loads per thread and view in flight
-  constexpr int KEEP = 2;                                // page partials per thread held in registers
-  constexpr int LPT = GG >= 2 ? GG / 2 : 1;              // lanes that share a token (two columns each)
-  const int tid = threadIdx.x;
-  const int nview = task == 2 ? 2 : 1;
-  const int ncols = nview * GG;
-  const int col0 = task == 1 ? GG : 0;
-  const int myc = tid % ncols;                           // SEL_T is a multiple of ncols
-  const int mycol = col0 + myc;
-  const int ntile = nC / GP_PAGE;
-  const int t0 = tid / ncols, tstep = SEL_T / ncols;
-  const bool table = ntile * ncols <= f_cap;
-  const int nv = nC * GG / 2;                            // 16-byte pieces of one view: consecutive lanes, consecutive pieces
-  const double* xb = x + (task == 1 ? view_stride : 0);
-  double2 keep[KEEP];
-#pragma unroll
-  for (int k = 0; k < KEEP; ++k) {
-    const int t = t0 + k * tstep;
-    keep[k] = make_double2(-INFINITY, 0.0);
-    if (t < ntile) keep[k] = ld_early2(zs + ((size_t)t * G2 + mycol) * 2);
-  }
-  double2 xv[2][U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int k = tid + u * SEL_T;
-    xv[0][u] = xv[1][u] = make_double2(0.0, 0.0);
-    if (k < nv) {
-      xv[0][u] = ld_early2(xb + 2 * (size_t)k);
-      if (task == 2) xv[1][u] = ld_early2(xb + view_stride + 2 * (size_t)k);
-    }
-  }
-  double m = fmax(keep[0].x, keep[1].x);
-  for (int t = t0 + KEEP * tstep; t < ntile; t += tstep) m = fmax(m, __ldcg(zs + ((size_t)t * G2 + mycol) * 2));
-  column_reduce<true>(m, ncols, red, sM);
-  const double mc = sM[myc];
-  double acc = 0.0;
-#pragma unroll
-  for (int k = 0; k < KEEP; ++k) {
-    const int t = t0 + k * tstep;
-    if (t < ntile) {
-      const double f = exp_once(keep[k].x - mc);
-      acc += keep[k].y * f;
-      if (table) F[t * ncols + myc] = f;
-    }
-  }
-  for (int t = t0 + KEEP * tstep; t < ntile; t += tstep) {
-    const double2 ms = __ldcg(reinterpret_cast<const double2*>(zs + ((size_t)t * G2 + mycol) * 2));
-    const double f = exp_once(ms.x - mc);
-    acc += ms.y * f;
-    if (table) F[t * ncols + myc] = f;
-  }
-  column_reduce<false>(acc, ncols, red, sZ);
-  if (tid < ncols) sZ[tid] = 1.0 / ((double)GG * sZ[tid]);     // group mean and normaliser in one factor
-  __syncthreads();
-  unsigned top_bits = 0;
-  for (int k0 = tid; k0 - tid < nv; k0 += U * SEL_T) {   // uniform trip count: the shuffles below need whole warps
-    if (k0 != tid) {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = k0 + u * SEL_T;
-        xv[0][u] = xv[1][u] = make_double2(0.0, 0.0);
-        if (k < nv) {
-          xv[0][u] = __ldcg(reinterpret_cast<const double2*>(xb + 2 * (size_t)k));
-          if (task == 2) xv[1][u] = __ldcg(reinterpret_cast<const double2*>(xb + view_stride + 2 * (size_t)k));
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = k0 + u * SEL_T;
-      const bool on = k < nv;
-      const int flat = 2 * (on ? k : 0);
-      const int tok = flat / GG, g = flat % GG;           // GG = 1: tokens tok and tok + 1 (same page), column 0
-      const int t = tok / GP_PAGE;
-      double part[2][2];                                  // [view][element of the piece]
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        part[q][0] = part[q][1] = 0.0;
-        if (q < nview && on) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int c = q * GG + (GG == 1 ? 0 : g + e); // column of this job: index into F, sM, sZ
-            const double f = table ? F[t * ncols + c] : factor_slow(zs + ((size_t)t * G2 + col0 + c) * 2, sM[c]);
-            part[q][e] = (e == 0 ? xv[q][u].x : xv[q][u].y) * f * sZ[c];
-          }
-        }
-      }
-      if (GG == 1) {
-        if (on) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const double s0 = task == 2 ? fmax(part[0][e], part[1][e]) : part[0][e];       // Eq. 9
-            a[tok + e] = s0;
-            top_bits |= 1u << (unsigned)(((unsigned long long)__double_as_longlong(s0) >> 58) & 31ull);
-          }
-        }
-      } else {
-        double sv0 = part[0][0] + part[0][1], sv1 = part[1][0] + part[1][1];
-#pragma unroll
-        for (int o = 1; o < LPT; o <<= 1) {
-          sv0 += __shfl_xor_sync(0xffffffffu, sv0, o);
-          sv1 += __shfl_xor_sync(0xffffffffu, sv1, o);
-        }
-        if (on && g == 0) {
-          const double s0 = task == 2 ? fmax(sv0, sv1) : sv0;                              // Eq. 9
-          a[tok] = s0;
-          top_bits |= 1u << (unsigned)(((unsigned long long)__double_as_longlong(s0) >> 58) & 31ull);
-        }
-      }
-    }
-  }
-  // bits 62..58 of every score, as a set: the fast selection path needs them all equal.  (The block-wide
-  // barrier reductions combine predicates, not words, so the sets are OR-ed by hand: per warp, then over the
-  // warps through shared memory; `red` is free here.)
-  top_bits = __reduce_or_sync(0xffffffffu, top_bits);
-  unsigned* sets = reinterpret_cast<unsigned*>(red);
-  if ((tid & 31) == 0) sets[tid >> 5] = top_bits;
-  __syncthreads();
-  unsigned all_bits = 0;
-#pragma unroll
-  for (int w = 0; w < SEL_NW; ++w) all_bits |= sets[w];
-  __syncthreads();
-  return __popc(all_bits) == 1;
-}
-
-// Attention outputs of requests that were split over several work items: merges the items' partial results
-// (running maximum in the log2 domain, sum of exponentials, unnormalised output) into the output row.  The
-// calling CTA takes merges first, first + stride, ...
-__device__ __noinline__ void merge_partials(const GpDev& p, int n_req, float* __restrict__ out, int n_mc, int n_rc,
-                                            int first_item, int stride, int lh0, int lh_n) {
-  const int G = p.G, D = p.d;
-  const int PSTRIDE = G * (D + 2);
-  for (long long mi = first_item; mi < (long long)n_mc * lh_n; mi += stride) {       // units [lh0, lh0 + lh_n)
-    const int4 mc = p.mc_list[mi / lh_n];
-    const int lh = lh0 + (int)(mi % lh_n), l = lh / p.Hkv, h = lh % p.Hkv;
-    const int bi = mc.x, nch = mc.z;
-    const float* first = p.partials + ((size_t)lh * n_rc + mc.y) * PSTRIDE;
-    float* orow = out + (((size_t)l * n_req + bi) * p.Hq + h * G) * D;
-    for (int idx = threadIdx.x; idx < G * D; idx += blockDim.x) {
-      const int g = idx / D, dc = idx % D;
-      const float* pg = first + g * (D + 2);
-      float M = -INFINITY, acc = 0.f, ls = 0.f;
-      for (int c0 = 0; c0 < nch; c0 += 4) {               // four items' values in flight together
-        float m[4], lv[4], vv[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float* pc = pg + (size_t)(c0 + k) * PSTRIDE;
-          const bool on = c0 + k < nch;
-          m[k] = on ? __ldcg(pc + D) : -INFINITY;
-          lv[k] = on ? __ldcg(pc + D + 1) : 0.f;
-          vv[k] = on ? __ldcg(pc + dc) : 0.f;
-        }
-        const float Mn = fmaxf(fmaxf(M, fmaxf(m[0], m[1])), fmaxf(m[2], m[3]));
-        const float sc = exp2f(M - Mn);
-        acc *= sc; ls *= sc;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float w = exp2f(m[k] - Mn);
-          acc += w * vv[k];
-          ls += w * lv[k];
-        }
-        M = Mn;
-      }
-      orow[idx] = acc / ls;
-    }
-  }
-}
-
-// ------------------------------------------------------------------------------------------------------
-// working sets + speculative eviction list; three independent jobs per unit (four under the Shrink policy: its
-// list of 2b evictions), one CTA each; the last CTA decides
-// ------------------------------------------------------------------------------------------------------
-struct SelGeom {
-  static constexpr size_t BUF_BYTES = SEL_CAP * sizeof(double);
-  static constexpr size_t H_BYTES = (size_t)FB_PAD * 12;
-  static constexpr size_t MISC_BYTES = SEL_NW * 8 + SEL_NW * 4 + 8 * 8 + 2 * GP_MAX_BLK * 4 + 16 * 4 + (SEL_NW * 16 + 32) * 8 + 32 * 8 + 32 * 4 + 3 * CBINS * 4;
+// shared memory of the selection; the arrays of scores come last, their size follows the pool's page cap
+constexpr int BIN_STRIDE = 256 + 32;              // 256 bins at b + (b >> 3): a lane's 8 bins and its neighbours' in other banks
+#define BIDX(b) ((b) + ((b) >> 3))
+constexpr int SEL_F = 1024;                       // page factors in shared memory at a time
+struct SelMisc {
+  double red[SEL_NW * 16];
+  double sM[16], sZ[16];                          // per column (view, head): maximum logit, 1 / (G sum of exponentials)
+  unsigned long long list[3][32], list_fix[2][32];     // members of the crossing bin, per task: bit pattern, fixed-point mass
+  int list_slot[32];
+  unsigned rng[3][2];                             // smallest and largest high word of a^S, a^L and max(a^S, a^L)
+  long long res[3][4];                            // crossing bin, members and mass before it, members in it
+  int cnt[4];                                     // evicted slots listed, list members per task
+  int K[2];
+  int s_i[8];
+  int ev[2 * GP_MAX_BLK];
+  unsigned bins[3][3][BIN_STRIDE];                // per task: members, mass (low, high word)
+  double F[SEL_F];
 };
-
-// shared memory of the selection kernel
 struct SelSmem {
-  double* sbuf;                      // [SEL_CAP] a^S, a^L or s
-  unsigned* hcnt;                    // histogram planes; the softmax factors F share them before the bins are used
-  unsigned long long* hsum;
-  unsigned long long* wsum;          // [SEL_NW]
-  unsigned* wc;                      // [SEL_NW]
-  long long* s_res;                  // [8]
-  int* ev;                           // [2 * GP_MAX_BLK] evicted slots of the job
-  int* s_i;                          // [16]
-  double* red;                       // [SEL_NW][16]
-  double* sM;                        // [16]
-  double* sZ;                        // [16]
-  double* flist;                     // [32] members of the crossing bin
-  int* flist_slot;                   // [32]
-  unsigned* loc;                     // [cap*b/32 + 1] block-local picks, one bit per candidate
-  FastHist H;
+  SelMisc* m;
+  unsigned* loc;                     // [cap * 16 / 32 + 2] block-local picks, one bit per candidate
+  double* sS;                        // [SEL_CAP or fewer] a^S, then as many of a^L
+  double* sL;
+  int n_cap;                         // candidates they have room for
 };
-constexpr int SEL_F_CAP = (int)(SelGeom::H_BYTES / sizeof(double));
-
-__device__ __forceinline__ SelSmem sel_smem_at(uint8_t* smem) {      // smem: 256-byte aligned, gp_bsel_smem bytes
+__host__ __device__ inline int sel_n_cap(long long cap) { return cap * GP_PAGE < SEL_CAP ? (int)(cap * GP_PAGE) : SEL_CAP; }
+__host__ __device__ inline size_t sel_loc_bytes(long long cap) { return (((size_t)cap * GP_PAGE / 32 + 2) * 4 + 15) / 16 * 16; }
+constexpr size_t DECIDE_SMEM = 8 * GP_MAX_REQ * 4;          // the decisions' scratch takes the place of bitmap and scores
+__device__ __forceinline__ SelSmem sel_smem_at(uint8_t* smem, int cap) {      // smem: 16-byte aligned, gp_sel_smem bytes
   SelSmem S;
-  S.sbuf = reinterpret_cast<double*>(smem);
-  S.hcnt = reinterpret_cast<unsigned*>(smem + SelGeom::BUF_BYTES);
-  S.hsum = reinterpret_cast<unsigned long long*>(S.hcnt + FB_PAD);           // two u32 planes (low, high)
-  S.wsum = S.hsum + FB_PAD;
-  S.wc = reinterpret_cast<unsigned*>(S.wsum + SEL_NW);
-  S.s_res = reinterpret_cast<long long*>(S.wc + SEL_NW);
-  S.ev = reinterpret_cast<int*>(S.s_res + 8);
-  S.s_i = S.ev + 2 * GP_MAX_BLK;
-  S.red = reinterpret_cast<double*>(S.s_i + 16);
-  S.sM = S.red + SEL_NW * 16;
-  S.sZ = S.sM + 16;
-  S.flist = S.sZ + 16;
-  S.flist_slot = reinterpret_cast<int*>(S.flist + 32);
-  unsigned* coarse = reinterpret_cast<unsigned*>(S.flist_slot + 32);           // [3][CBINS] summary bins
-  S.loc = coarse + 3 * CBINS;
-  S.H.cnt = S.hcnt; S.H.lo = reinterpret_cast<unsigned*>(S.hsum); S.H.hi = S.H.lo + FB_PAD;
-  S.H.ccnt = coarse; S.H.clo = coarse + CBINS; S.H.chi = coarse + 2 * CBINS;
+  S.m = reinterpret_cast<SelMisc*>(smem);
+  uint8_t* at = smem + (sizeof(SelMisc) + 15) / 16 * 16;
+  S.loc = reinterpret_cast<unsigned*>(at);
+  S.n_cap = sel_n_cap(cap);
+  S.sS = reinterpret_cast<double*>(at + sel_loc_bytes(cap));
+  S.sL = S.sS + S.n_cap;
   return S;
 }
 
-// One selection job of a boundary unit: per-head softmax over the candidate set and the group mean from the
-// attention kernel's per-page partials (`z`, `zs`), then either the working-set size of one view (task 0: K^S,
-// 1: K^L; Eq. 7) or the `ne` slots a compression would evict (task 2; Eq. 9, Eq. 10).  The outputs go to Kout / acc
-// (the request's running sum for Eq. 8) and evout.
-__device__ __forceinline__ void sel_job(const GpDev& p, const SelSmem& S, const double* z, size_t view_stride, const double* zs,
-                                     double* a, int nC, int task, int ne, int* Kout, int* acc, int* evout, double* Hout) {
+// Per-head softmax over the first `ntile` pages of the candidates and the group mean (Sec. 3.2): a^S and a^L of every
+// candidate.  The attention kernel left, per 16-token page t and column c (view, head), the page's maximum logit m_tc
+// and s_tc = sum of exp(z - m_tc), and per token x = exp(z - m_tc).  With M_c the maximum over pages and
+// f_tc = exp(m_tc - M_c):  softmax = x f_tc / Z_c,  Z_c = sum_t s_tc f_tc.  So this pass takes one exponential per page
+// and column instead of one per token and column; the factors f_tc / (G Z_c) of SEL_F / 2G pages at a time sit in
+// shared memory.  A thread takes whole tokens (a view's values of a token are contiguous).  All loads of the prologue
+// (page partials and the first tokens) are issued together.  `views`: bit 0 a^S, bit 1 a^L (a job that needs one view
+// reads only that one's logits).  Also leaves the range of the scores' high words.
+template <int GG>
+__device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __restrict__ x, size_t view_stride,
+                                             const double* __restrict__ zs, double* __restrict__ aS, double* __restrict__ aL, int ntile,
+                                             int views) {
+  constexpr int NC = 2 * GG;                             // columns
+  constexpr int U = GG >= 4 ? 2 : 4;                     // tokens per thread in flight
+  constexpr int KEEP = 2;                                // page partials per thread held in registers
+  constexpr int FT = SEL_F / NC;                         // pages whose factors are in shared memory at a time
+  SelMisc& m = *S.m;
   const int tid = threadIdx.x;
-  if (task == 2) for (int i = tid; i < (nC + 31) / 32; i += SEL_T) S.loc[i] = 0;
-  if (tid == 0) { S.s_res[0] = -1; S.s_i[0] = 0; S.s_i[5] = 0; S.s_i[6] = 0; S.s_i[7] = 0; }
-  bool uniform;
-  double* F = reinterpret_cast<double*>(S.hcnt);
-  switch (p.G) {
-    case 1: uniform = job_softmax<1>(p, z, view_stride, zs, a, nC, task, S.red, S.sM, S.sZ, F, SEL_F_CAP); break;
-    case 2: uniform = job_softmax<2>(p, z, view_stride, zs, a, nC, task, S.red, S.sM, S.sZ, F, SEL_F_CAP); break;
-    case 4: uniform = job_softmax<4>(p, z, view_stride, zs, a, nC, task, S.red, S.sM, S.sZ, F, SEL_F_CAP); break;
-    default: uniform = job_softmax<8>(p, z, view_stride, zs, a, nC, task, S.red, S.sM, S.sZ, F, SEL_F_CAP); break;
-  }
-  if (task < 2 && p.metric == GP_METRIC_ENTROPY) {
-    // the ablation's other metric: H = -sum a ln a of the view, summed in a fixed order (per thread over its
-    // strided candidates, then a fixed tree), so that the same input gives the same bits on every run
-    __syncthreads();
-    double hsum = 0.0;
-    for (int i = tid; i < nC; i += SEL_T) { const double v = a[i]; if (v > 0.0) hsum -= v * log(v); }
+  const int myc = tid % NC;                              // SEL_T is a multiple of NC
+  const int t0 = tid / NC;
+  constexpr int TSTEP = SEL_T / NC;
+  double2 keep[KEEP];
 #pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) hsum += __shfl_xor_sync(0xffffffffu, hsum, o2);
-    if ((tid & 31) == 0) S.red[tid >> 5] = hsum;
-    __syncthreads();
-    if (tid == 0) {
-      double tot = 0.0;
-      for (int w = 0; w < SEL_NW; ++w) tot += S.red[w];
-      Kout[task] = 0;
-      Hout[task] = tot;
-    }
-    __syncthreads();
-    return;
+  for (int k = 0; k < KEEP; ++k) {
+    const int t = t0 + k * TSTEP;
+    keep[k] = make_double2(-INFINITY, 0.0);
+    if (t < ntile) keep[k] = ld_early2(zs + ((size_t)t * NC + myc) * 2);
   }
-  fast_hist_zero(S.H, task < 2);                   // the factors' table shared this memory
-  if (task < 2) {
-    __syncthreads();
-    // ---- Eq. 7 -------------------------------------------------------------------------------------------
-    int K = uniform ? top_p_fast(p, a, nC, p.p_fix, S.H, S.wc, S.wsum, S.s_res, S.flist, &S.s_i[5]) : -1;
-    if (K < 0) { __syncthreads(); K = top_p_count<SEL_T>(p, a, nC, p.p_fix, S.hcnt, S.hsum, S.wc, S.wsum, S.s_res); }
-    if (tid == 0) {
-      Kout[task] = K;
-      atomicAdd(acc + task, K);                    // Eq. 8 needs only the sums over layers and heads
-    }
-    return;
-  }
-  // ---- Eq. 10, block-local quota: the k' best slots of every block of C (score desc, slot asc); a block is a
-  // page of the method, the last one short when the protected window is smaller than the page -----------------
-  const int blk = p.blk;
-  const int nblk = (nC + blk - 1) / blk;
-  const int K_t = nC - ne;
-  const int kq = min(p.k_loc, K_t / nblk);
-  if (kq > 0) {
-    for (int i = tid; i < nC; i += SEL_T) {
-      const double s = a[i];
-      int rank = 0;
-      if (blk == GP_PAGE) {
-        const int b0 = i & ~15;
+  double xv[U][2][GG];
+  auto load = [&](int tok0, int n_tok) {                 // tokens tok0 + tid, tok0 + tid + SEL_T, ... of both views
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const double sj = a[b0 + j];
-          rank += (sj > s) || (sj == s && (b0 + j) < i);
-        }
-      } else {
-        const int b0 = (i / blk) * blk, b1 = min(b0 + blk, nC);
-        for (int j = b0; j < b1; ++j) {
-          const double sj = a[j];
-          rank += (sj > s) || (sj == s && j < i);
+    for (int u = 0; u < U; ++u) {
+      const int tok = tok0 + tid + u * SEL_T;
+      if (tok < n_tok) {
+        if (views & 1) ld_early_row<GG>(x + (size_t)tok * GG, xv[u][0]);
+        if (views & 2) ld_early_row<GG>(x + view_stride + (size_t)tok * GG, xv[u][1]);
+      }
+    }
+  };
+  const int n = ntile * GP_PAGE;
+  load(0, n);
+  double mx = fmax(keep[0].x, keep[1].x);
+#pragma unroll 8
+  for (int t = t0 + KEEP * TSTEP; t < ntile; t += TSTEP) mx = fmax(mx, __ldcg(zs + ((size_t)t * NC + myc) * 2));
+  column_reduce<true>(mx, NC, m.red, m.sM);
+  const double mc = m.sM[myc];
+  double acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < KEEP; ++k) {
+    const int t = t0 + k * TSTEP;
+    if (t < ntile) {
+      const double f = exp(keep[k].x - mc);
+      acc += keep[k].y * f;
+      if (t < FT) m.F[t * NC + myc] = f;
+    }
+  }
+  for (int tb = t0 + KEEP * TSTEP; tb < ntile; tb += 4 * TSTEP) {
+    double2 ms[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int t = tb + k * TSTEP;
+      ms[k] = t < ntile ? ld_early2(zs + ((size_t)t * NC + myc) * 2) : make_double2(-INFINITY, 0.0);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int t = tb + k * TSTEP;
+      if (t < ntile) {
+        const double f = exp(ms[k].x - mc);
+        acc += ms[k].y * f;
+        if (t < FT) m.F[t * NC + myc] = f;
+      }
+    }
+  }
+  column_reduce<false>(acc, NC, m.red, m.sZ);
+  const double rz = 1.0 / ((double)GG * m.sZ[myc]);        // group mean and normaliser in one factor
+  for (int t = t0; t < min(ntile, FT); t += TSTEP) m.F[t * NC + myc] *= rz;       // (the thread that wrote the entry)
+  __syncthreads();
+  unsigned lo_w[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi_w[3] = {0u, 0u, 0u};
+  for (int tb = 0; tb < ntile; tb += FT) {               // a set of pages whose factors are in shared memory
+    const int k_begin = tb * GP_PAGE, k_end = min(n, k_begin + FT * GP_PAGE);
+    if (tb) {
+      load(k_begin, k_end);
+      __syncthreads();
+      for (int t = tb + t0; t < min(ntile, tb + FT); t += TSTEP)
+        m.F[(t - tb) * NC + myc] = exp(__ldcg(zs + ((size_t)t * NC + myc) * 2) - mc) * rz;
+      __syncthreads();
+    }
+    for (int k0 = k_begin; k0 < k_end; k0 += U * SEL_T) {
+      if (k0 != k_begin) load(k0, k_end);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tok = k0 + tid + u * SEL_T;
+        if (tok < k_end) {
+          const double* f = m.F + (tok / GP_PAGE - tb) * NC;
+          double a[2] = {0.0, 0.0};
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            if ((views >> q) & 1) {
+              a[q] = xv[u][q][0] * f[q * GG];
+#pragma unroll
+              for (int g = 1; g < GG; ++g) a[q] += xv[u][q][g] * f[q * GG + g];
+            }
+          }
+          if (aS == aL) aS[tok] = views == 3 ? fmax(a[0], a[1]) : a[views >> 1];       // a job of one array
+          else { aS[tok] = a[0]; aL[tok] = a[1]; }
+          const unsigned w0 = (unsigned)__double2hiint(a[0]), w1 = (unsigned)__double2hiint(a[1]), w2 = max(w0, w1);
+          lo_w[0] = min(lo_w[0], w0); lo_w[1] = min(lo_w[1], w1); lo_w[2] = min(lo_w[2], w2);
+          hi_w[0] = max(hi_w[0], w0); hi_w[1] = max(hi_w[1], w1); hi_w[2] = max(hi_w[2], w2);
         }
       }
-      if (rank < kq) atomicOr(&S.loc[i >> 5], 1u << (i & 31));
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const unsigned a = __reduce_min_sync(0xffffffffu, lo_w[q]), b = __reduce_max_sync(0xffffffffu, hi_w[q]);
+    if ((tid & 31) == 0) { atomicMin(&m.rng[q][0], a); atomicMax(&m.rng[q][1], b); }
+  }
+}
+
+__device__ __forceinline__ unsigned long long key_of(double v) { return (unsigned long long)__double_as_longlong(v); }
+
+// Eq. 10, block-local quota: the kq best slots of every block of `blk` candidates (score desc, slot asc; the last block
+// may be short) as bits of loc[].  Run by `nw` warps, warp w of them taking every nw-th 32 slots or block.
+__device__ __forceinline__ void mark_local(const double* aS, const double* aL, int n, int blk, int kq, unsigned* loc, int w, int nw) {
+  const int lane = threadIdx.x & 31;
+  if (blk == GP_PAGE) {                                   // two blocks to a warp: every score against its block's others
+    for (int b0 = w * 32; b0 < n; b0 += nw * 32) {
+      const int i = b0 + lane;
+      const unsigned long long key = i < n ? max(key_of(aS[i]), key_of(aL[i])) : 0ull;
+      // by the high words; where two of a block share one (about one block in ten thousand), by the whole keys
+      const unsigned hw = (unsigned)(key >> 32);
+      int rank = 0;
+      bool same = false;
+#pragma unroll
+      for (int o = 1; o < 16; ++o) {
+        const unsigned t = __shfl_xor_sync(0xffffffffu, hw, o);
+        rank += t > hw; same |= t == hw;
+      }
+      if (__any_sync(0xffffffffu, same && i < n)) {
+        rank = 0;
+#pragma unroll 1
+        for (int o = 1; o < 16; ++o) {
+          const unsigned long long t = __shfl_xor_sync(0xffffffffu, key, o);
+          rank += t > key || (t == key && (lane ^ o) < lane);
+        }
+      }
+      const unsigned bits = __ballot_sync(0xffffffffu, i < n && rank < kq);
+      if (lane == 0) loc[b0 >> 5] = bits;
+    }
+    return;
+  }
+  // A warp to a block of 32 to 256: descends the bits of the kq-th largest score, counting with ballots; it may stop
+  // where exactly kq scores lie at or above the candidate.
+  for (int b0 = w * blk; b0 < n; b0 += nw * blk) {
+    const int per = blk / 32, have = min(blk, n - b0);
+    unsigned long long key[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int i = j * 32 + lane;
+      key[j] = j < per && i < have ? max(key_of(aS[b0 + i]), key_of(aL[b0 + i])) + 1 : 0ull;        // 0: no candidate
+    }
+    auto count = [&](unsigned long long t) {
+      int c = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) if (j < per) c += __popc(__ballot_sync(0xffffffffu, key[j] >= t));
+      return c;
+    };
+    unsigned long long thr = 1ull;                        // every candidate
+    bool exact = have <= kq;
+    if (!exact) {
+      thr = 0ull;
+      unsigned top = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) top = max(top, (unsigned)(key[j] >> 32));
+      top = __reduce_max_sync(0xffffffffu, top);
+      for (int bit = top ? 63 - __clz((int)top) : 31; bit >= 0 && !exact; --bit) {
+        const unsigned long long t = thr | (1ull << bit);
+        const int c = count(t);
+        if (c >= kq) { thr = t; exact = c == kq; }
+      }
+    }
+    int spare = exact ? 0 : kq - count(thr + 1);           // scores equal to the threshold that still fit, lowest slots first
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j < per) {
+        const unsigned above = __ballot_sync(0xffffffffu, exact ? key[j] >= thr : key[j] > thr);
+        const unsigned eq = exact ? 0u : __ballot_sync(0xffffffffu, key[j] == thr);
+        const bool pick = (above >> lane & 1u) || ((eq >> lane & 1u) && __popc(eq & ((1u << lane) - 1u)) < spare);
+        spare -= min(spare, __popc(eq));
+        const unsigned bits = __ballot_sync(0xffffffffu, pick);
+        if (lane == 0 && b0 + j * 32 < n) loc[(b0 >> 5) + j] = bits;
+      }
+    }
+  }
+}
+
+// Selection of one boundary unit over its scores a^S, a^L (n candidates), all tasks side by side:
+//   task 0, 1   warps 0-1, 2-3: K^S, K^L (Eq. 7): smallest k such that the k largest scores sum to at least p
+//   task 2      warps 4-7: the `ne` lowest of max(a^S, a^L) outside the block-local quota (Eq. 10; score asc, slot desc)
+// `tasks` is the set to run (bits); a single task gets all warps.  The descent goes level by level with block barriers, so
+// the tasks stay in step.
+// What bounds it: the latency of a level (members counted with shared-memory atomics, a scan by one warp); two or three
+// levels for a thousand candidates.  Behind the attention kernel of 36 layers x 256 residents (4608 units) the selection
+// takes 330 us, with a block per task and 4096-bin histograms it took 480; on 32 units of 20 000 candidates, groups of 8, 560 us
+// against 1300 (scores in the pool's scratch: their loads are batched).
+__device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, const double* aS, const double* aL, int n, int tasks,
+                                         int ne, int kq, int* Kout, int* acc, int* evout) {
+  SelMisc& m = *S.m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool alone = (tasks & (tasks - 1)) == 0;
+  const int task = alone ? tasks >> 1 : warp < 2 ? 0 : (warp < 4 ? 1 : 2);
+  const int T = alone ? SEL_T : task == 2 ? 128 : 64;                             // threads of the task, and this one's index
+  const int gt = alone ? tid : task == 2 ? tid - 128 : tid & 63;
+  const double* a = task == 1 ? aL : aS;
+  const bool lead = gt < 32;                                                      // the task's first warp
+  bool run = (tasks >> task) & 1;
+  unsigned* bcnt = m.bins[task][0]; unsigned* blo = m.bins[task][1]; unsigned* bhi = m.bins[task][2];
+  for (int i = tid; i < 3 * 3 * BIN_STRIDE; i += SEL_T) (&m.bins[0][0][0])[i] = 0;
+  if (tid < 4) m.cnt[tid] = 0;
+  __syncthreads();                                         // the scores are there
+  if (tasks & 4) {
+    if (kq > 0) mark_local(aS, aL, n, p.blk, kq, S.loc, warp, SEL_NW);
+    else for (int i = tid; i < (n + 31) / 32; i += SEL_T) S.loc[i] = 0;
+  }
+  // (non-negative doubles order as their bit patterns do)
+  auto key2 = [&](int i) { return max(key_of(aS[i]), key_of(aL[i])); };
+  auto eligible = [&](int i) { return !((S.loc[i >> 5] >> (i & 31)) & 1u); };
+  // keys agree above bit `shift + 8`
+  const unsigned h0 = m.rng[task][0], h1 = m.rng[task][1];
+  int shift = h0 == h1 ? 24 : max(0, 32 + (31 - __clz((int)(h0 ^ h1))) - 7);
+  int width = 8;
+  unsigned long long prefix = ((unsigned long long)h1 << 32) >> (shift + 8);
+  unsigned before = 0;                                     // members before the crossing bin (above it; task 2: below it)
+  unsigned long long mass = 0;
+  unsigned in_bin = 0;
+  int K = -1;
+  bool ties = false, whole = false;
+  __syncthreads();
+  const bool mine = run;
+  for (;;) {
+    // four at a time: their loads, then their adds, in flight together
+    const unsigned mask = (1u << width) - 1u;
+    if (run && task != 2) {
+      for (int i0 = gt; i0 < n; i0 += 4 * T) {
+        unsigned long long f[4]; bool on[4]; int b[4]; unsigned old[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int i = i0 + e * T;
+          const double v = a[i < n ? i : gt];
+          const unsigned long long k = key_of(v) >> shift;
+          on[e] = i < n && (k >> width) == prefix;
+          b[e] = BIDX((int)((unsigned)k & mask));
+          f[e] = to_fix(v);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          old[e] = 0u;
+          if (on[e]) { atomicAdd(&bcnt[b[e]], 1u); old[e] = atomicAdd(&blo[b[e]], (unsigned)f[e]); }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {                      // the carry travels with the high word's add
+          const unsigned up = (unsigned)(f[e] >> 32) + (old[e] + (unsigned)f[e] < old[e] ? 1u : 0u);
+          if (on[e] && up) atomicAdd(&bhi[b[e]], up);
+        }
+      }
+    } else if (run) {
+      for (int i0 = gt; i0 < n; i0 += 4 * T) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int i = i0 + e * T, j = i < n ? i : gt;
+          const unsigned long long k = key2(j) >> shift;
+          if (i < n && (k >> width) == prefix && eligible(j)) atomicAdd(&bcnt[BIDX((int)((unsigned)k & mask))], 1u);
+        }
+      }
+    }
+    __syncthreads();
+    if (run && lead) {                                     // lane owns bins [8 lane, 8 lane + 8)
+      unsigned c8[8]; unsigned long long m8[8];
+      unsigned c = 0; unsigned long long s = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int b = lane * 9 + j;                        // BIDX(8 lane + j)
+        c8[j] = bcnt[b];
+        m8[j] = task != 2 ? ((unsigned long long)bhi[b] << 32) + blo[b] : 0ull;
+        c += c8[j]; s += m8[j];
+      }
+      unsigned ic = c; unsigned long long is = s;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        if (task != 2) {                                   // largest scores first
+          const unsigned tc = __shfl_down_sync(0xffffffffu, ic, o);
+          const unsigned long long ts = __shfl_down_sync(0xffffffffu, is, o);
+          if (lane + o < 32) { ic += tc; is += ts; }
+        } else {                                           // lowest scores first
+          const unsigned tc = __shfl_up_sync(0xffffffffu, ic, o);
+          if (lane >= o) ic += tc;
+        }
+      }
+      unsigned rc = before + ic - c; unsigned long long rs = mass + is - s;
+      bool hit = false;
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        const int j = task != 2 ? 7 - jj : jj;
+        const bool here = task != 2 ? rs < p.p_fix && rs + m8[j] >= p.p_fix : rc < (unsigned)ne && rc + c8[j] >= (unsigned)ne;
+        if (here) { m.res[task][0] = lane * 8 + j; m.res[task][1] = rc; m.res[task][2] = (long long)rs; m.res[task][3] = c8[j]; hit = true; }
+        rc += c8[j]; rs += m8[j];
+      }
+      if (!__any_sync(0xffffffffu, hit) && lane == 0) m.res[task][0] = -1;
+    }
+    __syncthreads();
+    if (run) {
+      const int bin = (int)m.res[task][0];
+      if (bin < 0) {
+        // rounding kept the total below p: everything.  (Task 2 has more than `ne` eligible candidates by the quota's size.)
+        K = n; run = false;
+        if (task == 2) {                                     // (scores that are not numbers: some list within bounds, and the error bit)
+          for (int t = gt; t < ne; t += T) m.ev[t] = t;
+          if (gt == 0) atomicOr(p.err, GP_E_BOUNDS);
+        }
+      } else {
+        before = (unsigned)m.res[task][1]; mass = (unsigned long long)m.res[task][2]; in_bin = (unsigned)m.res[task][3];
+        prefix = (prefix << width) | (unsigned long long)bin;
+        if (task != 2 && in_bin == 1) { K = (int)before + 1; run = false; }
+        else if (task == 2 && before + in_bin == (unsigned)ne) { whole = true; run = false; }       // the bin goes as a whole
+        else if (in_bin <= 32) run = false;
+        else if (shift == 0) { ties = true; run = false; }              // copies of one value
+        else { width = min(8, shift); shift -= width; }
+        for (int i = gt; i < BIN_STRIDE; i += T) { bcnt[i] = 0; blo[i] = 0; bhi[i] = 0; }
+      }
+    }
+    if (!__syncthreads_or(run)) break;
+  }
+  // ---- the members of the crossing bin, one by one (keys >> shift == prefix) -----------------------------------------
+  const bool listed = mine && K < 0 && !ties && !whole;
+  if (mine && K < 0) {
+    if (task != 2) {
+      if (listed) {
+#pragma unroll 4
+        for (int i = gt; i < n; i += T) {
+          const double v = a[i];
+          if ((key_of(v) >> shift) == prefix) {
+            const int at = atomicAdd(&m.cnt[1 + task], 1);
+            m.list[task][at] = key_of(v); m.list_fix[task][at] = to_fix(v);
+          }
+        }
+      }
+    } else {
+#pragma unroll 4
+      for (int i = gt; i < n; i += T) {
+        const unsigned long long full = key2(i), k = full >> shift;
+        if (k <= prefix && eligible(i)) {
+          if (k < prefix || whole) { const int at = atomicAdd(&m.cnt[0], 1); if (at < ne) m.ev[at] = i; }
+          else if (listed) { const int at = atomicAdd(&m.cnt[3], 1); m.list[2][at] = full; m.list_slot[at] = i; }
+        }
+      }
     }
   }
   __syncthreads();
-  // ---- global cut: the b lowest of the rest are evicted (score asc, slot desc) --------------------------------
-  if (!uniform || !evict_fast(a, nC, S.loc, S.H, S.wc, S.s_res, S.flist, S.flist_slot, &S.s_i[6], S.ev, (unsigned)ne))
-    evict_general(p, a, nC, S.loc, S.hcnt, S.wc, S.s_res, S.s_i, S.ev, (unsigned)ne);
+  if (mine && lead) {
+    if (task != 2) {
+      if (listed) {
+        // every member's place in the descending order and the mass up to and including it
+        const unsigned long long v = m.list[task][lane];
+        int rank = 0;
+        unsigned long long inc = 0;
+#pragma unroll 4
+        for (int j = 0; j < (int)in_bin; ++j) {
+          const unsigned long long t = m.list[task][j];
+          const bool first = t > v || (t == v && j <= lane);
+          rank += first;
+          inc += first ? m.list_fix[task][j] : 0ull;
+        }
+        K = (int)before + (int)__reduce_min_sync(0xffffffffu, lane < (int)in_bin && mass + inc >= p.p_fix ? (unsigned)rank : in_bin);
+      } else if (ties) {
+        const unsigned long long f = to_fix(__longlong_as_double((long long)prefix));
+        unsigned long long j = f ? (p.p_fix - mass + f - 1) / f : 1ull;
+        if (j < 1) j = 1;
+        if (j > in_bin) j = in_bin;
+        K = (int)before + (int)j;
+      }
+      if (lane == 0) {
+        Kout[task] = K;
+        atomicAdd(acc + task, K);                          // Eq. 8 needs only the sums over layers and heads
+      }
+    } else if (listed) {                                   // the lowest scores of the bin, later slots first among equals
+      const unsigned long long v = m.list[2][lane];
+      const int slot = m.list_slot[lane];
+      int rank = 0;
+#pragma unroll 4
+      for (int j = 0; j < (int)in_bin; ++j) {
+        const unsigned long long t = m.list[2][j];
+        rank += t < v || (t == v && m.list_slot[j] > slot);
+      }
+      if (lane < (int)in_bin && rank < ne - (int)before) m.ev[before + rank] = slot;
+    } else if (ties && lane == 0) {                        // rare: older (lower) slots win ties
+      int at = (int)before;
+      for (int i = n - 1; i >= 0 && at < ne; --i)
+        if (key2(i) == prefix && eligible(i)) m.ev[at++] = i;
+    }
+  }
+  if (!(tasks & 4)) return;
   __syncthreads();
   for (int t = tid; t < ne; t += SEL_T) {                    // the evicted slots in ascending order, by rank
-    const int mine = S.ev[t];
+    const int slot = m.ev[t];
     int rank = 0;
-    for (int j = 0; j < ne; ++j) rank += (S.ev[j] < mine);
-    evout[rank] = mine;
+#pragma unroll 16
+    for (int j = 0; j < ne; ++j) rank += (m.ev[j] < slot);           // (ne is a multiple of 16)
+    evout[rank] = slot;
+  }
+}
+
+// Attention outputs of requests that were split over several work items: merges the items' partial results
+// (running maximum in the log2 domain, sum of exponentials, unnormalised output) into the output row.  A merge is a few
+// dependent round trips to the L2 and next to no work, so a query head's row is one warp's: the calling CTA takes rows
+// first, first + stride, ... of all CTAs' warps.  (A merge of a whole head group per thread block: 36 layers x 256 residents,
+// 12 000 merges per step, 80 us behind the selection.)
+template <int PER>     // head_dim / 32
+__device__ __forceinline__ void merge_rows(const GpDev& p, int n_req, float* __restrict__ out, int n_mc, int n_rc,
+                                           int first_block, int blocks, int lh0, int lh_n) {
+  constexpr int D = PER * 32;
+  const int G = p.G;
+  const int PSTRIDE = G * (D + 2);
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const long long rows = (long long)n_mc * lh_n * G;
+  for (long long mi = (long long)first_block * nw + (threadIdx.x >> 5); mi < rows; mi += (long long)blocks * nw) {
+    const int g = (int)(mi % G);
+    const long long u = mi / G;
+    const int4 mc = p.mc_list[u / lh_n];
+    const int lh = lh0 + (int)(u % lh_n), l = lh / p.Hkv, h = lh % p.Hkv;       // units [lh0, lh0 + lh_n)
+    const int bi = mc.x, nch = mc.z;
+    const float* pg = p.partials + ((size_t)lh * n_rc + mc.y) * PSTRIDE + g * (D + 2);
+    float* orow = out + (((size_t)l * n_req + bi) * p.Hq + h * G + g) * D;
+    float M = -INFINITY, ls = 0.f, acc[PER];
+#pragma unroll
+    for (int e = 0; e < PER; ++e) acc[e] = 0.f;
+    for (int c0 = 0; c0 < nch; c0 += 4) {                 // four items' values in flight together
+      float m[4], lv[4], vv[4][PER];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float* pc = pg + (size_t)(c0 + k) * PSTRIDE;
+        const bool on = c0 + k < nch;
+        m[k] = on ? __ldcg(pc + D) : -INFINITY;
+        lv[k] = on ? __ldcg(pc + D + 1) : 0.f;
+#pragma unroll
+        for (int e = 0; e < PER; ++e) vv[k][e] = on ? __ldcg(pc + lane + 32 * e) : 0.f;
+      }
+      const float Mn = fmaxf(fmaxf(M, fmaxf(m[0], m[1])), fmaxf(m[2], m[3]));
+      const float sc = exp2f(M - Mn);
+      ls *= sc;
+#pragma unroll
+      for (int e = 0; e < PER; ++e) acc[e] *= sc;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float w = exp2f(m[k] - Mn);
+        ls += w * lv[k];
+#pragma unroll
+        for (int e = 0; e < PER; ++e) acc[e] += w * vv[k][e];
+      }
+      M = Mn;
+    }
+#pragma unroll
+    for (int e = 0; e < PER; ++e) orow[lane + 32 * e] = acc[e] / ls;
+  }
+}
+__device__ __noinline__ void merge_partials(const GpDev& p, int n_req, float* __restrict__ out, int n_mc, int n_rc,
+                                            int first_block, int blocks, int lh0, int lh_n) {
+  if (p.d == 128) merge_rows<4>(p, n_req, out, n_mc, n_rc, first_block, blocks, lh0, lh_n);
+  else merge_rows<2>(p, n_req, out, n_mc, n_rc, first_block, blocks, lh0, lh_n);
+}
+
+// ------------------------------------------------------------------------------------------------------
+// working sets + speculative eviction lists of a unit, one CTA; the last CTA decides
+// ------------------------------------------------------------------------------------------------------
+// Unit u = (boundary request bidx, layer and KV head lh): K^S and K^L go to Kx and, summed, to bnd_acc (Eq. 8), the `b`
+// slots a compression would evict to evict, the 2b of a Shrink to evict2.  `want`: the tasks of unit_select, 7 for the whole
+// unit; with few units a thread block takes one of its three tasks.
+template <int GG>      // query heads per KV head
+__device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int bidx, int lh, const int4 inf, const int4 inf2, int want) {
+  SelMisc& m = *S.m;
+  const int tid = threadIdx.x;
+  constexpr int G = GG;
+  const int LH = p.L * p.Hkv;
+  const int r = inf.y, Pr = inf.z;
+  const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
+  const size_t u = (size_t)bidx * LH + lh;
+  int* Kout = p.Kx + ((size_t)r * LH + lh) * 2;
+  int* acc = p.bnd_acc + 4 * bidx;
+  // two supports (they coincide when the page is 16 tokens): the working sets of Eq. 7 leave out the newest page
+  // of the method, the eviction candidates of Eq. 10 only the protected window, the newest 16-token tile
+  const int nt_d = Pr - p.sub, nt_e = Pr - 1;
+  if (nt_d == 0) {                           // one page of the method: nothing to estimate from, nothing to evict
+    if (tid < 2 && ((want >> tid) & 1)) Kout[tid] = 0;
+    return;
+  }
+  const size_t view_stride = (size_t)p.z_stride * G;
+  const double* z = p.zbuf + (size_t)lh * 2 * view_stride + (size_t)off * G;       // [2 views][n][G] exp(logit - page max)
+  const double* zs = p.zstat + ((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + off / GP_PAGE) * 2 * G * 2;
+  // the scores: in shared memory, or, for candidate sets too large for it, in the pool's scratch (three regions: a whole
+  // unit uses two, one per view, a single job the one of its number).  A job that lists evictions keeps only
+  // max(a^S, a^L), in the place of both.
+  const bool single = want != 7;
+  const bool small = nt_e * GP_PAGE <= (single ? 2 * S.n_cap : S.n_cap);
+  double* aS = small ? S.sS : p.scores + ((size_t)(single ? want >> 1 : 0) * LH + lh) * p.max_boundary_tokens + off;
+  double* aL = single ? aS : small ? S.sL : aS + (size_t)LH * p.max_boundary_tokens;
+  const int views = want == 1 ? 1 : want == 2 ? 2 : 3;
+  const bool one_support = p.sub == 1;
+  const bool entropy = p.metric == GP_METRIC_ENTROPY;
+  for (int pass = 0; pass < (one_support ? 1 : 2); ++pass) {
+    const int ntile = pass == 0 ? nt_d : nt_e, n = ntile * GP_PAGE;
+    int tasks = want & (one_support ? 7 : pass == 0 ? 3 : 4);
+    if (!tasks) continue;
+    __syncthreads();                                       // the unit or pass before is done with the shared arrays
+    if (tid < 3) { m.rng[tid][0] = 0xffffffffu; m.rng[tid][1] = 0u; }
+    unit_softmax<GG>(S, z, view_stride, zs, aS, aL, ntile, views);      // (its barriers order rng before the first use)
+    if (entropy && (tasks & 3)) {
+      __syncthreads();                                     // the scores are there
+      // the ablation's other metric: H = -sum a ln a of the view, summed in a fixed order (per thread over its
+      // strided candidates, then a fixed tree), so that the same input gives the same bits on every run
+      double* Hout = p.Hx + ((size_t)r * LH + lh) * 2;
+      for (int view = 0; view < 2; ++view) {
+        if (!((tasks >> view) & 1)) continue;
+        const double* a = view ? aL : aS;
+        double hsum = 0.0;
+        for (int i = tid; i < n; i += SEL_T) { const double v = a[i]; if (v > 0.0) hsum -= v * log(v); }
+#pragma unroll
+        for (int o2 = 16; o2 > 0; o2 >>= 1) hsum += __shfl_xor_sync(0xffffffffu, hsum, o2);
+        if ((tid & 31) == 0) m.red[tid >> 5] = hsum;
+        __syncthreads();
+        if (tid == 0) {
+          double tot = 0.0;
+          for (int w = 0; w < SEL_NW; ++w) tot += m.red[w];
+          Kout[view] = 0;
+          Hout[view] = tot;
+        }
+        __syncthreads();
+      }
+      tasks &= 4;
+    }
+    // the lists: b slots of a compression, then, where this boundary can be a Shrink, its 2b
+    const bool shrink = p.policy == GP_POLICY_SHRINK && (tasks & 4) && Pr - p.sub >= p.min_pages_after_shrink;
+    const int nblk = (n + p.blk - 1) / p.blk;
+#pragma unroll 1
+    for (int list = 0; list < (shrink ? 2 : 1); ++list) {
+      const int ne = (list + 1) * p.blk;
+      if (list || tasks)
+        unit_select(p, S, aS, aL, n, list ? 4 : tasks, ne, min(p.k_loc, (n - ne) / nblk), Kout, acc,
+                    list ? p.evict2 + u * ne : p.evict + u * ne);
+    }
   }
 }
 
@@ -974,7 +875,28 @@ __device__ __noinline__ void publish_shard_sums(const GpDev& p, int n_bnd) {
   }
 }
 
-template <bool SHR>      // SHR: the pool runs the Shrink policy (a fourth job per unit)
+// Thread blocks per unit: one that runs the three tasks side by side over one softmax pass, or, while the grid has
+// three for every unit, one per task, each with all its warps.  Measured on units of 730 candidates, groups of 4: a task's
+// block 6.6 us, a whole unit's 10.7 us (32 units on 296 blocks take the former); on 4608 units of 640 candidates the three
+// passes over the logits that blocks per task take cost 150 us per step more.
+__device__ __forceinline__ int jobs_per_unit(long long units, int grid) { return units * 3 <= grid ? 3 : 1; }
+
+// pages of C that other requests share: each needs a copy-on-write target if boundary request e compresses
+__device__ __forceinline__ void count_shared(const GpDev& p, int e) {
+  if (threadIdx.x >= 32) return;
+  const int4 inf = p.bnd_info[2 * e];
+  const int* table = p.page_table + (size_t)inf.y * p.cap;
+  int ksh = 0;
+#pragma unroll 4
+  for (int j = threadIdx.x; j < inf.z - p.sub; j += 32) ksh += (p.refcount[table[j]] > 1);
+#pragma unroll
+  for (int o2 = 16; o2 > 0; o2 >>= 1) ksh += __shfl_xor_sync(0xffffffffu, ksh, o2);
+  if (threadIdx.x == 0) p.bnd_acc[4 * e + 2] = ksh;
+}
+
+// The selection as a kernel of its own.  Two thread blocks to an SM at 128 registers; three at 80 spill and are slower
+// (20 000 cycles per unit become 36 000).
+template <int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions,
                float* __restrict__ out, int serial, int decide) {
@@ -983,32 +905,30 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // sums of all parts are added up
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((256u - (smem_u32(smem_raw) & 255u)) & 255u);
-  SelSmem S = sel_smem_at(smem);
-  int* s_i = S.s_i;
-  // the decision scratch aliases the score staging area: it is used after the last item only
+  const SelSmem S = sel_smem_at(smem, p.cap);
+  int* s_i = S.m->s_i;
 
   const int tid = threadIdx.x;
   const int LH = p.L * p.Hkv;
-  const int G = p.G, G2 = 2 * p.G;
-  constexpr int NT = SHR ? 4 : 3;                           // jobs per unit: K^S, K^L, eviction list(s)
   // What the plan kernel wrote (counts, boundary records) is read before the wait for the attention kernel: the
   // plan kernel had completed before any CTA of the attention kernel let this grid be scheduled, and the
   // attention kernel does not touch these words; the loads go to the L2 (an L1 line could date from the step
-  // before).  The first item's record is fetched before the number of items is known (same round trip); slots
+  // before).  The first unit's record is fetched before the number of units is known (same round trip); slots
   // of bnd_info past the count hold stale but readable data that is then not used.
   int4 inf_first = make_int4(0, 0, 0, 0), inf2_first = inf_first;
   {
-    const int b0 = (int)(blockIdx.x / (NT * LH));
+    const int b0 = (int)(blockIdx.x / LH);               // (one thread block per unit; with three they are fetched again)
     if (b0 < p.M) { inf_first = __ldcg(p.bnd_info + 2 * b0); inf2_first = __ldcg(p.bnd_info + 2 * b0 + 1); }
   }
   const int n_bnd = __ldcg(p.hdr + HDR_N_BND);
   const int n_mc = out ? __ldcg(p.hdr + HDR_N_MC) : 0, n_rc = __ldcg(p.hdr + HDR_N_RC);   // out == null: already merged layer by layer
-  const long long items = (long long)n_bnd * LH * NT;
+  const int NJ = jobs_per_unit((long long)n_bnd * LH, gridDim.x);
+  const long long items = (long long)n_bnd * LH * NJ;
   gp_pdl_wait();
   gp_pdl_launch_dependents();
 
-  // CTAs without a job merge the split requests' attention partials while the others work; when fewer than a
-  // quarter of the CTAs are idle, everybody merges after the jobs instead
+  // CTAs without a unit merge the split requests' attention partials while the others work; when fewer than a
+  // quarter of the CTAs are idle, everybody merges after the units instead
   const long long n_busy = items + n_bnd < (long long)gridDim.x ? items + n_bnd : (long long)gridDim.x;
   const int n_idle = (int)gridDim.x - (int)n_busy;
   const bool idle_merge = n_idle * 4 >= (int)gridDim.x;
@@ -1016,49 +936,12 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     merge_partials(p, n_req, out, n_mc, n_rc, (int)blockIdx.x - (int)n_busy, n_idle, 0, LH);
 
   for (long long item = blockIdx.x; item < items + n_bnd; item += gridDim.x) {
-    if (item >= items) {
-      // pages of C that other requests share: each needs a copy-on-write target if this request compresses
-      const int e = (int)(item - items);
-      if (tid < 32) {
-        const int4 inf = p.bnd_info[2 * e];
-        const int* table = p.page_table + (size_t)inf.y * p.cap;
-        int ksh = 0;
-        for (int j = tid; j < inf.z - p.sub; j += 32) ksh += (p.refcount[table[j]] > 1);
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) ksh += __shfl_xor_sync(0xffffffffu, ksh, o2);
-        if (tid == 0) p.bnd_acc[4 * e + 2] = ksh;
-      }
-      continue;
-    }
-    const long long u = item / NT;
-    const int job = (int)(item % NT);               // 0: K^S, 1: K^L, 2: eviction list, 3: a Shrink's eviction list
-    const int task = job < 2 ? job : 2;
-    const int ne = (SHR && job == 3) ? 2 * p.blk : p.blk;        // slots a compression (a Shrink) frees
-    const int bidx = (int)(u / LH), lh = (int)(u % LH);
-    const int l = lh / p.Hkv, h = lh % p.Hkv;
-    const bool is_first = item == (long long)blockIdx.x;
-    const int4 inf = is_first ? inf_first : p.bnd_info[2 * bidx];          // {slot in the batch, request, P}
-    const int4 inf2 = is_first ? inf2_first : p.bnd_info[2 * bidx + 1];    // {offset into the logit scratch}
-    const int r = inf.y, Pr = inf.z;
-    const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
-    // two supports (they coincide when the page is 16 tokens): the working sets of Eq. 7 leave out the newest page
-    // of the method, the eviction candidates of Eq. 10 only the protected window, the newest 16-token tile
-    const int nC_d = (Pr - p.sub) * GP_PAGE, nC_e = (Pr - 1) * GP_PAGE;
-    const int nC = task < 2 ? nC_d : nC_e;
-    int* Kout = p.Kx + (((size_t)r * p.L + l) * p.Hkv + h) * 2;
-    int* evout = (SHR && job == 3) ? p.evict2 + (size_t)u * 2 * p.blk : p.evict + (size_t)u * p.blk;
-    __syncthreads();
-    if (nC_d == 0) {                         // one page of the method: nothing to estimate from, nothing to evict
-      if (tid == 0 && task < 2) Kout[task] = 0;
-      continue;
-    }
-    if (SHR && job == 3 && Pr - p.sub < p.min_pages_after_shrink) continue;      // this boundary cannot be a Shrink
-    const size_t view_stride = (size_t)p.z_stride * G;
-    const double* z = p.zbuf + (size_t)lh * 2 * view_stride + (size_t)off * G;   // [2 views][nC][G] exp(logit - page max)
-    const double* zs = p.zstat + ((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + off / GP_PAGE) * G2 * 2;
-    double* a = nC <= SEL_CAP ? S.sbuf : p.scores + ((size_t)job * LH + lh) * p.max_boundary_tokens + off;
-    sel_job(p, S, z, view_stride, zs, a, nC, task, ne, Kout, p.bnd_acc + 4 * bidx, evout,
-              p.Hx + (((size_t)r * p.L + l) * p.Hkv + h) * 2);
+    if (item >= items) { count_shared(p, (int)(item - items)); continue; }
+    const int u = (int)(item / NJ), bidx = u / LH, lh = u % LH;
+    const bool is_first = NJ == 1 && item == (long long)blockIdx.x;
+    sel_unit<GG>(p, S, bidx, lh, is_first ? inf_first : p.bnd_info[2 * bidx],          // {slot in the batch, request, P}
+                  is_first ? inf2_first : p.bnd_info[2 * bidx + 1],                     // {offset into the logit scratch}
+                  NJ == 1 ? 7 : 1 << (int)(item % NJ));
   }
 
   // ---- the last CTA takes the decisions ----------------------------------------------------------------------
@@ -1073,7 +956,7 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   if (s_i[2]) {
     __threadfence();
     if (!out) advance_counters(p, n_rc);
-    if (decide) decide_and_allocate(p, req_ids, n_req, n_bnd, actions, reinterpret_cast<int*>(S.sbuf), serial);
+    if (decide) decide_and_allocate(p, req_ids, n_req, n_bnd, actions, reinterpret_cast<int*>(S.loc), serial);
     else publish_shard_sums(p, n_bnd);
   }
 
@@ -1123,7 +1006,7 @@ __device__ __forceinline__ CmpSmem cmp_smem_at(uint8_t* base) {       // base: 1
 // over: one unit per ticket, its chunks in ascending order by the same thread block (a chunk's destinations lie
 // below the next chunk's sources, and program order puts every chunk's reads before the next chunk's writes), which
 // saves the ticket, the eviction list and the waits per chunk and skips the chunks below the first evicted slot.
-template <int D, bool SHR>
+template <int D>
 __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, int serial) {
   constexpr int CH = D / 8;
   constexpr int ROW_BYTES = D * 2;
@@ -1183,7 +1066,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     const int n_src = Pr * GP_PAGE;
     // second round trip: the eviction list and, for every source slot of the chunk, its page and its
     // copy-on-write target
-    const bool shrink = SHR && (inf.z & CMP_SHRINK) != 0;
+    const bool shrink = (inf.z & CMP_SHRINK) != 0;
     const int e_bnd = inf.z & (CMP_SHRINK - 1);
     const int ne = shrink ? 2 * p.blk : p.blk;             // slots freed: one page of the method, two at a Shrink
     for (int t = tid; t < ne; t += CT)
@@ -1336,7 +1219,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
         if (lane == 0 && mask) *reinterpret_cast<volatile int*>(p.free_top) = base + __popc(mask);
         __syncwarp();
       }
-      if (SHR && (s_info[ci].z & CMP_SHRINK) && lane == 0) {      // the page of the method the request no longer owns
+      if ((s_info[ci].z & CMP_SHRINK) && lane == 0) {      // the page of the method the request no longer owns
         for (int t = p.sub; t >= 1; --t) {
           const int last = table[Pr - t];
           if (atomicSub(&p.refcount[last], 1) == 1) {
@@ -1352,13 +1235,13 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
 }
 
 
-template <int D, bool SHR>
+template <int D>
 __global__ void __launch_bounds__(CT, 4)
 gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int serial) {
   __shared__ __align__(16) uint8_t cmp_raw[CMP_SMEM_BYTES];
   gp_pdl_wait();
   gp_pdl_launch_dependents();
-  compact_body<D, SHR>(p, cmp_smem_at(cmp_raw), serial);
+  compact_body<D>(p, cmp_smem_at(cmp_raw), serial);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -1373,7 +1256,7 @@ gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_i
 // ends after both, and the plan of step t + 2, its programmatic dependent, finds the pages and counters of the
 // requests that sat step t + 1 out in their final state.  `p`: the view of step t (its scratch set, the copy of
 // the counters its decisions go to); `pa`: the view of step t + 1 (for the merge).
-template <int D, bool SHR>
+template <int D, int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev pa, int n_req_merge, float* __restrict__ out_merge,
                 int serial, int has_chain, const int* __restrict__ req_ids, int* __restrict__ actions,
@@ -1393,51 +1276,20 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
   const bool same_step = !p.async;
   if (!same_step) gp_pdl_launch_dependents();
   if (has_chain) {
-    SelSmem S = sel_smem_at(smem);
-    int* s_i = S.s_i;
-    const int G = p.G, G2 = 2 * p.G;
-    constexpr int NT = SHR ? 4 : 3;
+    const SelSmem S = sel_smem_at(smem, p.cap);
+    int* s_i = S.m->s_i;
     const int n_bnd = __ldcg(p.hdr + HDR_N_BND);
-    const long long items = (long long)n_bnd * LH * NT;
+    const int NJ = jobs_per_unit((long long)n_bnd * LH, gridDim.x);
+    const long long items = (long long)n_bnd * LH * NJ;
     for (long long item = blockIdx.x; item < items + n_bnd; item += gridDim.x) {
-      if (item >= items) {
-        const int e = (int)(item - items);
-        if (tid < 32) {
-          const int4 inf = p.bnd_info[2 * e];
-          const int* table = p.page_table + (size_t)inf.y * p.cap;
-          int ksh = 0;
-          for (int j = tid; j < inf.z - p.sub; j += 32) ksh += (p.refcount[table[j]] > 1);
-#pragma unroll
-          for (int o2 = 16; o2 > 0; o2 >>= 1) ksh += __shfl_xor_sync(0xffffffffu, ksh, o2);
-          if (tid == 0) p.bnd_acc[4 * e + 2] = ksh;
-        }
-        continue;
-      }
-      const long long u = item / NT;
-      const int job = (int)(item % NT);
-      const int task = job < 2 ? job : 2;
-      const int ne = (SHR && job == 3) ? 2 * p.blk : p.blk;        // slots a compression (a Shrink) frees
-      const int bidx = (int)(u / LH), lh = (int)(u % LH);
-      const int l = lh / p.Hkv, h = lh % p.Hkv;
+      if (item >= items) { count_shared(p, (int)(item - items)); continue; }
+      const int u = (int)(item / NJ), bidx = u / LH, lh = u % LH;
       const int4 inf = p.bnd_info[2 * bidx];
       const int4 inf2 = p.bnd_info[2 * bidx + 1];
-      const int r = inf.y, Pr = inf.z;
-      const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
-      // two supports (they coincide when the page is 16 tokens): the working sets of Eq. 7 leave out the newest page
-    // of the method, the eviction candidates of Eq. 10 only the protected window, the newest 16-token tile
-    const int nC_d = (Pr - p.sub) * GP_PAGE, nC_e = (Pr - 1) * GP_PAGE;
-    const int nC = task < 2 ? nC_d : nC_e;
-      int* Kout = p.Kx + (((size_t)r * p.L + l) * p.Hkv + h) * 2;
-      int* evout = (SHR && job == 3) ? p.evict2 + (size_t)u * 2 * p.blk : p.evict + (size_t)u * p.blk;
-      __syncthreads();
-      if (nC_d == 0) {                         // one page of the method: nothing to estimate from, nothing to evict
-        if (tid == 0 && task < 2) Kout[task] = 0;
-        continue;
-      }
-      if (SHR && job == 3 && Pr - p.sub < p.min_pages_after_shrink) continue;
-      if (same_step) {
+      if (same_step && inf.z > p.sub) {
         // every work item of the request reports once per consumer warp for this unit (bounded wait; the
         // attention kernel's thread blocks were all resident before this grid could be scheduled)
+        __syncthreads();
         if (tid == 0) {
           const volatile int* rdy = p.unit_ready + (size_t)bidx * LH + lh;
           unsigned it = 0;
@@ -1447,12 +1299,7 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
         }
         __syncthreads();
       }
-      const size_t view_stride = (size_t)p.z_stride * G;
-      const double* z = p.zbuf + (size_t)lh * 2 * view_stride + (size_t)off * G;
-      const double* zs = p.zstat + ((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + off / GP_PAGE) * G2 * 2;
-      double* a = nC <= SEL_CAP ? S.sbuf : p.scores + ((size_t)job * LH + lh) * p.max_boundary_tokens + off;
-      sel_job(p, S, z, view_stride, zs, a, nC, task, ne, Kout, p.bnd_acc + 4 * bidx, evout,
-              p.Hx + (((size_t)r * p.L + l) * p.Hkv + h) * 2);
+      sel_unit<GG>(p, S, bidx, lh, inf, inf2, NJ == 1 ? 7 : 1 << (int)(item % NJ));
     }
     // ---- the last CTA to finish its jobs takes the decisions and tells the others ------------------------------
     const int stamp = same_step ? p.hdr[HDR_STEP] : serial + 1;
@@ -1466,7 +1313,7 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
     __syncthreads();
     if (s_i[2]) {
       __threadfence();
-      decide_and_allocate(p, req_ids, n_req_merge, n_bnd, same_step ? actions : nullptr, reinterpret_cast<int*>(S.sbuf), serial);
+      decide_and_allocate(p, req_ids, n_req_merge, n_bnd, same_step ? actions : nullptr, reinterpret_cast<int*>(S.loc), serial);
       __syncthreads();
       if (tid == 0 && !(p.withhold & GP_WITHHOLD_DECIDED)) {      // (test support: see GP_WITHHOLD_DECIDED)
         __threadfence();
@@ -1493,7 +1340,7 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
       gp_pdl_launch_dependents();
     }
     // ---- compaction: its arrays take the place of the selection's -----------------------------------------------
-    compact_body<D, SHR>(p, cmp_smem_at(smem), serial);
+    compact_body<D>(p, cmp_smem_at(smem), serial);
   }
   if (same_step) return;
   gp_pdl_wait();              // the attention kernel beside which this grid ran has ended
@@ -1510,59 +1357,55 @@ gp_decide_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_id
 
 }  // namespace
 
-// the compaction kernel of a pool: head dimension, and whether the Shrink policy is on
+// the kernels of a pool: head dimension and query heads per KV head
 static auto compact_kernel_of(const GpDev& p) -> void (*)(const GpDev, const int*, int, int) {
-  const bool shr = p.policy == GP_POLICY_SHRINK;
-  if (p.d == 128) return shr ? gp_compact_kernel<128, true> : gp_compact_kernel<128, false>;
-  return shr ? gp_compact_kernel<64, true> : gp_compact_kernel<64, false>;
+  return p.d == 128 ? gp_compact_kernel<128> : gp_compact_kernel<64>;
 }
-
-// shared memory of the selection kernel for a per-request page cap (its bitmap of block-local picks has one bit
-// per candidate token)
-size_t gp_bsel_smem_for_cap(long long cap) {
-  return SelGeom::BUF_BYTES + SelGeom::H_BYTES + SelGeom::MISC_BYTES + ((size_t)cap * GP_PAGE / 32 + 2) * 4 + 512;
+typedef void (*SelKernel)(const GpDev, const int*, int, int*, float*, int, int);
+static SelKernel sel_kernel_of(const GpDev& p) {
+  return p.G == 1 ? gp_bsel_kernel<1> : p.G == 2 ? gp_bsel_kernel<2> : p.G == 4 ? gp_bsel_kernel<4> : gp_bsel_kernel<8>;
 }
-size_t gp_bsel_smem(const GpDev& p) { return gp_bsel_smem_for_cap(p.cap); }
+typedef void (*ChainKernel)(const GpDev, const GpDev, int, float*, int, int, const int*, int*, int*);
+template <int D> static ChainKernel chain_kernel_d(const GpDev& p) {
+  return p.G == 1 ? gp_chain_kernel<D, 1> : p.G == 2 ? gp_chain_kernel<D, 2> : p.G == 4 ? gp_chain_kernel<D, 4> : gp_chain_kernel<D, 8>;
+}
+static ChainKernel chain_kernel_of(const GpDev& p) { return p.d == 128 ? chain_kernel_d<128>(p) : chain_kernel_d<64>(p); }
 
-// one-time setup for a pool: opts the selection kernel into its shared memory and sizes both grids to
-// exactly one resident wave, so that no CTA waits for another to leave before it can start
-void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact) {
-  const size_t sel_sm = gp_bsel_smem(p);
-  const bool shr = p.policy == GP_POLICY_SHRINK;
-  auto sel = shr ? gp_bsel_kernel<true> : gp_bsel_kernel<false>;
-  cudaFuncSetAttribute(sel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_sm);
-  {                                                  // the kernel with the whole boundary chain: same shared memory
-    auto opt_in = [&](auto kern) { cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_sm); };
-    if (p.d == 128) { if (shr) opt_in(gp_chain_kernel<128, true>); else opt_in(gp_chain_kernel<128, false>); }
-    else { if (shr) opt_in(gp_chain_kernel<64, true>); else opt_in(gp_chain_kernel<64, false>); }
-  }
-  int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sel, SEL_T, sel_sm);
-  *grid_sel = num_sms * (occ > 0 ? occ : 1);
-  occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, compact_kernel_of(p), CT, 0);
-  *grid_compact = num_sms * (occ > 0 ? occ : 1);
+// shared memory of the selection for a per-request page cap
+static size_t gp_sel_smem(const GpDev& p) {
+  const size_t tail = sel_loc_bytes(p.cap) + 2 * (size_t)sel_n_cap(p.cap) * sizeof(double);
+  return (sizeof(SelMisc) + 15) / 16 * 16 + (tail > DECIDE_SMEM ? tail : DECIDE_SMEM) + 256;
+}
+static_assert((sizeof(SelMisc) + 15) / 16 * 16 + ((GP_MAX_TILES_PER_REQ / 2 + 2) * 4 + 15) / 16 * 16 + 2 * SEL_CAP * sizeof(double) + 256 <= GP_MAX_DYN_SMEM,
+              "the largest page cap fits");
+static_assert(CMP_SMEM_BYTES <= sizeof(SelMisc) + DECIDE_SMEM, "the compaction's arrays take the selection's place");
+
+// one-time setup for a pool: opts the selection kernels into their shared memory and sizes the grids to at most one
+// resident wave, so that no CTA waits for another to leave before it can start
+void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain) {
+  const size_t sel_sm = gp_sel_smem(p);
+  auto blocks = [&](auto kern, int threads, size_t smem, int most) {
+    if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
+    return num_sms * (occ > most ? most : occ > 0 ? occ : 1);
+  };
+  *grid_sel = blocks(sel_kernel_of(p), SEL_T, sel_sm, 32);
+  *grid_chain = blocks(chain_kernel_of(p), SEL_T, sel_sm, 2);
+  *grid_compact = blocks(compact_kernel_of(p), CT, 0, 32);
 }
 
 // asynchronous mode: the boundary chain of the step whose view is `p` (none when !has_chain), and afterwards the
 // merge of the split requests' partial outputs of the step whose view is `pa` (none when out_merge is null)
 void gp_launch_chain(const GpDev& p, const GpDev& pa, int n_req_merge, float* out_merge, int serial, int has_chain, int grid,
                      cudaStream_t s, bool pdl, const int* req_ids, int* actions, int* actions_copy) {
-  const size_t sm = gp_bsel_smem(p);
-  const bool shr = p.policy == GP_POLICY_SHRINK;
-  auto launch = [&](auto kern) {
-    gp_launch(kern, grid, SEL_T, sm, s, pdl, p, pa, n_req_merge, out_merge, serial, has_chain, req_ids, actions, actions_copy);
-  };
-  if (p.d == 128) { if (shr) launch(gp_chain_kernel<128, true>); else launch(gp_chain_kernel<128, false>); }
-  else { if (shr) launch(gp_chain_kernel<64, true>); else launch(gp_chain_kernel<64, false>); }
+  gp_launch(chain_kernel_of(p), grid, SEL_T, gp_sel_smem(p), s, pdl, p, pa, n_req_merge, out_merge, serial, has_chain, req_ids,
+            actions, actions_copy);
 }
 
 void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel, cudaStream_t s,
                            bool pdl, int serial) {
-  const size_t sel_sm = gp_bsel_smem(p);
-  const bool shr = p.policy == GP_POLICY_SHRINK;
-  gp_launch(shr ? gp_bsel_kernel<true> : gp_bsel_kernel<false>, grid_sel, SEL_T, sel_sm, s, pdl, p, req_ids, n_req, actions, out,
-            serial, 0);
+  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl, p, req_ids, n_req, actions, out, serial, 0);
 }
 
 // plain launches: what comes before them on the stream (the caller's reduction of the sums) is not this library's
@@ -1578,12 +1421,9 @@ void gp_launch_merge(const GpDev& p, int n_req, float* out, int lh0, int lh_n, i
 
 void gp_launch_boundary(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel,
                         int grid_compact, cudaStream_t s, cudaEvent_t ev, bool pdl, int serial) {
-  const size_t sel_sm = gp_bsel_smem(p);
-  const bool shr = p.policy == GP_POLICY_SHRINK;
   // asynchronous mode: the kernel before this one on its stream belongs to another step (an event wait lies in
   // between): plain launch; the compaction kernel follows as a programmatic dependent as usual
-  gp_launch(shr ? gp_bsel_kernel<true> : gp_bsel_kernel<false>, grid_sel, SEL_T, sel_sm, s, pdl && !p.async, p, req_ids,
-            n_req, actions, out, serial, 1);
+  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl && !p.async, p, req_ids, n_req, actions, out, serial, 1);
   if (ev) cudaEventRecord(ev, s);
   gp_launch(compact_kernel_of(p), grid_compact, CT, 0, s, pdl, p, req_ids, n_req, serial);
 }

@@ -21,6 +21,7 @@
                                // The method's page (gp_config.page_size, b = 16 ... 256 tokens: the unit in which capacity
                                // grows, blocks are formed and slots are freed) is `sub` of these, always taken together.
 #define GP_MAX_BLK 256         // largest page_size
+#define GP_MAX_TILES_PER_REQ 61773   // 16-token tiles a request may hold: the selection keeps a bit per candidate in shared memory
 #define GP_SPIN_LIMIT (1u << 21)
 #define GP_MAX_REQ 1024        // upper limit of max_requests (shared-memory arrays are sized by it)
 #define GP_MOVE_TOK 64         // source slots per compaction chunk
@@ -283,8 +284,7 @@ void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* a
 void gp_launch_decide_compact(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_compact, cudaStream_t s,
                               int serial);
 void gp_launch_merge(const GpDev& p, int n_req, float* out, int lh0, int lh_n, int grid, cudaStream_t s, bool pdl);
-void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact);
-size_t gp_bsel_smem_for_cap(long long cap);
+void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain);
 #define GP_MAX_DYN_SMEM (227 * 1024)   // opt-in shared memory per CTA on sm_100
 // boundary chain: probabilities + working sets + selection + decision, then compaction.
 // `ev`, when not null, is recorded between the two kernels.  `pdl`: launch with programmatic stream serialization.

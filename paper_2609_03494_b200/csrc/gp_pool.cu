@@ -30,6 +30,7 @@ struct gp_pool {
   size_t bytes;
   std::vector<uint8_t> live;      // host mirror of the slot free list
   int num_sms, attn_grid, sel_grid, compact_grid;
+  int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
   std::vector<uint8_t> step_layer_seen;             // layers gp_attn_layer has run in the open step
   // error bits set by the kernels (GP_E_*): one int of page-locked host memory that the device addresses directly,
@@ -100,7 +101,7 @@ bool valid_config(const gp_config* c) {
   const long long sub = c->page_size / GP_PAGE;
   if (c->max_requests < 1 || c->max_requests > GP_MAX_REQ) return false;
   if (c->max_pages_per_req < 1 || c->max_pages_per_req * sub > (1 << 20)) return false;
-  if (gp_bsel_smem_for_cap(c->max_pages_per_req * sub) > GP_MAX_DYN_SMEM) return false;   // about 61 000 tiles of 16 tokens
+  if (c->max_pages_per_req * sub > GP_MAX_TILES_PER_REQ) return false;
   if (c->n_pages < 1 || c->n_pages * sub > 0x7fffffffLL / GP_PAGE) return false;
   if (c->k_loc < 0 || c->k_loc > c->page_size) return false;
   if (c->max_batch_tokens < 0 || c->max_boundary_tokens < 0) return false;
@@ -899,7 +900,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.scores = reinterpret_cast<double*>(base + L.scores);
   d.counters = reinterpret_cast<long long*>(base + L.counters);
   gp_attention_setup(d);
-  gp_boundary_setup(d, pool->num_sms, &pool->sel_grid, &pool->compact_grid);
+  gp_boundary_setup(d, pool->num_sms, &pool->sel_grid, &pool->compact_grid, &pool->chain_grid_max);
   pool->dev_alt = d;
   pool->chain_pending = 0;
   pool->last_stream = nullptr;
@@ -928,7 +929,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   // compaction grid (36 layers x 256 residents: 4.8 ms against 5.2; 256 requests x 8 units: 0.49 against 0.52).
   const bool fused_auto = (long long)cfg->max_requests * cfg->n_layers * cfg->n_kv_heads <= 1024;
   if (!cfg->async_boundary && (cfg->overlap_slots == -2 || (cfg->overlap_slots == 0 && fused_auto))) {
-    pool->chain_grid_ov = pool->sel_grid;          // the whole grid, behind the attention kernel's
+    pool->chain_grid_ov = pool->chain_grid_max;    // the whole grid, behind the attention kernel's
   } else if (!cfg->async_boundary && cfg->overlap_slots > 0) {
     int slots = cfg->overlap_slots;
     if (slots > pool->attn_grid / 2) slots = pool->attn_grid / 2;
