@@ -1,17 +1,20 @@
-// Fused append + GQA paged decode attention (Sec. 4.1), plus, for requests that reach their capacity boundary
-// with this step, the logits of the two calibrated summaries against every candidate key (Eq. 12, App. D.1)
-// while the key tile is in shared memory.  (The summaries themselves, Eq. 6, and the calibrated q~ are updated
-// by the plan kernel's summary CTAs before this kernel starts.)
+// Fused append + GQA paged decode attention (Sec. 4.1) with the update of the two query summaries (Eq. 6, App. D.1),
+// plus, for requests that reach their capacity boundary with this step, the logits of the two calibrated summaries
+// (Eq. 12) against every candidate key while the key tile is in shared memory.
 //
 // Work decomposition.  The plan kernel cuts every stepped request into chunks of `chunk_pages` pages and
-// writes one descriptor per chunk, sorted by descending cost; a work item is (chunk, layer, KV head).  A
-// persistent grid (two CTAs per SM) deals the items out round by round, alternating the CTA order so that
-// every CTA gets about the same total.  Each CTA is warp-specialised:
+// writes one descriptor per chunk, sorted by descending cost; a work item is (chunk, layer, KV head).  The CTAs of a
+// persistent grid (two per SM) draw them in that order.  Each CTA is warp-specialised:
 //
-//   warp 0      producer: takes its items (a static deal of the cost-sorted list) and publishes each in a ring
-//               of item slots: descriptor, query rows (and the new key/value row) by bulk copy, page ids.  For
-//               boundary items it also brings q~ into the CTA's single q~ buffer.
-//   warps 4..7  consumers: take the tiles of an item round-robin (tile j belongs to warp (j - item number) mod 4,
+//   warp 0      producer: draws the CTA's items and publishes each in a ring of item slots: descriptor, query rows
+//               (and the new key/value row, and the position's cosines and sines) by bulk copy, page ids.
+//   warps 1, 3  summaries: the first item of a request's unit carries its summaries one step on (read from one of the
+//               request's two buffers, written to the other); every item with candidate pages of a request at its
+//               boundary gets the calibrated, rotated summaries q~ in the CTA's single q~ buffer, each item's CTA from
+//               the old buffer for itself.  (They were CTAs of the plan kernel: 8 us before the first key could be
+//               asked for in a layer-by-layer launch, 300 us of the step at 36 layers x 256 requests, and q~ went through
+//               global memory.)
+//   warps 4..7  consumers: take the tiles of an item round-robin (tile j belongs to warp (j - its item's number) mod 4,
 //               so the odd tiles of successive items fall on different warps).  Each warp
 //               fetches its own K|V tiles (one contiguous 8 KB per (layer, page, head)) with 16-byte
 //               asynchronous copies into a private ring of stages, running ahead across item boundaries, so
@@ -20,26 +23,32 @@
 //               Rows 8..15 of the A operand carry the bf16 rounding residual of rows 0..7 (of the rotated
 //               query when RoPE is on, of P always), which costs nothing and gives ~16 mantissa bits.  For
 //               boundary units the summary logits of a candidate page are an fp64 tensor-core contraction
-//               (m8n8k4 DMMA: 8 tokens x (2 views x G heads) x d).
+//               (m8n8k4 DMMA: 8 tokens x (2 views x G heads) x d).  With NORM the query rows and the new key row arrive
+//               raw: the summary warps normalise the queries in the slot (RMS over the head dimension, a learned weight
+//               per element), the warp that appends the key normalises that.
 //   warp 2      merger: combines the four consumers' partial (max, sum, O) of an item and writes the output
-//               or, for requests split over several items, the partial (the next kernel merges those).
+//               or, for requests split over several items, the partial; the merger whose partial is a unit's last merges
+//               them all, in the order of the chunks.
 //               Consumers hand over through a double buffer and go straight on to the next item.
-//   warps 1, 3  idle.
 //
-// The two warp groups re-split the register file (setmaxnreg): the service warps keep 56 registers per
-// thread, the consumers, which hold the output accumulators, get 200.
+// The two warp groups re-split the register file (setmaxnreg): the service warps keep 80 registers per
+// thread, the consumers, which hold the output accumulators, get 176 (at 160 their loop spills: 13.8 ms against 12.0 on
+// pages of 256).
 // All waits are bounded; a wait that gives up sets an error bit (with a code for which wait it was) and an
 // abort flag that drains the CTA.  No wait of an item depends on a later item being published.
 #include "gp_dev.cuh"
 
 namespace {
 
-constexpr int NI_MAX = 8;                  // item slots per CTA (4 when the group is 8 heads wide)
+constexpr int NI = 4;                      // item slots per CTA
 constexpr int NSW = 2;                     // tile stages per consumer warp (at most 3: see the wait in the tile loop)
 constexpr int NCW = 4;                     // consumer warps
-constexpr int NTHREADS = 256;              // warp group 0: producer, idle, merger, idle; warp group 1: consumers
-constexpr int REGS_SERVICE = 56;           // registers per thread after the split (setmaxnreg)
-constexpr int REGS_CONSUMER = 200;
+constexpr int NTHREADS = 256;              // warp group 0: producer, summaries, merger, summaries; warp group 1: consumers
+constexpr int REGS_SERVICE = 80;           // registers per thread after the split (setmaxnreg): 128 x (80 + 176) as launched
+constexpr int REGS_CONSUMER = 176;
+constexpr int NSUM = 2;                    // summary warps
+constexpr int MERGE_FAN = 8;               // partial outputs merged at a time
+constexpr double QT_SCALE = 0x1p896;       // of the q~ buffer: see bf16_lo_scaled
 constexpr int QT_PAD = 8;                  // doubles of padding per q~ row: rows alternate bank halves
 
 template <int D>
@@ -50,27 +59,26 @@ struct Geo {
   static constexpr int DTILES = D / 8;
   static constexpr int SLOT_DESC = 384;                                // 96 ints: descriptor (32), then up to 64 page ids
   static constexpr int SLOT_PAGES = 32;                                // first page id (int index)
-  static constexpr int SLOT_BYTES = (SLOT_DESC + 8 * ROW_BYTES + 2 * ROW_BYTES + 127) / 128 * 128;
+  static constexpr int SLOT_ROPE = SLOT_DESC + 10 * ROW_BYTES;         // cosine and sine of the position, D / 2 pairs of floats
+  static constexpr int SLOT_BYTES = (SLOT_ROPE + D / 2 * 8 + 127) / 128 * 128;
 };
 
 struct Lay {            // shared-memory layout, depends on the group size
-  int ni, ncomb, off_slots, off_qt, off_comb, comb_warp, off_bars, off_misc, total;
+  int ncomb, off_slots, off_qt, off_comb, comb_warp, off_bars, off_misc, total;
 };
 template <int D>
 __host__ __device__ inline Lay make_lay(int G) {
   using GEO = Geo<D>;
   Lay L;
-  const bool wide = (D == 128 && G == 8);
-  L.ni = wide ? 4 : NI_MAX;
-  L.ncomb = wide ? 1 : 2;
+  L.ncomb = (D == 128 && G == 8) ? 1 : 2;
   L.off_slots = NCW * NSW * GEO::TILE_BYTES;
-  L.off_qt = L.off_slots + L.ni * GEO::SLOT_BYTES;
+  L.off_qt = L.off_slots + NI * GEO::SLOT_BYTES;
   const int nrows = 2 * G < 8 ? 8 : 2 * G;
   L.off_comb = L.off_qt + nrows * (D + QT_PAD) * 8;
   L.comb_warp = (16 + G * D) * 4;
   L.off_bars = L.off_comb + L.ncomb * NCW * L.comb_warp;
-  L.off_misc = L.off_bars + (2 * NCW * NSW + 2 * NI_MAX + 2 + 4) * 8;
-  L.total = L.off_misc + 128 + 256;          // abort flag and code, then the queue of q~ copies
+  L.off_misc = L.off_bars + (3 * NI + 2 + 4) * 8;
+  L.total = L.off_misc + 128;                // abort flag and code
   return L;
 }
 
@@ -93,11 +101,264 @@ __device__ __forceinline__ void dmma(double& d0, double& d1, double a, double b)
                : "d"(a), "d"(b));
 }
 
-template <int D, bool ROPE>
+// double -> float -> bf16, each round-to-nearest-even (the order a host library takes)
+__device__ __forceinline__ __nv_bfloat16 to_bf16(double x) { return __float2bfloat16_rn((float)x); }
+__device__ __forceinline__ uint32_t pack_bf16_d(double lo, double hi) { return pack_bf16((float)lo, (float)hi); }
+
+// Partial outputs [n][G][D + 2] at `first`, `stride` floats apart (unnormalised output, running maximum in the log2 domain, sum
+// of exponentials), merged by one warp in ascending order, so that the result does not depend on who merges: into output
+// rows, or, with `into`, into a partial output again (the first one's place: a row is read before it is written).
+template <int D>
+__device__ __forceinline__ void merge_unit(float* first, size_t stride, int n, int G, float* __restrict__ orow, bool into) {
+  constexpr int PER2 = D / 64;                           // float2 pieces of a row per lane
+  const int lane = threadIdx.x & 31;
+  for (int g0 = 0; g0 < G; g0 += 4) {                    // four heads at a time
+    const int g = g0 + (lane & 3);                       // lane: head g0 + lane % 4, partials lane / 4, + 8, ...
+    const float* ml = first + (g < G ? g : 0) * (D + 2) + D;
+    float M = -INFINITY, ls = 0.f;
+    for (int c = lane >> 2; c < n; c += 8) {
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(ml + c * stride));
+      const float Mn = fmaxf(M, v.x);
+      ls = ls * exp2f(M - Mn) + exp2f(v.x - Mn) * v.y;
+      M = Mn;
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {                   // (a lane without a partial: M is -inf, weight 0)
+      const float Mo = __shfl_xor_sync(0xffffffffu, M, o), lo = __shfl_xor_sync(0xffffffffu, ls, o);
+      const float Mn = fmaxf(M, Mo);
+      ls = (M == -INFINITY ? 0.f : ls * exp2f(M - Mn)) + (Mo == -INFINITY ? 0.f : lo * exp2f(Mo - Mn));
+      M = Mn;
+    }
+    float2 acc[4][PER2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int e = 0; e < PER2; ++e) acc[q][e] = make_float2(0.f, 0.f);
+    for (int c0 = 0; c0 < n; c0 += 2) {                  // two partials' values in flight
+      float2 vv[2][4][PER2];
+      float mv[2][4];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float* pr = first + (c0 + k < n ? c0 + k : c0) * stride + (g0 + q < G ? g0 + q : 0) * (D + 2);
+          mv[k][q] = c0 + k < n ? __ldcg(pr + D) : -INFINITY;
+#pragma unroll
+          for (int e = 0; e < PER2; ++e) vv[k][q][e] = __ldcg(reinterpret_cast<const float2*>(pr) + lane + 32 * e);
+        }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float wgt = exp2f(mv[k][q] - __shfl_sync(0xffffffffu, M, q));
+#pragma unroll
+          for (int e = 0; e < PER2; ++e) { acc[q][e].x += wgt * vv[k][q][e].x; acc[q][e].y += wgt * vv[k][q][e].y; }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float tot = __shfl_sync(0xffffffffu, ls, q), Mq = __shfl_sync(0xffffffffu, M, q);
+      if (g0 + q < G) {
+        const float inv = into ? 1.f : 1.f / tot;
+        float2* dst = reinterpret_cast<float2*>(into ? first + (g0 + q) * (D + 2) : orow + (g0 + q) * D);
+#pragma unroll
+        for (int e = 0; e < PER2; ++e) dst[lane + 32 * e] = make_float2(acc[q][e].x * inv, acc[q][e].y * inv);
+        if (into && lane == 0) { first[(g0 + q) * (D + 2) + D] = Mq; first[(g0 + q) * (D + 2) + D + 1] = tot; }
+      }
+    }
+  }
+}
+
+// The summaries of one unit, the heads g = w, w + NSUM, ... by the calling warp (w): Eq. 6 on the un-rotated query from the
+// request's current buffer to the other one (`owner`), and, with `qt`, the calibrated (Eq. 12) and rotated summaries q~ into
+// the q~ buffer (times QT_SCALE), all in fp64.  What bounds it is the round trip for the old rows: two heads' (both views)
+// are in flight together, and the first ones' are asked for before anything else.  With NORM the warp first normalises its
+// heads' query rows in the slot and reports them on `norm_bar`: the consumers wait for that.
+template <int D, bool ROPE, bool NORM>
+__device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, uint8_t* qrows, uint64_t* norm_bar, int w, int G, int l,
+                                             int h, int r, int bi, int par, bool started, bool owner, double* qt) {
+  constexpr int PER = D / 32;
+  const int lane = threadIdx.x & 31;
+  __nv_bfloat16* q0 = reinterpret_cast<__nv_bfloat16*>(qrows);
+  double ov[2][2][PER];                                   // [head of the pair][view]
+  auto load_old = [&](int g0) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        if (g0 + NSUM * k < G) {
+          const double* o0 = p.summ + gp_summ_off(p, l, r, par, x, h * G + g0 + NSUM * k);
+#pragma unroll
+          for (int e = 0; e < PER; ++e) ov[k][x][e] = __ldcg(o0 + lane + 32 * e);
+        }
+  };
+  if (owner || qt) load_old(w);
+  if (NORM) {                    // the summaries follow the query after its normalisation and before its rotation (Sec. 3.2)
+    for (int g = w; g < G; g += NSUM) {
+      float qf[PER];
+      double ssq = 0.0;
+#pragma unroll
+      for (int e = 0; e < PER; ++e) { qf[e] = __bfloat162float(q0[g * D + lane + 32 * e]); ssq += (double)qf[e] * (double)qf[e]; }
+#pragma unroll
+      for (int o2 = 16; o2 > 0; o2 >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o2);
+      const double scale = 1.0 / sqrt(ssq / (double)D + nm.eps);
+#pragma unroll
+      for (int e = 0; e < PER; ++e) q0[g * D + lane + 32 * e] = to_bf16((double)qf[e] * scale * (double)__ldg(nm.wq + lane + 32 * e));
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(norm_bar);
+  }
+  if (!owner && !qt) return;
+  for (int g0 = w; g0 < G; g0 += 2 * NSUM) {
+    if (g0 != w) load_old(g0);
+    double ss[2][2], sq[2];                                // sums of squares: new summaries, query
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int g = g0 + NSUM * k;
+      ss[k][0] = ss[k][1] = sq[k] = 0.0;
+      if (g < G) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+          const double qv = (double)__bfloat162float(q0[g * D + lane + 32 * e]);
+          sq[k] += qv * qv;
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const double beta = x ? p.beta_l : p.beta_s;
+            const double nv = started ? beta * ov[k][x][e] + (1.0 - beta) * qv : qv;             // Eq. 6
+            ov[k][x][e] = nv;
+            ss[k][x] += nv * nv;
+          }
+        }
+        if (owner) {
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            double* newp = p.summ + gp_summ_off(p, l, r, par ^ 1, x, h * G + g);
+#pragma unroll
+            for (int e = 0; e < PER; ++e) newp[lane + 32 * e] = ov[k][x][e];
+          }
+        }
+      }
+    }
+    if (!qt) continue;
+#pragma unroll
+    for (int o2 = 16; o2 > 0; o2 >>= 1) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        sq[k] += __shfl_xor_sync(0xffffffffu, sq[k], o2);
+        ss[k][0] += __shfl_xor_sync(0xffffffffu, ss[k][0], o2);
+        ss[k][1] += __shfl_xor_sync(0xffffffffu, ss[k][1], o2);
+      }
+    }
+    // Eq. 12: lane 2k + x works out its gamma (roots and quotients once for the four rows)
+    const double my_ss = lane & 2 ? (lane & 1 ? ss[1][1] : ss[1][0]) : (lane & 1 ? ss[0][1] : ss[0][0]);
+    const double my_sq = lane & 2 ? sq[1] : sq[0];
+    const double gam = (my_ss > 0.0 ? sqrt(my_sq / (double)D) / sqrt(my_ss / (double)D) : 1.0) * QT_SCALE;
+    double2 cs[PER / 2];
+#pragma unroll
+    for (int e = 0; e < PER / 2; ++e)
+      if (ROPE) cs[e] = *reinterpret_cast<const double2*>(p.rope_cs + ((size_t)bi * (D / 2) + lane + 32 * e) * 2);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const double gamma = __shfl_sync(0xffffffffu, gam, 2 * k + x);
+        if (g0 + NSUM * k < G) {
+          double* dst = qt + (size_t)(x * G + g0 + NSUM * k) * (D + QT_PAD);
+#pragma unroll
+          for (int e = 0; e < PER / 2; ++e) {
+            const int j = lane + 32 * e;
+            const double x1 = gamma * ov[k][x][e], x2 = gamma * ov[k][x][e + PER / 2];
+            dst[j] = ROPE ? x1 * cs[e].x - x2 * cs[e].y : x1;
+            dst[j + D / 2] = ROPE ? x2 * cs[e].x + x1 * cs[e].y : x2;
+          }
+        }
+      }
+  }
+}
+
+// bf16 -> double by its bits, scaled by 2^-896 (an 8-bit exponent read as an 11-bit one): exact for every finite number, and
+// cheaper than the conversion unit.  The q~ buffer holds the summaries times 2^896, so that the products are what they were.
+__device__ __forceinline__ double bf16_lo_scaled(uint32_t w) { return __hiloint2double((int)((uint32_t)((int)(w << 16) >> 3) & 0x8fffffffu), 0); }
+__device__ __forceinline__ double bf16_hi_scaled(uint32_t w) { return __hiloint2double((int)((uint32_t)((int)(w & 0xffff0000u) >> 3) & 0x8fffffffu), 0); }
+
+// fp64 logits of a boundary unit's calibrated summaries against the 16 keys of a candidate page, by one warp:
+// Z[token][n] = sum_d K[token][d] q~[n][d], n = view * G + head.  One m8n8k4 DMMA covers 8 tokens,
+// 8 columns and 4 values of d; inside a 16-byte chunk of a key row lane t of a quad takes the
+// bf16 pair at byte 4t, whose low and high element feed two successive k-steps (q~ is read with
+// the same mapping, so the contraction is over the same d on both sides).  One block of eight columns at a time (nt of them: a
+// group of eight heads has two).  What bounds it: the fp64 pipe and four chains of dependent DMMAs; the registers it takes are
+// the consumers' (two blocks together spilled: 84.0 ms against 80.0 on 36 layers x 256 requests).  Stores the exponentials
+// per token and the page's softmax partials per column.
+template <int D>
+__device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* tile, const double* qt, int G, int lh, long long zoff,
+                                               int tok0, int nt) {
+  constexpr int CH = D / 8, ROW_BYTES = D * 2;
+  const int lane = threadIdx.x & 31, grp = lane >> 2, t4 = lane & 3;
+  double z[2][2][2];                                      // [even / odd chunks][token half][column pair]
+#pragma unroll
+  for (int i = 0; i < 8; ++i) (&z[0][0][0])[i] = 0.0;
+  const int n = nt * 8 + grp;                             // B column held by this lane's group (past 2G: another one's, not stored)
+  const double* qrow = qt + (size_t)(n < 2 * G ? n : 0) * (D + QT_PAD) + 2 * t4;
+  const uint8_t* krow0 = tile + grp * ROW_BYTES + 4 * t4;
+  const uint8_t* krow1 = tile + (8 + grp) * ROW_BYTES + 4 * t4;
+#pragma unroll 4
+  for (int c = 0; c < CH; c += 2) {
+#pragma unroll
+    for (int odd = 0; odd < 2; ++odd) {
+      const uint32_t ka = *reinterpret_cast<const uint32_t*>(krow0 + (((c + odd) ^ grp) << 4));   // grp == token & 7
+      const uint32_t kb = *reinterpret_cast<const uint32_t*>(krow1 + (((c + odd) ^ grp) << 4));
+      const double2 qq = *reinterpret_cast<const double2*>(qrow + (c + odd) * 8);
+      dmma(z[odd][0][0], z[odd][0][1], bf16_lo_scaled(ka), qq.x);
+      dmma(z[odd][1][0], z[odd][1][1], bf16_lo_scaled(kb), qq.x);
+      dmma(z[odd][0][0], z[odd][0][1], bf16_hi_scaled(ka), qq.y);
+      dmma(z[odd][1][0], z[odd][1][1], bf16_hi_scaled(kb), qq.y);
+    }
+  }
+  const double inv_sqrt_d = 1.0 / sqrt((double)D);
+  // D fragment: row = grp (token), columns 2*t4, 2*t4 + 1
+  const int col = nt * 8 + 2 * t4;
+  double z00 = (z[0][0][0] + z[1][0][0]) * inv_sqrt_d, z01 = (z[0][0][1] + z[1][0][1]) * inv_sqrt_d;
+  double z10 = (z[0][1][0] + z[1][1][0]) * inv_sqrt_d, z11 = (z[0][1][1] + z[1][1][1]) * inv_sqrt_d;
+  // the page's softmax partials per column: max and sum of exponentials over its 16 tokens; the
+  // exponentials themselves are what is stored per token
+  double m0 = fmax(z00, z10), m1 = fmax(z01, z11);
+#pragma unroll
+  for (int o2 = 4; o2 < 32; o2 <<= 1) {
+    m0 = fmax(m0, __shfl_xor_sync(0xffffffffu, m0, o2));
+    m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o2));
+  }
+  z00 = exp(z00 - m0); z10 = exp(z10 - m0); z01 = exp(z01 - m1); z11 = exp(z11 - m1);
+  double e0 = z00 + z10, e1 = z01 + z11;
+#pragma unroll
+  for (int o2 = 4; o2 < 32; o2 <<= 1) {
+    e0 += __shfl_xor_sync(0xffffffffu, e0, o2);
+    e1 += __shfl_xor_sync(0xffffffffu, e1, o2);
+  }
+  if (col < 2 * G) {
+    // view = col / G (short or long summary); a view's values of one unit are contiguous [token][G]
+    const size_t tokrow = (size_t)(zoff + tok0 + grp);
+    if (G >= 2) {
+      double* z0 = p.zbuf + (((size_t)lh * 2 + col / G) * p.z_stride + tokrow) * G + col % G;
+      *reinterpret_cast<double2*>(z0) = make_double2(z00, z01);
+      *reinterpret_cast<double2*>(z0 + (size_t)8 * G) = make_double2(z10, z11);
+    } else {
+      double* zS = p.zbuf + ((size_t)lh * 2 * p.z_stride + tokrow);
+      double* zL = zS + p.z_stride;
+      zS[0] = z00; zS[8] = z10; zL[0] = z01; zL[8] = z11;
+    }
+    if (grp == 0) {
+      double* st2 = p.zstat + (((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + (zoff + tok0) / GP_PAGE) * (2 * G) + col) * 2;
+      *reinterpret_cast<double2*>(st2) = make_double2(m0, e0);
+      *reinterpret_cast<double2*>(st2 + 2) = make_double2(m1, e1);
+    }
+  }
+}
+
+template <int D, bool ROPE, bool NORM, bool WIDE>       // WIDE: groups of eight query heads
 __global__ void __launch_bounds__(NTHREADS, 2)
 gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* __restrict__ q,
                const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, float* __restrict__ out, int lh0,
-               int lh_n, int adv_lh) {
+               int lh_n, int adv_lh, const GpNorm nm) {
   // lh0, lh_n: the (layer, KV head) units this launch covers, [lh0, lh0 + lh_n): all of them, or one layer's
   // adv_lh: the unit whose append also moves the request's counters on by one token (-1: none; the layer-by-layer
   // step does that at its end)
@@ -106,11 +367,12 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   uint8_t* smem = smem_raw + ((256u - (smem_u32(smem_raw) & 255u)) & 255u);
   const int G = p.G;
   const Lay L = make_lay<D>(G);
-  const uint32_t NI = (uint32_t)L.ni, NCOMB = (uint32_t)L.ncomb;
+  const uint32_t NCOMB = (uint32_t)L.ncomb;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.off_bars);
-  uint64_t* slot_full = bars + 2 * NCW * NSW;  // [NI]
-  uint64_t* slot_empty = slot_full + NI_MAX;   // [NI]
-  uint64_t* qt_full = slot_empty + NI_MAX;
+  uint64_t* slot_full = bars;                  // [NI]
+  uint64_t* slot_empty = slot_full + NI;       // [NI]
+  uint64_t* slot_norm = slot_empty + NI;       // [NI] the slot's query rows have been normalised
+  uint64_t* qt_full = slot_norm + NI;
   uint64_t* qt_empty = qt_full + 1;
   uint64_t* comb_full = qt_empty + 1;          // [2]
   uint64_t* comb_empty = comb_full + 2;        // [2]
@@ -122,8 +384,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t lim = p.spin_limit;
   if (tid == 0) {
-    for (int i = 0; i < NI_MAX; ++i) { mbar_init(&slot_full[i], 2); mbar_init(&slot_empty[i], NCW + 1); }
-    mbar_init(qt_full, 1);
+    for (int i = 0; i < NI; ++i) { mbar_init(&slot_full[i], 2); mbar_init(&slot_empty[i], NCW + 1 + NSUM); mbar_init(&slot_norm[i], NSUM); }
+    mbar_init(qt_full, NSUM);
     mbar_init(qt_empty, NCW);
     for (int i = 0; i < 2; ++i) { mbar_init(&comb_full[i], NCW); mbar_init(&comb_empty[i], 1); }
     s_misc[0] = 0;
@@ -134,6 +396,10 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   gp_pdl_launch_dependents();
   __syncthreads();
 
+  // the first item's descriptor is fetched before the number of items is known (same round trip): a slot past it holds
+  // stale but readable data that is then not used
+  int hFirst = 0;
+  if (warp == 0 && lane < GP_DESC_INTS && (int)(blockIdx.x / lh_n) < p.max_rc) hFirst = p.rcx[(size_t)(blockIdx.x / lh_n) * GP_DESC_INTS + lane];
   const int n_rc = p.hdr[HDR_N_RC];
   const int LH = p.L * p.Hkv;
   const long long total = (long long)n_rc * lh_n;
@@ -146,129 +412,66 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   }
   if (warp == 0) {
     // ================================= producer ===========================================
-    // Software pipeline over items, one stage per tick, so that no global round trip of one item delays
-    // another: A = item known, descriptor header load issued; B = header here: the slot is claimed, the
-    // descriptor written, the query rows (and the new key/value row) copied in, the page ids requested;
-    // C = page ids here: written to the slot, which completes its `full` barrier (two arrivals: B and C, plus
-    // the bytes of B's copies).  The ring of slots paces the producer: it runs NI items ahead at most.
-    const long long grid = gridDim.x;
-    // static schedule: items are sorted by descending cost; round k goes to the CTAs in alternating order
-    auto item_of_tick = [&](long long kk) -> long long {
-      const long long item = kk * grid + ((kk & 1) ? grid - 1 - (long long)blockIdx.x : (long long)blockIdx.x);
-      return item < total ? item : total;
-    };
-    long long itA = item_of_tick(0), itB = total, itC = total;
-    int hB = 0, hC = 0;                        // descriptor header, word `lane` (lanes 0..15)
-    int pC = -1, pC2 = -1;                     // page ids of tiles `lane` and `lane + 32` of the item
-    int slC = 0;                               // slot of the item in stage C
-    uint32_t n_pub = 0, n_comp = 0;          // items published (stage B), items completed (stage C)
-    bool sentinel_out = false;
-    // The q~ buffer is single: the copy for a boundary item is issued once the consumers are done with the
-    // previous boundary item.  The producer never blocks on that (it would hold back the slots of other
-    // items, possibly of the very item the consumers have to finish first): copies wait in a queue (never
-    // more entries than item slots) and are issued from the polls below, oldest first.
-    volatile int* qt_queue = s_misc + 16;          // [NI_MAX][2]: batch slot, layer/head
-    uint32_t qt_head = 0, qt_tail = 0;              // qt_head = copies issued so far
-    auto poll_qt = [&]() {
-      if (qt_head != qt_tail && mbar_test_wait(qt_empty, (qt_head & 1u) ^ 1u)) {
-        if (lane == 0) {
-          const int qbi = qt_queue[(qt_head % NI_MAX) * 2], qlh = qt_queue[(qt_head % NI_MAX) * 2 + 1];
-          fence_proxy_async();
-          mbar_expect_tx(qt_full, 2 * G * D * 8);
-          const double* src = p.qtil + ((size_t)qbi * LH + qlh) * 2 * G * D;
-          for (int row2 = 0; row2 < 2 * G; ++row2)
-            bulk_g2s(qt + (size_t)row2 * (D + QT_PAD), src + (size_t)row2 * D, D * 8, qt_full);
-        }
-        ++qt_head;
-      }
-    };
-    auto wait_polling = [&](uint64_t* bar, uint32_t parity) -> bool {     // bounded, abort-aware, keeps q~ moving
-      for (uint32_t w = 0; w < lim; ++w) {
-        if (mbar_try_wait(bar, parity)) return true;
-        poll_qt();
-        if ((w & 63u) == 63u && s_misc[0]) return false;
-      }
-      if (s_misc[0] == 0) s_misc[1] = 1;
-      s_misc[0] = 1;
-      return false;
-    };
-    for (uint32_t tick = 0;; ++tick) {
-      // ---- issue the loads of the young stages --------------------------------------------------
-      int hNew = 0;
-      if (itA < total && lane < GP_DESC_INTS) hNew = p.rcx[(size_t)(itA / lh_n) * GP_DESC_INTS + lane];
-      int pNew = -1, pNew2 = -1;
-      int slNew = 0;
-      // ---- page ids of stage C have arrived: into the slot, which is then complete ----------------------
-      if (itC < total) {
-        int* sd = reinterpret_cast<int*>(smem + L.off_slots + slC * GEO::SLOT_BYTES);
-        sd[GEO::SLOT_PAGES + lane] = pC;
-        sd[GEO::SLOT_PAGES + 32 + lane] = pC2;
+    // A CTA's first item is the one of its own number, the others are drawn from a counter, costliest first (numbering the
+    // items unit by unit instead, so that boundary items spread over the launch: 35.7 ms against 33.9 on the 32B shape), and
+    // only once the item before the one last published is done: a CTA holds the item it works on and the next, and what is
+    // left goes to whoever is free.  (Dealt out statically by an estimate of their cost, the CTAs of a one-layer step ended
+    // between 26 and 38 us; drawn as far ahead as a ring of eight slots allows, they hoarded.)  Which CTA takes an item does
+    // not change its result.
+    long long item = (long long)blockIdx.x < total ? (long long)blockIdx.x : total;
+    int hdr = hFirst;                          // descriptor header, word `lane` (lanes 0..15)
+    for (uint32_t n = 0;; ++n) {
+      const int sl = n % NI;
+      if (!wait_bar(&slot_empty[sl], ((n / NI) & 1u) ^ 1u, s_misc, 1, lim)) break;
+      uint8_t* slot = smem + L.off_slots + sl * GEO::SLOT_BYTES;
+      int* sd = reinterpret_cast<int*>(slot);
+      if (item >= total) {
+        if (lane == 0) sd[3] = -1;
         __syncwarp();
-        // (test support: the first CTA's second item can be withheld, so that the consumers' bounded wait runs out)
-        const bool withheld = (p.withhold & GP_WITHHOLD_ITEM) && blockIdx.x == 0 && n_comp == 1;
-        ++n_comp;
-        if (lane == 0 && !withheld) mbar_arrive(&slot_full[slC]);
+        if (lane == 0) { mbar_arrive(&slot_full[sl]); mbar_arrive(&slot_full[sl]); }
+        break;
       }
-      poll_qt();
-      // ---- header of stage B has arrived: load its page ids and fill its slot -----------------------
-      if (tick >= 1 && !sentinel_out) {
-        const int sl = n_pub % NI;
-        slNew = sl;
-        if (!wait_polling(&slot_empty[sl], ((n_pub / NI) & 1u) ^ 1u)) break;
-        uint8_t* slot = smem + L.off_slots + sl * GEO::SLOT_BYTES;
-        int* sd = reinterpret_cast<int*>(slot);
-        if (itB >= total) {
-          if (lane == 0) sd[3] = -1;
-          __syncwarp();
-          if (lane == 0) { mbar_arrive(&slot_full[sl]); mbar_arrive(&slot_full[sl]); }
-          sentinel_out = true;
-        } else {
-          const int lh = lh0 + (int)(itB % lh_n);
-          const int l = lh / p.Hkv, h = lh % p.Hkv;
-          const int bi = __shfl_sync(0xffffffffu, hB, 0);
-          const int r = __shfl_sync(0xffffffffu, hB, 1), pg0 = __shfl_sync(0xffffffffu, hB, 2);
-          const int npg = __shfl_sync(0xffffffffu, hB, 3);
-          const int chunk = __shfl_sync(0xffffffffu, hB, 4);
-          const int nchunks = __shfl_sync(0xffffffffu, hB, 5);
-          if (lane < npg) pNew = p.page_table[(size_t)r * p.cap + pg0 + lane];
-          if (lane + 32 < npg) pNew2 = p.page_table[(size_t)r * p.cap + pg0 + 32 + lane];
-          if (lane < 14) sd[lane] = hB;
-          if (lane == 14) sd[14] = lh;
-          if (lane == 15) sd[15] = hB;            // index among the step's boundary requests
-          __syncwarp();
-          if (lane == 0) {
-            const bool has_new = (chunk == nchunks - 1);
-            fence_proxy_async();
-            mbar_expect_tx(&slot_full[sl], q_bytes + (has_new ? 2 * GEO::ROW_BYTES : 0));
-            bulk_g2s(slot + GEO::SLOT_DESC, q + (((size_t)l * n_req + bi) * p.Hq + h * G) * D, q_bytes, &slot_full[sl]);
-            if (has_new) {
-              const size_t kvo = (((size_t)l * n_req + bi) * p.Hkv + h) * D;
-              bulk_g2s(slot + GEO::SLOT_DESC + 8 * GEO::ROW_BYTES, k + kvo, GEO::ROW_BYTES, &slot_full[sl]);
-              bulk_g2s(slot + GEO::SLOT_DESC + 9 * GEO::ROW_BYTES, v + kvo, GEO::ROW_BYTES, &slot_full[sl]);
-            }
-          }
-          // boundary unit with candidate pages in this chunk: its calibrated summaries q~ (written by the
-          // plan kernel's summary CTAs) go into the single q~ buffer once the previous such item is done
-          const int flags = __shfl_sync(0xffffffffu, hB, 8), Pr = __shfl_sync(0xffffffffu, hB, 9);
-          if ((flags & 1) && pg0 < Pr - 1) {
-            if (lane == 0) { qt_queue[(qt_tail % NI_MAX) * 2] = bi; qt_queue[(qt_tail % NI_MAX) * 2 + 1] = lh; }
-            __syncwarp();
-            ++qt_tail;
-            poll_qt();
-          }
+      const int lh = lh0 + (int)(item % lh_n);
+      const int l = lh / p.Hkv, h = lh % p.Hkv;
+      const int bi = __shfl_sync(0xffffffffu, hdr, 0);
+      const int r = __shfl_sync(0xffffffffu, hdr, 1), pg0 = __shfl_sync(0xffffffffu, hdr, 2);
+      const int npg = __shfl_sync(0xffffffffu, hdr, 3);
+      const int chunk = __shfl_sync(0xffffffffu, hdr, 4);
+      const int nchunks = __shfl_sync(0xffffffffu, hdr, 5);
+      int pg = -1, pg2 = -1;                   // page ids of tiles `lane` and `lane + 32` of the item
+      if (lane < npg) pg = p.page_table[(size_t)r * p.cap + pg0 + lane];
+      if (lane + 32 < npg) pg2 = p.page_table[(size_t)r * p.cap + pg0 + 32 + lane];
+      if (lane < 14) sd[lane] = hdr;
+      if (lane == 14) sd[14] = lh;
+      if (lane == 15) sd[15] = hdr;            // index among the step's boundary requests
+      if (lane == 16) sd[16] = (int)(item & (NCW - 1));       // the consumer warp that takes the item's first tile
+      __syncwarp();
+      if (lane == 0) {
+        const bool has_new = (chunk == nchunks - 1);
+        fence_proxy_async();
+        mbar_expect_tx(&slot_full[sl], q_bytes + (has_new ? 2 * GEO::ROW_BYTES : 0) + (ROPE ? D / 2 * 8 : 0));
+        bulk_g2s(slot + GEO::SLOT_DESC, q + (((size_t)l * n_req + bi) * p.Hq + h * G) * D, q_bytes, &slot_full[sl]);
+        if (ROPE) bulk_g2s(slot + GEO::SLOT_ROPE, p.rope_f + (size_t)bi * D, D / 2 * 8, &slot_full[sl]);
+        if (has_new) {
+          const size_t kvo = (((size_t)l * n_req + bi) * p.Hkv + h) * D;
+          bulk_g2s(slot + GEO::SLOT_DESC + 8 * GEO::ROW_BYTES, k + kvo, GEO::ROW_BYTES, &slot_full[sl]);
+          bulk_g2s(slot + GEO::SLOT_DESC + 9 * GEO::ROW_BYTES, v + kvo, GEO::ROW_BYTES, &slot_full[sl]);
         }
-        ++n_pub;
       }
-      if (sentinel_out && itC >= total) break;
-      // ---- rotate -----------------------------------------------------------------------------------------
-      itC = itB; hC = hB; pC = pNew; pC2 = pNew2; slC = slNew;
-      itB = itA; hB = hNew;
-      itA = item_of_tick((long long)tick + 1);
-    }
-    (void)hC;
-    while (qt_head != qt_tail && !s_misc[0]) {           // copies still queued when the last slot is out
-      if (!wait_polling(qt_empty, (qt_head & 1u) ^ 1u)) break;
-      poll_qt();
+      sd[GEO::SLOT_PAGES + lane] = pg;
+      sd[GEO::SLOT_PAGES + 32 + lane] = pg2;
+      __syncwarp();
+      // (test support: the first CTA's second item can be withheld, so that the consumers' bounded wait runs out)
+      const bool withheld = (p.withhold & GP_WITHHOLD_ITEM) && blockIdx.x == 0 && n == 1;
+      if (lane == 0 && !withheld) mbar_arrive(&slot_full[sl]);
+      // ---- the next item ----------------------------------------------------------------------------------
+      if (n > 0 && !wait_bar(&slot_empty[(n - 1) % NI], ((n - 1) / NI) & 1u, s_misc, 2, lim)) break;
+      int t = 0;
+      if (lane == 0) t = atomicAdd(p.tickets + lh0 / p.Hkv, 1);
+      item = (long long)gridDim.x + __shfl_sync(0xffffffffu, t, 0);
+      if (item > total) item = total;
+      hdr = 0;
+      if (item < total && lane < GP_DESC_INTS) hdr = p.rcx[(size_t)(item / lh_n) * GP_DESC_INTS + lane];
     }
   } else if (warp >= 4) {
     // ================================= consumers ==========================================
@@ -301,7 +504,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           f_npg = fsd[3];
           if (f_npg < 0) { f_done = true; break; }
           f_lh = fsd[14];
-          f_pgl = (cw + f_it) % NCW;                      // the first tile goes to another warp from item to item
+          f_pgl = (cw + fsd[16]) % NCW;                   // the first tile goes to another warp from item to item
           f_have = true;
         }
         if (f_pgl >= f_npg) { ++f_it; f_have = false; continue; }
@@ -335,6 +538,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const int n_new = n_old + 1;
       const bool need_qt = (flags & 1) && (pg0 < Pr - 1);
 
+      if (NORM && !wait_bar(&slot_norm[sl], (it / NI) & 1u, s_misc, 11, lim)) break;
       // ---- query fragments (A operand), rotated when RoPE is on ----------------------------------
       uint32_t qa[GEO::KSTEPS][2];
       uint32_t ql[GEO::KSTEPS][2];
@@ -342,40 +546,32 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
         const bool valid = row < G;
         const uint8_t* qrow = slot + GEO::SLOT_DESC + (valid ? row : 0) * GEO::ROW_BYTES;
 #pragma unroll
-        for (int kk = 0; kk < GEO::KSTEPS; ++kk) {
+        for (int kk = 0; kk < GEO::KSTEPS; ++kk)
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
-            const int col = kk * 16 + half * 8 + qc;
-            uint32_t hi = 0, lo = 0;
-            if (valid) {
-              if (!ROPE) {
-                hi = *reinterpret_cast<const uint32_t*>(qrow + col * 2);
-              } else {
-                const int j = col % (D / 2);
-                const uint32_t w1 = *reinterpret_cast<const uint32_t*>(qrow + j * 2);
-                const uint32_t w2 = *reinterpret_cast<const uint32_t*>(qrow + (j + D / 2) * 2);
-                const double* cs = p.rope_cs + ((size_t)bi * (D / 2) + j) * 2;
-                const float c0 = (float)cs[0], s0 = (float)cs[1], c1 = (float)cs[2], s1 = (float)cs[3];
-                float r0, r1;
-                if (col < D / 2) {
-                  r0 = bf16_lo_f(w1) * c0 - bf16_lo_f(w2) * s0;
-                  r1 = bf16_hi_f(w1) * c1 - bf16_hi_f(w2) * s1;
-                } else {
-                  r0 = bf16_lo_f(w2) * c0 + bf16_lo_f(w1) * s0;
-                  r1 = bf16_hi_f(w2) * c1 + bf16_hi_f(w1) * s1;
-                }
-                hi = pack_bf16(r0, r1);
-                lo = pack_bf16(r0 - bf16_lo_f(hi), r1 - bf16_hi_f(hi));
-              }
-            }
-            qa[kk][half] = hi;
-            ql[kk][half] = lo;
+            qa[kk][half] = valid ? *reinterpret_cast<const uint32_t*>(qrow + (kk * 16 + half * 8 + qc) * 2) : 0u;
+            ql[kk][half] = 0u;
           }
+        if (ROPE) {                                        // column col pairs with col + D / 2: the fragment KSTEPS / 2 on
+#pragma unroll
+          for (int kk = 0; kk < GEO::KSTEPS / 2; ++kk)
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              const int j = kk * 16 + half * 8 + qc;
+              const uint32_t w1 = qa[kk][half], w2 = qa[kk + GEO::KSTEPS / 2][half];
+              const float4 cs = *reinterpret_cast<const float4*>(slot + GEO::SLOT_ROPE + j * 8);     // (j is even)
+              const float c0 = cs.x, s0 = cs.y, c1 = cs.z, s1 = cs.w;
+              const float a0 = bf16_lo_f(w1) * c0 - bf16_lo_f(w2) * s0, a1 = bf16_hi_f(w1) * c1 - bf16_hi_f(w2) * s1;
+              const float b0 = bf16_lo_f(w2) * c0 + bf16_lo_f(w1) * s0, b1 = bf16_hi_f(w2) * c1 + bf16_hi_f(w1) * s1;
+              const uint32_t ha = pack_bf16(a0, a1), hb = pack_bf16(b0, b1);
+              qa[kk][half] = ha;
+              ql[kk][half] = pack_bf16(a0 - bf16_lo_f(ha), a1 - bf16_hi_f(ha));
+              qa[kk + GEO::KSTEPS / 2][half] = hb;
+              ql[kk + GEO::KSTEPS / 2][half] = pack_bf16(b0 - bf16_lo_f(hb), b1 - bf16_hi_f(hb));
+            }
         }
       }
-      if (need_qt) {
-        if (!wait_bar(qt_full, qt_uses & 1u, s_misc, 5, lim)) break;
-      }
+      bool qt_here = false;                                // the item's q~ is in the buffer
 
       const bool last_chunk = (chunk == nchunks - 1);
       float o[GEO::DTILES][4];
@@ -384,7 +580,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       float m_run = -INFINITY, l_run = 0.f;
       bool ok = true;
 
-      for (int pgl = (cw + it) % NCW; pgl < npg; pgl += NCW) {
+      for (int pgl = (cw + sd[16]) % NCW; pgl < npg; pgl += NCW) {
         const uint32_t st = cw * NSW + (my_tiles % NSW);
         {
           // one copy group per tile, in fetch order: all but the groups younger than this tile's must be done
@@ -401,9 +597,38 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           const int s = n_old - tok0;
           const int page = sd[GEO::SLOT_PAGES + npg - 1];
           constexpr int CH = D / 8;
+          uint4 k_new = make_uint4(0, 0, 0, 0);
+          if (NORM) {
+            // the raw key row (a chunk of eight elements per lane, CH lanes): normalised per head, rotated to the token's
+            // position, its cache form
+            const int c = lane % CH;
+            const uint4 raw = *reinterpret_cast<const uint4*>(slot + GEO::SLOT_DESC + 8 * GEO::ROW_BYTES + c * 16);
+            const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+            double e[8];
+            double ss = 0.0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              e[2 * i] = bf16_lo_f(w[i]); e[2 * i + 1] = bf16_hi_f(w[i]);
+              ss += e[2 * i] * e[2 * i] + e[2 * i + 1] * e[2 * i + 1];
+            }
+#pragma unroll
+            for (int o2 = 1; o2 < CH; o2 <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o2);
+            const double ks = 1.0 / sqrt(ss / (double)D + nm.eps);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              e[i] = e[i] * ks * (double)__ldg(nm.wk + c * 8 + i);
+              if (ROPE) {
+                const double other = __shfl_xor_sync(0xffffffffu, e[i], CH / 2);     // element j + D / 2 of j, and back
+                const double* cs = p.rope_cs + ((size_t)bi * (D / 2) + (c % (CH / 2)) * 8 + i) * 2;
+                e[i] = c < CH / 2 ? e[i] * cs[0] - other * cs[1] : e[i] * cs[0] + other * cs[1];
+              }
+            }
+            k_new = make_uint4(pack_bf16_d(e[0], e[1]), pack_bf16_d(e[2], e[3]), pack_bf16_d(e[4], e[5]), pack_bf16_d(e[6], e[7]));
+          }
           if (lane < 2 * CH) {
             const int isv = lane / CH, c = lane % CH;
-            const uint4 val = *reinterpret_cast<const uint4*>(slot + GEO::SLOT_DESC + (8 + isv) * GEO::ROW_BYTES + c * 16);
+            const uint4 val = NORM && !isv ? k_new
+                                           : *reinterpret_cast<const uint4*>(slot + GEO::SLOT_DESC + (8 + isv) * GEO::ROW_BYTES + c * 16);
             const int off = isv * GP_PAGE * GEO::ROW_BYTES + s * GEO::ROW_BYTES + ((c ^ (s & 7)) << 4);
             *reinterpret_cast<uint4*>(tile + off) = val;
             uint8_t* g = reinterpret_cast<uint8_t*>(p.kv + gp_tile_off(p, l, page, h)) + off;
@@ -412,8 +637,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           }
           if (lane == 0) p.tok[gp_tok_off(p, l, page, h) + s] = sd[7];
           if (lane == 1 && lh == adv_lh) {
-            // the request is one token further; the summary CTAs of this step have written the buffer not in use
-            // (the plan kernel had completed before this kernel passed its wait)
+            // the request is one token further, its summaries in the other buffer (nothing in this kernel looks at these
+            // words: what it needs is in the descriptors)
             const int r = sd[1];
             p.n[r] = n_new; p.pos[r] = (long long)sd[7] + 1; p.started[r] = 1; p.sum_par[r] = sd[12] ^ 1;
           }
@@ -487,87 +712,22 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             mma_bf16(o[jd + 1], pa[0], pa[1], pa[2], pa[3], v2, v3);
           }
         }
-        // Boundary unit: fp64 logits of the calibrated summaries against the 16 keys of a candidate page,
-        // Z[token][n] = sum_d K[token][d] q~[n][d], n = view * G + head.  One m8n8k4 DMMA covers 8 tokens,
-        // 8 columns and 4 values of d; inside a 16-byte chunk of a key row lane t of a quad takes the
-        // bf16 pair at byte 4t, whose low and high element feed two successive k-steps (q~ is read with
-        // the same mapping, so the contraction is over the same d on both sides).
+        // Boundary unit: fp64 logits of the calibrated summaries against the 16 keys of a candidate page
         if (need_qt && (pg0 + pgl) < Pr - 1) {
-          constexpr int CH = D / 8;
-          const int grp = lane >> 2, t4 = lane & 3;
-          const int n_tiles = (2 * G + 7) / 8;
-          const double sqrt_d = sqrt((double)D);
-          const long long zoff = ((long long)(unsigned)sd[10]) | ((long long)sd[11] << 32);
-          for (int nt = 0; nt < n_tiles; ++nt) {
-            const int n = nt * 8 + grp;                           // B column held by this lane's group
-            const bool ncol = n < 2 * G;
-            const double* qrow = qt + (size_t)(ncol ? n : 0) * (D + QT_PAD) + 2 * t4;
-            double z00 = 0.0, z01 = 0.0, z10 = 0.0, z11 = 0.0;    // [m-tile][column pair], even chunks
-            double y00 = 0.0, y01 = 0.0, y10 = 0.0, y11 = 0.0;    // odd chunks: four independent DMMA chains
-            const uint8_t* krow0 = tile + grp * GEO::ROW_BYTES + 4 * t4;
-            const uint8_t* krow1 = tile + (8 + grp) * GEO::ROW_BYTES + 4 * t4;
-#pragma unroll 4
-            for (int c = 0; c < CH; c += 2) {
-              const uint32_t ka = *reinterpret_cast<const uint32_t*>(krow0 + ((c ^ grp) << 4));   // grp == token & 7
-              const uint32_t kb = *reinterpret_cast<const uint32_t*>(krow1 + ((c ^ grp) << 4));
-              const uint32_t kc = *reinterpret_cast<const uint32_t*>(krow0 + (((c + 1) ^ grp) << 4));
-              const uint32_t kd = *reinterpret_cast<const uint32_t*>(krow1 + (((c + 1) ^ grp) << 4));
-              const double2 qq = *reinterpret_cast<const double2*>(qrow + c * 8);
-              const double2 qr = *reinterpret_cast<const double2*>(qrow + c * 8 + 8);
-              const double b0 = ncol ? qq.x : 0.0, b1 = ncol ? qq.y : 0.0;
-              const double b2 = ncol ? qr.x : 0.0, b3 = ncol ? qr.y : 0.0;
-              dmma(z00, z01, (double)bf16_lo_f(ka), b0);
-              dmma(z10, z11, (double)bf16_lo_f(kb), b0);
-              dmma(y00, y01, (double)bf16_lo_f(kc), b2);
-              dmma(y10, y11, (double)bf16_lo_f(kd), b2);
-              dmma(z00, z01, (double)bf16_hi_f(ka), b1);
-              dmma(z10, z11, (double)bf16_hi_f(kb), b1);
-              dmma(y00, y01, (double)bf16_hi_f(kc), b3);
-              dmma(y10, y11, (double)bf16_hi_f(kd), b3);
-            }
-            z00 += y00; z01 += y01; z10 += y10; z11 += y11;
-            // D fragment: row = grp (token), columns 2*t4, 2*t4 + 1
-            const int col = nt * 8 + 2 * t4;
-            z00 /= sqrt_d; z01 /= sqrt_d; z10 /= sqrt_d; z11 /= sqrt_d;
-            // the page's softmax partials per column: max and sum of exponentials over its 16 tokens; the
-            // exponentials themselves are what is stored per token
-            double m0 = fmax(z00, z10), m1 = fmax(z01, z11);
-#pragma unroll
-            for (int o2 = 4; o2 < 32; o2 <<= 1) {
-              m0 = fmax(m0, __shfl_xor_sync(0xffffffffu, m0, o2));
-              m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o2));
-            }
-            z00 = exp(z00 - m0); z10 = exp(z10 - m0); z01 = exp(z01 - m1); z11 = exp(z11 - m1);
-            double e0 = z00 + z10, e1 = z01 + z11;
-#pragma unroll
-            for (int o2 = 4; o2 < 32; o2 <<= 1) {
-              e0 += __shfl_xor_sync(0xffffffffu, e0, o2);
-              e1 += __shfl_xor_sync(0xffffffffu, e1, o2);
-            }
-            if (col < 2 * G) {
-              // view = col / G (short or long summary); a view's values of one unit are contiguous [token][G]
-              const size_t tokrow = (size_t)(zoff + tok0 + grp);
-              if (G >= 2) {
-                double* z0 = p.zbuf + (((size_t)lh * 2 + col / G) * p.z_stride + tokrow) * G + col % G;
-                *reinterpret_cast<double2*>(z0) = make_double2(z00, z01);
-                *reinterpret_cast<double2*>(z0 + (size_t)8 * G) = make_double2(z10, z11);
-              } else {
-                double* zS = p.zbuf + ((size_t)lh * 2 * p.z_stride + tokrow);
-                double* zL = zS + p.z_stride;
-                zS[0] = z00; zS[8] = z10; zL[0] = z01; zL[8] = z11;
-              }
-              if (grp == 0) {
-                double* st2 = p.zstat + (((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + (zoff + tok0) / GP_PAGE) * (2 * G) + col) * 2;
-                *reinterpret_cast<double2*>(st2) = make_double2(m0, e0);
-                *reinterpret_cast<double2*>(st2 + 2) = make_double2(m1, e1);
-              }
-            }
+          if (!qt_here) {
+            if (!wait_bar(qt_full, qt_uses & 1u, s_misc, 5, lim)) { ok = false; break; }
+            qt_here = true;
           }
+          const long long zoff = ((long long)(unsigned)sd[10]) | ((long long)sd[11] << 32);
+          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0);
+          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1);
         }
         __syncwarp();
         if (!top_up(it)) { ok = false; break; }            // the stage is free: fetch the next tile into it
       }
       if (!ok) break;
+      // (a warp without a candidate tile waits all the same: its next wait is for the phase after this one)
+      if (need_qt && !qt_here && !wait_bar(qt_full, qt_uses & 1u, s_misc, 5, lim)) break;
 
       // ---- a request at its boundary: this warp's share of the unit's summary logits (and the appended row, and the
       // request's counters) is written; the boundary work that may run beside this kernel counts the reports
@@ -608,7 +768,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const int* sd = reinterpret_cast<const int*>(slot);
       const int npg = sd[3];
       if (npg < 0) break;
-      const int bi = sd[0], nchunks = sd[5], rc_i = sd[13], lh = sd[14];
+      const int bi = sd[0], chunk = sd[4], nchunks = sd[5], rc_i = sd[13], lh = sd[14];
       const int l = lh / p.Hkv, h = lh % p.Hkv;
       const int cb = it % NCOMB;
       if (!wait_bar(&comb_full[cb], (it / NCOMB) & 1u, s_misc, 8, lim)) break;
@@ -616,29 +776,93 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const size_t out_row0 = (((size_t)l * n_req + bi) * p.Hq + h * G) * D;
       const int PSTRIDE = G * (D + 2);
       float* part = p.partials + ((size_t)lh * n_rc + rc_i) * PSTRIDE;
+      // weights of the four warps' rows, lane = 4 head + warp; then a row at a time, a lane owning D / 32 columns of it
+      static_assert(NCW == 4, "a quad of lanes per head");
+      const int mg = lane >> 2;
+      const float mw = mg < G ? cbuf[(lane & 3) * comb_w + mg] : 0.f;
+      float M = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, 1));
+      M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 2));
+      const float wgt = exp2f(mw - M);
+      float ls = mg < G ? wgt * cbuf[(lane & 3) * comb_w + 8 + mg] : 1.f;
+      ls += __shfl_xor_sync(0xffffffffu, ls, 1);
+      ls += __shfl_xor_sync(0xffffffffu, ls, 2);
+      if (nchunks > 1 && mg < G && (lane & 3) == 0) { part[mg * (D + 2) + D] = M; part[mg * (D + 2) + D + 1] = ls; }
+      const float inv = nchunks == 1 ? 1.f / ls : 1.f;
+      constexpr int PER2 = D / 64;                        // float2 pieces of a row per lane
+#pragma unroll 2
       for (int g = 0; g < G; ++g) {
-        float M = -INFINITY;
+        float2 acc[PER2];
 #pragma unroll
-        for (int w = 0; w < NCW; ++w) M = fmaxf(M, cbuf[w * comb_w + g]);
-        float wgt[NCW];
-        float ls = 0.f;
+        for (int e = 0; e < PER2; ++e) acc[e] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int w = 0; w < NCW; ++w) {
-          wgt[w] = exp2f(cbuf[w * comb_w + g] - M);
-          ls += wgt[w] * cbuf[w * comb_w + 8 + g];
-        }
-        const float inv = 1.f / ls;
-        for (int dc = lane; dc < D; dc += 32) {
-          float acc = 0.f;
+          const float ww = __shfl_sync(0xffffffffu, wgt, g * 4 + w);
 #pragma unroll
-          for (int w = 0; w < NCW; ++w) acc += wgt[w] * cbuf[w * comb_w + 16 + g * D + dc];
-          if (nchunks == 1) out[out_row0 + g * D + dc] = acc * inv;
-          else part[g * (D + 2) + dc] = acc;
+          for (int e = 0; e < PER2; ++e) {
+            const float2 x = *reinterpret_cast<const float2*>(cbuf + w * comb_w + 16 + g * D + 2 * lane + 64 * e);
+            acc[e].x += ww * x.x; acc[e].y += ww * x.y;
+          }
         }
-        if (nchunks > 1 && lane == 0) { part[g * (D + 2) + D] = M; part[g * (D + 2) + D + 1] = ls; }
+        const float sc2 = __shfl_sync(0xffffffffu, inv, g * 4);
+        float* dst = nchunks == 1 ? out + out_row0 + g * D : part + g * (D + 2);
+#pragma unroll
+        for (int e = 0; e < PER2; ++e) *reinterpret_cast<float2*>(dst + 2 * lane + 64 * e) = make_float2(acc[e].x * sc2, acc[e].y * sc2);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&comb_empty[cb]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&slot_empty[sl]);
+      if (nchunks > 1) {
+        // A split unit: whoever adds the last partial of a group of MERGE_FAN chunks merges the group, and whoever adds the
+        // last group's the groups (a tree of two levels, whatever the order of arrival).  The counters go back to zero
+        // for the next step.
+        const int n_grp = (nchunks + MERGE_FAN - 1) / MERGE_FAN, c_grp = chunk / MERGE_FAN * MERGE_FAN;
+        const int in_grp = min(MERGE_FAN, nchunks - c_grp);
+        float* unit = p.partials + ((size_t)lh * n_rc + rc_i - chunk) * PSTRIDE;
+        auto last_of = [&](int* cnt, int n) {
+          __threadfence();
+          __syncwarp();
+          int last = 0;
+          if (lane == 0 && atomicAdd(cnt, 1) == n - 1) { *cnt = 0; last = 1; }
+          last = __shfl_sync(0xffffffffu, last, 0);
+          __threadfence();
+          return last != 0;
+        };
+        int* cnt = p.merge_cnt + ((size_t)rc_i - chunk) * LH + (size_t)lh * nchunks;       // the unit's: one per chunk
+        if (last_of(cnt + c_grp, in_grp)) {
+          if (n_grp == 1) {
+            merge_unit<D>(unit, PSTRIDE, nchunks, G, out + out_row0, false);
+          } else {
+            if (in_grp > 1) merge_unit<D>(unit + (size_t)c_grp * PSTRIDE, PSTRIDE, in_grp, G, nullptr, true);
+            if (last_of(cnt + 1, n_grp)) merge_unit<D>(unit, (size_t)MERGE_FAN * PSTRIDE, n_grp, G, out + out_row0, false);
+          }
+        }
+      }
+    }
+  } else {
+    // ================================= summaries ==========================================
+    const int w = warp >> 1;
+    uint32_t qt_uses = 0;
+    for (uint32_t it = 0;; ++it) {
+      const int sl = it % NI;
+      if (!wait_bar(&slot_full[sl], (it / NI) & 1u, s_misc, 9, lim)) break;
+      uint8_t* slot = smem + L.off_slots + sl * GEO::SLOT_BYTES;
+      const int* sd = reinterpret_cast<const int*>(slot);
+      if (sd[3] < 0) break;
+      const int bi = sd[0], r = sd[1], flags = sd[8], par = sd[12], lh = sd[14];
+      const bool owner = sd[4] == 0;                       // this item writes the unit's new summaries
+      const bool need_qt = (flags & 1) && sd[2] < sd[9] - 1;
+      if (NORM || owner || need_qt) {
+        if (need_qt && !wait_bar(qt_empty, (qt_uses & 1u) ^ 1u, s_misc, 10, lim)) break;
+        const int l = lh / p.Hkv, h = lh % p.Hkv;
+        summary_rows<D, ROPE, NORM>(p, nm, slot + GEO::SLOT_DESC, &slot_norm[sl], w, G, l, h, r, bi, par, (flags & 2) != 0, owner,
+                                    need_qt ? qt : nullptr);
+        __syncwarp();
+        if (need_qt) {
+          ++qt_uses;
+          if (lane == 0) mbar_arrive(qt_full);
+        }
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&slot_empty[sl]);
     }
@@ -653,34 +877,26 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
 size_t gp_attention_smem(int d, int G) { return d == 128 ? make_lay<128>(G).total : make_lay<64>(G).total; }
 int gp_attention_ctas_per_sm(int d) { (void)d; return 2; }
 
-void gp_attention_setup(const GpDev& p) {           // once per pool: opt into the kernel's shared memory
-  const int sm = (int)gp_attention_smem(p.d, p.G);
-  if (p.d == 128) {
-    cudaFuncSetAttribute(gp_attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(gp_attn_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  } else {
-    cudaFuncSetAttribute(gp_attn_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(gp_attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  }
+typedef void (*AttnKernel)(const GpDev, int, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, float*, int, int, int,
+                           const GpNorm);
+template <int D, bool WIDE> static AttnKernel attn_kernel_d(bool rope, bool norm) {
+  return rope ? (norm ? gp_attn_kernel<D, true, true, WIDE> : gp_attn_kernel<D, true, false, WIDE>)
+              : (norm ? gp_attn_kernel<D, false, true, WIDE> : gp_attn_kernel<D, false, false, WIDE>);
+}
+static AttnKernel attn_kernel_of(const GpDev& p, bool norm) {
+  const bool rope = p.rope_theta != 0.0;
+  if (p.d == 128) return p.G == 8 ? attn_kernel_d<128, true>(rope, norm) : attn_kernel_d<128, false>(rope, norm);
+  return p.G == 8 ? attn_kernel_d<64, true>(rope, norm) : attn_kernel_d<64, false>(rope, norm);
 }
 
-void gp_launch_attention(const GpDev& p, const int* req_ids, int n_req, const void* q, const void* k, const void* v,
-                         float* out, int grid, cudaStream_t s, bool pdl, int lh0, int lh_n, int adv_lh) {
-  (void)req_ids;
-  const __nv_bfloat16* qq = static_cast<const __nv_bfloat16*>(q);
-  const __nv_bfloat16* kk = static_cast<const __nv_bfloat16*>(k);
-  const __nv_bfloat16* vv = static_cast<const __nv_bfloat16*>(v);
-  const bool rope = p.rope_theta != 0.0;
-  const int sm = (int)gp_attention_smem(p.d, p.G);
-#define GP_LAUNCH(DD, RR)                                                                 \
-  do {                                                                                    \
-    auto kern = gp_attn_kernel<DD, RR>;                                                   \
-    gp_launch(kern, grid, NTHREADS, (size_t)sm, s, pdl, p, n_req, qq, kk, vv, out, lh0, lh_n, adv_lh); \
-  } while (0)
-  if (p.d == 128) {
-    if (rope) GP_LAUNCH(128, true); else GP_LAUNCH(128, false);
-  } else {
-    if (rope) GP_LAUNCH(64, true); else GP_LAUNCH(64, false);
-  }
-#undef GP_LAUNCH
+void gp_attention_setup(const GpDev& p) {           // once per pool: opt into the kernels' shared memory
+  for (int norm = 0; norm < 2; ++norm)
+    cudaFuncSetAttribute(attn_kernel_of(p, norm != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp_attention_smem(p.d, p.G));
+}
+
+void gp_launch_attention(const GpDev& p, int n_req, const void* q, const void* k, const void* v, float* out, int grid, cudaStream_t s,
+                         bool pdl, int lh0, int lh_n, int adv_lh, const GpNorm& nm) {
+  gp_launch(attn_kernel_of(p, nm.wq != nullptr), grid, NTHREADS, gp_attention_smem(p.d, p.G), s, pdl, p, n_req,
+            static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), out, lh0,
+            lh_n, adv_lh, nm);
 }

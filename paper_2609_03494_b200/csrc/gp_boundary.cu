@@ -16,7 +16,6 @@
 //                     read" before the next chunk may overwrite their tail) or, with many units, a unit at a
 //                     time.  The last CTA swaps in the target pages, drops the references to the replaced ones
 //                     and returns the last page of every request that shrank.
-//   merge             of the partial attention outputs of requests that were split over several work items.
 //
 // It comes in two shapes that run the same device functions:
 //   gp_chain_kernel                       all of it in one kernel (the deciding CTA tells the others through a flag):
@@ -712,65 +711,6 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
   }
 }
 
-// Attention outputs of requests that were split over several work items: merges the items' partial results
-// (running maximum in the log2 domain, sum of exponentials, unnormalised output) into the output row.  A merge is a few
-// dependent round trips to the L2 and next to no work, so a query head's row is one warp's: the calling CTA takes rows
-// first, first + stride, ... of all CTAs' warps.  (A merge of a whole head group per thread block: 36 layers x 256 residents,
-// 12 000 merges per step, 80 us behind the selection.)
-template <int PER>     // head_dim / 32
-__device__ __forceinline__ void merge_rows(const GpDev& p, int n_req, float* __restrict__ out, int n_mc, int n_rc,
-                                           int first_block, int blocks, int lh0, int lh_n) {
-  constexpr int D = PER * 32;
-  const int G = p.G;
-  const int PSTRIDE = G * (D + 2);
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const long long rows = (long long)n_mc * lh_n * G;
-  for (long long mi = (long long)first_block * nw + (threadIdx.x >> 5); mi < rows; mi += (long long)blocks * nw) {
-    const int g = (int)(mi % G);
-    const long long u = mi / G;
-    const int4 mc = p.mc_list[u / lh_n];
-    const int lh = lh0 + (int)(u % lh_n), l = lh / p.Hkv, h = lh % p.Hkv;       // units [lh0, lh0 + lh_n)
-    const int bi = mc.x, nch = mc.z;
-    const float* pg = p.partials + ((size_t)lh * n_rc + mc.y) * PSTRIDE + g * (D + 2);
-    float* orow = out + (((size_t)l * n_req + bi) * p.Hq + h * G + g) * D;
-    float M = -INFINITY, ls = 0.f, acc[PER];
-#pragma unroll
-    for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-    for (int c0 = 0; c0 < nch; c0 += 4) {                 // four items' values in flight together
-      float m[4], lv[4], vv[4][PER];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float* pc = pg + (size_t)(c0 + k) * PSTRIDE;
-        const bool on = c0 + k < nch;
-        m[k] = on ? __ldcg(pc + D) : -INFINITY;
-        lv[k] = on ? __ldcg(pc + D + 1) : 0.f;
-#pragma unroll
-        for (int e = 0; e < PER; ++e) vv[k][e] = on ? __ldcg(pc + lane + 32 * e) : 0.f;
-      }
-      const float Mn = fmaxf(fmaxf(M, fmaxf(m[0], m[1])), fmaxf(m[2], m[3]));
-      const float sc = exp2f(M - Mn);
-      ls *= sc;
-#pragma unroll
-      for (int e = 0; e < PER; ++e) acc[e] *= sc;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float w = exp2f(m[k] - Mn);
-        ls += w * lv[k];
-#pragma unroll
-        for (int e = 0; e < PER; ++e) acc[e] += w * vv[k][e];
-      }
-      M = Mn;
-    }
-#pragma unroll
-    for (int e = 0; e < PER; ++e) orow[lane + 32 * e] = acc[e] / ls;
-  }
-}
-__device__ __noinline__ void merge_partials(const GpDev& p, int n_req, float* __restrict__ out, int n_mc, int n_rc,
-                                            int first_block, int blocks, int lh0, int lh_n) {
-  if (p.d == 128) merge_rows<4>(p, n_req, out, n_mc, n_rc, first_block, blocks, lh0, lh_n);
-  else merge_rows<2>(p, n_req, out, n_mc, n_rc, first_block, blocks, lh0, lh_n);
-}
-
 // ------------------------------------------------------------------------------------------------------
 // working sets + speculative eviction lists of a unit, one CTA; the last CTA decides
 // ------------------------------------------------------------------------------------------------------
@@ -899,7 +839,7 @@ __device__ __forceinline__ void count_shared(const GpDev& p, int e) {
 template <int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions,
-               float* __restrict__ out, int serial, int decide) {
+               int by_layer, int serial, int decide) {
   // decide == 0: the step of a pool that holds a part of the model's KV heads: the last thread block only hands
   // out the sums of K^S and K^L per boundary request; the decisions follow in a kernel of their own once the
   // sums of all parts are added up
@@ -921,19 +861,11 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     if (b0 < p.M) { inf_first = __ldcg(p.bnd_info + 2 * b0); inf2_first = __ldcg(p.bnd_info + 2 * b0 + 1); }
   }
   const int n_bnd = __ldcg(p.hdr + HDR_N_BND);
-  const int n_mc = out ? __ldcg(p.hdr + HDR_N_MC) : 0, n_rc = __ldcg(p.hdr + HDR_N_RC);   // out == null: already merged layer by layer
+  const int n_rc = __ldcg(p.hdr + HDR_N_RC);
   const int NJ = jobs_per_unit((long long)n_bnd * LH, gridDim.x);
   const long long items = (long long)n_bnd * LH * NJ;
   gp_pdl_wait();
   gp_pdl_launch_dependents();
-
-  // CTAs without a unit merge the split requests' attention partials while the others work; when fewer than a
-  // quarter of the CTAs are idle, everybody merges after the units instead
-  const long long n_busy = items + n_bnd < (long long)gridDim.x ? items + n_bnd : (long long)gridDim.x;
-  const int n_idle = (int)gridDim.x - (int)n_busy;
-  const bool idle_merge = n_idle * 4 >= (int)gridDim.x;
-  if (idle_merge && (long long)blockIdx.x >= n_busy)
-    merge_partials(p, n_req, out, n_mc, n_rc, (int)blockIdx.x - (int)n_busy, n_idle, 0, LH);
 
   for (long long item = blockIdx.x; item < items + n_bnd; item += gridDim.x) {
     if (item >= items) { count_shared(p, (int)(item - items)); continue; }
@@ -955,23 +887,10 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   __syncthreads();
   if (s_i[2]) {
     __threadfence();
-    if (!out) advance_counters(p, n_rc);
+    if (by_layer) advance_counters(p, n_rc);
     if (decide) decide_and_allocate(p, req_ids, n_req, n_bnd, actions, reinterpret_cast<int*>(S.loc), serial);
     else publish_shard_sums(p, n_bnd);
   }
-
-  if (!idle_merge) merge_partials(p, n_req, out, n_mc, n_rc, (int)gridDim.x - 1 - (int)blockIdx.x, (int)gridDim.x, 0, LH);
-}
-
-// merges the partial outputs of the split requests for the units [lh0, lh0 + lh_n): the per-layer entry point
-// needs a layer's output complete before the next layer's query exists
-__global__ void __launch_bounds__(256)
-gp_merge_kernel(const __grid_constant__ GpDev p, int n_req, float* __restrict__ out, int lh0, int lh_n) {
-  // the kernel after this one may be scheduled at once: it waits for this grid's end where it needs to, and this
-  // grid ends after the attention kernel (the wait below), so completion stays transitive
-  gp_pdl_launch_dependents();
-  gp_pdl_wait();
-  merge_partials(p, n_req, out, p.hdr[HDR_N_MC], p.hdr[HDR_N_RC], (int)blockIdx.x, (int)gridDim.x, lh0, lh_n);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -1249,18 +1168,16 @@ gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_i
 // ------------------------------------------------------------------------------------------------------
 // Launched right behind the attention kernel of step t + 1 as its programmatic dependent, this grid works on the
 // boundary chain of step t: it does not wait for that attention kernel before it starts (everything it reads
-// was complete before that kernel could start), runs the selection jobs, lets the last CTA to finish them
+// was complete before that kernel could start), runs the selection, lets the last CTA to finish it
 // decide and allocate, waits inside the grid for that (a bounded wait on a flag: the grid is sized to be
 // resident at once, on the room the attention kernel leaves), compacts, and only then waits for the attention
-// kernel to end; after that it merges the split requests' partial outputs of step t + 1.  The grid therefore
-// ends after both, and the plan of step t + 2, its programmatic dependent, finds the pages and counters of the
-// requests that sat step t + 1 out in their final state.  `p`: the view of step t (its scratch set, the copy of
-// the counters its decisions go to); `pa`: the view of step t + 1 (for the merge).
+// kernel to end.  The grid therefore ends after both, and the plan of step t + 2, its programmatic dependent, finds the
+// pages and counters of the requests that sat step t + 1 out in their final state.  `p`: the view of step t (its
+// scratch set, the copy of the counters its decisions go to).
 template <int D, int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
-gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev pa, int n_req_merge, float* __restrict__ out_merge,
-                int serial, int has_chain, const int* __restrict__ req_ids, int* __restrict__ actions,
-                int* __restrict__ actions_copy) {
+gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_chain, const int* __restrict__ req_ids,
+                int* __restrict__ actions, int* __restrict__ actions_copy) {
   // actions_copy: where the step's actions are wanted as well once they are final (the host entry points: the
   // caller's array in page-locked host memory; writing them there from the plan kernel made that kernel wait
   // for the bus)
@@ -1313,7 +1230,7 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
     __syncthreads();
     if (s_i[2]) {
       __threadfence();
-      decide_and_allocate(p, req_ids, n_req_merge, n_bnd, same_step ? actions : nullptr, reinterpret_cast<int*>(S.loc), serial);
+      decide_and_allocate(p, req_ids, n_req, n_bnd, same_step ? actions : nullptr, reinterpret_cast<int*>(S.loc), serial);
       __syncthreads();
       if (tid == 0 && !(p.withhold & GP_WITHHOLD_DECIDED)) {      // (test support: see GP_WITHHOLD_DECIDED)
         __threadfence();
@@ -1328,15 +1245,13 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
     }
     __syncthreads();
     if (same_step) {
-      // The attention kernel of this step has ended by now (the decisions needed its last reports): the split
-      // requests' outputs are merged first, and then the next kernel on the stream may be scheduled.  With early
-      // planning that is the next step's plan, which so runs beside the compaction below: the decisions it reads
-      // are taken, the attention kernel has moved the requests on, and the compaction reads nothing the plan writes
-      // (the merge does: the lists of split requests, hence its place before).
+      // The attention kernel of this step has all but ended by now (the decisions needed its last reports).  From here on the
+      // next kernel on the stream may be scheduled.  With early planning that is the next step's plan, which so runs
+      // beside the compaction below: the decisions it reads are taken, the attention kernel has moved the requests on, and
+      // the compaction reads nothing the plan writes.
       gp_pdl_wait();
       if (actions_copy && blockIdx.x == gridDim.x - 1)
-        for (int i = tid; i < n_req_merge; i += SEL_T) actions_copy[i] = __ldcg(actions + i);
-      if (out_merge) merge_partials(pa, n_req_merge, out_merge, pa.hdr[HDR_N_MC], pa.hdr[HDR_N_RC], (int)blockIdx.x, (int)gridDim.x, 0, LH);
+        for (int i = tid; i < n_req; i += SEL_T) actions_copy[i] = __ldcg(actions + i);
       gp_pdl_launch_dependents();
     }
     // ---- compaction: its arrays take the place of the selection's -----------------------------------------------
@@ -1344,7 +1259,6 @@ gp_chain_kernel(const __grid_constant__ GpDev p, const __grid_constant__ GpDev p
   }
   if (same_step) return;
   gp_pdl_wait();              // the attention kernel beside which this grid ran has ended
-  if (out_merge) merge_partials(pa, n_req_merge, out_merge, pa.hdr[HDR_N_MC], pa.hdr[HDR_N_RC], (int)blockIdx.x, (int)gridDim.x, 0, LH);
 }
 
 // the decisions of a step whose sums of K^S and K^L were completed outside (KV heads spread over several pools)
@@ -1361,11 +1275,11 @@ gp_decide_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_id
 static auto compact_kernel_of(const GpDev& p) -> void (*)(const GpDev, const int*, int, int) {
   return p.d == 128 ? gp_compact_kernel<128> : gp_compact_kernel<64>;
 }
-typedef void (*SelKernel)(const GpDev, const int*, int, int*, float*, int, int);
+typedef void (*SelKernel)(const GpDev, const int*, int, int*, int, int, int);
 static SelKernel sel_kernel_of(const GpDev& p) {
   return p.G == 1 ? gp_bsel_kernel<1> : p.G == 2 ? gp_bsel_kernel<2> : p.G == 4 ? gp_bsel_kernel<4> : gp_bsel_kernel<8>;
 }
-typedef void (*ChainKernel)(const GpDev, const GpDev, int, float*, int, int, const int*, int*, int*);
+typedef void (*ChainKernel)(const GpDev, int, int, int, const int*, int*, int*);
 template <int D> static ChainKernel chain_kernel_d(const GpDev& p) {
   return p.G == 1 ? gp_chain_kernel<D, 1> : p.G == 2 ? gp_chain_kernel<D, 2> : p.G == 4 ? gp_chain_kernel<D, 4> : gp_chain_kernel<D, 8>;
 }
@@ -1395,17 +1309,15 @@ void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_com
   *grid_compact = blocks(compact_kernel_of(p), CT, 0, 32);
 }
 
-// asynchronous mode: the boundary chain of the step whose view is `p` (none when !has_chain), and afterwards the
-// merge of the split requests' partial outputs of the step whose view is `pa` (none when out_merge is null)
-void gp_launch_chain(const GpDev& p, const GpDev& pa, int n_req_merge, float* out_merge, int serial, int has_chain, int grid,
-                     cudaStream_t s, bool pdl, const int* req_ids, int* actions, int* actions_copy) {
-  gp_launch(chain_kernel_of(p), grid, SEL_T, gp_sel_smem(p), s, pdl, p, pa, n_req_merge, out_merge, serial, has_chain, req_ids,
-            actions, actions_copy);
+// the boundary chain of the step whose view is `p` (asynchronous mode: none when !has_chain)
+void gp_launch_chain(const GpDev& p, int n_req, int serial, int has_chain, int grid, cudaStream_t s, bool pdl, const int* req_ids,
+                     int* actions, int* actions_copy) {
+  gp_launch(chain_kernel_of(p), grid, SEL_T, gp_sel_smem(p), s, pdl, p, n_req, serial, has_chain, req_ids, actions, actions_copy);
 }
 
-void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel, cudaStream_t s,
-                           bool pdl, int serial) {
-  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl, p, req_ids, n_req, actions, out, serial, 0);
+void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_sel, cudaStream_t s, bool pdl,
+                           int serial) {
+  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl, p, req_ids, n_req, actions, 0, serial, 0);
 }
 
 // plain launches: what comes before them on the stream (the caller's reduction of the sums) is not this library's
@@ -1415,15 +1327,11 @@ void gp_launch_decide_compact(const GpDev& p, const int* req_ids, int n_req, int
   gp_launch(compact_kernel_of(p), grid_compact, CT, 0, s, true, p, req_ids, n_req, serial);
 }
 
-void gp_launch_merge(const GpDev& p, int n_req, float* out, int lh0, int lh_n, int grid, cudaStream_t s, bool pdl) {
-  gp_launch(gp_merge_kernel, grid, 256, 0, s, pdl, p, n_req, out, lh0, lh_n);
-}
-
-void gp_launch_boundary(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel,
+void gp_launch_boundary(const GpDev& p, const int* req_ids, int n_req, int* actions, bool by_layer, int grid_sel,
                         int grid_compact, cudaStream_t s, cudaEvent_t ev, bool pdl, int serial) {
   // asynchronous mode: the kernel before this one on its stream belongs to another step (an event wait lies in
   // between): plain launch; the compaction kernel follows as a programmatic dependent as usual
-  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl && !p.async, p, req_ids, n_req, actions, out, serial, 1);
+  gp_launch(sel_kernel_of(p), grid_sel, SEL_T, gp_sel_smem(p), s, pdl && !p.async, p, req_ids, n_req, actions, by_layer ? 1 : 0, serial, 1);
   if (ev) cudaEventRecord(ev, s);
   gp_launch(compact_kernel_of(p), grid_compact, CT, 0, s, pdl, p, req_ids, n_req, serial);
 }

@@ -41,7 +41,7 @@ enum {
   HDR_DONE_SEL,      // CTAs of the selection kernel that have finished
   HDR_WORK_CMP,      // ticket counter of the compaction kernel
   HDR_N_CITEM,       // compaction work items (chunks x layers x heads)
-  HDR_N_MC,          // requests whose attention was split over several work items
+  HDR_FREE,          // (not in use)
   HDR_N_COW,         // copy-on-write targets allotted this step
   HDR_COUNT = 16
 };
@@ -111,7 +111,7 @@ struct GpDev {
                                          //   6 n before the append, 7 position, 8 flags (1 boundary, 2 started),
                                          //   9 P, 10-11 offset into the logit scratch, 12 summary buffer in use,
                                          //   13 index of its partial-output slot
-  int4* mc_list;                         // [M] split requests: {batch index, first partial, chunks, 0}
+  int* merge_cnt;                        // [max_rc * L H_kv] per unit of a split request and chunk: partial outputs that are there (zero between steps)
   int4* bnd_info;                        // [M][2] requests at a boundary: {slot in the batch, request, P, position of the step's token}, {score offset lo, hi, 0, 0}
   int* shard_sums;                       // [M][2] per boundary request: sum of K^S, sum of K^L over this pool's units (to be
                                          // summed over the pools that hold the other KV heads), then over all units
@@ -124,13 +124,15 @@ struct GpDev {
   int4* cmp_info;                        // [M+1] compressing requests: {request, P, index in bnd_info, first compaction chunk}
   double* zbuf;                          // [L*H_kv][2][z_stride][G] boundary units, per view (short, long): exp(summary logit - its page's max)
   long long z_stride;                    // max_boundary_tokens rounded up to a multiple of the page size
-  double* qtil;                          // [M][L*H_kv][2][G][d] calibrated, rotated summaries q~ of boundary requests, by batch slot
   double* zstat;                         // [L*H_kv][max_boundary_tokens / b][2][G][2] per-page softmax partials (max, sum)
   int* sum_par;                          // [M] which of the two summary buffers is current
   int* evict;                            // [M][L*H_kv][page_size] slots a compression evicts, ascending
   int* evict2;                           // [M][L*H_kv][2 page_size] slots a Shrink evicts, ascending (Shrink policy only)
   int* cflags;                           // compaction chunk flags, stamped with the step number
-  double* rope_cs;                       // [M][d/2][2] cos, sin at the step's position
+  int* tickets;                          // [L] next attention work item to draw: of the whole step (0) or of a layer's launch
+  double* inv_freq;                      // [d/2] rope_theta^(-2j/d)
+  float* rope_f;                         // [M][d/2][2] cos, sin at the step's position in fp32 (the queries' rotation)
+  double* rope_cs;                       // [M][d/2][2] the same in fp64
   float* partials;
   double* scores;
   long long* counters;                   // [16]
@@ -247,8 +249,14 @@ __device__ __forceinline__ float bf16_lo_f(uint32_t w) { return __uint_as_float(
 __device__ __forceinline__ float bf16_hi_f(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // ---- host-visible launchers (one per translation unit) -------------------------------------------
-void gp_launch_attention(const GpDev& p, const int* req_ids, int n_req, const void* q, const void* k, const void* v,
-                         float* out, int grid, cudaStream_t s, bool pdl, int lh0, int lh_n, int adv_lh);
+// Fused QK-norm of the layer-by-layer entry (null weights: queries and keys arrive normalised): queries and keys of the call
+// are raw, the attention kernel normalises them per head (RMS over the head dimension, a learned weight per element).
+struct GpNorm {
+  const float* wq; const float* wk;
+  double eps;
+};
+void gp_launch_attention(const GpDev& p, int n_req, const void* q, const void* k, const void* v, float* out, int grid, cudaStream_t s,
+                         bool pdl, int lh0, int lh_n, int adv_lh, const GpNorm& nm);
 size_t gp_attention_smem(int d, int G);
 int gp_attention_ctas_per_sm(int d);
 // ---- programmatic dependent launch -------------------------------------------------------------------
@@ -276,17 +284,16 @@ inline cudaError_t gp_launch(void (*kern)(KArgs...), int grid, int block, size_t
 #endif
 
 void gp_attention_setup(const GpDev& p);
-void gp_launch_chain(const GpDev& p, const GpDev& pa, int n_req_merge, float* out_merge, int serial, int has_chain, int grid,
-                     cudaStream_t s, bool pdl, const int* req_ids = nullptr, int* actions = nullptr, int* actions_copy = nullptr);
-// merge of the split requests' partial outputs for the units [lh0, lh0 + lh_n) (per-layer entry point)
-void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel, cudaStream_t s,
-                           bool pdl, int serial);
+void gp_launch_chain(const GpDev& p, int n_req, int serial, int has_chain, int grid, cudaStream_t s, bool pdl,
+                     const int* req_ids = nullptr, int* actions = nullptr, int* actions_copy = nullptr);
+void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_sel, cudaStream_t s, bool pdl,
+                           int serial);
 void gp_launch_decide_compact(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_compact, cudaStream_t s,
                               int serial);
-void gp_launch_merge(const GpDev& p, int n_req, float* out, int lh0, int lh_n, int grid, cudaStream_t s, bool pdl);
 void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain);
 #define GP_MAX_DYN_SMEM (227 * 1024)   // opt-in shared memory per CTA on sm_100
 // boundary chain: probabilities + working sets + selection + decision, then compaction.
 // `ev`, when not null, is recorded between the two kernels.  `pdl`: launch with programmatic stream serialization.
-void gp_launch_boundary(const GpDev& p, const int* req_ids, int n_req, int* actions, float* out, int grid_sel,
+// `by_layer`: the step's end after layer-by-layer launches (the requests' counters move on here).
+void gp_launch_boundary(const GpDev& p, const int* req_ids, int n_req, int* actions, bool by_layer, int grid_sel,
                         int grid_compact, cudaStream_t s, cudaEvent_t ev, bool pdl, int serial);

@@ -47,7 +47,6 @@ struct gp_pool {
   long long host_waited;                            // gp_decode_step_host_async calls whose results have been waited for
   long long host_async_issued;                      // ... and issued
   int host_async_set[2];                            // the staging sets of the (at most two) calls not yet waited for
-  __nv_bfloat16* qn; __nv_bfloat16* kn;             // one layer's normalised queries and keys (gp_attn_layer_qknorm)
   // small device words
   int* d_status;
   uint8_t* dbg;                   // gather target of the debug getters
@@ -68,10 +67,10 @@ namespace {
 
 struct Layout {
   size_t kv, tok, refcount, free_stack, words, page_table, shadow, reqi, pos, summ, Kx, Hx, delta, rc,
-      mc_list, bnd_info, bnd_acc, free_peek, cmp_info, zbuf, qtil, zstat, sum_par,
-      unit_ready, shard_sums, bnd_info2, bnd_acc2, zbuf2, zstat2, rc2, mc_list2, qtil2, rope_cs2,
+      merge_cnt, bnd_info, bnd_acc, free_peek, cmp_info, zbuf, zstat, sum_par, inv_freq, tickets, rope_f,
+      unit_ready, shard_sums, bnd_info2, bnd_acc2, zbuf2, zstat2, rc2, rope_cs2, rope_f2,
       evict, evict2, cflags, rope_cs, partials, scores, counters, dbg,
-      st_ids, st_q, st_k, st_v, st_out, st_act, st2_ids, st2_q, st2_k, st2_v, qn, kn, total;
+      st_ids, st_q, st_k, st_v, st_out, st_act, st2_ids, st2_q, st2_k, st2_v, total;
   int max_rc;
   long long max_batch_tokens, max_boundary_tokens;
 };
@@ -153,7 +152,7 @@ Layout make_layout(const gp_config& c) {
   L.Hx = take(c.demand_metric == GP_METRIC_ENTROPY ? M * LH * 2 * 8 : 16);
   L.delta = take(M * 8);
   L.rc = take((size_t)L.max_rc * GP_DESC_INTS * 4);
-  L.mc_list = take(M * 16);
+  L.merge_cnt = take((size_t)L.max_rc * LH * 4);
   L.bnd_info = take(M * 32);
   L.bnd_acc = take(M * 16);
   L.unit_ready = take((size_t)M * LH * 4);
@@ -161,11 +160,13 @@ Layout make_layout(const gp_config& c) {
   L.free_peek = take((M + 1) * 4);
   L.cmp_info = take((M + 1) * 16);
   L.zbuf = take(LH * (Tb + b) * 2 * G * 8);
-  L.qtil = take(M * LH * 2 * (size_t)G * d * 8);
   L.zstat = take(LH * (Tb / b + 1) * 2 * G * 2 * 8);
   L.evict = take(M * LH * blk * 4);
   L.evict2 = take(c.policy == GP_POLICY_SHRINK ? M * LH * 2 * blk * 4 : 16);
   L.cflags = take(LH * ((Tb + M * b) / GP_MOVE_TOK + 2 * M + 1) * 4);
+  L.inv_freq = take(d / 2 * 8);
+  L.tickets = take((size_t)c.n_layers * 4);
+  L.rope_f = take(M * (d / 2) * 2 * 4);
   L.rope_cs = take(M * (d / 2) * 2 * 8);
   L.partials = take((size_t)L.max_rc * LH * G * (d + 2) * 4);
   L.scores = take((c.policy == GP_POLICY_SHRINK ? 4 : 3) * LH * Tb * 8);
@@ -176,11 +177,10 @@ Layout make_layout(const gp_config& c) {
     L.zstat2 = take(LH * (Tb / b + 1) * 2 * G * 2 * 8);
     // and of what the plan of a step writes while the attention kernel of the step before may still read its own
     L.rc2 = take((size_t)L.max_rc * GP_DESC_INTS * 4);
-    L.mc_list2 = take(M * 16);
-    L.qtil2 = take(M * LH * 2 * (size_t)G * d * 8);
     L.rope_cs2 = take(M * (d / 2) * 2 * 8);
+    L.rope_f2 = take(M * (d / 2) * 2 * 4);
   } else {
-    L.bnd_info2 = L.bnd_acc2 = L.zbuf2 = L.zstat2 = L.rc2 = L.mc_list2 = L.qtil2 = L.rope_cs2 = 0;
+    L.bnd_info2 = L.bnd_acc2 = L.zbuf2 = L.zstat2 = L.rc2 = L.rope_cs2 = L.rope_f2 = 0;
   }
   L.counters = take(16 * 8);
   L.dbg = take(cap * b * (4 + 2 * d * 2));
@@ -198,8 +198,6 @@ Layout make_layout(const gp_config& c) {
   } else {
     L.st_ids = L.st_q = L.st_k = L.st_v = L.st_out = L.st_act = L.st2_ids = L.st2_q = L.st2_k = L.st2_v = 0;
   }
-  L.qn = take(M * c.n_q_heads * d * 2);              // one layer's normalised queries and keys (fused QK-norm)
-  L.kn = take(M * c.n_kv_heads * d * 2);
   L.total = o;
   return L;
 }
@@ -214,6 +212,7 @@ __global__ void gp_init_kernel(GpDev p) {
   for (long long i = i0; i < p.n_pages; i += stride) p.free_stack[i] = (int)(p.n_pages - 1 - i);
   for (long long i = i0; i < (long long)p.M * p.cap; i += stride) p.shadow[i] = -1;
   for (long long i = i0; i < p.M; i += stride) p.bstep[i] = GP_NEVER;
+  for (long long i = i0; i < p.d / 2; i += stride) p.inv_freq[i] = p.rope_theta != 0.0 ? pow(p.rope_theta, -2.0 * (double)i / (double)p.d) : 0.0;
   if (i0 == 0) *p.free_top = (int)p.n_pages;
 }
 
@@ -250,216 +249,54 @@ __device__ __forceinline__ void plan_scan(int v, long long w, int& ev, long long
   __syncthreads();
 }
 
-// Fused QK-norm of the layer-by-layer entry (null weights: queries and keys arrive normalised).  Queries and keys
-// of the call are raw; the summary CTAs, which read every query row anyway, normalise them per head (RMS over the
-// head dimension, a learned weight per element), rotate the key to its cache form and leave both, rounded to
-// bf16, where the attention kernel then finds them.
-struct GpNorm {
-  const float* wq; const float* wk;
-  double eps;
-  const __nv_bfloat16* k_raw;
-  __nv_bfloat16* qn; __nv_bfloat16* kn;
-};
-
-// double -> float -> bf16, each round-to-nearest-even (the order a host library takes)
-__device__ __forceinline__ __nv_bfloat16 to_bf16(double x) { return __float2bfloat16_rn((float)x); }
-
-// Summary update of one (batch slot, layer, KV head) unit, run by the CTAs of the plan kernel other than the
-// first, concurrently with the planning: Eq. 6 on the un-rotated query of every head of the group (read from
-// one of the request's two buffers, written to the other; the decision step flips the buffers of the requests
-// that were really stepped, so a unit that turns out not to step leaves no trace), and, for a request that
-// reaches its capacity boundary, the calibrated (Eq. 12) and rotated summaries q~ in fp64 for the attention
-// kernel's logits.  One warp per (view, head) row; a CTA takes as many units at a time as its warps cover.
-template <int D>
-__device__ void prepare_row(const GpDev& p, int n_req, const __nv_bfloat16* __restrict__ q, int bi, int lh, int row, int r,
-                            int n_old, int Pr, int started, int par, long long pos, const GpNorm& nm) {
-  constexpr int PER = D / 32;
-  const int lane = threadIdx.x & 31;
-  const int G = p.G;
-  const int l = lh / p.Hkv, h = lh % p.Hkv;
-  const int x = row / G, g = row % G;
-  const int head = h * G + g;
-  // one round trip: the query row and the old summary from the request's current buffer (the request's state
-  // was staged in shared memory by the CTA)
-  const __nv_bfloat16* qrow = q + (((size_t)l * n_req + bi) * p.Hq + head) * D;
-  float qf[PER];
-#pragma unroll
-  for (int e = 0; e < PER; ++e) qf[e] = __bfloat162float(qrow[lane + 32 * e]);
-  if (nm.wq) {
-    // the raw query row becomes the normalised one (Sec. 3.2: the summaries follow the query after its
-    // normalisation and before its rotation); the short view's warp leaves it for the attention kernel
-    double ssq = 0.0;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) ssq += (double)qf[e] * (double)qf[e];
-#pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o2);
-    const double scale = 1.0 / sqrt(ssq / (double)D + nm.eps);
-    __nv_bfloat16* qout = nm.qn + (((size_t)l * n_req + bi) * p.Hq + head) * D;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      const __nv_bfloat16 v = to_bf16((double)qf[e] * scale * (double)nm.wq[lane + 32 * e]);
-      qf[e] = __bfloat162float(v);
-      if (x == 0) qout[lane + 32 * e] = v;
-    }
-    if (row == 0) {                        // the unit's key row: normalise, rotate to the token's position, leave
-      const __nv_bfloat16* krow = nm.k_raw + (((size_t)l * n_req + bi) * p.Hkv + h) * D;
-      double kv[PER];
-      double ks = 0.0;
-#pragma unroll
-      for (int e = 0; e < PER; ++e) { kv[e] = (double)__bfloat162float(krow[lane + 32 * e]); ks += kv[e] * kv[e]; }
-#pragma unroll
-      for (int o2 = 16; o2 > 0; o2 >>= 1) ks += __shfl_xor_sync(0xffffffffu, ks, o2);
-      const double kscale = 1.0 / sqrt(ks / (double)D + nm.eps);
-#pragma unroll
-      for (int e = 0; e < PER; ++e) kv[e] = kv[e] * kscale * (double)nm.wk[lane + 32 * e];
-      __nv_bfloat16* kout = nm.kn + (((size_t)l * n_req + bi) * p.Hkv + h) * D;
-      if (p.rope_theta != 0.0) {
-#pragma unroll
-        for (int e = 0; e < PER / 2; ++e) {
-          const int j = lane + 32 * e;
-          const double inv = pow(p.rope_theta, -2.0 * (double)j / (double)D);
-          double si, co;
-          sincos((double)pos * inv, &si, &co);
-          kout[j] = to_bf16(kv[e] * co - kv[e + PER / 2] * si);
-          kout[j + D / 2] = to_bf16(kv[e + PER / 2] * co + kv[e] * si);
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < PER; ++e) kout[lane + 32 * e] = to_bf16(kv[e]);
-      }
-    }
-  }
-  double ovv[PER];
-  {
-    const double* o0 = p.summ + gp_summ_off(p, l, r, par, x, head);
-#pragma unroll
-    for (int e = 0; e < PER; ++e) ovv[e] = __ldcg(o0 + lane + 32 * e);
-  }
-  const bool need_qt = (n_old + 1 == Pr * GP_PAGE) && Pr > 1;
-  {
-    const double beta = x ? p.beta_l : p.beta_s;
-    double* newp = p.summ + gp_summ_off(p, l, r, par ^ 1, x, head);
-    double nv[PER];
-    double sq = 0.0, ss = 0.0;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      const double qv = (double)qf[e];
-      const double ov = ovv[e];
-      sq += qv * qv;
-      nv[e] = started ? beta * ov + (1.0 - beta) * qv : qv;              // Eq. 6
-      newp[lane + 32 * e] = nv[e];
-      ss += nv[e] * nv[e];
-    }
-    if (need_qt) {
-#pragma unroll
-      for (int o2 = 16; o2 > 0; o2 >>= 1) {
-        sq += __shfl_xor_sync(0xffffffffu, sq, o2);
-        ss += __shfl_xor_sync(0xffffffffu, ss, o2);
-      }
-      // Eq. 12
-      const double gamma = ss > 0.0 ? sqrt(sq / (double)D) / sqrt(ss / (double)D) : 1.0;
-      double* dst = p.qtil + (((size_t)bi * p.L * p.Hkv + lh) * 2 * G + row) * D;
-      if (p.rope_theta != 0.0) {
-#pragma unroll
-        for (int e = 0; e < PER / 2; ++e) {
-          const int j = lane + 32 * e;
-          const double inv = pow(p.rope_theta, -2.0 * (double)j / (double)D);
-          double si, co;
-          sincos((double)pos * inv, &si, &co);
-          const double x1 = gamma * nv[e], x2 = gamma * nv[e + PER / 2];
-          dst[j] = x1 * co - x2 * si;
-          dst[j + D / 2] = x2 * co + x1 * si;
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < PER; ++e) dst[lane + 32 * e] = gamma * nv[e];
-      }
-    }
-  }
-}
-
 // Step plan: validates the batch, cuts every stepped request into chunks and writes one work descriptor
 // per chunk for the attention kernel, lists the requests that reach their capacity boundary with this
-// step's append (trailing check: n + 1 == P b) and hands each a slice of the logit scratch.
+// step's append (trailing check: n + 1 == P b) and hands each a slice of the logit scratch.  With rotary embeddings the other
+// CTAs write the cosines and sines of the requests' positions.
 __global__ void __launch_bounds__(GP_PLAN_THREADS)
-gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions,
-               const __nv_bfloat16* __restrict__ q, int plan_on, int lh0, int lh_n, int cp_norm, int cp_bnd,
-               int launch_units, int launch_grid, int serial, const GpNorm nm) {
+gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions, int early,
+               int cp_norm, int cp_bnd, int launch_units, int launch_grid, int serial) {
   // serial: number of this decode step (asynchronous boundary mode: a request that reached its boundary at
   // step serial - 1 sits this step out; its counters and pages belong to that step's boundary chain, which may
   // still be running)
   // cp_norm, cp_bnd: pages per work item, for requests in general and for those at their capacity boundary, when
   // the attention launch has work for large items; launch_units: (layer, head) units per request in one
   // attention launch; launch_grid: its CTAs
-  // plan_on: 0: no planning (the per-layer calls after the step's first); 1: CTA 0 plans; 2: CTA 0 plans and
-  // the caller's inputs may be read before the wait for the preceding kernel (see below).  The summary CTAs
-  // cover the (layer, KV head) units [lh0, lh0 + lh_n) (none when lh_n is 0: the query rows come layer by layer)
+  // early: the caller's request ids may be read before the wait for the preceding kernel (see below)
   __shared__ int sv[33];
   __shared__ long long sw[33];
   __shared__ __align__(16) int s_first[GP_MAX_REQ];      // lowest batch index naming a request
-  __shared__ int s_chunks[GP_MAX_REQ], s_pos[GP_MAX_REQ];
-  __shared__ int s_req[GP_MAX_REQ], s_state[GP_MAX_REQ];     // summary CTAs: request of a batch slot, flags
-  __shared__ long long s_pos64[GP_MAX_REQ];
-  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS], s_nmc;
+  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS];
   const int i = threadIdx.x;
   const bool in = i < n_req;
   // What runs before the wait for the kernel before this one.  In a whole-step launch that kernel is the
   // compaction of the step before (or something the caller put in between, which then has completed): this
   // grid became schedulable only after that step's decisions had completed, and compaction touches neither the
-  // requests' counters, nor the summaries, nor anything the plan writes except the step stamp.  So the summary
-  // CTAs do not wait at all, and CTA 0 plans the whole step first and waits only before it looks at the free
-  // list (which compaction's last CTA may still change) and stamps the step.  CTA 0 does wait, so the grid as
-  // a whole still ends after everything before it.  The layer-by-layer launches (plan_on == 0) have no CTA 0
-  // work and keep the wait in every CTA, so that completion stays transitive.  The next kernel may be scheduled
+  // requests' counters nor anything the plan writes except the step stamp.  So CTA 0 plans the whole step first and waits
+  // only before it looks at the free list (which compaction's last CTA may still change) and stamps the step.  CTA 0 does
+  // wait, so the grid as a whole still ends after everything before it.  The next kernel may be scheduled
   // as soon as every CTA of this grid has started; it waits for this grid's end at its own top.
-  // All of this reads the caller's request ids and queries before the wait, which is only right if they were
-  // complete before the preceding kernel could signal: the caller says so (plan_on == 2); otherwise every CTA
+  // All of this reads the caller's request ids before the wait, which is only right if they were
+  // complete before the preceding kernel could signal: the caller says so (`early`); otherwise every CTA
   // waits first (the later wait of CTA 0 is then a no-op).
-  if (plan_on != 2) gp_pdl_wait();
+  if (!early) gp_pdl_wait();
   gp_pdl_launch_dependents();
-  if (blockIdx.x > 0) {                       // summary CTAs: one warp per (unit, view, head)
-    // The state of the batch's requests is staged once per CTA, from the L2 (these CTAs may run before the wait,
-    // and an L1 line could date from the step before): request of a slot (-1: not stepped by these CTAs:
-    // out of range, dead, or named by an earlier slot), tokens, pages, flags, position.
-    if (i < GP_MAX_REQ) s_first[i] = 0x7fffffff;
-    __syncthreads();
-    int r = -1;
-    if (in) {
-      r = req_ids[i];
-      if (r >= 0 && r < p.M) atomicMin(&s_first[r], i); else r = -1;
-    }
-    __syncthreads();
-    if (in) {
-      int ok = 0;
-      if (r >= 0 && s_first[r] == i && __ldcg(p.live + r) && !(p.async && __ldcg(p.bstep + r) == serial - 1)) {
-        ok = 1;
-        s_chunks[i] = __ldcg(p.n + r);
-        s_pos[i] = __ldcg(p.P + r);
-        s_state[i] = (__ldcg(p.started + r) ? 1 : 0) | (__ldcg(p.sum_par + r) ? 2 : 0);
-        s_pos64[i] = __ldcg(p.pos + r);
-      }
-      s_req[i] = ok ? r : -1;
-    }
-    __syncthreads();
-    const int rows = 2 * p.G, upc = 32 / rows;             // units per CTA and pass
-    const int warp = threadIdx.x >> 5;
-    const long long units = (long long)n_req * lh_n;
-    if (warp < upc * rows) {
-      for (long long u = ((long long)blockIdx.x - 1) * upc + warp / rows; u < units; u += ((long long)gridDim.x - 1) * upc) {
-        const int bi = (int)(u / lh_n), lh = lh0 + (int)(u % lh_n);
-        const int rr = s_req[bi];
-        if (rr < 0) continue;
-        const int st = s_state[bi];
-        if (p.d == 128) prepare_row<128>(p, n_req, q, bi, lh, warp % rows, rr, s_chunks[bi], s_pos[bi], st & 1, (st >> 1) & 1, s_pos64[bi], nm);
-        else prepare_row<64>(p, n_req, q, bi, lh, warp % rows, rr, s_chunks[bi], s_pos[bi], st & 1, (st >> 1) & 1, s_pos64[bi], nm);
+  if (blockIdx.x > 0) {                       // cos / sin of the step's position (from the L2: these CTAs may run before the wait)
+    const int half = p.d / 2;
+    const int idx = ((int)blockIdx.x - 1) * GP_PLAN_THREADS + i;
+    if (idx < n_req * half) {
+      const int r = req_ids[idx / half];
+      if (r >= 0 && r < p.M) {
+        double sn, cs;
+        sincos((double)__ldcg(p.pos + r) * p.inv_freq[idx % half], &sn, &cs);
+        *reinterpret_cast<double2*>(p.rope_cs + (size_t)idx * 2) = make_double2(cs, sn);
+        *reinterpret_cast<float2*>(p.rope_f + (size_t)idx * 2) = make_float2((float)cs, (float)sn);
       }
     }
     return;
   }
-  if (!plan_on) return;
   s_first[i] = 0x7fffffff;
   if (i < GP_COST_BINS) s_bin[i] = 0;
-  if (i == 0) s_nmc = 0;
   // The number this step goes by: the host's count of decode steps in the asynchronous mode (the two scratch sets
   // count on their own); otherwise the pool's own counter on the device, so that a step replayed from a CUDA graph
   // still gets a number of its own.
@@ -561,7 +398,6 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   }
   __syncthreads();
   const int sorted0 = s_binbase[key] + within;
-  s_chunks[i] = chunks; s_pos[i] = (int)pos;
   if (in) {
     if (isb) { p.bstep[r] = step_no; if (p.async) act = GP_ACT_PENDING; }
     actions[i] = act;
@@ -581,29 +417,13 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
       d[2] = make_int4(flags, Pr, (int)(unsigned)(tok_off & 0xffffffffLL), (int)(tok_off >> 32));
       d[3] = make_int4(par, rc_off + c, 0, isb ? bnd_idx : 0);
     }
-    if (chunks > 1) p.mc_list[atomicAdd(&s_nmc, 1)] = make_int4(i, rc_off, chunks, 0);
-  }
-  __syncthreads();
-  if (p.rope_theta != 0.0) {                                      // cos / sin of the step's position
-    __syncthreads();
-    const int half = p.d / 2;
-    for (int idx = threadIdx.x; idx < n_req * half; idx += GP_PLAN_THREADS) {
-      const int bi = idx / half, j = idx % half;
-      if (s_chunks[bi] > 0) {
-        const double inv = pow(p.rope_theta, -2.0 * (double)j / (double)p.d);
-        const double ang = (double)s_pos[bi] * inv;
-        double sn, cs;
-        sincos(ang, &sn, &cs);
-        p.rope_cs[(size_t)idx * 2] = cs;
-        p.rope_cs[(size_t)idx * 2 + 1] = sn;
-      }
-    }
   }
   // the attention kernel counts, per unit of a boundary request, the work items its consumer warps have finished
   for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += GP_PLAN_THREADS) p.unit_ready[idx] = 0;
+  // (the attention kernel of the step before, the last to draw from these, has ended: the decisions waited for it)
+  for (int idx = threadIdx.x; idx < p.L; idx += GP_PLAN_THREADS) p.tickets[idx] = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
-    p.hdr[HDR_N_MC] = s_nmc;
     p.hdr[HDR_N_RC] = n_rc;
     p.hdr[HDR_N_BND] = n_bnd;
     p.hdr[HDR_N_ACTIVE] = n_active;
@@ -746,7 +566,7 @@ int flush_chain(gp_pool* pool, cudaStream_t s) {
   if (!pool->cfg.async_boundary || !pool->chain_pending) return GP_OK;
   const long long t = pool->serial - 1;                       // the step the chain belongs to
   const GpDev& d = (t & 1) ? pool->dev_alt : pool->dev;
-  gp_launch_chain(d, d, 0, nullptr, (int)(t & 0x3fffffff), 1, pool->chain_grid, s, false);
+  gp_launch_chain(d, 0, (int)(t & 0x3fffffff), 1, pool->chain_grid, s, false);
   pool->chain_pending = 0;
   pool->launch_count += 1;
   return cudaGetLastError() == cudaSuccess ? GP_OK : GP_ERR_CUDA;
@@ -881,7 +701,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.metric = cfg->demand_metric;
   d.delta = reinterpret_cast<double*>(base + L.delta);
   d.rcx = reinterpret_cast<int*>(base + L.rc);
-  d.mc_list = reinterpret_cast<int4*>(base + L.mc_list);
+  d.merge_cnt = reinterpret_cast<int*>(base + L.merge_cnt);
   d.bnd_info = reinterpret_cast<int4*>(base + L.bnd_info);
   d.bnd_acc = reinterpret_cast<int*>(base + L.bnd_acc);
   d.unit_ready = reinterpret_cast<int*>(base + L.unit_ready);
@@ -890,11 +710,13 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.free_peek = reinterpret_cast<int*>(base + L.free_peek);
   d.cmp_info = reinterpret_cast<int4*>(base + L.cmp_info);
   d.zbuf = reinterpret_cast<double*>(base + L.zbuf);
-  d.qtil = reinterpret_cast<double*>(base + L.qtil);
   d.zstat = reinterpret_cast<double*>(base + L.zstat);
   d.evict = reinterpret_cast<int*>(base + L.evict);
   d.evict2 = reinterpret_cast<int*>(base + L.evict2);
   d.cflags = reinterpret_cast<int*>(base + L.cflags);
+  d.inv_freq = reinterpret_cast<double*>(base + L.inv_freq);
+  d.tickets = reinterpret_cast<int*>(base + L.tickets);
+  d.rope_f = reinterpret_cast<float*>(base + L.rope_f);
   d.rope_cs = reinterpret_cast<double*>(base + L.rope_cs);
   d.partials = reinterpret_cast<float*>(base + L.partials);
   d.scores = reinterpret_cast<double*>(base + L.scores);
@@ -912,8 +734,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
     a.zbuf = reinterpret_cast<double*>(base + L.zbuf2);
     a.zstat = reinterpret_cast<double*>(base + L.zstat2);
     a.rcx = reinterpret_cast<int*>(base + L.rc2);
-    a.mc_list = reinterpret_cast<int4*>(base + L.mc_list2);
-    a.qtil = reinterpret_cast<double*>(base + L.qtil2);
+    a.rope_f = reinterpret_cast<float*>(base + L.rope_f2);
     a.rope_cs = reinterpret_cast<double*>(base + L.rope_cs2);
     // the chain kernel runs beside the attention kernel on the room it leaves: `slots` of its thread blocks
     int slots = cfg->async_slots > 0 ? cfg->async_slots : 64;
@@ -938,8 +759,6 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   }
   pool->dev.report_units = pool->dev_alt.report_units = pool->chain_grid_ov > 0;
   pool->dbg = base + L.dbg;
-  pool->qn = reinterpret_cast<__nv_bfloat16*>(base + L.qn);
-  pool->kn = reinterpret_cast<__nv_bfloat16*>(base + L.kn);
   if (cfg->host_staging) {
     pool->st_ids = reinterpret_cast<int*>(base + L.st_ids);
     pool->st_q = base + L.st_q; pool->st_k = base + L.st_k; pool->st_v = base + L.st_v;
@@ -1016,19 +835,15 @@ int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, co
   return GP_OK;
 }
 
-// CTA 0 plans (when plan_on); the others update the query summaries of the units [lh0, lh0 + lh_n)
-static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_t* actions, const void* q, int plan_on,
-                        int lh0, int lh_n, cudaStream_t s, bool pdl, bool by_layer = false, const GpDev* dev = nullptr,
-                        int attn_grid = 0, const GpNorm* norm = nullptr) {
+static const GpNorm kNoNorm = {nullptr, nullptr, 0.0};
+
+// CTA 0 plans; the others fill the table of cosines and sines (a thread per entry)
+static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_t* actions, bool early, cudaStream_t s, bool pdl,
+                        bool by_layer = false, const GpDev* dev = nullptr, int attn_grid = 0) {
   const GpDev& d = dev ? *dev : pool->dev;
-  const int upc = 32 / (2 * d.G);                            // units a CTA takes per pass (one warp per row)
-  const long long want = ((long long)n_req * lh_n + upc - 1) / upc;
-  const long long room = 2LL * pool->num_sms - 1;            // two 1024-thread CTAs per SM, one wave
-  const int prep = (int)(want < room ? want : room);
-  gp_launch(gp_plan_kernel, 1 + prep, GP_PLAN_THREADS, 0, s, pdl, d, ids, n_req, actions,
-            static_cast<const __nv_bfloat16*>(q), plan_on, lh0, lh_n, d.chunk_pages, d.bchunk_pages,
-            by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff),
-            norm ? *norm : GpNorm{nullptr, nullptr, 0.0, nullptr, nullptr, nullptr});
+  const int table = d.rope_theta != 0.0 ? (n_req * (d.d / 2) + GP_PLAN_THREADS - 1) / GP_PLAN_THREADS : 0;
+  gp_launch(gp_plan_kernel, 1 + table, GP_PLAN_THREADS, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
+            by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff));
 }
 
 int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, const void* q, const void* k,
@@ -1056,23 +871,22 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
       // split outputs) is one kernel behind the attention kernel.  Its thread blocks take their places as that
       // kernel's leave (or, with overlap_slots > 0, run beside it on slots its grid leaves free), and a selection job
       // starts as soon as the attention kernel has reported its unit's summary logits complete.
-      launch_plan(pool, dev_req_ids, n_req, dev_actions, q, pool->early_plan ? 2 : 1, 0, LH, s, pdl && !pool->first_plain, false,
-                  nullptr, pool->attn_grid_ov);
+      launch_plan(pool, dev_req_ids, n_req, dev_actions, pool->early_plan != 0, s, pdl && !pool->first_plain, false, nullptr,
+                  pool->attn_grid_ov);
       if (prof) cudaEventRecord(pool->ev[1], s);
-      gp_launch_attention(d, dev_req_ids, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0);
+      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
-      gp_launch_chain(d, d, n_req, static_cast<float*>(out), serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions,
-                      pool->actions_copy);
+      gp_launch_chain(d, n_req, serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy);
       if (prof) { cudaEventRecord(pool->ev[3], s); cudaEventRecord(pool->ev[4], s); }    // the last interval stays empty
       pool->launch_count += 3;
     } else {
       // Four kernels, one after the other (overlap_slots = -1): the selection and compaction kernels of the
       // layer-by-layer step
-      launch_plan(pool, dev_req_ids, n_req, dev_actions, q, pool->early_plan ? 2 : 1, 0, LH, s, pdl && !pool->first_plain);
+      launch_plan(pool, dev_req_ids, n_req, dev_actions, pool->early_plan != 0, s, pdl && !pool->first_plain);
       if (prof) cudaEventRecord(pool->ev[1], s);
-      gp_launch_attention(d, dev_req_ids, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, pdl, 0, LH, 0);
+      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, pdl, 0, LH, 0, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
-      gp_launch_boundary(d, dev_req_ids, n_req, dev_actions, static_cast<float*>(out), pool->sel_grid, pool->compact_grid, s,
+      gp_launch_boundary(d, dev_req_ids, n_req, dev_actions, false, pool->sel_grid, pool->compact_grid, s,
                          prof ? pool->ev[3] : nullptr, pdl, serial);
       if (prof) cudaEventRecord(pool->ev[4], s);
       pool->launch_count += GP_N_KERNELS;
@@ -1088,14 +902,13 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
     if (prof) cudaEventRecord(pool->ev[0], s);
     // no early planning here: the plan reads the pages and slots of the requests that return from their step out,
     // which the chain kernel of the step before (the kernel before this one on the stream) has just written
-    launch_plan(pool, dev_req_ids, n_req, dev_actions, q, 1, 0, LH, s, pdl && !pool->first_plain, false, &d, pool->attn_grid_async);
+    launch_plan(pool, dev_req_ids, n_req, dev_actions, false, s, pdl && !pool->first_plain, false, &d, pool->attn_grid_async);
     if (prof) cudaEventRecord(pool->ev[1], s);
-    gp_launch_attention(d, dev_req_ids, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_async, s, pdl, 0, LH, 0);
+    gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_async, s, pdl, 0, LH, 0, kNoNorm);
     if (prof) cudaEventRecord(pool->ev[2], s);
     // the decisions of the step before set pages and slots of requests that sit this step out: nothing else of
     // this step looks at those words
-    gp_launch_chain(dprev, d, n_req, static_cast<float*>(out), (int)((pool->serial - 1) & 0x3fffffff),
-                    pool->chain_pending, pool->chain_grid, s, pdl);
+    gp_launch_chain(dprev, n_req, (int)((pool->serial - 1) & 0x3fffffff), pool->chain_pending, pool->chain_grid, s, pdl);
     if (prof) { cudaEventRecord(pool->ev[3], s); cudaEventRecord(pool->ev[4], s); }
     pool->chain_pending = 1;
     pool->last_stream = s;
@@ -1145,7 +958,7 @@ int gp_step_begin(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, int3
   if (n_req == 0) return GP_OK;
   if (!dev_req_ids || !dev_actions || misaligned(dev_req_ids, 4) || misaligned(dev_actions, 4)) return GP_ERR_INVALID;
   GP_CUDA(cudaSetDevice(pool->device));
-  launch_plan(pool, dev_req_ids, n_req, dev_actions, nullptr, 1, 0, 0, static_cast<cudaStream_t>(stream), true, true);
+  launch_plan(pool, dev_req_ids, n_req, dev_actions, false, static_cast<cudaStream_t>(stream), true, true);
   pool->launch_count += 1;
   pool->step_open = 1;
   pool->step_n_req = n_req;
@@ -1173,10 +986,8 @@ int gp_attn_layer(gp_pool* pool, int32_t layer, const int32_t* dev_req_ids, int3
   const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(reinterpret_cast<uintptr_t>(v) - ks * 2);
   float* ob = reinterpret_cast<float*>(reinterpret_cast<uintptr_t>(out) - qs * 4);
   const int lh0 = layer * d.Hkv, lh_n = d.Hkv;
-  launch_plan(pool, dev_req_ids, n_req, nullptr, qb, 0, lh0, lh_n, s, true);
-  gp_launch_attention(d, dev_req_ids, n_req, qb, kb, vb, ob, pool->attn_grid, s, true, lh0, lh_n, -1);
-  gp_launch_merge(d, n_req, ob, lh0, lh_n, pool->num_sms, s, true);
-  pool->launch_count += 3;
+  gp_launch_attention(d, n_req, qb, kb, vb, ob, pool->attn_grid, s, true, lh0, lh_n, -1, kNoNorm);
+  pool->launch_count += 1;
   pool->step_layers_done += 1;
   pool->step_layer_seen[layer] = 1;
   GP_CUDA(cudaGetLastError());
@@ -1201,16 +1012,10 @@ int gp_attn_layer_qknorm(gp_pool* pool, int32_t layer, const int32_t* dev_req_id
   const __nv_bfloat16* qb = reinterpret_cast<const __nv_bfloat16*>(shifted(q_raw, qs * 2));
   const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(shifted(v, ks * 2));
   float* ob = reinterpret_cast<float*>(shifted(out, qs * 4));
-  GpNorm nm;
-  nm.wq = q_weight; nm.wk = k_weight; nm.eps = eps;
-  nm.k_raw = reinterpret_cast<const __nv_bfloat16*>(shifted(k_raw, ks * 2));
-  nm.qn = reinterpret_cast<__nv_bfloat16*>(shifted(pool->qn, qs * 2));
-  nm.kn = reinterpret_cast<__nv_bfloat16*>(shifted(pool->kn, ks * 2));
-  const int lh0 = layer * d.Hkv, lh_n = d.Hkv;
-  launch_plan(pool, dev_req_ids, n_req, nullptr, qb, 0, lh0, lh_n, s, true, false, nullptr, 0, &nm);
-  gp_launch_attention(d, dev_req_ids, n_req, nm.qn, nm.kn, vb, ob, pool->attn_grid, s, true, lh0, lh_n, -1);
-  gp_launch_merge(d, n_req, ob, lh0, lh_n, pool->num_sms, s, true);
-  pool->launch_count += 3;
+  const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(shifted(k_raw, ks * 2));
+  const GpNorm nm = {q_weight, k_weight, eps};
+  gp_launch_attention(d, n_req, qb, kb, vb, ob, pool->attn_grid, s, true, layer * d.Hkv, d.Hkv, -1, nm);
+  pool->launch_count += 1;
   pool->step_layers_done += 1;
   pool->step_layer_seen[layer] = 1;
   GP_CUDA(cudaGetLastError());
@@ -1222,8 +1027,7 @@ int gp_step_end(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, int32_
   if (n_req != pool->step_n_req || !dev_req_ids || !dev_actions) return GP_ERR_INVALID;
   if (pool->step_layers_done != pool->cfg.n_layers) return GP_ERR_STATE;       // layers missing: run them, or gp_step_abort
   GP_CUDA(cudaSetDevice(pool->device));
-  gp_launch_boundary(pool->dev, dev_req_ids, n_req, dev_actions, nullptr,
-                     pool->sel_grid, pool->compact_grid,
+  gp_launch_boundary(pool->dev, dev_req_ids, n_req, dev_actions, true, pool->sel_grid, pool->compact_grid,
                      static_cast<cudaStream_t>(stream), nullptr, true, (int)(pool->serial & 0x3fffffff));
   pool->serial += 1;
   pool->launch_count += 2;
@@ -1255,9 +1059,9 @@ int gp_decode_step_local(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_re
   const GpDev& d = pool->dev;
   const int LH = d.L * d.Hkv;
   const int serial = (int)(pool->serial & 0x3fffffff);
-  launch_plan(pool, dev_req_ids, n_req, dev_actions, q, 1, 0, LH, s, true);
-  gp_launch_attention(d, dev_req_ids, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, true, 0, LH, 0);
-  gp_launch_select_only(d, dev_req_ids, n_req, dev_actions, static_cast<float*>(out), pool->sel_grid, s, true, serial);
+  launch_plan(pool, dev_req_ids, n_req, dev_actions, false, s, true);
+  gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, true, 0, LH, 0, kNoNorm);
+  gp_launch_select_only(d, dev_req_ids, n_req, dev_actions, pool->sel_grid, s, true, serial);
   pool->launch_count += 3;
   pool->step_open = 2;                           // between the two halves the pool takes nothing else
   pool->step_n_req = n_req;
