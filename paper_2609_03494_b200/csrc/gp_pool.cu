@@ -11,7 +11,8 @@
 #include "../../include/growpage.h"
 #include "gp_dev.cuh"
 
-#define GP_PLAN_THREADS 1024
+#define GP_PLAN_THREADS 1024       // threads of the plan kernel for batches of up to GP_MAX_REQ requests (a thread each) ...
+#define GP_PLAN_SMALL 256          // ... and for batches of up to this many: its time is block barriers, which 8 warps pass faster than 32
 #define GP_NEVER (-(1 << 30))      // bstep of a request that has not reached a boundary
 
 struct gp_pool {
@@ -216,7 +217,7 @@ __global__ void gp_init_kernel(GpDev p) {
   if (i0 == 0) *p.free_top = (int)p.n_pages;
 }
 
-// exclusive scan over the CTA (1024 threads) of an int and a long long; also returns the totals
+// exclusive scan over the CTA (up to 32 warps) of an int and a long long; also returns the totals
 __device__ __forceinline__ void plan_scan(int v, long long w, int& ev, long long& ew, int& tv, long long& tw,
                                           int* sv, long long* sw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -230,7 +231,8 @@ __device__ __forceinline__ void plan_scan(int v, long long w, int& ev, long long
   if (lane == 31) { sv[warp] = iv; sw[warp] = iw; }
   __syncthreads();
   if (warp == 0) {                       // scan of the 32 warp totals: exclusive prefix in [0..31], total in [32]
-    int xv = sv[lane]; long long xw = sw[lane];
+    const bool has = lane < (int)(blockDim.x >> 5);
+    int xv = has ? sv[lane] : 0; long long xw = has ? sw[lane] : 0;
     const int ov = xv; const long long ow = xw;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -283,7 +285,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   gp_pdl_launch_dependents();
   if (blockIdx.x > 0) {                       // cos / sin of the step's position (from the L2: these CTAs may run before the wait)
     const int half = p.d / 2;
-    const int idx = ((int)blockIdx.x - 1) * GP_PLAN_THREADS + i;
+    const int idx = ((int)blockIdx.x - 1) * (int)blockDim.x + i;
     if (idx < n_req * half) {
       const int r = req_ids[idx / half];
       if (r >= 0 && r < p.M) {
@@ -295,8 +297,8 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     }
     return;
   }
-  s_first[i] = 0x7fffffff;
-  if (i < GP_COST_BINS) s_bin[i] = 0;
+  for (int t = i; t < p.M; t += blockDim.x) s_first[t] = 0x7fffffff;
+  for (int t = i; t < GP_COST_BINS; t += blockDim.x) s_bin[t] = 0;
   // The number this step goes by: the host's count of decode steps in the asynchronous mode (the two scratch sets
   // count on their own); otherwise the pool's own counter on the device, so that a step replayed from a CUDA graph
   // still gets a number of its own.
@@ -419,9 +421,10 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     }
   }
   // the attention kernel counts, per unit of a boundary request, the work items its consumer warps have finished
-  for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += GP_PLAN_THREADS) p.unit_ready[idx] = 0;
+  if (p.report_units)
+    for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += blockDim.x) p.unit_ready[idx] = 0;
   // (the attention kernel of the step before, the last to draw from these, has ended: the decisions waited for it)
-  for (int idx = threadIdx.x; idx < p.L; idx += GP_PLAN_THREADS) p.tickets[idx] = 0;
+  for (int idx = threadIdx.x; idx < p.L; idx += blockDim.x) p.tickets[idx] = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
     p.hdr[HDR_N_RC] = n_rc;
@@ -874,8 +877,9 @@ static const GpNorm kNoNorm = {nullptr, nullptr, 0.0};
 static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_t* actions, bool early, cudaStream_t s, bool pdl,
                         bool by_layer = false, const GpDev* dev = nullptr, int attn_grid = 0) {
   const GpDev& d = dev ? *dev : pool->dev;
-  const int table = d.rope_theta != 0.0 ? (n_req * (d.d / 2) + GP_PLAN_THREADS - 1) / GP_PLAN_THREADS : 0;
-  gp_launch(gp_plan_kernel, 1 + table, GP_PLAN_THREADS, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
+  const int threads = n_req <= GP_PLAN_SMALL ? GP_PLAN_SMALL : GP_PLAN_THREADS;
+  const int table = d.rope_theta != 0.0 ? (n_req * (d.d / 2) + threads - 1) / threads : 0;
+  gp_launch(gp_plan_kernel, 1 + table, threads, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
             by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff));
 }
 
