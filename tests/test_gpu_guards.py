@@ -136,6 +136,55 @@ def test_pool_is_closed_to_admissions_and_releases_inside_an_open_step_and_a_ste
     assert a1.tolist() == [B.GP_ACT_GROW, B.GP_ACT_NONE, B.GP_ACT_GROW]      # 32 and 48 tokens fill two and three pages
 
 
+def test_early_planned_steps_behind_abandoned_ones_are_undisturbed():
+    """Layers of a step that is abandoned may still run when the next step is issued, early planning or not: no host wait lies in
+    between.  About 650 items a layer (more than two rounds of the grid), requests of up to nine items, boundaries at most steps."""
+    import torch
+    layers, hq, hkv, d, steps = 3, 16, 8, 64, 5
+    lens = [15 + 16 * i for i in range(12)] + [600 + 331 * i for i in range(12)]
+    n_req, cap = len(lens), max(lens) // 16 + 3
+    rng = np.random.default_rng(41)
+    prompts = [(_bits(rng, layers, n, hkv, d), _bits(rng, layers, n, hkv, d), n) for n in lens]
+    ins = [tuple(_dev(torch, _bits(rng, layers, n_req, h, d)) for h in (hq, hkv, hkv)) for _ in range(2 * steps)]
+    ids = torch.arange(n_req, dtype=torch.int32, device="cuda")
+    backwards = ids.flip(0).contiguous()
+    results = []
+    for disturb in (False, True):
+        pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(n // 16 + 3 for n in lens), max_pages_per_req=cap, max_requests=n_req,
+                                    tau=-0.02))
+        try:
+            for kt, vt, n in prompts:
+                assert pool.request_add(-1, 0, kt, vt, n, 0)[0] == B.GP_OK
+            B.gp_set_early_plan(pool.handle, disturb)
+            outs = [torch.zeros((layers, n_req, hq, d), dtype=torch.float32, device="cuda") for _ in range(steps)]
+            acts = torch.zeros((steps, n_req), dtype=torch.int32, device="cuda")
+            waste, waste_act = torch.zeros_like(outs[0]), torch.zeros(n_req, dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            s = pool.stream()
+            for t in range(steps):
+                if disturb:
+                    q, k, v = ins[steps + t]
+                    B.gp_step_begin(pool.handle, backwards.data_ptr(), n_req, waste_act.data_ptr(), s)
+                    for l in (2, 0)[:t % 3]:                     # none, one or two of the layers
+                        B.gp_attn_layer(pool.handle, l, backwards.data_ptr(), n_req, q[l].data_ptr(), k[l].data_ptr(), v[l].data_ptr(),
+                                        waste[l].data_ptr(), s)
+                    B.gp_step_abort(pool.handle)
+                q, k, v = ins[t]
+                pool.decode_step(ids, q, k, v, outs[t], acts[t])
+            torch.cuda.synchronize()
+            assert B.gp_pool_status(pool.handle) == (B.GP_OK, 0)
+            state = [B.gp_debug_request(pool.handle, r, cap) for r in range(n_req)]
+            kept = [B.gp_debug_retained(pool.handle, r, l, h, state[r][1]) for r in range(n_req) for l in range(layers) for h in (0, hkv - 1)]
+            summ = [B.gp_debug_summaries(pool.handle, r, layers, hq, d) for r in range(n_req)]
+            results.append((torch.stack(outs).cpu().numpy(), acts.cpu().numpy(), state, kept, summ))
+        finally:
+            pool.close()
+    (o1, a1, s1, k1, m1), (o2, a2, s2, k2, m2) = results
+    assert np.array_equal(a1, a2) and (a1 != B.GP_ACT_NONE).any()
+    assert [tuple(map(str, x)) for x in s1] == [tuple(map(str, x)) for x in s2]
+    assert all(np.array_equal(x, y) for x, y in zip(k1 + m1, k2 + m2)) and np.array_equal(o1, o2)
+
+
 # ----------------------------------------------------------------------------------------------------------------
 # bounded waits that run out: the kernel gives up, says so, and ends; nothing hangs, nothing faults
 # ----------------------------------------------------------------------------------------------------------------
