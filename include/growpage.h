@@ -175,7 +175,8 @@ int gp_pool_destroy(gp_pool* pool);
  * leading ones possibly shared (App. D.2 prefix sharing).  Its first `n_shared_pages` pages are shared by reference
  * count with live request `share_from` (-1 for none), which must still hold them as untouched
  * full prompt pages.  The rest of the prompt, `n_tail` tokens, is copied from k_tail / v_tail:
- * device pointers, bf16 [L][n_tail][H_kv][d], keys already in cache form (post-RoPE).
+ * device pointers, 16-byte aligned (the copy moves 16-byte pieces), bf16 [L][n_tail][H_kv][d], keys already in cache form
+ * (post-RoPE).
  * The request starts with max(initial_pages, floor(n_prompt / b) + 1) pages.
  * On success *out_req receives the request id (the lowest free slot).  The summaries of the slot
  * are not cleared: the first decode step overwrites them.  Synchronises `stream`.

@@ -830,7 +830,7 @@ int gp_pool_destroy(gp_pool* pool) {
 int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, const void* k_tail, const void* v_tail,
                    int32_t n_tail, int32_t initial_pages, void* stream, int32_t* out_req) {
   if (!pool || !out_req || n_tail < 0 || n_shared_pages < 0 || initial_pages < 0) return GP_ERR_INVALID;
-  if (n_tail > 0 && (!k_tail || !v_tail)) return GP_ERR_INVALID;
+  if (n_tail > 0 && (!k_tail || !v_tail || misaligned(k_tail, 16) || misaligned(v_tail, 16))) return GP_ERR_INVALID;
   *out_req = -1;
   if (pool->step_open) return GP_ERR_STATE;      // the open step's plan holds a snapshot of the free list
   if (n_shared_pages > 0 && check_req(pool, share_from) != GP_OK) return GP_ERR_INVALID;

@@ -94,3 +94,19 @@ def test_pages_replaced_in_one_step_return_once_in_the_last_sharers_order(sharer
         assert st == B.GP_OK and list(B.gp_debug_request(pool.handle, b, P)[3][:P - 1]) == list(shared[::-1])
     finally:
         pool.close()
+
+
+def test_misaligned_prompt_is_refused_before_any_launch():
+    import torch
+    pool = B.Pool(B.make_config(1, 2, 2, 64, n_pages=8, max_pages_per_req=4, max_requests=4))
+    try:
+        rows = torch.zeros(20 * 2 * 64 + 64, dtype=torch.int16, device="cuda")
+        good = rows.data_ptr()
+        launches = B.gp_launch_count(pool.handle)
+        for k, v in ((good + 2, good), (good, good + 8), (good + 14, good + 14)):
+            assert B.gp_request_add(pool.handle, -1, 0, k, v, 20, 0, pool.stream()) == (B.GP_ERR_INVALID, -1)
+        assert B.gp_launch_count(pool.handle) == launches and B.gp_debug_pool(pool.handle)[0] == 8
+        assert B.gp_request_add(pool.handle, -1, 0, good, good, 20, 0, pool.stream()) == (B.GP_OK, 0)
+        assert B.gp_request_add(pool.handle, 0, 1, 2, 2, 0, 0, pool.stream()) == (B.GP_OK, 1)       # no tail: the pointers are not looked at
+    finally:
+        pool.close()
