@@ -858,7 +858,7 @@ int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, co
                                               pool->dev.err + 1);
   pool->launch_count++;
   GP_CUDA(cudaGetLastError());
-  if (n_tail > 0 && slot >= 0) {
+  if (n_tail > 0 && slot >= 0 && P <= c.max_pages_per_req) {       // (otherwise the admission refuses: nothing to copy, and no bound on n_tail)
     const long long blocks = 2LL * ((n_tail + GP_PAGE - 1) / GP_PAGE) * c.n_layers;
     GP_CUDA(gp_launch(gp_ingest_kernel, (int)blocks, INGEST_THREADS, 0, s, true, pool->dev, slot, n_shared_pages * sub, (int)n_tail,
                       static_cast<const __nv_bfloat16*>(k_tail), static_cast<const __nv_bfloat16*>(v_tail),

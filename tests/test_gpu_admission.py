@@ -110,3 +110,21 @@ def test_misaligned_prompt_is_refused_before_any_launch():
         assert B.gp_request_add(pool.handle, 0, 1, 2, 2, 0, 0, pool.stream()) == (B.GP_OK, 1)       # no tail: the pointers are not looked at
     finally:
         pool.close()
+
+
+def test_a_prompt_past_the_page_cap_is_refused_without_copying_it():
+    """With shared pages the refusal comes from the device (a bad donor is reported first): the prompt is not copied meanwhile, however
+    long the caller says it is."""
+    import torch
+    pool = B.Pool(B.make_config(36, 2, 2, 64, n_pages=8, max_pages_per_req=4, max_requests=4))
+    try:
+        rows = torch.zeros(36 * 20 * 2 * 64, dtype=torch.int16, device="cuda").data_ptr()
+        assert B.gp_request_add(pool.handle, -1, 0, rows, rows, 20, 0, pool.stream()) == (B.GP_OK, 0)
+        for donor_pages, n_tail, want in ((1, 49, B.GP_ERR_NO_PAGES), (1, 2 ** 30, B.GP_ERR_NO_PAGES), (1, 2 ** 31 - 1, B.GP_ERR_NO_PAGES),
+                                          (2, 2 ** 30, B.GP_ERR_INVALID)):
+            launches = B.gp_launch_count(pool.handle)
+            assert B.gp_request_add(pool.handle, 0, donor_pages, rows, rows, n_tail, 0, pool.stream()) == (want, -1)
+            assert B.gp_launch_count(pool.handle) == launches + 1
+        assert B.gp_debug_pool(pool.handle)[0] == 6 and B.gp_debug_request(pool.handle, 0, 4)[:3] == (2, 20, 20)
+    finally:
+        pool.close()
