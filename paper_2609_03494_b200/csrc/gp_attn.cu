@@ -66,10 +66,11 @@ struct Geo {
 struct Lay {            // shared-memory layout, depends on the group size
   int ncomb, off_slots, off_qt, off_comb, comb_warp, off_bars, off_misc, total;
 };
+constexpr int SMEM_ALIGN = 256;          // the kernel rounds the start of its shared memory up to this
 template <int D>
-__host__ __device__ inline Lay make_lay(int G) {
+__host__ __device__ constexpr Lay make_lay(int G) {
   using GEO = Geo<D>;
-  Lay L;
+  Lay L = {};
   L.ncomb = (D == 128 && G == 8) ? 1 : 2;
   L.off_slots = NCW * NSW * GEO::TILE_BYTES;
   L.off_qt = L.off_slots + NI * GEO::SLOT_BYTES;
@@ -78,9 +79,12 @@ __host__ __device__ inline Lay make_lay(int G) {
   L.comb_warp = (16 + G * D) * 4;
   L.off_bars = L.off_comb + L.ncomb * NCW * L.comb_warp;
   L.off_misc = L.off_bars + (3 * NI + 2 + 4) * 8;
-  L.total = L.off_misc + 128;                // abort flag and code
+  L.total = L.off_misc + 128 + SMEM_ALIGN;   // abort flag and code; room for the rounding
   return L;
 }
+// two thread blocks to an SM, each with the 1 KB the system takes of its own
+static_assert(2 * (make_lay<128>(8).total + 1024) <= 228 * 1024 && 2 * (make_lay<128>(4).total + 1024) <= 228 * 1024 &&
+              2 * (make_lay<64>(8).total + 1024) <= 228 * 1024, "shared memory of two thread blocks");
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -364,7 +368,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   // step does that at its end)
   using GEO = Geo<D>;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + ((256u - (smem_u32(smem_raw) & 255u)) & 255u);
+  uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & (SMEM_ALIGN - 1u));
   const int G = p.G;
   const Lay L = make_lay<D>(G);
   const uint32_t NCOMB = (uint32_t)L.ncomb;
