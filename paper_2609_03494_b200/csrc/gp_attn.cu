@@ -145,10 +145,11 @@ __device__ __forceinline__ void merge_unit(float* first, size_t stride, int n, i
       for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float* pr = first + (c0 + k < n ? c0 + k : c0) * stride + (g0 + q < G ? g0 + q : 0) * (D + 2);
-          mv[k][q] = c0 + k < n ? __ldcg(pr + D) : -INFINITY;
+          const bool here = c0 + k < n;                  // (past the last one: weight 0 and values 0, whatever that one holds)
+          const float* pr = first + (c0 + k) * stride + (g0 + q < G ? g0 + q : 0) * (D + 2);
+          mv[k][q] = here ? __ldcg(pr + D) : -INFINITY;
 #pragma unroll
-          for (int e = 0; e < PER2; ++e) vv[k][q][e] = __ldcg(reinterpret_cast<const float2*>(pr) + lane + 32 * e);
+          for (int e = 0; e < PER2; ++e) vv[k][q][e] = here ? __ldcg(reinterpret_cast<const float2*>(pr) + lane + 32 * e) : make_float2(0.f, 0.f);
         }
 #pragma unroll
       for (int k = 0; k < 2; ++k)
