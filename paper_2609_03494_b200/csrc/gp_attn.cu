@@ -48,7 +48,8 @@ constexpr int REGS_SERVICE = 80;           // registers per thread after the spl
 constexpr int REGS_CONSUMER = 176;
 constexpr int NSUM = 2;                    // summary warps
 constexpr int MERGE_FAN = 8;               // partial outputs merged at a time
-constexpr double QT_SCALE = 0x1p896;       // of the q~ buffer: see bf16_lo_scaled
+constexpr double QT_SCALE = 0x1p880;       // of the q~ buffer: see bf16_lo_scaled
+constexpr double Z_SCALE = 0x1p16;         // of the logits made from it
 constexpr int QT_PAD = 8;                  // doubles of padding per q~ row: rows alternate bank halves
 
 template <int D>
@@ -282,7 +283,10 @@ __device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, u
 }
 
 // bf16 -> double by its bits, scaled by 2^-896 (an 8-bit exponent read as an 11-bit one): exact for every finite number, and
-// cheaper than the conversion unit.  The q~ buffer holds the summaries times 2^896, so that the products are what they were.
+// cheaper than the conversion unit.  The q~ buffer holds the summaries times 2^880, the logits are scaled by the remaining 2^16:
+// all powers of two, so that the logits are what they were.  (The calibrated summary of a query whose elements are near the
+// largest bf16, 2^128, can be sqrt(d) times as large and twice that after its rotation: 2^133 at most, and 2^896 times that is
+// past the largest double.)
 __device__ __forceinline__ double bf16_lo_scaled(uint32_t w) { return __hiloint2double((int)((uint32_t)((int)(w << 16) >> 3) & 0x8fffffffu), 0); }
 __device__ __forceinline__ double bf16_hi_scaled(uint32_t w) { return __hiloint2double((int)((uint32_t)((int)(w & 0xffff0000u) >> 3) & 0x8fffffffu), 0); }
 
@@ -319,7 +323,7 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
       dmma(z[odd][1][0], z[odd][1][1], bf16_hi_scaled(kb), qq.y);
     }
   }
-  const double inv_sqrt_d = 1.0 / sqrt((double)D);
+  const double inv_sqrt_d = Z_SCALE / sqrt((double)D);
   // D fragment: row = grp (token), columns 2*t4, 2*t4 + 1
   const int col = nt * 8 + 2 * t4;
   double z00 = (z[0][0][0] + z[1][0][0]) * inv_sqrt_d, z01 = (z[0][0][1] + z[1][0][1]) * inv_sqrt_d;
