@@ -297,10 +297,11 @@ __device__ __forceinline__ double bf16_hi_scaled(uint32_t w) { return __hiloint2
 // the same mapping, so the contraction is over the same d on both sides).  One block of eight columns at a time (nt of them: a
 // group of eight heads has two).  What bounds it: the fp64 pipe and four chains of dependent DMMAs; the registers it takes are
 // the consumers' (two blocks together spilled: 84.0 ms against 80.0 on 36 layers x 256 requests).  Stores the exponentials
-// per token and the page's softmax partials per column.
+// per token and the page's softmax partials per column.  `odd`: keys of the page may be infinite or not numbers, which their
+// bits read as a double's are not: the same contraction over converted keys.
 template <int D>
 __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* tile, const double* qt, int G, int lh, long long zoff,
-                                               int tok0, int nt) {
+                                               int tok0, int nt, bool odd) {
   constexpr int CH = D / 8, ROW_BYTES = D * 2;
   const int lane = threadIdx.x & 31, grp = lane >> 2, t4 = lane & 3;
   double z[2][2][2];                                      // [even / odd chunks][token half][column pair]
@@ -321,6 +322,24 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
       dmma(z[odd][1][0], z[odd][1][1], bf16_lo_scaled(kb), qq.x);
       dmma(z[odd][0][0], z[odd][0][1], bf16_hi_scaled(ka), qq.y);
       dmma(z[odd][1][0], z[odd][1][1], bf16_hi_scaled(kb), qq.y);
+    }
+  }
+  if (odd) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) (&z[0][0][0])[i] = 0.0;
+#pragma unroll 1
+    for (int c = 0; c < CH; c += 2) {
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const uint32_t ka = *reinterpret_cast<const uint32_t*>(krow0 + (((c + w) ^ grp) << 4));
+        const uint32_t kb = *reinterpret_cast<const uint32_t*>(krow1 + (((c + w) ^ grp) << 4));
+        const double2 qq = *reinterpret_cast<const double2*>(qrow + (c + w) * 8);
+        const double q0 = qq.x * 0x1p-896, q1 = qq.y * 0x1p-896;
+        dmma(z[w][0][0], z[w][0][1], (double)bf16_lo_f(ka), q0);
+        dmma(z[w][1][0], z[w][1][1], (double)bf16_lo_f(kb), q0);
+        dmma(z[w][0][0], z[w][0][1], (double)bf16_hi_f(ka), q1);
+        dmma(z[w][1][0], z[w][1][1], (double)bf16_hi_f(kb), q1);
+      }
     }
   }
   const double inv_sqrt_d = Z_SCALE / sqrt((double)D);
@@ -672,6 +691,9 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             mma_bf16(s_acc[1], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b10, b11);
           }
         }
+        // a key that is infinite or not a number leaves no finite score with any query (of row 0, which is always one of the group)
+        const bool odd_keys = need_qt && __any_sync(0xffffffffu, !(fabsf(s_acc[0][0]) + fabsf(s_acc[0][1]) + fabsf(s_acc[1][0]) +
+                                                                  fabsf(s_acc[1][1]) < INFINITY));
         // online softmax in the log2 domain
         float sv[2][2];
         const int n_valid = has_new ? (n_new - tok0) : GP_PAGE;
@@ -728,8 +750,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             qt_here = true;
           }
           const long long zoff = ((long long)(unsigned)sd[10]) | ((long long)sd[11] << 32);
-          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0);
-          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1);
+          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0, odd_keys);
+          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1, odd_keys);
         }
         __syncwarp();
         if (!top_up(it)) { ok = false; break; }            // the stage is free: fetch the next tile into it

@@ -300,6 +300,8 @@ __device__ __forceinline__ SelSmem sel_smem_at(uint8_t* smem, int cap) {      //
   return S;
 }
 
+__device__ __forceinline__ unsigned long long key_of(double v) { return (unsigned long long)__double_as_longlong(v); }
+
 // Per-head softmax over the first `ntile` pages of the candidates and the group mean (Sec. 3.2): a^S and a^L of every
 // candidate.  The attention kernel left, per 16-token page t and column c (view, head), the page's maximum logit m_tc
 // and s_tc = sum of exp(z - m_tc), and per token x = exp(z - m_tc).  With M_c the maximum over pages and
@@ -403,7 +405,8 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
               for (int g = 1; g < GG; ++g) a[q] += xv[u][q][g] * f[q * GG + g];
             }
           }
-          if (aS == aL) aS[tok] = views == 3 ? fmax(a[0], a[1]) : a[views >> 1];       // a job of one array
+          // a job of one array; the larger score by its bits, as everywhere (one that is not a number is the largest)
+          if (aS == aL) aS[tok] = views == 3 ? __longlong_as_double((long long)max(key_of(a[0]), key_of(a[1]))) : a[views >> 1];
           else { aS[tok] = a[0]; aL[tok] = a[1]; }
           const unsigned w0 = (unsigned)__double2hiint(a[0]), w1 = (unsigned)__double2hiint(a[1]), w2 = max(w0, w1);
           lo_w[0] = min(lo_w[0], w0); lo_w[1] = min(lo_w[1], w1); lo_w[2] = min(lo_w[2], w2);
@@ -418,8 +421,6 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
     if ((tid & 31) == 0) { atomicMin(&m.rng[q][0], a); atomicMax(&m.rng[q][1], b); }
   }
 }
-
-__device__ __forceinline__ unsigned long long key_of(double v) { return (unsigned long long)__double_as_longlong(v); }
 
 // Eq. 10, block-local quota: the kq best slots of every block of `blk` candidates (score desc, slot asc; the last block
 // may be short) as bits of loc[].  Run by `nw` warps, warp w of them taking every nw-th 32 slots or block.

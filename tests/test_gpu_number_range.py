@@ -1,4 +1,5 @@
-"""Numbers at and past the edges of their formats: outputs that overflow, queries near the largest bf16."""
+"""Numbers at and past the edges of their formats: outputs that overflow, queries near the largest bf16, keys that are
+infinite or not numbers."""
 import numpy as np
 import pytest
 
@@ -75,6 +76,51 @@ def test_boundary_after_queries_near_the_largest_bf16(hq, d, rope_theta):
         left = ora.request_state(0)[1]
         for h in range(hkv):
             assert np.array_equal(B.gp_debug_retained(pool.handle, 0, 0, h, left), ora.retained(0, 0, h))
+        assert B.gp_debug_pool(pool.handle)[2][7] == 0
+    finally:
+        pool.close()
+
+
+# With few units a thread block takes one task of a unit; with overlap_slots = 1 the boundary kernel has one block, which takes
+# whole units.
+@pytest.mark.parametrize("hq,d", [(2, 64), (8, 64), (16, 128)])
+@pytest.mark.parametrize("slots", [0, 1])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_a_key_that_is_no_finite_number_shows_in_its_units_scores(value, slots, hq, d):
+    """Against positive query elements a key element of -inf is a token without weight.  With +inf or NaN no score of the unit is a number:
+    its working sets are all candidates and, all scores being equal, the evicted slots go by their order.  The other unit is untouched."""
+    rng = np.random.default_rng(7)
+    L, hkv, pages, k_loc = 1, 2, 6, 4
+    n = pages * 16 - 1
+    kw = dict(n_pages=pages, max_pages_per_req=pages, max_requests=2, tau=2.0, k_loc=k_loc)
+    pool = B.Pool(B.make_config(L, hq, hkv, d, overlap_slots=slots, **kw))
+    ora = O.OraclePool(O.OracleConfig(L, hq, hkv, d, **kw))
+    f = W.bf16_bits_to_f64
+    try:
+        keys, vals = _bits(rng, L, n + 1, hkv, d), _bits(rng, L, n + 1, hkv, d)
+        q = W.f32_to_bf16_bits(np.abs(rng.standard_normal((L, 1, hq, d))).astype(np.float32) + 0.1)
+        bad = keys.copy()
+        bad[0, 37, 1, 5] = {True: 0x7fc0, False: 0x7f80 if value > 0 else 0xff80}[bool(np.isnan(value))]
+        exact = bad if value == -np.inf else keys                  # what the oracle can follow
+        assert pool.request_add(-1, 0, bad[:, :n], vals[:, :n], n, 0)[0] == B.GP_OK
+        ora.request_add(-1, 0, f(exact[:, :n]), f(vals[:, :n]), n, 0)
+        out, act = _step(pool, q, keys[:, n:], vals[:, n:])
+        rec = ora.decode_step([0], f(q), f(keys[:, n:]), f(vals[:, n:]))
+        assert act == B.GP_ACT_COMPRESS and rec.actions.tolist() == [act]
+        ks, kl, _ = B.gp_debug_boundary(pool.handle, 0, L, hkv)
+        G, n_c = hq // hkv, (pages - 1) * 16
+        slots_left = np.arange(n_c)
+        rest = slots_left[slots_left % 16 >= k_loc]
+        by_order = np.setdiff1d(np.arange(n + 1), rest[len(rest) - 16:])
+        for h in range(hkv):
+            kept = B.gp_debug_retained(pool.handle, 0, 0, h, n_c)
+            if h == 1 and value != -np.inf:
+                assert np.isnan(out[0, G:]).all() and (ks[0, h], kl[0, h]) == (n_c, n_c)
+                assert np.array_equal(kept, by_order)
+            else:
+                assert np.abs(out[0, h * G:(h + 1) * G] - rec.out[0, 0, h * G:(h + 1) * G]).max() <= 1e-2
+                assert (ks[0, h], kl[0, h]) == (rec.boundary[0].K_s[0, h], rec.boundary[0].K_l[0, h])
+                assert np.array_equal(kept, ora.retained(0, 0, h))
         assert B.gp_debug_pool(pool.handle)[2][7] == 0
     finally:
         pool.close()
