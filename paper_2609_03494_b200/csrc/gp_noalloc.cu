@@ -51,40 +51,49 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
   return y;
 }
 
-// The tokens [t0, t1) of one (request, KV head) with plain loads of single elements and fp32 arithmetic throughout:
-// for keys and values whose addresses are not 16-byte aligned, and for a split whose tensor-core result is not finite
-// (below).  Writes the split's partial results.  `smem`: NA_THREADS / 32 + 1 arrays of 8 rows.
-__device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qrow0, const __nv_bfloat16* __restrict__ kbase,
-                                            const __nv_bfloat16* __restrict__ vbase, int G, int d, int t0, int t1, float* smem,
-                                            float* __restrict__ part, size_t row_stride) {
+// The tokens [t0, t1) of one (request, KV head) with plain loads of single elements and fp32 arithmetic throughout.
+// Writes the split's partial results.  `smem`: NA_PLAIN_FLOATS floats.  Bound by the latency of a warp's chain of loads, sums over
+// the warp and exponentials, so by the warps an SM holds.  AHEAD: the next token's elements are on their way while one is worked on,
+// which pays where they are few (twelve in the tensor-core kernel: 507 us for 64 requests of 60 to 4000 tokens, groups of 4, d = 128,
+// against 805) and costs where they are many (twenty-four in the plain kernel: 664 us against 507, both with the width a variable).
+constexpr int NA_PLAIN_FLOATS = 8 * NA_MAX_D + NA_WARPS * 8 * NA_STRIDE;
+template <int D, bool AHEAD>
+__device__ __forceinline__ void na_plain_tokens(const __nv_bfloat16* __restrict__ qrow0, const __nv_bfloat16* __restrict__ kbase,
+                                                const __nv_bfloat16* __restrict__ vbase, int G, int t0, int t1, float* smem,
+                                                float* __restrict__ part, size_t row_stride) {
+  constexpr int PER = D / 32;                                              // elements of a row per lane
   float* s_q = smem;                                                       // [8][NA_MAX_D]
   float (*s_part)[8][NA_STRIDE] = reinterpret_cast<float (*)[8][NA_STRIDE]>(smem + 8 * NA_MAX_D);     // [warps]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int per = d / 32;
   __syncthreads();                                                         // whatever the memory held before is done with
-  for (int i = tid; i < G * d; i += NA_THREADS) s_q[(i / d) * NA_MAX_D + i % d] = __bfloat162float(qrow0[i]);
+  for (int i = tid; i < G * D; i += NA_THREADS) s_q[(i / D) * NA_MAX_D + i % D] = __bfloat162float(qrow0[i]);
   __syncthreads();
-  const float scale = 1.4426950408889634f * rsqrtf((float)d);
-  float m[8], l[8], acc[8][4];
+  const float scale = 1.4426950408889634f * rsqrtf((float)D);
+  float m[8], l[8], acc[8][PER];
 #pragma unroll
   for (int g = 0; g < 8; ++g) {
     m[g] = -INFINITY; l[g] = 0.f;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[g][e] = 0.f;
+    for (int e = 0; e < PER; ++e) acc[g][e] = 0.f;
   }
-  for (int t = t0 + warp; t < t1; t += NA_WARPS) {
-    float kv[4], vv[4];
+  __nv_bfloat16 kn[PER], vn[PER];                         // AHEAD: as loaded, converted where they are used, so that nothing waits for them before
+  auto load = [&](int t) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      kv[e] = e < per ? __bfloat162float(kbase[(size_t)t * d + lane + 32 * e]) : 0.f;
-      vv[e] = e < per ? __bfloat162float(vbase[(size_t)t * d + lane + 32 * e]) : 0.f;
-    }
+    for (int e = 0; e < PER; ++e) { kn[e] = kbase[(size_t)t * D + lane + 32 * e]; vn[e] = vbase[(size_t)t * D + lane + 32 * e]; }
+  };
+  if (AHEAD && t0 + warp < t1) load(t0 + warp);
+  for (int t = t0 + warp; t < t1; t += NA_WARPS) {
+    if (!AHEAD) load(t);
+    float kv[PER], vv[PER];
+#pragma unroll
+    for (int e = 0; e < PER; ++e) { kv[e] = __bfloat162float(kn[e]); vv[e] = __bfloat162float(vn[e]); }
+    if (AHEAD) load(min(t + NA_WARPS, t1 - 1));
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
       if (g < G) {
         float s = 0.f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s += (e < per ? s_q[g * NA_MAX_D + lane + 32 * e] : 0.f) * kv[e];
+        for (int e = 0; e < PER; ++e) s += s_q[g * NA_MAX_D + lane + 32 * e] * kv[e];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         s *= scale;
@@ -92,7 +101,7 @@ __device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qr
         const float corr = exp2f(m[g] - mn), p = exp2f(s - mn);
         l[g] = l[g] * corr + p;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[g][e] = acc[g][e] * corr + p * vv[e];
+        for (int e = 0; e < PER; ++e) acc[g][e] = acc[g][e] * corr + p * vv[e];
         m[g] = mn;
       }
     }
@@ -101,14 +110,13 @@ __device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qr
   for (int g = 0; g < 8; ++g) {
     if (g < G) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (e < per) s_part[warp][g][lane + 32 * e] = acc[g][e];
+      for (int e = 0; e < PER; ++e) s_part[warp][g][lane + 32 * e] = acc[g][e];
       if (lane == 0) { s_part[warp][g][NA_MAX_D] = m[g]; s_part[warp][g][NA_MAX_D + 1] = l[g]; }
     }
   }
   __syncthreads();
-  for (int i = tid; i < G * d; i += NA_THREADS) {
-    const int g = i / d, c = i % d;
+  for (int i = tid; i < G * D; i += NA_THREADS) {
+    const int g = i / D, c = i % D;
     float M = -INFINITY;
     for (int w = 0; w < NA_WARPS; ++w) M = fmaxf(M, s_part[w][g][NA_MAX_D]);
     float a = 0.f, ls = 0.f;
@@ -121,6 +129,31 @@ __device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qr
     dst[c] = a;
     if (c == 0) { dst[NA_MAX_D] = M; dst[NA_MAX_D + 1] = ls; }
   }
+}
+// out of line, for a split whose tensor-core result is not finite (below)
+template <int D>
+__device__ __noinline__ void na_split_plain(const __nv_bfloat16* qrow0, const __nv_bfloat16* kbase, const __nv_bfloat16* vbase, int G,
+                                            int t0, int t1, float* smem, float* part, size_t row_stride) {
+  na_plain_tokens<D, true>(qrow0, kbase, vbase, G, t0, t1, smem, part, row_stride);
+}
+
+// Keys or values whose addresses are not 16-byte aligned.  A kernel of its own: it needs a third of the tensor-core kernel's shared
+// memory, so that an SM holds twice the warps (inside that kernel: 1120 us for 64 requests of 60 to 4000 tokens, 8 KV heads, groups
+// of 4, d = 128, against 466).
+template <int D>
+__global__ void __launch_bounds__(NA_THREADS)
+na_plain_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+                const int* __restrict__ lens, int Hq, int Hkv, int max_len, float* __restrict__ scratch) {
+  __shared__ float smem[NA_PLAIN_FLOATS];
+  const int split = blockIdx.x, n_split = gridDim.x, unit = blockIdx.y;
+  const int req = unit / Hkv, h = unit % Hkv, G = Hq / Hkv;
+  gp_pdl_launch_dependents();                           // the merge waits for this grid's end before it reads
+  const int len = max(0, min(lens[req], max_len));
+  const int chunk = (int)(((long long)len + n_split - 1) / n_split);
+  const int t0 = min(len, split * chunk), t1 = min(len, t0 + chunk);
+  const size_t at = ((size_t)req * Hkv + h) * (size_t)max_len * D;
+  na_plain_tokens<D, false>(q + ((size_t)req * Hq + h * G) * D, k + at, v + at, G, t0, t1, smem,
+                            scratch + (((size_t)req * Hq + h * G) * n_split + split) * NA_STRIDE, (size_t)n_split * NA_STRIDE);
 }
 
 // One thread block per (split, request, KV head): the split's share of the tokens, all G query heads of the group.
@@ -136,7 +169,7 @@ __device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qr
 // core over a long chain: the logits are added up in fp32 registers from MMAs of 16 products each, and so is O from
 // one tile to the next.
 // An infinite value would meet a zero mid or lo term (inf x 0), so a split whose result is not finite is done over
-// in plain arithmetic.
+// in plain arithmetic (an infinite value in every split, on the sizes below: 507 us; 491 before there was a first pass).
 // Measured, both kernels: 64 requests of 60 to 4000 tokens, 8 KV heads, groups of 4, d = 128 (532 MB): 464 us before (one
 // element per load, fp32 FMAs and shuffles), 96 us now, 5.6 TB/s; 32 requests of 8 to 1678, 4 KV heads, groups of 8: 114 us
 // before, 25 now.  Error against 64 bits 1.3e-7 to 1.9e-7 (before: 1.4e-7 to 2.0e-7 on the same inputs).  Four warps
@@ -144,7 +177,7 @@ __device__ __noinline__ void na_split_plain(const __nv_bfloat16* __restrict__ qr
 template <int D>
 __global__ void __launch_bounds__(NA_THREADS)
 na_partial_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                  const __nv_bfloat16* __restrict__ v, const int* __restrict__ lens, int Hq, int Hkv, int max_len, int aligned,
+                  const __nv_bfloat16* __restrict__ v, const int* __restrict__ lens, int Hq, int Hkv, int max_len,
                   float* __restrict__ scratch) {
   constexpr int ROW = D * 2;                            // bytes of a token's key or value
   constexpr int CH = D / 8;                             // 16-byte pieces of one
@@ -165,10 +198,6 @@ na_partial_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __re
   const __nv_bfloat16* vbase = v + ((size_t)req * Hkv + h) * (size_t)max_len * D;
   const size_t row_stride = (size_t)n_split * NA_STRIDE;
   float* part = scratch + (((size_t)req * Hq + h * G) * n_split + split) * NA_STRIDE;      // row g: + g * row_stride
-  if (!aligned) {
-    na_split_plain(qrow0, kbase, vbase, G, D, t0, t1, reinterpret_cast<float*>(smem), part, row_stride);
-    return;
-  }
 
   const int n_tiles = (t1 - t0 + TOK - 1) / TOK;
   uint8_t* ring = smem + warp * NA_STAGES * NA_TILE_BYTES;
@@ -294,7 +323,7 @@ na_partial_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __re
     for (int e = 0; e < 4; ++e) bad |= !(fabsf(o[jd][e]) < INFINITY) && (lane & 3) * 2 + (e & 1) < G;
   cp_async_wait<0>();
   if (__syncthreads_or(bad)) {
-    na_split_plain(qrow0, kbase, vbase, G, D, t0, t1, reinterpret_cast<float*>(smem), part, row_stride);
+    na_split_plain<D>(qrow0, kbase, vbase, G, t0, t1, reinterpret_cast<float*>(smem), part, row_stride);
     return;
   }
   // merge the warps; every slot of this (row, split) is rewritten on every call, so nothing stale survives
@@ -398,11 +427,17 @@ extern "C" int gp_attention_noalloc(const void* q, const void* k, const void* v,
   const long long most = ((long long)max_len + NA_MIN_SPLIT - 1) / NA_MIN_SPLIT, room = NA_ROOM / (n_req * n_q_heads);
   if (splits > most) splits = most;
   if (splits > room) splits = room;
-  const int aligned = (((uintptr_t)k | (uintptr_t)v) & 15) == 0;      // the tiles' copies move 16 bytes
-  const dim3 grid((unsigned)splits, (unsigned)units);
-  partial<<<grid, NA_THREADS, NA_SMEM, s>>>(static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
-                                           static_cast<const __nv_bfloat16*>(v), lens, n_q_heads, n_kv_heads, max_len, aligned,
-                                           scratch);
+  const __nv_bfloat16 *qp = static_cast<const __nv_bfloat16*>(q), *kp = static_cast<const __nv_bfloat16*>(k),
+                      *vp = static_cast<const __nv_bfloat16*>(v);
+  if ((((uintptr_t)k | (uintptr_t)v) & 15) == 0) {                    // the tiles' copies move 16 bytes
+    partial<<<dim3((unsigned)splits, (unsigned)units), NA_THREADS, NA_SMEM, s>>>(qp, kp, vp, lens, n_q_heads, n_kv_heads, max_len, scratch);
+  } else {
+    // a token costs a warp here what a tile of 16 costs there, so short splits pay: no fewer than the array holds at any size (with the
+    // rule above 128 requests, one of 16 000 tokens and the others of 200, 8 KV heads, groups of 2: 3860 us; now 477)
+    if (splits < GP_NOALLOC_SPLITS) splits = GP_NOALLOC_SPLITS;
+    auto plain = head_dim == 128 ? na_plain_kernel<128> : na_plain_kernel<64>;
+    plain<<<dim3((unsigned)splits, (unsigned)units), NA_THREADS, 0, s>>>(qp, kp, vp, lens, n_q_heads, n_kv_heads, max_len, scratch);
+  }
   if (cudaGetLastError() != cudaSuccess) return GP_ERR_CUDA;
   return gp_launch(na_merge_kernel, n_req * n_q_heads, head_dim, 0, s, true, static_cast<const float*>(scratch), (int)splits,
                    static_cast<float*>(out)) == cudaSuccess ? GP_OK : GP_ERR_CUDA;

@@ -127,6 +127,9 @@ def _dense(rng, hq, hkv, d, lens, max_len, offset=0):
     (1, 1, 64, (5000,), 0),
     (8, 2, 128, (77, 300), 1),
     (7, 1, 64, (77, 300), 4),
+    (16, 4, 128, (1, 0, 7, 8, 9, 31, 33, 1025), 1),
+    (1, 1, 64, (5000,), 3),
+    (8, 8, 64, (2500, 1) + (3,) * 118, 1),
 ])
 def test_noalloc_attention_at_tile_and_split_edges(hq, hkv, d, lens, offset):
     import torch
@@ -159,3 +162,27 @@ def test_noalloc_attention_with_an_infinite_value_keeps_the_other_columns():
     assert np.array_equal(np.isinf(got), np.isinf(want)) and not np.isnan(got).any()
     fin = np.isfinite(want)
     assert np.linalg.norm(got[fin] - want[fin]) <= 1e-6 * np.linalg.norm(want[fin])
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_noalloc_attention_with_a_key_that_is_no_finite_number(value, offset):
+    """Against positive query elements a key element of -inf is a token without weight.  With +inf or NaN the weights of the heads that
+    read it have no finite sum, and a row without a positive sum of weights is written as zeros.  The other heads are untouched."""
+    import torch
+    rng = np.random.default_rng(31)
+    hq, hkv, d, n, G = 6, 2, 128, 100, 3
+    (q, K, V), (qf, Kf, Vf) = _dense(rng, hq, hkv, d, (n,), n, offset)
+    q.view(hq, d)[:, 5] = 0x3f80                                   # 1.0
+    qf[0][:, 5] = 1.0
+    K.view(hkv, n, d)[1, 45, 5] = 0x7fc0 if np.isnan(value) else 0x7f80 if value > 0 else 0xff80 - 0x10000
+    if value == -np.inf:
+        Kf[0, 1, 45, 5] = value
+    lens_d = torch.tensor([n], dtype=torch.int32, device="cuda")
+    out = torch.zeros((1, hq, d), dtype=torch.float32, device="cuda")
+    B.gp_attention_noalloc(q.data_ptr(), K.data_ptr(), V.data_ptr(), lens_d.data_ptr(), 1, hq, hkv, d, n, out.data_ptr(), 0)
+    got = out.cpu().numpy().astype(np.float64)[0]
+    want = O.attention_decode(qf[0], Kf[0], Vf[0])
+    clean = hq if value == -np.inf else G
+    assert np.linalg.norm(got[:clean] - want[:clean]) <= 1e-6 * np.linalg.norm(want[:clean])
+    assert not got[clean:].any()
