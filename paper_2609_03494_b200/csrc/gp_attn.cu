@@ -33,7 +33,8 @@
 //
 // The two warp groups re-split the register file (setmaxnreg): the service warps keep 80 registers per
 // thread, the consumers, which hold the output accumulators, get 176 (at 160 their loop spills: 13.8 ms against 12.0 on
-// pages of 256).
+// pages of 256).  At this split the kernel still spills: 60 bytes a thread at d = 64, 128 to 184 at d = 128.  All of it at d = 64 and
+// most at d = 128 is the merge of split outputs (a service warp, once per split unit); without it 24 to 72 bytes are left.
 // All waits are bounded; a wait that gives up sets an error bit (with a code for which wait it was) and an
 // abort flag that drains the CTA.  No wait of an item depends on a later item being published.
 #include "gp_dev.cuh"
@@ -297,11 +298,11 @@ __device__ __forceinline__ double bf16_hi_scaled(uint32_t w) { return __hiloint2
 // the same mapping, so the contraction is over the same d on both sides).  One block of eight columns at a time (nt of them: a
 // group of eight heads has two).  What bounds it: the fp64 pipe and four chains of dependent DMMAs; the registers it takes are
 // the consumers' (two blocks together spilled: 84.0 ms against 80.0 on 36 layers x 256 requests).  Stores the exponentials
-// per token and the page's softmax partials per column.  `odd`: keys of the page may be infinite or not numbers, which their
-// bits read as a double's are not: the same contraction over converted keys.
+// per token and the page's softmax partials per column.  Keys that are infinite or not numbers, which their bits read as a
+// double's are not, are looked for on the way and put in afterwards.
 template <int D>
 __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* tile, const double* qt, int G, int lh, long long zoff,
-                                               int tok0, int nt, bool odd) {
+                                               int tok0, int nt) {
   constexpr int CH = D / 8, ROW_BYTES = D * 2;
   const int lane = threadIdx.x & 31, grp = lane >> 2, t4 = lane & 3;
   double z[2][2][2];                                      // [even / odd chunks][token half][column pair]
@@ -311,6 +312,7 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
   const double* qrow = qt + (size_t)(n < 2 * G ? n : 0) * (D + QT_PAD) + 2 * t4;
   const uint8_t* krow0 = tile + grp * ROW_BYTES + 4 * t4;
   const uint8_t* krow1 = tile + (8 + grp) * ROW_BYTES + 4 * t4;
+  uint32_t most = 0;                                      // the largest magnitudes among the keys' low and high halves, as bits
 #pragma unroll 4
   for (int c = 0; c < CH; c += 2) {
 #pragma unroll
@@ -318,28 +320,11 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
       const uint32_t ka = *reinterpret_cast<const uint32_t*>(krow0 + (((c + odd) ^ grp) << 4));   // grp == token & 7
       const uint32_t kb = *reinterpret_cast<const uint32_t*>(krow1 + (((c + odd) ^ grp) << 4));
       const double2 qq = *reinterpret_cast<const double2*>(qrow + (c + odd) * 8);
+      most = __vmaxu2(most, __vmaxu2(ka & 0x7fff7fffu, kb & 0x7fff7fffu));
       dmma(z[odd][0][0], z[odd][0][1], bf16_lo_scaled(ka), qq.x);
       dmma(z[odd][1][0], z[odd][1][1], bf16_lo_scaled(kb), qq.x);
       dmma(z[odd][0][0], z[odd][0][1], bf16_hi_scaled(ka), qq.y);
       dmma(z[odd][1][0], z[odd][1][1], bf16_hi_scaled(kb), qq.y);
-    }
-  }
-  if (odd) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) (&z[0][0][0])[i] = 0.0;
-#pragma unroll 1
-    for (int c = 0; c < CH; c += 2) {
-#pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        const uint32_t ka = *reinterpret_cast<const uint32_t*>(krow0 + (((c + w) ^ grp) << 4));
-        const uint32_t kb = *reinterpret_cast<const uint32_t*>(krow1 + (((c + w) ^ grp) << 4));
-        const double2 qq = *reinterpret_cast<const double2*>(qrow + (c + w) * 8);
-        const double q0 = qq.x * 0x1p-896, q1 = qq.y * 0x1p-896;
-        dmma(z[w][0][0], z[w][0][1], (double)bf16_lo_f(ka), q0);
-        dmma(z[w][1][0], z[w][1][1], (double)bf16_lo_f(kb), q0);
-        dmma(z[w][0][0], z[w][0][1], (double)bf16_hi_f(ka), q1);
-        dmma(z[w][1][0], z[w][1][1], (double)bf16_hi_f(kb), q1);
-      }
     }
   }
   const double inv_sqrt_d = Z_SCALE / sqrt((double)D);
@@ -347,6 +332,20 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
   const int col = nt * 8 + 2 * t4;
   double z00 = (z[0][0][0] + z[1][0][0]) * inv_sqrt_d, z01 = (z[0][0][1] + z[1][0][1]) * inv_sqrt_d;
   double z10 = (z[0][1][0] + z[1][1][0]) * inv_sqrt_d, z11 = (z[0][1][1] + z[1][1][1]) * inv_sqrt_d;
+  if (__any_sync(0xffffffffu, (most & 0xffffu) >= 0x7f80u || most >= 0x7f800000u)) {       // such a key adds infinity, or no number
+#pragma unroll 1
+    for (int j = 0; j < D; ++j) {
+      const double* qj = qt + (size_t)(col < 2 * G ? col : 0) * (D + QT_PAD) + j;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const uint32_t kw = *reinterpret_cast<const uint16_t*>(tile + (half * 8 + grp) * ROW_BYTES + (((j >> 3) ^ grp) << 4) + (j & 7) * 2);
+        if ((kw & 0x7f80u) == 0x7f80u) {
+          (half ? z10 : z00) += (double)bf16_lo_f(kw) * qj[0];
+          (half ? z11 : z01) += (double)bf16_lo_f(kw) * qj[D + QT_PAD];
+        }
+      }
+    }
+  }
   // the page's softmax partials per column: max and sum of exponentials over its 16 tokens; the
   // exponentials themselves are what is stored per token
   double m0 = fmax(z00, z10), m1 = fmax(z01, z11);
@@ -691,9 +690,6 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             mma_bf16(s_acc[1], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b10, b11);
           }
         }
-        // a key that is infinite or not a number leaves no finite score with any query (of row 0, which is always one of the group)
-        const bool odd_keys = need_qt && __any_sync(0xffffffffu, !(fabsf(s_acc[0][0]) + fabsf(s_acc[0][1]) + fabsf(s_acc[1][0]) +
-                                                                  fabsf(s_acc[1][1]) < INFINITY));
         // online softmax in the log2 domain
         float sv[2][2];
         const int n_valid = has_new ? (n_new - tok0) : GP_PAGE;
@@ -750,8 +746,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             qt_here = true;
           }
           const long long zoff = ((long long)(unsigned)sd[10]) | ((long long)sd[11] << 32);
-          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0, odd_keys);
-          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1, odd_keys);
+          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0);
+          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1);
         }
         __syncwarp();
         if (!top_up(it)) { ok = false; break; }            // the stage is free: fetch the next tile into it

@@ -22,7 +22,7 @@
 //                                         behind the attention kernel of its own step, with every job waiting for the
 //                                         attention kernel's report that its unit is complete (synchronous mode), or
 //                                         beside the attention kernel of the next step (asynchronous mode);
-//   gp_bsel_kernel, gp_compact_kernel     selection + decisions + merge, then compaction, as kernels of their own
+//   gp_bsel_kernel, gp_compact_kernel     selection + decisions, then compaction, as kernels of their own
 //   (and gp_decide_kernel)                (large pools, the layer-by-layer step; with the KV heads spread over several
 //                                         pools the decisions wait for the sums of all pools in a kernel of their own).
 //
@@ -406,7 +406,7 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
             }
           }
           // a job of one array; the larger score by its bits, as everywhere (one that is not a number is the largest)
-          if (aS == aL) aS[tok] = views == 3 ? __longlong_as_double((long long)max(key_of(a[0]), key_of(a[1]))) : a[views >> 1];
+          if (aS == aL) aS[tok] = views == 3 ? (key_of(a[0]) > key_of(a[1]) ? a[0] : a[1]) : a[views >> 1];
           else { aS[tok] = a[0]; aL[tok] = a[1]; }
           const unsigned w0 = (unsigned)__double2hiint(a[0]), w1 = (unsigned)__double2hiint(a[1]), w2 = max(w0, w1);
           lo_w[0] = min(lo_w[0], w0); lo_w[1] = min(lo_w[1], w1); lo_w[2] = min(lo_w[2], w2);
@@ -836,7 +836,8 @@ __device__ __forceinline__ void count_shared(const GpDev& p, int e) {
 }
 
 // The selection as a kernel of its own.  Two thread blocks to an SM at 128 registers; three at 80 spill and are slower
-// (20 000 cycles per unit become 36 000).
+// (20 000 cycles per unit become 36 000).  Groups of eight spill at 128 as well (240 bytes a thread here, 192 in gp_chain_kernel: the
+// values of a token, eight per view, are loaded two tokens ahead), the smaller groups by 8 to 24 bytes.
 template <int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions,
