@@ -938,3 +938,72 @@ def test_layer_entry_with_fused_query_key_normalisation(rope_theta, hq, hkv, d):
         assert B.gp_debug_pool(gpu.handle)[2][7] == 0
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("rope_theta,hq,hkv,d", [(1e4, 3, 3, 64), (0.0, 4, 2, 128), (1e6, 8, 2, 128), (0.0, 16, 2, 64)])
+def test_fused_query_key_normalisation_of_requests_in_many_pieces(rope_theta, hq, hkv, d):
+    """Every work item normalises its own copy of the queries.  Requests of 1, 2, 3, 8, 9 and 17 items of 32 pages, and at their capacity
+    boundary (the first step, items of 8 pages) of 2, 8, 9 and 17: merged in one level and in two, with a last group of one.  Groups of 1,
+    2, 4 and 8: with one head per group the second summary warp has none.  Three steps, every layer of a step in another order."""
+    import torch
+    L, eps = 2, 1e-6
+    plain, boundary = [20, 64, 70, 250, 288, 540], [10, 64, 72, 136]             # pages
+    lens = [16 * p - 9 for p in plain] + [16 * p - 1 for p in boundary]
+    caps = plain + boundary
+    kw = dict(n_pages=sum(caps), max_pages_per_req=max(caps), max_requests=len(lens), k_loc=4, tau=2.0, rope_theta=rope_theta)
+    gpu = B.Pool(B.make_config(L, hq, hkv, d, **kw))
+    ora = O.OraclePool(O.OracleConfig(L, hq, hkv, d, **kw))
+    rng = np.random.default_rng(37)
+    bits = lambda *shape: W.f32_to_bf16_bits((2.0 * rng.standard_normal(shape)).astype(np.float32))
+    f = W.bf16_bits_to_f64
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to("cuda:0")
+    wq, wk = ((1.0 + 0.3 * rng.standard_normal((L, d))).astype(np.float32) for _ in range(2))
+    wq_d, wk_d = torch.from_numpy(wq).cuda(), torch.from_numpy(wk).cuda()
+    round_bf16 = lambda x: W.f32_to_bf16_bits(x.astype(np.float32))
+
+    def normalise(x_bits, w):
+        x = f(x_bits)
+        return x / np.sqrt((x * x).mean(axis=-1, keepdims=True) + eps) * w.astype(np.float64)
+
+    try:
+        for n0 in lens:
+            kp, vp = bits(L, n0, hkv, d), bits(L, n0, hkv, d)
+            assert gpu.request_add(-1, 0, kp, vp, n0, 0)[0] == B.GP_OK
+            assert ora.request_add(-1, 0, f(kp), f(vp), n0, 0)[0] == O.OK
+        n_req = len(lens)
+        ids = torch.arange(n_req, dtype=torch.int32, device="cuda:0")
+        for t in range(3):
+            q_raw, k_raw, v = bits(L, n_req, hq, d), bits(L, n_req, hkv, d), bits(L, n_req, hkv, d)
+            pos = [ora.request_state(r)[2] for r in range(n_req)]
+            q_n = np.stack([round_bf16(normalise(q_raw[l], wq[l])) for l in range(L)])
+            k_n = np.stack([np.stack([round_bf16(O.rope(normalise(k_raw[l, r], wk[l]), pos[r], rope_theta)) for r in range(n_req)])
+                            for l in range(L)])
+            rec = ora.decode_step(list(range(n_req)), f(q_n), f(k_n), f(v))
+            out = torch.zeros((L, n_req, hq, d), dtype=torch.float32, device="cuda:0")
+            act = torch.zeros(n_req, dtype=torch.int32, device="cuda:0")
+            qd, kd, vd = dev(q_raw), dev(k_raw), dev(v)
+            s_ = gpu.stream()
+            B.gp_step_begin(gpu.handle, ids.data_ptr(), n_req, act.data_ptr(), s_)
+            for l in rng.permutation(L):
+                l = int(l)
+                B.gp_attn_layer_qknorm(gpu.handle, l, ids.data_ptr(), n_req, qd[l].data_ptr(), kd[l].data_ptr(), vd[l].data_ptr(),
+                                       wq_d[l].data_ptr(), wk_d[l].data_ptr(), eps, out[l].data_ptr(), s_)
+            B.gp_step_end(gpu.handle, ids.data_ptr(), n_req, act.data_ptr(), s_)
+            assert act.cpu().tolist() == rec.actions.tolist(), t
+            assert np.abs(out.cpu().numpy() - rec.out).max() <= LS.ATTN_MAX_ABS, t
+            if t == 0:
+                for r, info in rec.boundary.items():
+                    ks, kl, _ = B.gp_debug_boundary(gpu.handle, r, L, hkv)
+                    assert np.array_equal(ks, info.K_s) and np.array_equal(kl, info.K_l)
+                assert sorted(rec.boundary) == list(range(len(plain), n_req))
+        for r in range(n_req):
+            assert B.gp_debug_request(gpu.handle, r, max(caps))[:3] == ora.request_state(r)[:3]
+            g, o = B.gp_debug_summaries(gpu.handle, r, L, hq, d), ora.summaries(r)
+            assert (np.linalg.norm(g - o, axis=-1) / np.linalg.norm(o, axis=-1)).max() <= LS.SUMMARY_REL
+            n = ora.request_state(r)[1]
+            for l in range(L):
+                for h in range(hkv):
+                    assert np.array_equal(B.gp_debug_retained(gpu.handle, r, l, h, n), ora.retained(r, l, h))
+        assert B.gp_debug_pool(gpu.handle)[2][7] == 0
+    finally:
+        gpu.close()
