@@ -41,7 +41,6 @@ enum {
   HDR_DONE_SEL,      // CTAs of the selection kernel that have finished
   HDR_WORK_CMP,      // ticket counter of the compaction kernel
   HDR_N_CITEM,       // compaction work items (chunks x layers x heads)
-  HDR_FREE,          // (not in use)
   HDR_N_COW,         // copy-on-write targets allotted this step
   HDR_COUNT = 16
 };
@@ -187,13 +186,6 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: returns false when the limit ran out (the caller records GP_E_SPIN and goes on).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (uint32_t it = 0; it < GP_SPIN_LIMIT; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-  }
-  return false;
-}
 // 1-D bulk copy global -> shared of this CTA (this CTA only), completion counted on an mbarrier.
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {
   asm volatile(
@@ -202,12 +194,9 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       "l"(src_gmem), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
-// 16-byte asynchronous copy global -> shared (L2 only), tracked per thread in commit groups
-__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void* src_gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src_gmem) : "memory");
-}
-// the same with an L2 eviction-priority hint (createpolicy): streamed data marked evict-first leaves the L2 before
-// the small, reused state and the code of the step's other kernels
+// 16-byte asynchronous copy global -> shared (L2 only), tracked per thread in commit groups, with an L2 eviction-priority
+// hint (createpolicy): streamed data marked evict-first leaves the L2 before the small, reused state and the code of the
+// step's other kernels
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));

@@ -171,7 +171,7 @@ Layout make_layout(const gp_config& c) {
   L.rope_f = take(M * (d / 2) * 2 * 4);
   L.rope_cs = take(M * (d / 2) * 2 * 8);
   L.partials = take((size_t)L.max_rc * LH * G * (d + 2) * 4);
-  L.scores = take((c.policy == GP_POLICY_SHRINK ? 4 : 3) * LH * Tb * 8);
+  L.scores = take(3 * LH * Tb * 8);                // a whole unit uses two regions, a job of one task the one of its number
   if (c.async_boundary) {                        // the second set of what a boundary chain reads beside the next step
     L.bnd_info2 = take(M * 32);
     L.bnd_acc2 = take(M * 16);
