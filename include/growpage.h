@@ -139,7 +139,7 @@ typedef struct gp_config {
                                 an error: requests that do not fit report GP_ACT_SCRATCH          */
   int64_t max_boundary_tokens; /* bound on the summed candidate tokens of the requests that reach their
                                 boundary in one step; sizes the boundary scratch (summary logits,
-                                per-page softmax partials, large-set scores), 50 to 60 bytes per token,
+                                per-page softmax partials, large-set scores), 18 G + 24 bytes per token,
                                 layer and KV head.  0 = max_batch_tokens: every request of a batch may be
                                 at its boundary (equal prompts reach it together).  On average one
                                 request in sixteen is, so a large pool can set an eighth of that, at
@@ -333,6 +333,7 @@ int gp_release(gp_pool* pool, int32_t req, void* stream);
  * call this after synchronising its stream.  The bits are sticky for the life of the pool:
  *   1 a bounded wait inside the attention kernel gave up   2 free-list accounting out of range
  *   4 an index failed a bounds check (the access was skipped)   8 a bounded wait inside the compaction kernel gave up
+ *  16 a selection job's bounded wait for its unit's summary logits gave up
  * (bits 7 and up say which wait of the attention kernel it was). */
 int gp_pool_status(gp_pool* pool, int32_t* error_bits);
 
@@ -377,9 +378,9 @@ int gp_debug_pool(gp_pool* pool, int64_t* n_free, int32_t* refcounts, int64_t co
 
 /* ---- measurement ----------------------------------------------------------------------------- */
 
-#define GP_N_KERNELS 4   /* plan, attention (+ boundary logits), selection + decision, compaction; with the boundary
-                            work in one kernel (overlap_slots >= 0, the default) the third entry is that kernel and
-                            the fourth stays zero */
+#define GP_N_KERNELS 4   /* plan, attention (+ summaries, boundary logits), selection + decision, compaction; with the
+                            boundary work in one kernel (see overlap_slots) the third entry is that kernel and the
+                            fourth an empty interval */
 
 /* With profiling on, every kernel of gp_decode_step is bracketed by CUDA events on the step's
  * stream (this serialises nothing but adds event records).  Off by default. */
@@ -387,15 +388,15 @@ int gp_set_profiling(gp_pool* pool, int32_t enable);
 
 /* Early planning (off by default).  The first kernel of gp_decode_step is launched as a programmatic
  * dependent of whatever kernel precedes it on the stream.  With the option off it waits for that
- * kernel to end before it reads anything: always safe.  With it on, it reads dev_req_ids and q, plans
- * the step and updates the query summaries before that wait, beside the compaction kernel of the
- * step before, and waits only before it looks at the free list.  That is correct only if
- * dev_req_ids and q are complete in memory by the time the preceding kernel on the stream lets
- * its dependents be scheduled: true when they were produced by copies or by kernels that do not
- * signal programmatic launch completion (or when nothing was enqueued since the step before);
- * not true when the query projection enqueued just before the step signals completion ahead of its
- * stores.  gp_decode_step_host always plans early (its inputs arrive by copies).  The
- * layer-by-layer calls are not affected. */
+ * kernel to end before it reads anything: always safe.  With it on, it reads dev_req_ids and plans
+ * the step before that wait, beside the compaction of the step before, and waits only before it looks
+ * at the free list.  That is correct only if dev_req_ids is complete in memory by the time the preceding
+ * kernel on the stream lets its dependents be scheduled: true when it was produced by copies or by
+ * kernels that do not signal programmatic launch completion (or when nothing was enqueued since the
+ * step before); not true when a kernel enqueued just before the step writes the ids and signals completion
+ * ahead of its stores.  (Queries, keys and values are read by the step's second kernel: nothing is asked of
+ * them.)  gp_decode_step_host always plans early (its inputs arrive by copies).  The layer-by-layer
+ * calls are not affected; the step after a gp_step_abort waits whatever the option says. */
 int gp_set_early_plan(gp_pool* pool, int32_t enable);
 
 /* Synchronises, then returns the accumulated device time in milliseconds and the launch count of
@@ -433,10 +434,12 @@ int gp_test_withhold(gp_pool* pool, int32_t what, int32_t spin_limit);
  * the library holds that array until the process exits.
  *
  *   q     device bf16 [n_req][n_q_heads][d]
- *   k, v  device bf16 [n_req][n_kv_heads][max_len][d], rows in plain order (no page layout, no swizzle)
+ *   k, v  device bf16 [n_req][n_kv_heads][max_len][d], rows in plain order (no page layout, no swizzle); any
+ *         alignment, but off a 16-byte boundary the call takes about five times as long
  *   lens  device int32 [n_req]: tokens of each request, 1..max_len (values above max_len are clipped;
  *         a request with lens <= 0 attends to nothing and gets an output row of zeros)
- *   out   device fp32 [n_req][n_q_heads][d]: softmax(q.K/sqrt(d)).V per query head, KV head g / G
+ *   out   device fp32 [n_req][n_q_heads][d]: softmax(q.K/sqrt(d)).V per query head, KV head g / G (zeros where
+ *         the weights have no positive finite sum: a key that is +inf or not a number)
  *
  * Limits: d is 64 or 128, G = n_q_heads / n_kv_heads <= 8, n_req * n_q_heads <= GP_NOALLOC_MAX_ROWS;
  * beyond that the call returns GP_ERR_TOO_LARGE and does nothing.  It calls no cudaMalloc, cudaFree or

@@ -82,8 +82,8 @@ inline size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 // Pages per attention work item: 64 (two page ids per producer lane), and half of that for requests at their
 // capacity boundary, whose pages also pay for the fp64 logits.  When an attention launch has less than one such
 // item of work per CTA (small batches, short sequences; a layer-by-layer launch, which covers one layer's heads
-// only), smaller items (32 and 8 pages) keep more CTAs busy (measured: the 36-layer shape with 16 requests,
-// layer by layer, takes 1030 us per step that way, 1252 with the large items).
+// only), smaller items (32 and 8 pages) keep more CTAs busy (measured when a layer was three launches: the 36-layer shape
+// with 16 requests, layer by layer, 1030 us per step that way, 1252 with the large items; a layer is one launch now, 900 us).
 constexpr int GP_CHUNK = 64, GP_BCHUNK = 32;
 constexpr int GP_FINE_CHUNK = 32, GP_FINE_BCHUNK = 8;
 int chunk_pages_setting() { return GP_CHUNK; }
@@ -367,8 +367,9 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // fp64 logits): the attention kernel deals them out in that order, largest first.  Counting sort.
   const int key = chunks > 0 ? min(GP_COST_BINS - 1, cp * (isb ? 4 : 1)) : 0;
   // Items of equal cost keep the batch's order (a rank counted over the earlier batch slots, not the order in
-  // which atomics land), so that the same batch is dealt to the thread blocks the same way every time and the
-  // attention outputs repeat bit for bit.
+  // which atomics land), so that the same batch gives the same numbered list every time.  An item's number says which of a
+  // block's warps takes which of its tiles, and split outputs are merged in chunk order: with the numbers fixed, the attention outputs
+  // repeat bit for bit whichever thread block draws an item.
   s_first[i] = chunks > 0 ? (key << 16) | chunks : 0;        // s_first has served its purpose: cost class and items
   if (chunks > 0) atomicAdd(&s_bin[key], chunks);
   __syncthreads();
@@ -782,9 +783,10 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   pool->attn_grid_ov = pool->attn_grid;
   pool->chain_grid_ov = 0;
   // One kernel behind the attention kernel pays while a step's boundary work is a few hundred jobs: it saves a kernel
-  // boundary and starts its jobs while the attention kernel drains (64 requests x 8 units: 68 us per step against
-  // 75).  With thousands of units the compaction moves hundreds of megabytes and wants the four-kernel path's larger
-  // compaction grid (36 layers x 256 residents: 4.8 ms against 5.2; 256 requests x 8 units: 0.49 against 0.52).
+  // boundary and starts its jobs while the attention kernel drains (requests of 200 to 1200 tokens, 64 x 8 units: 72.6 us per
+  // step against 79.5).  From about a thousand units on the compaction wants the four-kernel path's larger grid, few as the
+  // boundaries of a step may be (8 layers x 16 requests: 109.0 us in one kernel, 108.5 in four; 36 layers x 4: 104.5, 99.6;
+  // x 16: 393, 378; x 64: 1403, 1393; x 256: 4866, 4754; 1 layer x 256: 181, 178).
   const bool fused_auto = (long long)cfg->max_requests * cfg->n_layers * cfg->n_kv_heads <= 1024;
   if (!cfg->async_boundary && (cfg->overlap_slots == -2 || (cfg->overlap_slots == 0 && fused_auto))) {
     pool->chain_grid_ov = pool->chain_grid_max;    // the whole grid, behind the attention kernel's
@@ -909,8 +911,8 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
     // first_plain: the kernel before the plan on the stream is not one of this library's (the host entry point's
     // fetch of the inputs): no programmatic dependence on it
     if (pool->chain_grid_ov > 0) {
-      // Three kernels.  The boundary work of the step (selection jobs, decisions, compaction, then the merge of the
-      // split outputs) is one kernel behind the attention kernel.  Its thread blocks take their places as that
+      // Three kernels.  The boundary work of the step (selection jobs, decisions, compaction) is one kernel behind the
+      // attention kernel.  Its thread blocks take their places as that
       // kernel's leave (or, with overlap_slots > 0, run beside it on slots its grid leaves free), and a selection job
       // starts as soon as the attention kernel has reported its unit's summary logits complete.
       launch_plan(pool, dev_req_ids, n_req, dev_actions, pool->early_plan != 0, s, pdl && !pool->first_plain, false, nullptr,
@@ -936,7 +938,7 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
   } else {
     // Asynchronous boundary work, all on the caller's stream: plan and attention of this step, then one kernel
     // with the boundary chain of the step before (working sets, decisions, compaction), which runs beside the
-    // attention kernel, ends after it and then merges this step's split outputs.  Step t uses scratch set t mod 2.
+    // attention kernel and ends after it.  Step t uses scratch set t mod 2.
     const int par = (int)(pool->serial & 1);
     const GpDev& d = par ? pool->dev_alt : pool->dev;
     const GpDev& dprev = par ? pool->dev : pool->dev_alt;

@@ -1,7 +1,6 @@
 """The ways a synchronous step can launch its boundary work (gp_config.overlap_slots).
 
-With -2 the selection jobs, the decisions, the compaction and the merge of split outputs are one kernel behind the
-attention kernel, whose jobs start when that kernel has reported their unit's summary logits complete; with -1 a
+With -2 the selection jobs, the decisions and the compaction are one kernel behind the attention kernel, whose jobs start when that kernel has reported their unit's summary logits complete; with -1 a
 selection and a compaction kernel run one after the other (four launches); the default (0) picks between the two
 by the pool's size, so the other tests of the synchronous mode run one or the other.  Here both are forced, and
 the one kernel also runs beside the attention kernel on thread-block slots that kernel's grid gives up (N > 0).  Nothing about the results may change: the same lockstep comparison against the oracle
