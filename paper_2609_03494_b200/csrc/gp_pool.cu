@@ -1,5 +1,5 @@
 // Host side of the C ABI, the blob layout, and the small bookkeeping kernels:
-// step plan, decision + device allocator, admission, prompt ingest, release, debug gathers.
+// step plan, admission, prompt ingest, release, debug gathers.
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
