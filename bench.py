@@ -353,7 +353,7 @@ def run_ours(args):
     head.reset()
     head.roll(S0)
     torch.cuda.synchronize(device)
-    moved0 = int(head.counters()[8])
+    counters0 = head.counters()
     B.gp_set_profiling(head.pool.handle, True)
     attn_bytes = score_bytes = 0.0
     n_tok = n_kv = 0
@@ -369,8 +369,11 @@ def run_ours(args):
     kms, kn = B.gp_get_kernel_times(head.pool.handle)
     B.gp_set_profiling(head.pool.handle, False)
     head.by_layer = by_layer
-    moved = int(head.counters()[8]) - moved0
-    compact_bytes = 2.0 * moved * (2 * s.head_dim * 2 + 4)
+    # a compression moves one page worth of rows per (layer, KV head), a Shrink two, and rewrites the order index of every row behind
+    # the first evicted one
+    done = [int(x) - int(y) for x, y in zip(head.counters(), counters0)]
+    rows = (done[1] + done[2] + 2 * done[10]) * s.n_layers * s.n_kv_heads * s.page_size
+    compact_bytes = 2.0 * (rows * (2 * s.head_dim * 2 + 4) + done[8] * 4)
     summ_bytes = float(n_tok) * s.n_layers * 2 * s.n_q_heads * s.head_dim * 8 * 2      # both views, read + write, fp64
     step_bytes = attn_bytes + score_bytes + compact_bytes + summ_bytes
     peak, peak_kind = measured_peak()

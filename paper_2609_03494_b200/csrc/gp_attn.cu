@@ -662,7 +662,11 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             *reinterpret_cast<uint4*>(g) = val;
             fence_proxy_async();
           }
-          if (lane == 0) p.tok[gp_tok_off(p, l, page, h) + s] = sd[7];
+          if (lane == 0) {
+            const size_t at = gp_tok_off(p, l, page, h) + s;
+            p.tok[at] = sd[7];
+            p.rank[at] = n_old;                            // the newest token: last in the order
+          }
           if (lane == 1 && lh == adv_lh) {
             // the request is one token further, its summaries in the other buffer (nothing in this kernel looks at these
             // words: what it needs is in the descriptors)

@@ -10,11 +10,10 @@
 //   decisions         by the CTA that finishes its jobs last: Eq. 8 per request, the action (grow, compress,
 //                     shrink), the device allocator: grants first, then copy-on-write targets, each in ascending
 //                     request id.
-//   compaction        per compressing unit: stable in-place compaction into (P-1) b slots ((P-2) b at a Shrink),
-//                     writing to copy-on-write targets where the source page is shared.  Work is claimed from a
-//                     ticket counter, a chunk of 64 source slots at a time (a chunk publishes "my sources are
-//                     read" before the next chunk may overwrite their tail) or, with many units, a unit at a
-//                     time.  The last CTA swaps in the target pages, drops the references to the replaced ones
+//   compaction        per compressing unit: stable in-place compaction into (P-1) b slots ((P-2) b at a Shrink):
+//                     the rows behind the new end fill the evicted slots before it, the order of the tokens is kept in
+//                     a word per slot; shared pages are copied to their targets.  Work is claimed from a
+//                     ticket counter.  The last CTA swaps in the target pages, drops the references to the replaced ones
 //                     and returns the last page of every request that shrank.
 //
 // It comes in two shapes that run the same device functions:
@@ -41,11 +40,19 @@ constexpr int SEL_T = 256;           // threads of the selection kernel
 constexpr int SEL_NW = SEL_T / 32;
 constexpr int SEL_CAP = 5120;        // candidate tokens whose scores (both views) are kept in shared memory, at most
 constexpr int CT = 256;              // threads of the compaction kernel
-constexpr int MOVE_TOK = GP_MOVE_TOK;     // source slots per compaction chunk
 constexpr int CMP_SHRINK = 1 << 30;       // flag on a compressing request's boundary index: the action is a Shrink
 
 __device__ __forceinline__ unsigned long long to_fix(double a) {
   return (unsigned long long)__double2ll_rn(a * TWO62);
+}
+
+// slots per compaction ticket, and the tickets of a unit that keeps n_end slots: the last one has what lies behind them as well
+// (test support: see GP_WITHHOLD_CHUNK)
+__device__ __forceinline__ int part_slots_of(const GpDev& p) {
+  return (p.withhold & (GP_WITHHOLD_CHUNK | GP_TEST_COMPACT_BY_PART)) ? GP_PART_MIN : GP_PART_SLOTS;
+}
+__device__ __forceinline__ int parts_of(const GpDev& p, int n_end) {
+  return (p.withhold & GP_TEST_COMPACT_BY_UNIT) ? 1 : (n_end + part_slots_of(p) - 1) / part_slots_of(p);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -174,7 +181,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
       cow += s_ksh[e];
       const bool shrink = (s_want[e] & 16) != 0;
       p.cmp_info[n_cmp] = make_int4(r, s_P[e], e | (shrink ? CMP_SHRINK : 0), chunks);
-      chunks += (s_P[e] * GP_PAGE + MOVE_TOK - 1) / MOVE_TOK;
+      chunks += parts_of(p, (s_P[e] - (shrink ? 2 : 1) * sub) * GP_PAGE);
       ++n_cmp;
       if (s_want[e] & 1) { report(bi, r, GP_ACT_COMPRESS_FALLBACK); ++fall; }
       else if (shrink) { report(bi, r, GP_ACT_SHRINK); ++shr; }
@@ -303,17 +310,21 @@ __device__ __forceinline__ SelSmem sel_smem_at(uint8_t* smem, int cap) {      //
 __device__ __forceinline__ unsigned long long key_of(double v) { return (unsigned long long)__double_as_longlong(v); }
 
 // Per-head softmax over the first `ntile` pages of the candidates and the group mean (Sec. 3.2): a^S and a^L of every
-// candidate.  The attention kernel left, per 16-token page t and column c (view, head), the page's maximum logit m_tc
+// candidate, in the order of the tokens (`ord`; the logits lie in the order of the slots).  The attention kernel left, per 16-token page t and column c (view, head), the page's maximum logit m_tc
 // and s_tc = sum of exp(z - m_tc), and per token x = exp(z - m_tc).  With M_c the maximum over pages and
 // f_tc = exp(m_tc - M_c):  softmax = x f_tc / Z_c,  Z_c = sum_t s_tc f_tc.  So this pass takes one exponential per page
 // and column instead of one per token and column; the factors f_tc / (G Z_c) of SEL_F / 2G pages at a time sit in
 // shared memory.  A thread takes whole tokens (a view's values of a token are contiguous).  All loads of the prologue
 // (page partials and the first tokens) are issued together.  `views`: bit 0 a^S, bit 1 a^L (a job that needs one view
 // reads only that one's logits).  Also leaves the range of the scores' high words.
+struct UnitOrder {          // the unit's order indices: of slot s, rank[table[s / 16] * page_stride + s % 16]
+  const int* table; const int* rank;
+  size_t page_stride;
+};
 template <int GG>
 __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __restrict__ x, size_t view_stride,
                                              const double* __restrict__ zs, double* __restrict__ aS, double* __restrict__ aL, int ntile,
-                                             int views) {
+                                             int views, const UnitOrder& ord) {
   constexpr int NC = 2 * GG;                             // columns
   constexpr int U = GG >= 4 ? 2 : 4;                     // tokens per thread in flight
   constexpr int KEEP = 2;                                // page partials per thread held in registers
@@ -331,6 +342,19 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
     if (t < ntile) keep[k] = ld_early2(zs + ((size_t)t * NC + myc) * 2);
   }
   double xv[U][2][GG];
+  int pg[U], at[U];                                      // page of a token (of the next pass of the loop), its place in the order
+  auto load_pages = [&](int tok0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) { const int t = (tok0 + tid + u * SEL_T) / GP_PAGE; pg[u] = t < ntile ? __ldg(ord.table + t) : 0; }
+  };
+  auto load_order = [&](int tok0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int tok = tok0 + tid + u * SEL_T;
+      if (tok < ntile * GP_PAGE) at[u] = __ldcg(ord.rank + (size_t)pg[u] * ord.page_stride + tok % GP_PAGE);
+    }
+  };
+  load_pages(0);
   auto load = [&](int tok0, int n_tok) {                 // tokens tok0 + tid, tok0 + tid + SEL_T, ... of both views
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -346,6 +370,8 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
   double mx = fmax(keep[0].x, keep[1].x);
 #pragma unroll 8
   for (int t = t0 + KEEP * TSTEP; t < ntile; t += TSTEP) mx = fmax(mx, __ldcg(zs + ((size_t)t * NC + myc) * 2));
+  load_order(0);
+  load_pages(U * SEL_T);
   column_reduce<true>(mx, NC, m.red, m.sM);
   const double mc = m.sM[myc];
   double acc = 0.0;
@@ -384,13 +410,15 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
     const int k_begin = tb * GP_PAGE, k_end = min(n, k_begin + FT * GP_PAGE);
     if (tb) {
       load(k_begin, k_end);
+      load_order(k_begin);
+      load_pages(k_begin + U * SEL_T);
       __syncthreads();
       for (int t = tb + t0; t < min(ntile, tb + FT); t += TSTEP)
         m.F[(t - tb) * NC + myc] = exp(__ldcg(zs + ((size_t)t * NC + myc) * 2) - mc) * rz;
       __syncthreads();
     }
     for (int k0 = k_begin; k0 < k_end; k0 += U * SEL_T) {
-      if (k0 != k_begin) load(k0, k_end);
+      if (k0 != k_begin) { load(k0, k_end); load_order(k0); load_pages(k0 + U * SEL_T); }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int tok = k0 + tid + u * SEL_T;
@@ -406,8 +434,9 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
             }
           }
           // a job of one array; the larger score by its bits, as everywhere (one that is not a number is the largest)
-          if (aS == aL) aS[tok] = views == 3 ? (key_of(a[0]) > key_of(a[1]) ? a[0] : a[1]) : a[views >> 1];
-          else { aS[tok] = a[0]; aL[tok] = a[1]; }
+          const int i = min(max(at[u], 0), n - 1);           // (within bounds whatever a wait that gave up left behind)
+          if (aS == aL) aS[i] = views == 3 ? (key_of(a[0]) > key_of(a[1]) ? a[0] : a[1]) : a[views >> 1];
+          else { aS[i] = a[0]; aL[i] = a[1]; }
           const unsigned w0 = (unsigned)__double2hiint(a[0]), w1 = (unsigned)__double2hiint(a[1]), w2 = max(w0, w1);
           lo_w[0] = min(lo_w[0], w0); lo_w[1] = min(lo_w[1], w1); lo_w[2] = min(lo_w[2], w2);
           hi_w[0] = max(hi_w[0], w0); hi_w[1] = max(hi_w[1], w1); hi_w[2] = max(hi_w[2], w2);
@@ -747,6 +776,7 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
   double* aS = small ? S.sS : p.scores + ((size_t)(single ? want >> 1 : 0) * LH + lh) * p.max_boundary_tokens + off;
   double* aL = single ? aS : small ? S.sL : aS + (size_t)LH * p.max_boundary_tokens;
   const int views = want == 1 ? 1 : want == 2 ? 2 : 3;
+  const UnitOrder ord = {p.page_table + (size_t)r * p.cap, p.rank + gp_tok_off(p, lh / p.Hkv, 0, lh % p.Hkv), (size_t)p.Hkv * GP_PAGE};
   const bool one_support = p.sub == 1;
   const bool entropy = p.metric == GP_METRIC_ENTROPY;
   for (int pass = 0; pass < (one_support ? 1 : 2); ++pass) {
@@ -755,7 +785,7 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
     if (!tasks) continue;
     __syncthreads();                                       // the unit or pass before is done with the shared arrays
     if (tid < 3) { m.rng[tid][0] = 0xffffffffu; m.rng[tid][1] = 0u; }
-    unit_softmax<GG>(S, z, view_stride, zs, aS, aL, ntile, views);      // (its barriers order rng before the first use)
+    unit_softmax<GG>(S, z, view_stride, zs, aS, aL, ntile, views, ord);      // (its barriers order rng before the first use)
     if (entropy && (tasks & 3)) {
       __syncthreads();                                     // the scores are there
       // the ablation's other metric: H = -sum a ln a of the view, summed in a fixed order (per thread over its
@@ -900,24 +930,31 @@ gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
 // ------------------------------------------------------------------------------------------------------
 // shared memory of the compaction
 struct CmpSmem {
-  int4* s_info;      // [GP_MAX_REQ + 1] compressing requests: {request, P, boundary index, first chunk}
-  int* ev;           // [2 * GP_MAX_BLK] slots the unit's compression (or Shrink) evicts
+  int4* s_info;      // [GP_MAX_REQ + 1] compressing requests: {request, P, boundary index, first part}
+  int* ev;           // [CMP_EV] the order indices that the unit's compression (or Shrink) evicts, ascending
+  int* ev_slot;      // [CMP_EV] where they lie: slot and page (its copy-on-write target, where it has one) of each
+  int* ev_page;
+  int* mv_page;      // [CMP_EV] slots from the unit's new end on: page, and new order index (-1: evicted)
+  int* mv_rank;
+  int* hole;         // [CMP_EV] evicted slots below the new end, as entries of `ev`
+  int* mover;        // [CMP_EV] retained slots from the new end on, as entries of mv_page
   int* s_i;          // [8]
-  int* s_dst;        // [MOVE_TOK] per source slot of the chunk: destination slot (-1: stays or goes)
-  int* s_spage;      // [MOVE_TOK] source page
-  int* s_dpage;      // [MOVE_TOK] destination page
   int* order;        // [GP_MAX_REQ + 1] last CTA: pages each request gives back
 };
-constexpr size_t CMP_SMEM_BYTES = (GP_MAX_REQ + 1) * 16 + (2 * GP_MAX_BLK + 8 + 3 * MOVE_TOK + GP_MAX_REQ + 1) * 4;
+constexpr int CMP_EV = 2 * GP_MAX_BLK;
+constexpr size_t CMP_SMEM_BYTES = (GP_MAX_REQ + 1) * 16 + (7 * CMP_EV + 8 + GP_MAX_REQ + 1) * 4;
 __device__ __forceinline__ CmpSmem cmp_smem_at(uint8_t* base) {       // base: 16-byte aligned, CMP_SMEM_BYTES
   CmpSmem C;
   C.s_info = reinterpret_cast<int4*>(base);
   C.ev = reinterpret_cast<int*>(base + (GP_MAX_REQ + 1) * 16);
-  C.s_i = C.ev + 2 * GP_MAX_BLK;
-  C.s_dst = C.s_i + 8;
-  C.s_spage = C.s_dst + MOVE_TOK;
-  C.s_dpage = C.s_spage + MOVE_TOK;
-  C.order = C.s_dpage + MOVE_TOK;
+  C.ev_slot = C.ev + CMP_EV;
+  C.ev_page = C.ev_slot + CMP_EV;
+  C.mv_page = C.ev_page + CMP_EV;
+  C.mv_rank = C.mv_page + CMP_EV;
+  C.hole = C.mv_rank + CMP_EV;
+  C.mover = C.hole + CMP_EV;
+  C.s_i = C.mover + CMP_EV;
+  C.order = C.s_i + 8;
   return C;
 }
 
@@ -987,186 +1024,236 @@ __device__ __noinline__ void swap_pages(const GpDev& p, const int4* s_info, int 
   if (threadIdx.x == 0) *p.free_top += order[n_cmp];
 }
 
-// The compaction of a step, run by every CTA of the calling grid (CT threads): work is claimed from the ticket
-// counter until none is left; the last CTA to finish swaps in the copy-on-write targets.  What a ticket stands for
-// depends on how much there is.  A few units (one layer, a handful of requests at their boundary): one 64-slot chunk
-// of a unit per ticket, so that all thread blocks have work; a chunk says when its sources are read, and waits for
-// that word from the chunks before it whose sources its destinations reach.  Units for every thread block twice
-// over: one unit per ticket, its chunks in ascending order by the same thread block (a chunk's destinations lie
-// below the next chunk's sources, and program order puts every chunk's reads before the next chunk's writes), which
-// saves the ticket, the eviction list and the waits per chunk and skips the chunks below the first evicted slot.
+// entries [0, n) whose flag is set, in ascending order into `out`, by one warp; returns their number
+template <typename F>
+__device__ __forceinline__ int warp_pack(int n, int* out, F flag) {
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const bool f = i0 + lane < n && flag(i0 + lane);
+    const unsigned m = __ballot_sync(0xffffffffu, f);
+    if (f) out[at + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
+    at += __popc(m);
+  }
+  return at;
+}
+
+// The compaction of a step, run by every CTA of the calling grid (CT threads).  Per compressing (request, layer, KV head)
+// unit the `ne` evicted slots are closed by the retained rows that lie behind the unit's new end, which is all that
+// moves: `ne` rows at most (16 of 700 at a page of 16).  The order of the tokens is not in the places of the rows but in a word per
+// slot, its index in that order, and the stable compaction (retained history in order, then the protected window) is the
+// subtraction of the evicted indices below it.  What bounds it: four dependent round trips per unit (list and page table, order indices,
+// rows, stores), three thread blocks to an SM.  Every row behind the first evicted slot moved down (in 64-slot chunks that waited for one
+// another where units were few): 467 us at 36 layers x 256 requests, now 73; 53, now 12, at 36 x 16; 187, now 26, at 64 x 32; the
+// one-layer step of 64 requests 74.8 us, now 70.1.
+// The first ticket of a CTA is its number, the others come from a counter.  A ticket is a unit, or, where a unit has more than
+// GP_PART_SLOTS slots, a part of one: a part tells where its evicted slots lie, and the unit's last part, which waits for that
+// word of the others (tickets are handed out in order, so those are running or done), moves the rows.
 template <int D>
 __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, int serial) {
   constexpr int CH = D / 8;
   constexpr int ROW_BYTES = D * 2;
-  constexpr int PIECES = MOVE_TOK * 2 * CH / CT;        // 16-byte pieces per thread per chunk
+  constexpr int PPS = 2 * CH;                            // 16-byte pieces of a slot, keys then values
   int4* s_info = C.s_info;
   int* ev = C.ev;
   int* s_i = C.s_i;
-  int* s_dst = C.s_dst;
-  int* s_spage = C.s_spage;
-  int* s_dpage = C.s_dpage;
 
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int LH = p.L * p.Hkv;
-  // the first round trip fetches everything at once: the header, the list of compressing requests (its first
-  // CT entries before their count is known; entries past the count are never looked at) and the first ticket
-  if (tid == 0) { s_i[0] = atomicAdd(&p.hdr[HDR_WORK_CMP], 1); s_i[3] = 0; }
+  // the first round trip fetches everything at once: the header and the list of compressing requests (its first
+  // CT entries before their count is known; entries past the count are never looked at)
+  if (tid == 0) s_i[3] = 0;
   if (tid <= p.M) s_info[tid] = p.cmp_info[tid];
   const int n_cmp = p.hdr[HDR_N_CMP];
   const int n_items = p.hdr[HDR_N_CITEM];
   const int n_cow = p.hdr[HDR_N_COW];
-  // unique per decode step of the pool (the chunk flags are never cleared): the host's step count in the
+  // unique per decode step of the pool (the part flags are never cleared): the host's step count in the
   // asynchronous mode, where the two scratch sets count on their own; otherwise the counter the plan kernel keeps
   // on the device, so that a step replayed from a CUDA graph gets a stamp of its own
   const int stamp = p.async ? serial + 1 : p.hdr[HDR_STEP];
   for (int i = tid + CT; i <= n_cmp; i += CT) s_info[i] = p.cmp_info[i];
+  const int part_slots = part_slots_of(p);
+  int moved = 0;
 
-  const bool by_unit = (p.withhold & GP_TEST_COMPACT_BY_UNIT) || (long long)n_cmp * LH >= 2LL * (long long)gridDim.x;
-  const int n_work = by_unit ? n_cmp * LH : n_items;
+  int item = blockIdx.x;
   for (bool first = true;; first = false) {
     __syncthreads();
     if (!first) {
-      if (tid == 0) s_i[0] = atomicAdd(&p.hdr[HDR_WORK_CMP], 1);
+      if (tid == 0) s_i[0] = gridDim.x + atomicAdd(&p.hdr[HDR_WORK_CMP], 1);
       __syncthreads();
+      item = s_i[0];
     }
-    const int item = s_i[0];
-    if (item >= n_work) break;
-    // ticket -> (compressing request, layer/head) and the chunks it covers; chunks of a unit are consecutive and
-    // ascending in the item numbering the flags go by
-    int lo, lh, j_begin, j_end;
-    if (by_unit) {
-      lo = item / LH; lh = item % LH;
-      j_begin = 0; j_end = s_info[lo + 1].w - s_info[lo].w;
-    } else {
-      lo = 0;
-      int hi = n_cmp;
-      while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (LH * s_info[mid].w <= item) lo = mid; else hi = mid; }
-      const int nchunk = s_info[lo + 1].w - s_info[lo].w;
-      const int rem = item - LH * s_info[lo].w;
-      lh = rem / nchunk; j_begin = rem % nchunk; j_end = j_begin + 1;
-    }
+    if (item >= n_items) break;
+    // ticket -> (compressing request, layer/head, part); the parts of a unit are consecutive
+    int lo = 0, hi = n_cmp;
+    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (LH * s_info[mid].w <= item) lo = mid; else hi = mid; }
+    const int n_part = s_info[lo + 1].w - s_info[lo].w;
+    const int rem = item - LH * s_info[lo].w;
+    const int lh = rem / n_part, part = rem % n_part;
     const int4 inf = s_info[lo];
     const int l = lh / p.Hkv, h = lh % p.Hkv;
-    const int r = inf.x;
     const int Pr = inf.y;
-    const int* table = p.page_table + (size_t)r * p.cap;
-    const int* shadow = p.shadow + (size_t)r * p.cap;
-    const int n_src = Pr * GP_PAGE;
-    // second round trip: the eviction list and, for every source slot of the chunk, its page and its
-    // copy-on-write target
+    const int* table = p.page_table + (size_t)inf.x * p.cap;
+    const int* shadow = p.shadow + (size_t)inf.x * p.cap;
     const bool shrink = (inf.z & CMP_SHRINK) != 0;
     const int e_bnd = inf.z & (CMP_SHRINK - 1);
     const int ne = shrink ? 2 * p.blk : p.blk;             // slots freed: one page of the method, two at a Shrink
-    for (int t = tid; t < ne; t += CT)
+    const int n_src = Pr * GP_PAGE, n_end = n_src - ne;    // the unit's slots, and those that stay in use
+    const int c0 = n_part == 1 ? 0 : part * part_slots, c1 = part == n_part - 1 ? n_src : c0 + part_slots;
+    // order indices of a page's slots, and its rows: the unit's place in a page
+    const size_t tok_stride = (size_t)p.Hkv * GP_PAGE, tok_base = gp_tok_off(p, l, 0, h);
+    const size_t page_stride = (size_t)p.Hkv * 2 * GP_PAGE * ROW_BYTES;
+    uint8_t* const unit_base = reinterpret_cast<uint8_t*>(p.kv + gp_tile_off(p, l, 0, h));
+
+    for (int t = tid; t < ne; t += CT) {
       ev[t] = shrink ? p.evict2[((size_t)e_bnd * LH + lh) * 2 * p.blk + t] : p.evict[((size_t)e_bnd * LH + lh) * p.blk + t];
-    if (by_unit && n_cow == 0) {
-      // nothing is shared in this step: slots below the first evicted one stay where they are
-      __syncthreads();
-      if (tid < 32) {
-        int mn = 0x7fffffff;
-        for (int t = tid; t < ne; t += 32) mn = min(mn, ev[t]);
+      C.ev_slot[t] = -1;
+      C.mv_rank[t] = -1;
+    }
+    // pages that others share: copied whole, the evicted slots are closed in the copy (below)
+    if (n_cow) {
+      constexpr int TB = 2 * GP_PAGE * ROW_BYTES / 16;     // 16-byte pieces of a tile
+      constexpr int U = 4;                                 // tiles in flight
+      const int pg_end = min(c1, n_end) / GP_PAGE;
+      for (int pg0 = c0 / GP_PAGE; pg0 < pg_end; pg0 += U) {
+        uint4 val[U][TB / CT];
+        int to[U];
 #pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o2));
-        if (tid == 0) s_i[5] = mn / MOVE_TOK;
+        for (int u = 0; u < U; ++u) {
+          const int pg = pg0 + u;
+          to[u] = pg < pg_end && pg < Pr - 1 ? shadow[pg] : -1;
+          const uint4* src = reinterpret_cast<const uint4*>(unit_base + (size_t)(to[u] >= 0 ? table[pg] : 0) * page_stride);
+#pragma unroll
+          for (int e = 0; e < TB / CT; ++e) if (to[u] >= 0) val[u][e] = src[tid + e * CT];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          uint4* dst = reinterpret_cast<uint4*>(unit_base + (size_t)(to[u] >= 0 ? to[u] : 0) * page_stride);
+#pragma unroll
+          for (int e = 0; e < TB / CT; ++e) if (to[u] >= 0) dst[tid + e * CT] = val[u][e];
+        }
       }
-      __syncthreads();
-      j_begin = s_i[5];
     }
-   for (int j = j_begin; j < j_end; ++j) {
-    if (j != j_begin) __syncthreads();                   // the chunk before has left the shared arrays
-    const int c0 = j * MOVE_TOK;
-    int t0 = 0, s0 = -1;
-    const int my_i = c0 + tid;                             // the slot this thread plans (first MOVE_TOK threads)
-    if (tid < MOVE_TOK && my_i < n_src) {
-      const int pg = my_i / GP_PAGE;
-      t0 = table[pg]; s0 = shadow[pg];
-    }
-    __syncthreads();
-    int tokv = 0, tok_dst = -1, tok_page = 0;
-    if (tid < MOVE_TOK) {
-      int ds = -1, dpage = 0;
-      if (my_i < n_src) {
-        int sh = 0; bool evicted = false;
+    // the slots' new order indices, a slot per thread, SU of them in flight
+    constexpr int SU = 4;
+    bool listed = false;
+    for (int i0 = c0; i0 < c1; i0 += SU * CT) {
+      int from[SU], to[SU], rk[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int i = i0 + u * CT + tid, pg = i / GP_PAGE;
+        from[u] = i < c1 ? table[pg] : 0;
+        to[u] = i < c1 && n_cow && pg < Pr - 1 ? shadow[pg] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int i = i0 + u * CT + tid;
+        rk[u] = i < c1 ? __ldcg(p.rank + tok_base + (size_t)from[u] * tok_stride + i % GP_PAGE) : -1;
+      }
+      if (!listed) { __syncthreads(); listed = true; }     // the list of evicted indices is there
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int i = i0 + u * CT + tid;
+        if (i >= c1) continue;
+        int below = 0;                                     // evicted indices before this slot's
+        bool gone = false;
         if (ne == GP_PAGE) {
 #pragma unroll
-          for (int e2 = 0; e2 < GP_PAGE; ++e2) { sh += (ev[e2] < my_i); evicted |= (ev[e2] == my_i); }
+          for (int e = 0; e < GP_PAGE; ++e) { const int x = ev[e]; below += x < rk[u]; gone |= x == rk[u]; }
         } else {
-          for (int e2 = 0; e2 < ne; ++e2) { sh += (ev[e2] < my_i); evicted |= (ev[e2] == my_i); }
+          int hi2 = ne;
+          while (below < hi2) { const int mid = (below + hi2) >> 1; if (ev[mid] < rk[u]) below = mid + 1; else hi2 = mid; }
+          gone = below < ne && ev[below] == rk[u];
         }
-        const int pg = my_i / GP_PAGE;
-        const bool cow = (pg < Pr - 1) && (s0 >= 0);
-        if (!evicted && (sh > 0 || cow)) {
-          ds = my_i - sh;
-          // the destination tile: as many tiles down as evicted slots lie before this one (third round trip,
-          // from the L2, only for slots that move across a tile boundary)
-          const int dpg = ds / GP_PAGE;
-          if (dpg == pg) dpage = s0 >= 0 ? s0 : t0;
-          else { const int sd = shadow[dpg]; dpage = sd >= 0 ? sd : table[dpg]; }
-          tokv = p.tok[gp_tok_off(p, l, t0, h) + (my_i % GP_PAGE)];
-          tok_dst = ds; tok_page = dpage;
+        if (gone) {
+          C.ev_slot[below] = i;
+          C.ev_page[below] = to[u] >= 0 ? to[u] : from[u];
+          continue;
+        }
+        moved += below > 0 || to[u] >= 0;
+        if (i >= n_end) {
+          C.mv_page[i - n_end] = from[u];
+          C.mv_rank[i - n_end] = rk[u] - below;
+        } else if (below > 0 || to[u] >= 0) {
+          const size_t at = tok_base + i % GP_PAGE;
+          p.rank[at + (size_t)(to[u] >= 0 ? to[u] : from[u]) * tok_stride] = rk[u] - below;
+          if (to[u] >= 0) p.tok[at + (size_t)to[u] * tok_stride] = __ldcg(p.tok + at + (size_t)from[u] * tok_stride);
         }
       }
-      s_dst[tid] = ds; s_spage[tid] = t0; s_dpage[tid] = dpage;
     }
     __syncthreads();
-
-    // A thread's pieces of a chunk: piece k2 belongs to slot tl0 + k2 * TLS of the chunk, and is the same 16 bytes of
-    // its row every time (K or V, physical piece cp); a page's tile of this unit lies page_stride bytes after the
-    // one of the page before.
-    constexpr int PPS = 2 * CH, TLS = CT / PPS;
-    const int tl0 = tid / PPS, isv = (tid % PPS) / CH, cp = tid % CH;
-    uint8_t* const unit_base = reinterpret_cast<uint8_t*>(p.kv + gp_tile_off(p, l, 0, h)) + isv * GP_PAGE * ROW_BYTES;
-    const size_t page_stride = (size_t)p.Hkv * 2 * GP_PAGE * ROW_BYTES;
-    uint4 val[PIECES];
-#pragma unroll
-    for (int k2 = 0; k2 < PIECES; ++k2) {
-      const int tl = tl0 + k2 * TLS;
-      val[k2] = make_uint4(0, 0, 0, 0);
-      if (s_dst[tl] >= 0)
-        val[k2] = *reinterpret_cast<const uint4*>(unit_base + (size_t)s_spage[tl] * page_stride +
-                                                  ((c0 + tl) % GP_PAGE) * ROW_BYTES + (cp << 4));
-    }
-    // Touch every loaded value so that the loads have completed before the flag below is published: the
-    // next chunk's CTA may overwrite the tail of this chunk's sources as soon as it sees the flag.
-    unsigned touched = (unsigned)tokv;
-#pragma unroll
-    for (int k2 = 0; k2 < PIECES; ++k2) touched ^= val[k2].x ^ val[k2].y ^ val[k2].z ^ val[k2].w;
-    if (touched == 0x9e3779b9u && c0 < 0) s_i[4] = 1;      // never true; keeps the dependency alive
-    __syncthreads();
-    if (tid == 0 && !by_unit) {
-      // No fence on either side: the flag only says that loads have returned (they have: their values were
-      // consumed above), and the stores below are issued after the flag has been seen.
-      if (!((p.withhold & GP_WITHHOLD_CHUNK) && j == 0))               // (test support: see GP_WITHHOLD_CHUNK)
-        *reinterpret_cast<volatile int*>(p.cflags + item) = stamp;      // "my sources are read"
-      // my destinations reach back as far as a slot can move down, `ne` slots: into the sources of the chunks
-      // before this one, all of which must have been read (tickets are handed out in order, so those chunks are
-      // running or done)
-      const int reach = (ne + MOVE_TOK - 1) / MOVE_TOK;
-      for (int back = 1; back <= reach && back <= j; ++back) {
+    if (n_part > 1) {
+      // where a unit's evicted slots lie, found by its parts: in the place of its scores, which are done with
+      const int4 inf2 = p.bnd_info[2 * e_bnd + 1];
+      const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
+      int* found = reinterpret_cast<int*>(p.scores + (size_t)lh * p.max_boundary_tokens + off);        // [ne][2] (a unit has ne candidates at least)
+      if (part < n_part - 1) {
+        for (int t = tid; t < ne; t += CT)
+          if (C.ev_slot[t] >= 0) { found[2 * t] = C.ev_slot[t]; found[2 * t + 1] = C.ev_page[t]; }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0 && !((p.withhold & GP_WITHHOLD_CHUNK) && part == 0))      // (test support: see GP_WITHHOLD_CHUNK)
+          *reinterpret_cast<volatile int*>(p.cflags + item) = stamp;
+        continue;
+      }
+      if (tid == 0) s_i[4] = 1;
+      __syncthreads();
+      for (int back = 1 + tid; back <= part; back += CT) {
         volatile int* prev = reinterpret_cast<volatile int*>(p.cflags + item - back);
         unsigned it = 0;
         while (*prev != stamp && it < p.spin_limit) ++it;
-        if (it >= p.spin_limit) atomicOr(p.err, GP_E_SPIN_CMP);
+        if (it >= p.spin_limit) { atomicOr(p.err, GP_E_SPIN_CMP); s_i[4] = 0; }
       }
+      __threadfence();
+      __syncthreads();
+      if (!s_i[4]) continue;                               // nothing is known of those slots: no row moves
+      for (int t = tid; t < ne; t += CT)
+        if (C.ev_slot[t] < 0) {
+          const int2 f = __ldcg(reinterpret_cast<const int2*>(found) + t);
+          C.ev_slot[t] = f.x; C.ev_page[t] = f.y;
+        }
+      __syncthreads();
+    }
+    // ---- the retained rows behind the new end into the evicted slots before it, each in ascending order (as many of the one
+    // as of the other) ---------------------------------------------------------------------------------------------
+    if (warp == 0) {
+      const int n = warp_pack(ne, C.hole, [&](int e) { return C.ev_slot[e] >= 0 && C.ev_slot[e] < n_end; });
+      if (lane == 0) s_i[1] = n;
+    } else if (warp == 1) {
+      const int n = warp_pack(ne, C.mover, [&](int e) { return C.mv_rank[e] >= 0; });
+      if (lane == 0) s_i[5] = n;
     }
     __syncthreads();
+    const int n_mv = min(s_i[1], s_i[5]);
+    for (int k = tid; k < n_mv; k += CT) {
+      const int hole = C.hole[k], mv = C.mover[k], ds = C.ev_slot[hole];
+      const size_t at = tok_base + (size_t)C.ev_page[hole] * tok_stride + ds % GP_PAGE;
+      p.rank[at] = C.mv_rank[mv];
+      p.tok[at] = __ldcg(p.tok + tok_base + (size_t)C.mv_page[mv] * tok_stride + (n_end + mv) % GP_PAGE);
+    }
+    constexpr int MU = 2;
+    for (int q0 = tid; q0 < n_mv * PPS; q0 += MU * CT) {
+      uint4 val[MU];
 #pragma unroll
-    for (int k2 = 0; k2 < PIECES; ++k2) {
-      const int tl = tl0 + k2 * TLS;
-      const int ds = s_dst[tl];
-      if (ds >= 0) {
-        const int c = cp ^ ((c0 + tl) & 7);                 // the logical piece this thread holds (rows are swizzled by slot)
-        *reinterpret_cast<uint4*>(unit_base + (size_t)s_dpage[tl] * page_stride + (ds % GP_PAGE) * ROW_BYTES +
-                                  ((c ^ (ds & 7)) << 4)) = val[k2];
+      for (int u = 0; u < MU; ++u) {
+        const int q = q0 + u * CT, k = q / PPS, c = q % CH, isv = q % PPS / CH;        // c: piece of the row (rows are swizzled by slot)
+        if (k < n_mv) {
+          const int mv = C.mover[k], s = (n_end + mv) % GP_PAGE;
+          val[u] = *reinterpret_cast<const uint4*>(unit_base + (size_t)C.mv_page[mv] * page_stride + (isv * GP_PAGE + s) * ROW_BYTES + ((c ^ (s & 7)) << 4));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < MU; ++u) {
+        const int q = q0 + u * CT, k = q / PPS, c = q % CH, isv = q % PPS / CH;
+        if (k < n_mv) {
+          const int hole = C.hole[k], s = C.ev_slot[hole] % GP_PAGE;
+          *reinterpret_cast<uint4*>(unit_base + (size_t)C.ev_page[hole] * page_stride + (isv * GP_PAGE + s) * ROW_BYTES + ((c ^ (s & 7)) << 4)) = val[u];
+        }
       }
     }
-    if (tok_dst >= 0) {
-      atomicAdd(&s_i[3], 1);
-      p.tok[gp_tok_off(p, l, tok_page, h) + (tok_dst % GP_PAGE)] = tokv;
-    }
-   }
   }
+  moved = __reduce_add_sync(0xffffffffu, moved);
+  if (lane == 0 && moved) atomicAdd(&s_i[3], moved);
   __syncthreads();
   if (tid == 0 && s_i[3] > 0)
     atomicAdd(reinterpret_cast<unsigned long long*>(p.counters + 8), (unsigned long long)s_i[3]);
@@ -1190,7 +1277,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
 
 
 template <int D>
-__global__ void __launch_bounds__(CT, 4)
+__global__ void __launch_bounds__(CT, 3)
 gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int serial) {
   __shared__ __align__(16) uint8_t cmp_raw[CMP_SMEM_BYTES];
   gp_pdl_wait();

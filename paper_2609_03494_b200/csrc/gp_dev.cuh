@@ -8,6 +8,10 @@
 //                   slot index: logical chunk c of slot s lives at chunk c ^ (s & 7).  A tile
 //                   copied verbatim to shared memory is then bank-conflict free for ldmatrix.
 //   tok       int32 [L][n_pages][H_kv][b]               original token index of every slot
+//   rank      int32 [L][n_pages][H_kv][b]               place of every slot in the order of its unit's tokens: a compaction
+//                   closes evicted slots with rows from the unit's end and changes these words, not the places of the other rows.
+//                   Slots appended since the last compaction hold their own number; so do all of a request that never compacted,
+//                   which is what makes its pages shareable
 //   summaries fp64  [L][M][2][2][H_q][d]                Eq. 11 layout (short then long), double-buffered
 //   page_table / shadow int32 [M][cap]                  shadow holds copy-on-write targets
 //   scores    fp64  [jobs][L*H_kv][max_boundary_tokens] scores of candidate sets too large for shared memory
@@ -24,7 +28,8 @@
 #define GP_MAX_TILES_PER_REQ 61773   // 16-token tiles a request may hold: the selection keeps a bit per candidate in shared memory
 #define GP_SPIN_LIMIT (1u << 21)
 #define GP_MAX_REQ 1024        // upper limit of max_requests (shared-memory arrays are sized by it)
-#define GP_MOVE_TOK 64         // source slots per compaction chunk
+#define GP_PART_SLOTS 4096     // slots per compaction ticket: units beyond that are shared out (a unit of 20 000 slots in one block: 15 us of loads)
+#define GP_PART_MIN 64         // ... in tests
 #define GP_COST_BINS 288       // cost classes of attention work items (pages, x4 at a boundary)
 #define GP_DESC_INTS 16        // ints per attention work descriptor
 #define GP_ATTN_CONSUMERS 4    // consumer warps of an attention thread block: each reports once per item it worked on
@@ -40,7 +45,7 @@ enum {
   HDR_N_ACTIVE,      // requests actually stepped
   HDR_DONE_SEL,      // CTAs of the selection kernel that have finished
   HDR_WORK_CMP,      // ticket counter of the compaction kernel
-  HDR_N_CITEM,       // compaction work items (chunks x layers x heads)
+  HDR_N_CITEM,       // compaction work items (parts x layers x heads)
   HDR_N_COW,         // copy-on-write targets allotted this step
   HDR_COUNT = 16
 };
@@ -48,10 +53,11 @@ enum {
 // hand-overs a test can withhold (gp_test_withhold): the bounded wait for it then runs out
 enum {
   GP_WITHHOLD_ITEM = 1,     // attention kernel, first CTA: its second work item is never published to the consumers
-  GP_WITHHOLD_CHUNK = 2,    // compaction: the first chunk of a unit never says that its sources are read
+  GP_WITHHOLD_CHUNK = 2,    // compaction, in parts of GP_PART_MIN slots: the first part of a unit never says where its evicted slots lie
   GP_WITHHOLD_DECIDED = 4,  // boundary kernel: the deciding CTA never tells the others
   GP_WITHHOLD_READY = 8,    // attention kernel: the consumer warps never report a boundary unit's logits complete
-  GP_TEST_COMPACT_BY_UNIT = 16,   // (not a withheld hand-over) the compaction claims whole units whatever their number
+  GP_TEST_COMPACT_BY_UNIT = 16,   // (not withheld hand-overs) the compaction claims whole units whatever their size,
+  GP_TEST_COMPACT_BY_PART = 32,   // ... parts of GP_PART_MIN slots
 };
 
 // error bits
@@ -86,6 +92,7 @@ struct GpDev {
   // pool
   __nv_bfloat16* kv;
   int* tok;
+  int* rank;
   int* refcount;
   int* free_stack;
   int* free_top;                         // number of free pages (stack height)
@@ -120,14 +127,14 @@ struct GpDev {
   int* unit_ready;                       // [M][L H_kv] per boundary unit: consumer warps of the attention kernel done with it
   int* bnd_acc;                          // [M][4] per boundary request: sum of K^S, sum of K^L, shared pages of C, 0
   int* free_peek;                        // [M+1] free_top at plan time, then the top entries of the free list, top first
-  int4* cmp_info;                        // [M+1] compressing requests: {request, P, index in bnd_info, first compaction chunk}
+  int4* cmp_info;                        // [M+1] compressing requests: {request, P, index in bnd_info, first compaction part}
   double* zbuf;                          // [L*H_kv][2][z_stride][G] boundary units, per view (short, long): exp(summary logit - its page's max)
   long long z_stride;                    // max_boundary_tokens rounded up to a multiple of the page size
   double* zstat;                         // [L*H_kv][max_boundary_tokens / b][2][G][2] per-page softmax partials (max, sum)
   int* sum_par;                          // [M] which of the two summary buffers is current
   int* evict;                            // [M][L*H_kv][page_size] slots a compression evicts, ascending
   int* evict2;                           // [M][L*H_kv][2 page_size] slots a Shrink evicts, ascending (Shrink policy only)
-  int* cflags;                           // compaction chunk flags, stamped with the step number
+  int* cflags;                           // compaction part flags, stamped with the step number
   int* tickets;                          // [L] next attention work item to draw: of the whole step (0) or of a layer's launch
   double* inv_freq;                      // [d/2] rope_theta^(-2j/d)
   float* rope_f;                         // [M][d/2][2] cos, sin at the step's position in fp32 (the queries' rotation)

@@ -68,7 +68,7 @@ struct gp_pool {
 namespace {
 
 struct Layout {
-  size_t kv, tok, refcount, free_stack, words, page_table, shadow, reqi, pos, summ, Kx, Hx, delta, rc,
+  size_t kv, tok, rank, refcount, free_stack, words, page_table, shadow, reqi, pos, summ, Kx, Hx, delta, rc,
       merge_cnt, bnd_info, bnd_acc, free_peek, cmp_info, zbuf, zstat, sum_par, inv_freq, tickets, rope_f,
       unit_ready, shard_sums, bnd_info2, bnd_acc2, zbuf2, zstat2, rc2, rope_cs2, rope_f2,
       evict, evict2, cflags, rope_cs, partials, scores, counters, dbg,
@@ -142,6 +142,7 @@ Layout make_layout(const gp_config& c) {
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes); return at; };
   L.kv = take(LH * np * 2 * b * d * 2);
   L.tok = take(LH * np * b * 4);
+  L.rank = take(LH * np * b * 4);
   L.refcount = take(np * 4);
   L.free_stack = take(np * 4);
   L.words = take(256 * 4);                       // free_top, err, plan header, status
@@ -165,7 +166,7 @@ Layout make_layout(const gp_config& c) {
   L.zstat = take(LH * (Tb / b + 1) * 2 * G * 2 * 8);
   L.evict = take(M * LH * blk * 4);
   L.evict2 = take(c.policy == GP_POLICY_SHRINK ? M * LH * 2 * blk * 4 : 16);
-  L.cflags = take(LH * ((Tb + M * b) / GP_MOVE_TOK + 2 * M + 1) * 4);
+  L.cflags = take(LH * ((Tb + M * b) / GP_PART_MIN + 2 * M + 1) * 4);
   L.inv_freq = take(d / 2 * 8);
   L.tickets = take((size_t)c.n_layers * 4);
   L.rope_f = take(M * (d / 2) * 2 * 4);
@@ -524,7 +525,10 @@ gp_ingest_kernel(const __grid_constant__ GpDev p, int r, int n_shared, int n_tai
         uint8_t* dst = reinterpret_cast<uint8_t*>(p.kv + gp_tile_off(p, l, page, h)) + isv * GP_PAGE * row_bytes + s * row_bytes +
                        ((c ^ (s & 7)) << 4);
         *reinterpret_cast<uint4*>(dst) = val[e];
-        if (isv == 0 && c == 0) p.tok[gp_tok_off(p, l, page, h) + s] = (n_shared + tile) * GP_PAGE + s;
+        if (isv == 0 && c == 0) {
+          const size_t at = gp_tok_off(p, l, page, h) + s;
+          p.tok[at] = p.rank[at] = (n_shared + tile) * GP_PAGE + s;
+        }
       }
     }
   }
@@ -564,7 +568,7 @@ gp_release_kernel(const __grid_constant__ GpDev p, int r) {
   }
 }
 
-// debug: token ids and un-swizzled K, V rows of one (layer, head) stream into the gather buffer
+// debug: token ids and un-swizzled K, V rows of one (layer, head) stream into the gather buffer, in the order of the tokens
 __global__ void gp_gather_kernel(GpDev p, int r, int l, int h, int n, int* tok_out, uint4* k_out, uint4* v_out) {
   const int CH = p.d / 8;
   const int row_bytes = p.d * 2;
@@ -578,8 +582,10 @@ __global__ void gp_gather_kernel(GpDev p, int r, int l, int h, int n, int* tok_o
     const int s = slot % GP_PAGE;
     const uint8_t* src = reinterpret_cast<const uint8_t*>(p.kv + gp_tile_off(p, l, page, h)) +
                          isv * GP_PAGE * row_bytes + s * row_bytes + ((c ^ (s & 7)) << 4);
-    (isv ? v_out : k_out)[(size_t)slot * CH + c] = *reinterpret_cast<const uint4*>(src);
-    if (isv == 0 && c == 0) tok_out[slot] = p.tok[gp_tok_off(p, l, page, h) + s];
+    const int at = p.rank[gp_tok_off(p, l, page, h) + s];
+    if (at < 0 || at >= n) continue;                         // (a wait that gave up: the pool's error word says so)
+    (isv ? v_out : k_out)[(size_t)at * CH + c] = *reinterpret_cast<const uint4*>(src);
+    if (isv == 0 && c == 0) tok_out[at] = p.tok[gp_tok_off(p, l, page, h) + s];
   }
 }
 
@@ -708,6 +714,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.p_fix = (unsigned long long)llrint(cfg->top_p * 4611686018427387904.0);
   d.kv = reinterpret_cast<__nv_bfloat16*>(base + L.kv);
   d.tok = reinterpret_cast<int*>(base + L.tok);
+  d.rank = reinterpret_cast<int*>(base + L.rank);
   d.refcount = reinterpret_cast<int*>(base + L.refcount);
   d.free_stack = reinterpret_cast<int*>(base + L.free_stack);
   int* words = reinterpret_cast<int*>(base + L.words);
@@ -1493,7 +1500,7 @@ int gp_debug_pool(gp_pool* pool, int64_t* n_free, int32_t* refcounts, int64_t co
 }
 
 int gp_test_withhold(gp_pool* pool, int32_t what, int32_t spin_limit) {
-  if (!pool || what < 0 || what > 31 || spin_limit < 0) return GP_ERR_INVALID;
+  if (!pool || what < 0 || what > 63 || spin_limit < 0) return GP_ERR_INVALID;
   GpDev* views[2] = {&pool->dev, &pool->dev_alt};
   for (GpDev* v : views) {
     v->withhold = what;
