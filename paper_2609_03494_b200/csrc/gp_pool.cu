@@ -13,6 +13,7 @@
 
 #define GP_PLAN_THREADS 1024       // threads of the plan kernel for batches of up to GP_MAX_REQ requests (a thread each) ...
 #define GP_PLAN_SMALL 256          // ... and for batches of up to this many: its time is block barriers, which 8 warps pass faster than 32
+#define PLAN_STATES 512            // requests of a pool whose counters the plan kernel reads ahead (8 KB: it starts beside the boundary kernel)
 #define GP_NEVER (-(1 << 30))      // bstep of a request that has not reached a boundary
 
 struct gp_pool {
@@ -219,44 +220,40 @@ __global__ void gp_init_kernel(GpDev p) {
   if (i0 == 0) *p.free_top = (int)p.n_pages;
 }
 
-// exclusive scan over the CTA (up to 32 warps) of an int and a long long; also returns the totals
-__device__ __forceinline__ void plan_scan(int v, long long w, int& ev, long long& ew, int& tv, long long& tw,
-                                          int* sv, long long* sw) {
+// exclusive scan over the CTA (up to 32 warps) of two ints and a long long, with the totals: one barrier (every warp scans the
+// warps' sums for itself).  The arrays are free again after the caller's next barrier.
+struct PlanScan { int a[32], b[32]; long long w[32]; };
+__device__ __forceinline__ void plan_scan(PlanScan& S, int a, int b, long long w, int& ea, int& eb, long long& ew, int& ta, int& tb,
+                                          long long& tw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int iv = v; long long iw = w;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int a = __shfl_up_sync(0xffffffffu, iv, off);
-    const long long b2 = __shfl_up_sync(0xffffffffu, iw, off);
-    if (lane >= off) { iv += a; iw += b2; }
-  }
-  if (lane == 31) { sv[warp] = iv; sw[warp] = iw; }
-  __syncthreads();
-  if (warp == 0) {                       // scan of the 32 warp totals: exclusive prefix in [0..31], total in [32]
-    const bool has = lane < (int)(blockDim.x >> 5);
-    int xv = has ? sv[lane] : 0; long long xw = has ? sw[lane] : 0;
-    const int ov = xv; const long long ow = xw;
+  auto scan = [&](int& x, int& y, long long& z) {          // inclusive, over the warp
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const int a = __shfl_up_sync(0xffffffffu, xv, off);
-      const long long b2 = __shfl_up_sync(0xffffffffu, xw, off);
-      if (lane >= off) { xv += a; xw += b2; }
+      const int x2 = __shfl_up_sync(0xffffffffu, x, off), y2 = __shfl_up_sync(0xffffffffu, y, off);
+      const long long z2 = __shfl_up_sync(0xffffffffu, z, off);
+      if (lane >= off) { x += x2; y += y2; z += z2; }
     }
-    sv[lane] = xv - ov; sw[lane] = xw - ow;
-    if (lane == 31) { sv[32] = xv; sw[32] = xw; }
-  }
+  };
+  int ia = a, ib = b; long long iw = w;
+  scan(ia, ib, iw);
+  if (lane == 31) { S.a[warp] = ia; S.b[warp] = ib; S.w[warp] = iw; }
   __syncthreads();
-  ev = sv[warp] + iv - v;
-  ew = sw[warp] + iw - w;
-  tv = sv[32];
-  tw = sw[32];
-  __syncthreads();
+  const bool has = lane < (int)(blockDim.x >> 5);
+  int xa = has ? S.a[lane] : 0, xb = has ? S.b[lane] : 0; long long xw = has ? S.w[lane] : 0;
+  scan(xa, xb, xw);
+  ta = __shfl_sync(0xffffffffu, xa, 31); tb = __shfl_sync(0xffffffffu, xb, 31); tw = __shfl_sync(0xffffffffu, xw, 31);
+  const int pa = __shfl_sync(0xffffffffu, xa, (warp + 31) & 31), pb = __shfl_sync(0xffffffffu, xb, (warp + 31) & 31);
+  const long long pw = __shfl_sync(0xffffffffu, xw, (warp + 31) & 31);
+  ea = ia - a + (warp ? pa : 0); eb = ib - b + (warp ? pb : 0); ew = iw - w + (warp ? pw : 0);
 }
 
 // Step plan: validates the batch, cuts every stepped request into chunks and writes one work descriptor
 // per chunk for the attention kernel, lists the requests that reach their capacity boundary with this
 // step's append (trailing check: n + 1 == P b) and hands each a slice of the logit scratch.  With rotary embeddings the other
 // CTAs write the cosines and sines of the requests' positions.
+// What bounds it: two dependent round trips (request ids; descriptors out) and six block barriers between them.  (With the counters read
+// behind the ids, three scans and a scan of the cost bins of 45 dependent steps: 12.3 us between events for 64 requests, now 10.2;
+// 16 steps of four requests 317 us, now 280.)
 __global__ void __launch_bounds__(GP_PLAN_THREADS)
 gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions, int early,
                int cp_norm, int cp_bnd, int launch_units, int launch_grid, int serial) {
@@ -267,22 +264,36 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // the attention launch has work for large items; launch_units: (layer, head) units per request in one
   // attention launch; launch_grid: its CTAs
   // early: the caller's request ids may be read before the wait for the preceding kernel (see below)
-  __shared__ int sv[33];
-  __shared__ long long sw[33];
-  __shared__ __align__(16) int s_first[GP_MAX_REQ];      // lowest batch index naming a request
-  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS];
+  __shared__ PlanScan s_scan[2];
+  __shared__ __align__(16) int s_first[GP_MAX_REQ];      // lowest batch index naming a request; then cost classes and items
+  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS], s_pages;
+  // .x slots in use, .y pages, .z position, .w: 1 live, 2 has decoded, 4 summary buffer in use, 8 sits this step out
+  __shared__ int4 s_state[PLAN_STATES];
   const int i = threadIdx.x;
   const bool in = i < n_req;
   // What runs before the wait for the kernel before this one.  In a whole-step launch that kernel is the
-  // compaction of the step before (or something the caller put in between, which then has completed): this
+  // compaction of the step before (or something the caller put in between, which could not start before that): this
   // grid became schedulable only after that step's decisions had completed, and compaction touches neither the
-  // requests' counters nor anything the plan writes except the step stamp.  So CTA 0 plans the whole step first and waits
-  // only before it looks at the free list (which compaction's last CTA may still change) and stamps the step.  CTA 0 does
+  // requests' counters nor anything the plan writes except the step stamp.  So the counters of the pool's requests are read before
+  // the wait.  (In the asynchronous mode the chain kernel before this one writes counters until it ends.)
+  // The caller's request ids are read before it only where the caller says that they were complete before the
+  // preceding kernel could signal (`early`); CTA 0 then plans the whole step first and waits only before it looks at the free list
+  // (which compaction's last CTA may still change) and stamps the step.  CTA 0 does
   // wait, so the grid as a whole still ends after everything before it.  The next kernel may be scheduled
   // as soon as every CTA of this grid has started; it waits for this grid's end at its own top.
-  // All of this reads the caller's request ids before the wait, which is only right if they were
-  // complete before the preceding kernel could signal: the caller says so (`early`); otherwise every CTA
-  // waits first (the later wait of CTA 0 is then a no-op).
+  auto load_state = [&](int r) {                         // from the L2: before the wait
+    const int live = __ldcg(p.live + r), started = __ldcg(p.started + r), par = __ldcg(p.sum_par + r);
+    const int held = p.async && __ldcg(p.bstep + r) == serial - 1;
+    return make_int4(__ldcg(p.n + r), __ldcg(p.P + r), (int)__ldcg(p.pos + r), (live ? 1 : 0) | (started ? 2 : 0) | (par ? 4 : 0) | (held ? 8 : 0));
+  };
+  const bool preloaded = !p.async && p.M <= PLAN_STATES;
+  if (blockIdx.x == 0) {
+    if (preloaded) for (int t = i; t < p.M; t += blockDim.x) s_state[t] = load_state(t);
+    for (int t = i; t < p.M; t += blockDim.x) s_first[t] = 0x7fffffff;
+    for (int t = i; t < GP_COST_BINS; t += blockDim.x) s_bin[t] = 0;
+    if (i == 0) s_pages = 0;
+    __syncthreads();
+  }
   if (!early) gp_pdl_wait();
   gp_pdl_launch_dependents();
   if (blockIdx.x > 0) {                       // cos / sin of the step's position (from the L2: these CTAs may run before the wait)
@@ -299,35 +310,32 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     }
     return;
   }
-  for (int t = i; t < p.M; t += blockDim.x) s_first[t] = 0x7fffffff;
-  for (int t = i; t < GP_COST_BINS; t += blockDim.x) s_bin[t] = 0;
+  int r = -1;
+  if (in) r = req_ids[i];
   // The number this step goes by: the host's count of decode steps in the asynchronous mode (the two scratch sets
   // count on their own); otherwise the pool's own counter on the device, so that a step replayed from a CUDA graph
   // still gets a number of its own.
-  const int step_no = p.async ? serial : __ldcg(p.hdr + HDR_STEP);
+  const int hdr_step = __ldcg(p.hdr + HDR_STEP);           // (this kernel alone writes it)
+  const int step_no = p.async ? serial : hdr_step;
+  const int free_top0 = early ? 0 : __ldcg(p.free_top);
+  const bool inrange = in && r >= 0 && r < p.M;
+  if (inrange) atomicMin(&s_first[r], i);
+  int4 st = make_int4(0, 0, 0, 0);
+  if (inrange) st = preloaded ? s_state[r] : load_state(r);
+  // the attention kernel draws its items from these (the one of the step before, the last to draw, has ended: that step's
+  // decisions waited for it, or, where it was abandoned before it had any, this launch did)
+  for (int idx = threadIdx.x; idx < p.L; idx += blockDim.x) p.tickets[idx] = 0;
   __syncthreads();
-  int r = -1;
-  if (in) {
-    r = req_ids[i];
-    if (r >= 0 && r < p.M) atomicMin(&s_first[r], i);
-  }
-  __syncthreads();
-  int chunks = 0, pages = 0, n_old = 0, act = GP_ACT_NONE, Pr = 0, started = 0, par = 0;
-  long long nc = 0, pos = 0;
+  int chunks = 0, pages = 0, act = GP_ACT_NONE;
+  const int n_old = st.x, Pr = st.y, pos = st.z;
+  long long nc = 0;
   int isb = 0;
   int cp = cp_norm;                       // pages per work item of this request
-  int live = 0, held = 0;
-  if (in && r >= 0 && r < p.M) {          // independent loads, issued together (from the L2: before the wait)
-    live = __ldcg(p.live + r); n_old = __ldcg(p.n + r); Pr = __ldcg(p.P + r); pos = __ldcg(p.pos + r);
-    started = __ldcg(p.started + r); par = __ldcg(p.sum_par + r);
-    if (p.async) held = __ldcg(p.bstep + r) == serial - 1;
-  }
   if (in) {
-    const bool inrange = r >= 0 && r < p.M;
-    const bool valid = inrange && live && s_first[r] == i;
+    const bool valid = inrange && (st.w & 1) && s_first[r] == i;
     if (!valid) {
       act = GP_ACT_INVALID;
-    } else if (held) {
+    } else if (st.w & 8) {
       act = GP_ACT_HELD;                  // its boundary chain may still be running: nothing of it is looked at
     } else if (n_old >= Pr * GP_PAGE) {
       act = GP_ACT_STALLED;
@@ -341,9 +349,10 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     // request / CTAs >= an item), fine ones otherwise: small batches, short sequences, layer-by-layer launches.
     // Measured on one layer of the 8B shape: 8 to 48 requests of 30 to 50 pages are 2 to 8 us per step faster
     // with fine items, 64 requests of 44 pages and more 3 us faster with large ones.
-    int e0, tot_pages; long long d0, d1;
-    plan_scan(pages, 0, e0, d0, tot_pages, d1, sv, sw);
-    if ((long long)tot_pages * launch_units < (long long)cp_norm * launch_grid) { cp_norm = GP_FINE_CHUNK; cp_bnd = GP_FINE_BCHUNK; }
+    const int warp_pages = __reduce_add_sync(0xffffffffu, pages);
+    if ((i & 31) == 0 && warp_pages) atomicAdd(&s_pages, warp_pages);
+    __syncthreads();
+    if ((long long)s_pages * launch_units < (long long)cp_norm * launch_grid) { cp_norm = GP_FINE_CHUNK; cp_bnd = GP_FINE_BCHUNK; }
   }
   if (pages > 0) {
     // a page of a boundary request also pays for the fp64 summary logits: its items are half as large
@@ -352,18 +361,20 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     chunks = (pages + cp - 1) / cp;
     cp = (pages + chunks - 1) / chunks;              // equal sizes: chunks of cp pages, the last one shorter
   }
-  int rc_off, n_rc; long long tok_off, tok_tot;
-  plan_scan(chunks, nc, rc_off, tok_off, n_rc, tok_tot, sv, sw);
+  // (boundary requests and stepped requests in one word: at most GP_MAX_REQ of each)
+  int rc_off, n_rc, both, both_tot; long long tok_off, tok_tot;
+  plan_scan(s_scan[0], chunks, isb << 16 | (chunks > 0), nc, rc_off, both, tok_off, n_rc, both_tot, tok_tot);
   // A batch whose summed lengths exceed max_batch_tokens (the caller's bound; with shared prompt pages the sum
   // can exceed what the pool holds) does not fit the scratch: a request whose boundary logits or whose work
   // items do not fit is not stepped (its state stays as it is, it can be stepped again in a later batch).  The
   // offsets are then taken again over what is left, so that the item list has no holes.
-  const bool dropped = chunks > 0 && ((isb && tok_off + nc > p.max_boundary_tokens) || rc_off + chunks > p.max_rc);
-  if (dropped) { chunks = 0; isb = 0; nc = 0; act = GP_ACT_SCRATCH; }
-  if (__syncthreads_or(dropped)) plan_scan(chunks, nc, rc_off, tok_off, n_rc, tok_tot, sv, sw);
-  int bnd_idx, n_bnd, n_active; long long d0, d1;
-  plan_scan(isb, chunks > 0, bnd_idx, d0, n_bnd, d1, sv, sw);
-  n_active = (int)d1;
+  if (tok_tot > p.max_boundary_tokens || n_rc > p.max_rc) {         // (the same for every thread)
+    if (chunks > 0 && ((isb && tok_off + nc > p.max_boundary_tokens) || rc_off + chunks > p.max_rc)) {
+      chunks = 0; isb = 0; nc = 0; act = GP_ACT_SCRATCH;
+    }
+    plan_scan(s_scan[1], chunks, isb << 16 | (chunks > 0), nc, rc_off, both, tok_off, n_rc, both_tot, tok_tot);
+  }
+  const int bnd_idx = both >> 16, n_bnd = both_tot >> 16, n_active = both_tot & 0xffff;
   // Work items are listed by descending cost (pages, times four for boundary requests, which also pay for the
   // fp64 logits): the attention kernel deals them out in that order, largest first.  Counting sort.
   const int key = chunks > 0 ? min(GP_COST_BINS - 1, cp * (isb ? 4 : 1)) : 0;
@@ -371,9 +382,24 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // which atomics land), so that the same batch gives the same numbered list every time.  An item's number says which of a
   // block's warps takes which of its tiles, and split outputs are merged in chunk order: with the numbers fixed, the attention outputs
   // repeat bit for bit whichever thread block draws an item.
-  s_first[i] = chunks > 0 ? (key << 16) | chunks : 0;        // s_first has served its purpose: cost class and items
+  s_first[i] = chunks > 0 ? (key << 16) | chunks : 0;        // s_first has served its purpose
   if (chunks > 0) atomicAdd(&s_bin[key], chunks);
   __syncthreads();
+  if (threadIdx.x < 32) {                             // descending exclusive scan over the cost bins, nine to a lane
+    constexpr int PER = GP_COST_BINS / 32;
+    int v[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) { v[j] = s_bin[GP_COST_BINS - 1 - ((int)threadIdx.x * PER + j)]; sum += v[j]; }
+    int inc = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int a = __shfl_up_sync(0xffffffffu, inc, off);
+      if ((int)threadIdx.x >= off) inc += a;
+    }
+    int at = inc - sum;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) { s_binbase[GP_COST_BINS - 1 - ((int)threadIdx.x * PER + j)] = at; at += v[j]; }
+  }
   int within = 0;
   if (chunks > 0) {
     const int4* e4 = reinterpret_cast<const int4*>(s_first);
@@ -386,50 +412,30 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     for (; j < i; ++j) { const int e = s_first[j]; within += (e >> 16) == key ? (e & 0xffff) : 0; }
   }
   __syncthreads();
-  if (threadIdx.x < 32) {                             // descending exclusive scan over the cost bins
-    int carry = 0;
-    for (int b0 = GP_COST_BINS - 32; b0 >= 0; b0 -= 32) {
-      const int b = b0 + 31 - (int)threadIdx.x;       // lane 0 takes the costliest bin of the block of 32
-      const int v = s_bin[b];
-      int inc = v;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, inc, off);
-        if ((int)threadIdx.x >= off) inc += a;
-      }
-      s_binbase[b] = carry + inc - v;
-      carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-  }
-  __syncthreads();
   const int sorted0 = s_binbase[key] + within;
   if (in) {
     if (isb) { p.bstep[r] = step_no; if (p.async) act = GP_ACT_PENDING; }
     actions[i] = act;
     if (isb) {
-      p.bnd_info[2 * bnd_idx] = make_int4(i, r, Pr, (int)pos);     // pos: position of this step's token
+      p.bnd_info[2 * bnd_idx] = make_int4(i, r, Pr, pos);     // pos: position of this step's token
       // .z: reports the attention kernel makes per (layer, head) unit of this request (one per consumer warp and item)
       p.bnd_info[2 * bnd_idx + 1] = make_int4((int)(unsigned)(tok_off & 0xffffffffLL), (int)(tok_off >> 32), GP_ATTN_CONSUMERS * chunks, 0);
       reinterpret_cast<int4*>(p.bnd_acc)[bnd_idx] = make_int4(0, 0, 0, 0);
     }
     // descriptors of this request's chunks: four 16-byte stores each
-    const int flags = isb | (started ? 2 : 0);
+    const int flags = isb | (st.w & 2);
     for (int c = 0; c < chunks; ++c) {
       const int pg0 = c * cp;
       int4* d = reinterpret_cast<int4*>(p.rcx + (size_t)(sorted0 + c) * GP_DESC_INTS);
       d[0] = make_int4(i, r, pg0, min(cp, pages - pg0));
-      d[1] = make_int4(c, chunks, n_old, (int)pos);
+      d[1] = make_int4(c, chunks, n_old, pos);
       d[2] = make_int4(flags, Pr, (int)(unsigned)(tok_off & 0xffffffffLL), (int)(tok_off >> 32));
-      d[3] = make_int4(par, rc_off + c, 0, isb ? bnd_idx : 0);
+      d[3] = make_int4((st.w >> 2) & 1, rc_off + c, 0, isb ? bnd_idx : 0);
     }
   }
   // the attention kernel counts, per unit of a boundary request, the work items its consumer warps have finished
   if (p.report_units)
     for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += blockDim.x) p.unit_ready[idx] = 0;
-  // (the attention kernel of the step before, the last to draw from these, has ended: that step's decisions waited for it, or,
-  // where it was abandoned before it had any, this launch did)
-  for (int idx = threadIdx.x; idx < p.L; idx += blockDim.x) p.tickets[idx] = 0;
-  __syncthreads();
   if (threadIdx.x == 0) {
     p.hdr[HDR_N_RC] = n_rc;
     p.hdr[HDR_N_BND] = n_bnd;
@@ -441,11 +447,11 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     // the top of the free list, one page per boundary request: what this step's grants can take.  (In the
     // asynchronous mode the free list belongs to the boundary chains, which run one after the other: the
     // decision step reads it itself.)
-    const int free_top0 = *p.free_top;
-    if (in && isb && bnd_idx < free_top0) p.free_peek[1 + bnd_idx] = p.free_stack[free_top0 - 1 - bnd_idx];
-    if (threadIdx.x == 0) p.free_peek[0] = free_top0;
+    const int top = early ? __ldcg(p.free_top) : free_top0;
+    if (in && isb && bnd_idx < top) p.free_peek[1 + bnd_idx] = __ldcg(p.free_stack + top - 1 - bnd_idx);
+    if (threadIdx.x == 0) p.free_peek[0] = top;
   }
-  if (threadIdx.x == 0) p.hdr[HDR_STEP] += 1;
+  if (threadIdx.x == 0) p.hdr[HDR_STEP] = hdr_step + 1;
 }
 
 constexpr int ADMIT_THREADS = 256;
