@@ -80,7 +80,7 @@ __host__ __device__ constexpr Lay make_lay(int G) {
   L.off_comb = L.off_qt + nrows * (D + QT_PAD) * 8;
   L.comb_warp = (16 + G * D) * 4;
   L.off_bars = L.off_comb + L.ncomb * NCW * L.comb_warp;
-  L.off_misc = L.off_bars + (3 * NI + 2 + 4) * 8;
+  L.off_misc = L.off_bars + (4 * NI + 2 + 4) * 8;
   L.total = L.off_misc + 128 + SMEM_ALIGN;   // abort flag and code; room for the rounding
   return L;
 }
@@ -179,11 +179,12 @@ __device__ __forceinline__ void merge_unit(float* first, size_t stride, int n, i
 // The summaries of one unit, the heads g = w, w + NSUM, ... by the calling warp (w): Eq. 6 on the un-rotated query from the
 // request's current buffer to the other one (`owner`), and, with `qt`, the calibrated (Eq. 12) and rotated summaries q~ into
 // the q~ buffer (times QT_SCALE), all in fp64.  What bounds it is the round trip for the old rows: two heads' (both views)
-// are in flight together, and the first ones' are asked for before anything else.  With NORM the warp first normalises its
+// are in flight together, and the first ones' are asked for before anything else, the wait for the query rows (`rows_there`; false: it gave
+// up) included.  With NORM the warp first normalises its
 // heads' query rows in the slot and reports them on `norm_bar`: the consumers wait for that.
-template <int D, bool ROPE, bool NORM>
-__device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, uint8_t* qrows, uint64_t* norm_bar, int w, int G, int l,
-                                             int h, int r, int bi, int par, bool started, bool owner, double* qt) {
+template <int D, bool ROPE, bool NORM, typename Rows>
+__device__ __forceinline__ bool summary_rows(const GpDev& p, const GpNorm& nm, uint8_t* qrows, Rows rows_there, uint64_t* norm_bar, int w, int G,
+                                             int l, int h, int r, int bi, int par, bool started, bool owner, double* qt) {
   constexpr int PER = D / 32;
   const int lane = threadIdx.x & 31;
   __nv_bfloat16* q0 = reinterpret_cast<__nv_bfloat16*>(qrows);
@@ -200,6 +201,7 @@ __device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, u
         }
   };
   if (owner || qt) load_old(w);
+  if (!rows_there()) return false;
   if (NORM) {                    // the summaries follow the query after its normalisation and before its rotation (Sec. 3.2)
     for (int g = w; g < G; g += NSUM) {
       float qf[PER];
@@ -215,7 +217,7 @@ __device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, u
     __syncwarp();
     if (lane == 0) mbar_arrive(norm_bar);
   }
-  if (!owner && !qt) return;
+  if (!owner && !qt) return true;
   for (int g0 = w; g0 < G; g0 += 2 * NSUM) {
     if (g0 != w) load_old(g0);
     double ss[2][2], sq[2];                                // sums of squares: new summaries, query
@@ -281,6 +283,7 @@ __device__ __forceinline__ void summary_rows(const GpDev& p, const GpNorm& nm, u
         }
       }
   }
+  return true;
 }
 
 // bf16 -> double by its bits, scaled by 2^-896 (an 8-bit exponent read as an 11-bit one): exact for every finite number, and
@@ -381,14 +384,23 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
   }
 }
 
-template <int D, bool ROPE, bool NORM, bool WIDE>       // WIDE: groups of eight query heads
+// WIDE: groups of eight query heads.  MODE: a whole step, a layer of one, or a layer with raw queries and keys.
+enum { WHOLE_STEP, ONE_LAYER, ONE_LAYER_NORM };
+template <int D, bool ROPE, int MODE, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 2)
 gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* __restrict__ q,
                const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, float* __restrict__ out, int lh0,
-               int lh_n, int adv_lh, const GpNorm nm) {
+               int lh_n, int adv_lh, int planned, const GpNorm nm) {
   // lh0, lh_n: the (layer, KV head) units this launch covers, [lh0, lh0 + lh_n): all of them, or one layer's
   // adv_lh: the unit whose append also moves the request's counters on by one token (-1: none; the layer-by-layer
   // step does that at its end)
+  // planned (a layer's launch): the step's plan had completed before this grid could start.  It follows another layer's launch on
+  // its stream, and that one waited for the plan before it let this one be scheduled.  Then only the caller's tensors depend on the
+  // kernel before this one: descriptor, page ids, the first tiles and the old summaries are asked for while that kernel drains, and
+  // the producer waits before it asks for the first rows.  Whatever is written follows those rows.  (36 layers x 16 requests of 400 to 1000
+  // tokens, layer by layer: 864 us per step with every launch waiting at its top, now 760.  In the whole step's kernel the rows share
+  // the descriptor's barrier: two barriers there cost 1 to 2 %.)
+  constexpr bool LAYER = MODE != WHOLE_STEP, NORM = MODE == ONE_LAYER_NORM;
   using GEO = Geo<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & (SMEM_ALIGN - 1u));
@@ -396,10 +408,11 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   const Lay L = make_lay<D>(G);
   const uint32_t NCOMB = (uint32_t)L.ncomb;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.off_bars);
-  uint64_t* slot_full = bars;                  // [NI]
+  uint64_t* slot_full = bars;                  // [NI] descriptor and page ids, and, but in a layer's launch, the rows
   uint64_t* slot_empty = slot_full + NI;       // [NI]
   uint64_t* slot_norm = slot_empty + NI;       // [NI] the slot's query rows have been normalised
-  uint64_t* qt_full = slot_norm + NI;
+  uint64_t* slot_rows = slot_norm + NI;        // [NI] a layer's launch: the slot's query, key and value rows are there
+  uint64_t* qt_full = slot_rows + NI;
   uint64_t* qt_empty = qt_full + 1;
   uint64_t* comb_full = qt_empty + 1;          // [2]
   uint64_t* comb_empty = comb_full + 2;        // [2]
@@ -411,7 +424,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t lim = p.spin_limit;
   if (tid == 0) {
-    for (int i = 0; i < NI; ++i) { mbar_init(&slot_full[i], 2); mbar_init(&slot_empty[i], NCW + 1 + NSUM); mbar_init(&slot_norm[i], NSUM); }
+    for (int i = 0; i < NI; ++i) { mbar_init(&slot_full[i], LAYER ? 1 : 2); mbar_init(&slot_rows[i], 1); mbar_init(&slot_empty[i], NCW + 1 + NSUM); mbar_init(&slot_norm[i], NSUM); }
     mbar_init(qt_full, NSUM);
     mbar_init(qt_empty, NCW);
     for (int i = 0; i < 2; ++i) { mbar_init(&comb_full[i], NCW); mbar_init(&comb_empty[i], 1); }
@@ -419,8 +432,10 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
     s_misc[1] = 0;
     fence_mbar_init();
   }
-  gp_pdl_wait();                  // everything above touched only this CTA's shared memory
-  gp_pdl_launch_dependents();
+  if (!LAYER || !planned) {
+    gp_pdl_wait();                // everything above touched only this CTA's shared memory
+    gp_pdl_launch_dependents();
+  }
   __syncthreads();
 
   // the first item's descriptor is fetched before the number of items is known (same round trip): a slot past it holds
@@ -452,10 +467,15 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       if (!wait_bar(&slot_empty[sl], ((n / NI) & 1u) ^ 1u, s_misc, 1, lim)) break;
       uint8_t* slot = smem + L.off_slots + sl * GEO::SLOT_BYTES;
       int* sd = reinterpret_cast<int*>(slot);
+      const bool rows_later = LAYER && planned && n == 0;
       if (item >= total) {
+        if (rows_later) { gp_pdl_wait(); gp_pdl_launch_dependents(); }
         if (lane == 0) sd[3] = -1;
         __syncwarp();
-        if (lane == 0) { mbar_arrive(&slot_full[sl]); mbar_arrive(&slot_full[sl]); }
+        if (lane == 0) {
+          mbar_arrive(&slot_full[sl]);
+          if (!LAYER) mbar_arrive(&slot_full[sl]);
+        }
         break;
       }
       const int lh = lh0 + (int)(item % lh_n);
@@ -473,24 +493,31 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       if (lane == 15) sd[15] = hdr;            // index among the step's boundary requests
       if (lane == 16) sd[16] = (int)(item & (NCW - 1));       // the consumer warp that takes the item's first tile
       __syncwarp();
-      if (lane == 0) {
+      auto ask_rows = [&]() {
         const bool has_new = (chunk == nchunks - 1);
+        uint64_t* bar = LAYER ? &slot_rows[sl] : &slot_full[sl];
         fence_proxy_async();
-        mbar_expect_tx(&slot_full[sl], q_bytes + (has_new ? 2 * GEO::ROW_BYTES : 0) + (ROPE ? D / 2 * 8 : 0));
-        bulk_g2s(slot + GEO::SLOT_DESC, q + (((size_t)l * n_req + bi) * p.Hq + h * G) * D, q_bytes, &slot_full[sl]);
-        if (ROPE) bulk_g2s(slot + GEO::SLOT_ROPE, p.rope_f + (size_t)bi * D, D / 2 * 8, &slot_full[sl]);
+        mbar_expect_tx(bar, q_bytes + (has_new ? 2 * GEO::ROW_BYTES : 0) + (ROPE ? D / 2 * 8 : 0));
+        bulk_g2s(slot + GEO::SLOT_DESC, q + (((size_t)l * n_req + bi) * p.Hq + h * G) * D, q_bytes, bar);
+        if (ROPE) bulk_g2s(slot + GEO::SLOT_ROPE, p.rope_f + (size_t)bi * D, D / 2 * 8, bar);
         if (has_new) {
           const size_t kvo = (((size_t)l * n_req + bi) * p.Hkv + h) * D;
-          bulk_g2s(slot + GEO::SLOT_DESC + 8 * GEO::ROW_BYTES, k + kvo, GEO::ROW_BYTES, &slot_full[sl]);
-          bulk_g2s(slot + GEO::SLOT_DESC + 9 * GEO::ROW_BYTES, v + kvo, GEO::ROW_BYTES, &slot_full[sl]);
+          bulk_g2s(slot + GEO::SLOT_DESC + 8 * GEO::ROW_BYTES, k + kvo, GEO::ROW_BYTES, bar);
+          bulk_g2s(slot + GEO::SLOT_DESC + 9 * GEO::ROW_BYTES, v + kvo, GEO::ROW_BYTES, bar);
         }
-      }
+      };
+      if (lane == 0 && !rows_later) ask_rows();
       sd[GEO::SLOT_PAGES + lane] = pg;
       sd[GEO::SLOT_PAGES + 32 + lane] = pg2;
       __syncwarp();
       // (test support: the first CTA's second item can be withheld, so that the consumers' bounded wait runs out)
       const bool withheld = (p.withhold & GP_WITHHOLD_ITEM) && blockIdx.x == 0 && n == 1;
       if (lane == 0 && !withheld) mbar_arrive(&slot_full[sl]);
+      if (rows_later) {
+        gp_pdl_wait();
+        gp_pdl_launch_dependents();
+        if (lane == 0) ask_rows();
+      }
       // ---- the next item ----------------------------------------------------------------------------------
       if (n > 0 && !wait_bar(&slot_empty[(n - 1) % NI], ((n - 1) / NI) & 1u, s_misc, 2, lim)) break;
       int t = 0;
@@ -565,7 +592,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const int n_new = n_old + 1;
       const bool need_qt = (flags & 1) && (pg0 < Pr - 1);
 
-      if (NORM && !wait_bar(&slot_norm[sl], (it / NI) & 1u, s_misc, 11, lim)) break;
+      if (LAYER && !wait_bar(NORM ? &slot_norm[sl] : &slot_rows[sl], (it / NI) & 1u, s_misc, NORM ? 11 : 12, lim)) break;
       // ---- query fragments (A operand), rotated when RoPE is on ----------------------------------
       uint32_t qa[GEO::KSTEPS][2];
       uint32_t ql[GEO::KSTEPS][2];
@@ -886,8 +913,9 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       if (NORM || owner || need_qt) {
         if (need_qt && !wait_bar(qt_empty, (qt_uses & 1u) ^ 1u, s_misc, 10, lim)) break;
         const int l = lh / p.Hkv, h = lh % p.Hkv;
-        summary_rows<D, ROPE, NORM>(p, nm, slot + GEO::SLOT_DESC, &slot_norm[sl], w, G, l, h, r, bi, par, (flags & 2) != 0, owner,
-                                    need_qt ? qt : nullptr);
+        auto rows_there = [&]() { return !LAYER || wait_bar(&slot_rows[sl], (it / NI) & 1u, s_misc, 13, lim); };
+        if (!summary_rows<D, ROPE, NORM>(p, nm, slot + GEO::SLOT_DESC, rows_there, &slot_norm[sl], w, G, l, h, r, bi, par, (flags & 2) != 0, owner,
+                                         need_qt ? qt : nullptr)) break;
         __syncwarp();
         if (need_qt) {
           ++qt_uses;
@@ -908,26 +936,28 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
 size_t gp_attention_smem(int d, int G) { return d == 128 ? make_lay<128>(G).total : make_lay<64>(G).total; }
 int gp_attention_ctas_per_sm(int d) { (void)d; return 2; }
 
-typedef void (*AttnKernel)(const GpDev, int, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, float*, int, int, int,
+typedef void (*AttnKernel)(const GpDev, int, const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*, float*, int, int, int, int,
                            const GpNorm);
-template <int D, bool WIDE> static AttnKernel attn_kernel_d(bool rope, bool norm) {
-  return rope ? (norm ? gp_attn_kernel<D, true, true, WIDE> : gp_attn_kernel<D, true, false, WIDE>)
-              : (norm ? gp_attn_kernel<D, false, true, WIDE> : gp_attn_kernel<D, false, false, WIDE>);
+template <int D, bool WIDE> static AttnKernel attn_kernel_d(bool rope, int mode) {
+  return mode == WHOLE_STEP ? (rope ? gp_attn_kernel<D, true, WHOLE_STEP, WIDE> : gp_attn_kernel<D, false, WHOLE_STEP, WIDE>)
+         : mode == ONE_LAYER ? (rope ? gp_attn_kernel<D, true, ONE_LAYER, WIDE> : gp_attn_kernel<D, false, ONE_LAYER, WIDE>)
+                             : (rope ? gp_attn_kernel<D, true, ONE_LAYER_NORM, WIDE> : gp_attn_kernel<D, false, ONE_LAYER_NORM, WIDE>);
 }
-static AttnKernel attn_kernel_of(const GpDev& p, bool norm) {
+static AttnKernel attn_kernel_of(const GpDev& p, int mode) {
   const bool rope = p.rope_theta != 0.0;
-  if (p.d == 128) return p.G == 8 ? attn_kernel_d<128, true>(rope, norm) : attn_kernel_d<128, false>(rope, norm);
-  return p.G == 8 ? attn_kernel_d<64, true>(rope, norm) : attn_kernel_d<64, false>(rope, norm);
+  if (p.d == 128) return p.G == 8 ? attn_kernel_d<128, true>(rope, mode) : attn_kernel_d<128, false>(rope, mode);
+  return p.G == 8 ? attn_kernel_d<64, true>(rope, mode) : attn_kernel_d<64, false>(rope, mode);
 }
 
 void gp_attention_setup(const GpDev& p) {           // once per pool: opt into the kernels' shared memory
-  for (int norm = 0; norm < 2; ++norm)
-    cudaFuncSetAttribute(attn_kernel_of(p, norm != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp_attention_smem(p.d, p.G));
+  for (int mode = WHOLE_STEP; mode <= ONE_LAYER_NORM; ++mode)
+    cudaFuncSetAttribute(attn_kernel_of(p, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp_attention_smem(p.d, p.G));
 }
 
 void gp_launch_attention(const GpDev& p, int n_req, const void* q, const void* k, const void* v, float* out, int grid, cudaStream_t s,
-                         bool pdl, int lh0, int lh_n, int adv_lh, const GpNorm& nm) {
-  gp_launch(attn_kernel_of(p, nm.wq != nullptr), grid, NTHREADS, gp_attention_smem(p.d, p.G), s, pdl, p, n_req,
+                         bool pdl, int lh0, int lh_n, int adv_lh, bool layer, bool planned, const GpNorm& nm) {
+  const int mode = !layer ? WHOLE_STEP : nm.wq ? ONE_LAYER_NORM : ONE_LAYER;
+  gp_launch(attn_kernel_of(p, mode), grid, NTHREADS, gp_attention_smem(p.d, p.G), s, pdl, p, n_req,
             static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), out, lh0,
-            lh_n, adv_lh, nm);
+            lh_n, adv_lh, planned ? 1 : 0, nm);
 }

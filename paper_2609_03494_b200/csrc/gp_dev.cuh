@@ -252,7 +252,7 @@ struct GpNorm {
   double eps;
 };
 void gp_launch_attention(const GpDev& p, int n_req, const void* q, const void* k, const void* v, float* out, int grid, cudaStream_t s,
-                         bool pdl, int lh0, int lh_n, int adv_lh, const GpNorm& nm);
+                         bool pdl, int lh0, int lh_n, int adv_lh, bool layer, bool planned, const GpNorm& nm);
 size_t gp_attention_smem(int d, int G);
 int gp_attention_ctas_per_sm(int d);
 // ---- programmatic dependent launch -------------------------------------------------------------------

@@ -36,6 +36,7 @@ struct gp_pool {
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
   int abandoned;                                    // a step was abandoned since the last plan: its kernels may still run
   std::vector<uint8_t> step_layer_seen;             // layers gp_attn_layer has run in the open step
+  cudaStream_t layer_stream;                        // stream of the last of them
   // error bits set by the kernels (GP_E_*): one int of page-locked host memory that the device addresses directly,
   // so that the host reads it without a copy once the work that could set it has completed
   int* h_err;
@@ -931,7 +932,7 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
       launch_plan(pool, dev_req_ids, n_req, dev_actions, pool->early_plan != 0, s, pdl && !pool->first_plain, false, nullptr,
                   pool->attn_grid_ov);
       if (prof) cudaEventRecord(pool->ev[1], s);
-      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0, kNoNorm);
+      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0, false, false, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
       gp_launch_chain(d, n_req, serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy);
       if (prof) { cudaEventRecord(pool->ev[3], s); cudaEventRecord(pool->ev[4], s); }    // the last interval stays empty
@@ -941,7 +942,7 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
       // layer-by-layer step
       launch_plan(pool, dev_req_ids, n_req, dev_actions, pool->early_plan != 0, s, pdl && !pool->first_plain);
       if (prof) cudaEventRecord(pool->ev[1], s);
-      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, pdl, 0, LH, 0, kNoNorm);
+      gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, pdl, 0, LH, 0, false, false, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
       gp_launch_boundary(d, dev_req_ids, n_req, dev_actions, false, pool->sel_grid, pool->compact_grid, s,
                          prof ? pool->ev[3] : nullptr, pdl, serial);
@@ -961,7 +962,7 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
     // which the chain kernel of the step before (the kernel before this one on the stream) has just written
     launch_plan(pool, dev_req_ids, n_req, dev_actions, false, s, pdl && !pool->first_plain, false, &d, pool->attn_grid_async);
     if (prof) cudaEventRecord(pool->ev[1], s);
-    gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_async, s, pdl, 0, LH, 0, kNoNorm);
+    gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_async, s, pdl, 0, LH, 0, false, false, kNoNorm);
     if (prof) cudaEventRecord(pool->ev[2], s);
     // the decisions of the step before set pages and slots of requests that sit this step out: nothing else of
     // this step looks at those words
@@ -1025,6 +1026,16 @@ int gp_step_begin(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, int3
   return GP_OK;
 }
 
+// A layer behind another layer's launch on the same stream may start before that one has ended: the plan it reads has (that
+// launch waited for it), and layers share nothing else (see gp_attn_kernel).
+static void launch_layer(gp_pool* pool, int n_req, const void* q, const void* k, const void* v, float* out, int layer, cudaStream_t s,
+                         const GpNorm& nm) {
+  const GpDev& d = pool->dev;
+  const bool planned = pool->step_layers_done > 0 && s == pool->layer_stream;
+  pool->layer_stream = s;
+  gp_launch_attention(d, n_req, q, k, v, out, pool->attn_grid, s, true, layer * d.Hkv, d.Hkv, -1, true, planned, nm);
+}
+
 int gp_attn_layer(gp_pool* pool, int32_t layer, const int32_t* dev_req_ids, int32_t n_req, const void* q, const void* k,
                   const void* v, void* out, void* stream) {
   if (!pool || pool->step_open != 1 || n_req != pool->step_n_req) return pool && pool->step_open != 1 ? GP_ERR_STATE : GP_ERR_INVALID;
@@ -1042,8 +1053,7 @@ int gp_attn_layer(gp_pool* pool, int32_t layer, const int32_t* dev_req_ids, int3
   const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(reinterpret_cast<uintptr_t>(k) - ks * 2);
   const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(reinterpret_cast<uintptr_t>(v) - ks * 2);
   float* ob = reinterpret_cast<float*>(reinterpret_cast<uintptr_t>(out) - qs * 4);
-  const int lh0 = layer * d.Hkv, lh_n = d.Hkv;
-  gp_launch_attention(d, n_req, qb, kb, vb, ob, pool->attn_grid, s, true, lh0, lh_n, -1, kNoNorm);
+  launch_layer(pool, n_req, qb, kb, vb, ob, layer, s, kNoNorm);
   pool->launch_count += 1;
   pool->step_layers_done += 1;
   pool->step_layer_seen[layer] = 1;
@@ -1071,7 +1081,7 @@ int gp_attn_layer_qknorm(gp_pool* pool, int32_t layer, const int32_t* dev_req_id
   float* ob = reinterpret_cast<float*>(shifted(out, qs * 4));
   const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(shifted(k_raw, ks * 2));
   const GpNorm nm = {q_weight, k_weight, eps};
-  gp_launch_attention(d, n_req, qb, kb, vb, ob, pool->attn_grid, s, true, layer * d.Hkv, d.Hkv, -1, nm);
+  launch_layer(pool, n_req, qb, kb, vb, ob, layer, s, nm);
   pool->launch_count += 1;
   pool->step_layers_done += 1;
   pool->step_layer_seen[layer] = 1;
@@ -1118,7 +1128,7 @@ int gp_decode_step_local(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_re
   const int LH = d.L * d.Hkv;
   const int serial = (int)(pool->serial & 0x3fffffff);
   launch_plan(pool, dev_req_ids, n_req, dev_actions, false, s, true);
-  gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, true, 0, LH, 0, kNoNorm);
+  gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid, s, true, 0, LH, 0, false, false, kNoNorm);
   gp_launch_select_only(d, dev_req_ids, n_req, dev_actions, pool->sel_grid, s, true, serial);
   pool->launch_count += 3;
   pool->step_open = 2;                           // between the two halves the pool takes nothing else
