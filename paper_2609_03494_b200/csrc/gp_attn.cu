@@ -3,8 +3,8 @@
 // (Eq. 12) against every candidate key while the key tile is in shared memory.
 //
 // Work decomposition.  The plan kernel cuts every stepped request into chunks of `chunk_pages` pages and
-// writes one descriptor per chunk, sorted by descending cost; a work item is (chunk, layer, KV head).  The CTAs of a
-// persistent grid (two per SM) draw them in that order.  Each CTA is warp-specialised:
+// writes one descriptor per chunk, those of requests at their boundary first, each part sorted by descending cost; a work item is
+// (chunk, layer, KV head).  The CTAs of a persistent grid (two per SM) draw them in that order.  Each CTA is warp-specialised:
 //
 //   warp 0      producer: draws the CTA's items and publishes each in a ring of item slots: descriptor, query rows
 //               (and the new key/value row, and the position's cosines and sines) by bulk copy, page ids.
@@ -368,7 +368,8 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
     // view = col / G (short or long summary); a view's values of one unit are contiguous [token][G]
     const size_t tokrow = (size_t)(zoff + tok0 + grp);
     if (G >= 2) {
-      double* z0 = p.zbuf + (((size_t)lh * 2 + col / G) * p.z_stride + tokrow) * G + col % G;
+      const int lg = 31 - __clz(G);                       // (a power of two)
+      double* z0 = p.zbuf + (((((size_t)lh * 2 + (col >> lg)) * p.z_stride + tokrow) << lg) + (col & (G - 1)));
       *reinterpret_cast<double2*>(z0) = make_double2(z00, z01);
       *reinterpret_cast<double2*>(z0 + (size_t)8 * G) = make_double2(z10, z11);
     } else {
@@ -377,7 +378,7 @@ __device__ __forceinline__ void summary_logits(const GpDev& p, const uint8_t* ti
       zS[0] = z00; zS[8] = z10; zL[0] = z01; zL[8] = z11;
     }
     if (grp == 0) {
-      double* st2 = p.zstat + (((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + (zoff + tok0) / GP_PAGE) * (2 * G) + col) * 2;
+      double* st2 = p.zstat + (((size_t)lh * ((unsigned long long)p.max_boundary_tokens / GP_PAGE) + (unsigned long long)(zoff + tok0) / GP_PAGE) * (2 * G) + col) * 2;
       *reinterpret_cast<double2*>(st2) = make_double2(m0, e0);
       *reinterpret_cast<double2*>(st2 + 2) = make_double2(m1, e1);
     }
@@ -438,13 +439,13 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   }
   __syncthreads();
 
-  // the first item's descriptor is fetched before the number of items is known (same round trip): a slot past it holds
-  // stale but readable data that is then not used
+  // the descriptor of the item of this CTA's own number, which its first one nearly always is, is fetched before the numbers of items
+  // are known (same round trip): a slot past them holds stale but readable data that is then not used
   int hFirst = 0;
   if (warp == 0 && lane < GP_DESC_INTS && (int)(blockIdx.x / lh_n) < p.max_rc) hFirst = p.rcx[(size_t)(blockIdx.x / lh_n) * GP_DESC_INTS + lane];
-  const int n_rc = p.hdr[HDR_N_RC];
+  const int n_rc = __ldcg(p.hdr + HDR_N_RC), n_brc = __ldcg(p.hdr + HDR_N_BRC);
   const int LH = p.L * p.Hkv;
-  const long long total = (long long)n_rc * lh_n;
+  const long long total_b = (long long)n_brc * lh_n, total = (long long)n_rc * lh_n;
   const int q_bytes = G * GEO::ROW_BYTES;
 
   if (warp < 4) {
@@ -454,14 +455,25 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   }
   if (warp == 0) {
     // ================================= producer ===========================================
-    // A CTA's first item is the one of its own number, the others are drawn from a counter, costliest first (numbering the
-    // items unit by unit instead, so that boundary items spread over the launch: 35.7 ms against 33.9 on the 32B shape), and
+    // Two lists: the items of requests at their boundary, whose tiles also pay for the fp64 logits (bound by the DMMA pipe, 26 cycles
+    // each, which keeps a sub-partition from much else), and the others, which are bound by memory; costliest first in each.  A part of
+    // the grid draws from the former as long as there are any, the rest from the latter, so that the logits hide behind other
+    // blocks' loads: half of the grid where the boundary items fit there at once (their requests' selection waits for them), else a
+    // third (36 layers x 256 requests 4375 us per step with half, 4312 with a third, 4336 with a quarter).  One list, boundary
+    // items first, so that all blocks were at them and the memory idle: 4478; 36 x 16: 328, now 313; 64 x 32 with groups of 8: 1813, now 1774.
+    // A CTA's first item follows from its number, the others are drawn from a counter per list, and
     // only once the item before the one last published is done: a CTA holds the item it works on and the next, and what is
     // left goes to whoever is free.  (Dealt out statically by an estimate of their cost, the CTAs of a one-layer step ended
     // between 26 and 38 us; drawn as far ahead as a ring of eight slots allows, they hoarded.)  Which CTA takes an item does
     // not change its result.
-    long long item = (long long)blockIdx.x < total ? (long long)blockIdx.x : total;
+    const long long total_p = total - total_b, cta = blockIdx.x, grid = gridDim.x;
+    const long long b_ctas = total_b <= grid / 2 ? total_b : grid / 3;      // blocks that draw boundary items first
+    const long long first_p = min(total_p, grid - b_ctas), first_b = min(total_b, grid - first_p);
+    // an item's number: of the first list, then of the second
+    long long item = cta < b_ctas ? cta : cta - b_ctas < first_p ? total_b + cta - b_ctas : cta - first_p < first_b ? cta - first_p : total;
+    bool left[2] = {true, true};               // items of the lists this CTA still asks for
     int hdr = hFirst;                          // descriptor header, word `lane` (lanes 0..15)
+    if (item != cta && item < total && lane < GP_DESC_INTS) hdr = p.rcx[(size_t)(item / lh_n) * GP_DESC_INTS + lane];
     for (uint32_t n = 0;; ++n) {
       const int sl = n % NI;
       if (!wait_bar(&slot_empty[sl], ((n / NI) & 1u) ^ 1u, s_misc, 1, lim)) break;
@@ -520,10 +532,17 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       }
       // ---- the next item ----------------------------------------------------------------------------------
       if (n > 0 && !wait_bar(&slot_empty[(n - 1) % NI], ((n - 1) / NI) & 1u, s_misc, 2, lim)) break;
-      int t = 0;
-      if (lane == 0) t = atomicAdd(p.tickets + lh0 / p.Hkv, 1);
-      item = (long long)gridDim.x + __shfl_sync(0xffffffffu, t, 0);
-      if (item > total) item = total;
+      item = total;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int list = cta < b_ctas ? k : 1 - k;
+        if (item < total || !left[list]) continue;
+        int t = 0;
+        if (lane == 0) t = atomicAdd(p.tickets + 2 * (lh0 / p.Hkv) + list, 1);
+        const long long at = (list ? first_p : first_b) + __shfl_sync(0xffffffffu, t, 0);
+        left[list] = at < (list ? total_p : total_b);
+        if (left[list]) item = list ? total_b + at : at;
+      }
       hdr = 0;
       if (item < total && lane < GP_DESC_INTS) hdr = p.rcx[(size_t)(item / lh_n) * GP_DESC_INTS + lane];
     }

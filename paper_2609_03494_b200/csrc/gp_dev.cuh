@@ -30,7 +30,7 @@
 #define GP_MAX_REQ 1024        // upper limit of max_requests (shared-memory arrays are sized by it)
 #define GP_PART_SLOTS 4096     // slots per compaction ticket: units beyond that are shared out (a unit of 20 000 slots in one block: 15 us of loads)
 #define GP_PART_MIN 64         // ... in tests
-#define GP_COST_BINS 288       // cost classes of attention work items (pages, x4 at a boundary)
+#define GP_COST_BINS 160       // cost classes of attention work items: pages, from the middle on those of requests at a boundary
 #define GP_DESC_INTS 16        // ints per attention work descriptor
 #define GP_ATTN_CONSUMERS 4    // consumer warps of an attention thread block: each reports once per item it worked on
 
@@ -47,6 +47,7 @@ enum {
   HDR_WORK_CMP,      // ticket counter of the compaction kernel
   HDR_N_CITEM,       // compaction work items (parts x layers x heads)
   HDR_N_COW,         // copy-on-write targets allotted this step
+  HDR_N_BRC,         // (request, chunk) work items of requests at their boundary: the first of the list
   HDR_COUNT = 16
 };
 
@@ -135,7 +136,7 @@ struct GpDev {
   int* evict;                            // [M][L*H_kv][page_size] slots a compression evicts, ascending
   int* evict2;                           // [M][L*H_kv][2 page_size] slots a Shrink evicts, ascending (Shrink policy only)
   int* cflags;                           // compaction part flags, stamped with the step number
-  int* tickets;                          // [L] next attention work item to draw: of the whole step (0) or of a layer's launch
+  int* tickets;                          // [L][2] next attention work item to draw, per list: of the whole step (0) or of a layer's launch
   double* inv_freq;                      // [d/2] rope_theta^(-2j/d)
   float* rope_f;                         // [M][d/2][2] cos, sin at the step's position in fp32 (the queries' rotation)
   double* rope_cs;                       // [M][d/2][2] the same in fp64

@@ -386,7 +386,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   s_first[i] = chunks > 0 ? (key << 16) | chunks : 0;        // s_first has served its purpose
   if (chunks > 0) atomicAdd(&s_bin[key], chunks);
   __syncthreads();
-  if (threadIdx.x < 32) {                             // descending exclusive scan over the cost bins, nine to a lane
+  if (threadIdx.x < 32) {                             // descending exclusive scan over the cost bins, five to a lane
     constexpr int PER = GP_COST_BINS / 32;
     int v[PER], sum = 0;
 #pragma unroll
