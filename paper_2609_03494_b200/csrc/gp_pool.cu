@@ -170,7 +170,7 @@ Layout make_layout(const gp_config& c) {
   L.evict2 = take(c.policy == GP_POLICY_SHRINK ? M * LH * 2 * blk * 4 : 16);
   L.cflags = take(LH * ((Tb + M * b) / GP_PART_MIN + 2 * M + 1) * 4);
   L.inv_freq = take(d / 2 * 8);
-  L.tickets = take((size_t)c.n_layers * 4);
+  L.tickets = take((size_t)c.n_layers * 2 * 4);
   L.rope_f = take(M * (d / 2) * 2 * 4);
   L.rope_cs = take(M * (d / 2) * 2 * 8);
   L.partials = take((size_t)L.max_rc * LH * G * (d + 2) * 4);
@@ -325,7 +325,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   if (inrange) st = preloaded ? s_state[r] : load_state(r);
   // the attention kernel draws its items from these (the one of the step before, the last to draw, has ended: that step's
   // decisions waited for it, or, where it was abandoned before it had any, this launch did)
-  for (int idx = threadIdx.x; idx < p.L; idx += blockDim.x) p.tickets[idx] = 0;
+  for (int idx = threadIdx.x; idx < 2 * p.L; idx += blockDim.x) p.tickets[idx] = 0;
   __syncthreads();
   int chunks = 0, pages = 0, act = GP_ACT_NONE;
   const int n_old = st.x, Pr = st.y, pos = st.z;
@@ -376,9 +376,9 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     plan_scan(s_scan[1], chunks, isb << 16 | (chunks > 0), nc, rc_off, both, tok_off, n_rc, both_tot, tok_tot);
   }
   const int bnd_idx = both >> 16, n_bnd = both_tot >> 16, n_active = both_tot & 0xffff;
-  // Work items are listed by descending cost (pages, times four for boundary requests, which also pay for the
-  // fp64 logits): the attention kernel deals them out in that order, largest first.  Counting sort.
-  const int key = chunks > 0 ? min(GP_COST_BINS - 1, cp * (isb ? 4 : 1)) : 0;
+  // Work items are listed by descending cost (pages), those of boundary requests, which also pay for the fp64 logits, before the
+  // others: the attention kernel draws from the two parts in that order, largest first.  Counting sort.
+  const int key = chunks > 0 ? cp + (isb ? GP_COST_BINS / 2 : 0) : 0;
   // Items of equal cost keep the batch's order (a rank counted over the earlier batch slots, not the order in
   // which atomics land), so that the same batch gives the same numbered list every time.  An item's number says which of a
   // block's warps takes which of its tiles, and split outputs are merged in chunk order: with the numbers fixed, the attention outputs
@@ -439,6 +439,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += blockDim.x) p.unit_ready[idx] = 0;
   if (threadIdx.x == 0) {
     p.hdr[HDR_N_RC] = n_rc;
+    p.hdr[HDR_N_BRC] = s_binbase[GP_COST_BINS / 2] + s_bin[GP_COST_BINS / 2];
     p.hdr[HDR_N_BND] = n_bnd;
     p.hdr[HDR_N_ACTIVE] = n_active;
   }
