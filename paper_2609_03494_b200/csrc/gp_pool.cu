@@ -797,16 +797,16 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   }
   pool->attn_grid_ov = pool->attn_grid;
   pool->chain_grid_ov = 0;
-  // One kernel behind the attention kernel pays while a step's boundary work is a few hundred jobs: it saves a kernel
-  // boundary and starts its jobs while the attention kernel drains (requests of 200 to 1200 tokens, 64 x 8 units: 72.6 us per
-  // step against 79.5).  From about a thousand units on the compaction wants the four-kernel path's larger grid, few as the
-  // boundaries of a step may be (8 layers x 16 requests: 109.0 us in one kernel, 108.5 in four; 36 layers x 4: 104.5, 99.6;
-  // x 16: 393, 378; x 64: 1403, 1393; x 256: 4866, 4754; 1 layer x 256: 181, 178).
-  const bool fused_auto = (long long)cfg->max_requests * cfg->n_layers * cfg->n_kv_heads <= 1024;
-  if (!cfg->async_boundary && (cfg->overlap_slots == -2 || (cfg->overlap_slots == 0 && fused_auto))) {
+  // How the boundary work of a step is launched where the caller leaves it open.  One kernel behind the attention kernel saves a kernel
+  // boundary and starts its jobs while the attention kernel drains (us per step, four kernels / one, layers x requests, 8 KV heads:
+  // 1 x 64 73.5 / 65.7; 8 x 16 91 / 87; 36 x 4 84 / 83; 36 x 16 314 / 310); from about ten thousand units on the two kernels'
+  // larger grids are worth as much (64 x 32: 1790 / 1810; 36 x 64: 1177 / 1180; 36 x 256: 4388 / 4420).
+  const long long units = (long long)cfg->n_layers * cfg->n_kv_heads * cfg->max_requests;
+  int slots = cfg->overlap_slots;
+  if (slots == 0) slots = units <= 8192 ? -2 : -1;
+  if (!cfg->async_boundary && slots == -2) {
     pool->chain_grid_ov = pool->chain_grid_max;    // the whole grid, behind the attention kernel's
-  } else if (!cfg->async_boundary && cfg->overlap_slots > 0) {
-    int slots = cfg->overlap_slots;
+  } else if (!cfg->async_boundary && slots > 0) {
     if (slots > pool->attn_grid / 2) slots = pool->attn_grid / 2;
     pool->attn_grid_ov = pool->attn_grid - slots;
     pool->chain_grid_ov = slots;
