@@ -14,7 +14,7 @@
 //               the old buffer for itself.  (They were CTAs of the plan kernel: 8 us before the first key could be
 //               asked for in a layer-by-layer launch, 300 us of the step at 36 layers x 256 requests, and q~ went through
 //               global memory.)
-//   warps 4..7  consumers: take the tiles of an item round-robin (tile j belongs to warp (j - its item's number) mod 4,
+//   warps 4..7  consumers: take the tiles of an item round-robin (tile j, at d = 64 pair j of tiles, belongs to warp (j - its item's number) mod 4,
 //               so the odd tiles of successive items fall on different warps).  Each warp
 //               fetches its own K|V tiles (one contiguous 8 KB per (layer, page, head)) with 16-byte
 //               asynchronous copies into a private ring of stages, running ahead across item boundaries, so
@@ -57,6 +57,10 @@ template <int D>
 struct Geo {
   static constexpr int ROW_BYTES = D * 2;
   static constexpr int TILE_BYTES = 2 * GP_PAGE * ROW_BYTES;
+  // Tiles a consumer warp takes at a time: two of 4 KB at d = 64, where one cost nearly the instructions (softmax, its shuffles, the ring) of
+  // one of 8 KB (64 layers x 32 requests of 200 to 1800 tokens, groups of 4: 774 us one by one, 5.6 TB/s; now 676, 6.4 TB/s)
+  static constexpr int PAIR = 128 / D;
+  static constexpr int STAGE_BYTES = PAIR * TILE_BYTES;                // 8 KB
   static constexpr int KSTEPS = D / 16;
   static constexpr int DTILES = D / 8;
   static constexpr int SLOT_DESC = 384;                                // 96 ints: descriptor (32), then up to 64 page ids
@@ -74,7 +78,7 @@ __host__ __device__ constexpr Lay make_lay(int G) {
   using GEO = Geo<D>;
   Lay L = {};
   L.ncomb = (D == 128 && G == 8) ? 1 : 2;
-  L.off_slots = NCW * NSW * GEO::TILE_BYTES;
+  L.off_slots = NCW * NSW * GEO::STAGE_BYTES;
   L.off_qt = L.off_slots + NI * GEO::SLOT_BYTES;
   const int nrows = 2 * G < 8 ? 8 : 2 * G;
   L.off_comb = L.off_qt + nrows * (D + QT_PAD) * 8;
@@ -559,6 +563,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
     // boundaries, but never further than the ring of item slots allows).  No other warp touches the ring, so
     // program order plus a proxy fence orders the reads of a stage before the copy that overwrites it.
     const uint64_t kv_policy = l2_policy_evict_first();    // the K/V stream is read once per step: first out of the L2
+    constexpr int PAIR = GEO::PAIR;
     uint32_t my_fetch = 0, f_it = 0;
     int f_pgl = 0, f_npg = 0, f_lh = 0;
     bool f_have = false, f_done = false;
@@ -577,21 +582,23 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           f_npg = fsd[3];
           if (f_npg < 0) { f_done = true; break; }
           f_lh = fsd[14];
-          f_pgl = (cw + fsd[16]) % NCW;                   // the first tile goes to another warp from item to item
+          f_pgl = (cw + fsd[16]) % NCW;                   // in units of PAIR tiles; the first goes to another warp from item to item
           f_have = true;
         }
-        if (f_pgl >= f_npg) { ++f_it; f_have = false; continue; }
-        const int page = fsd[GEO::SLOT_PAGES + f_pgl];
+        if (f_pgl * PAIR >= f_npg) { ++f_it; f_have = false; continue; }
         const uint32_t fst = cw * NSW + (my_fetch % NSW);
-        {
+#pragma unroll
+        for (int sub = 0; sub < PAIR; ++sub) {
+          if (sub && f_pgl * PAIR + sub >= f_npg) break;
+          const int page = fsd[GEO::SLOT_PAGES + f_pgl * PAIR + sub];
           // 16-byte asynchronous copies through the load/store path, 512 contiguous bytes per warp instruction:
           // the bulk-copy engine takes several hundred cycles to accept an 8 KB copy, which paced the kernel
           const uint8_t* src = reinterpret_cast<const uint8_t*>(p.kv + gp_tile_off(p, f_lh / p.Hkv, page, f_lh % p.Hkv)) + lane * 16;
-          const uint32_t dst = smem_u32(smem + fst * GEO::TILE_BYTES) + lane * 16;
+          const uint32_t dst = smem_u32(smem + fst * GEO::STAGE_BYTES + sub * GEO::TILE_BYTES) + lane * 16;
 #pragma unroll
           for (int c = 0; c < GEO::TILE_BYTES / 512; ++c) cp_async16_hint(dst + c * 512, src + c * 512, kv_policy);
-          cp_async_commit();
         }
+        cp_async_commit();
         ++my_fetch;
         f_pgl += NCW;
       }
@@ -653,7 +660,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       float m_run = -INFINITY, l_run = 0.f;
       bool ok = true;
 
-      for (int pgl = (cw + sd[16]) % NCW; pgl < npg; pgl += NCW) {
+      for (int pgl = (cw + sd[16]) % NCW * PAIR; pgl < npg; pgl += NCW * PAIR) {
         const uint32_t st = cw * NSW + (my_tiles % NSW);
         {
           // one copy group per tile, in fetch order: all but the groups younger than this tile's must be done
@@ -662,12 +669,14 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           __syncwarp();
         }
         ++my_tiles;
-        uint8_t* tile = smem + st * GEO::TILE_BYTES;
+        uint8_t* stage = smem + st * GEO::STAGE_BYTES;
         const int tok0 = (pg0 + pgl) * GP_PAGE;
-        const bool has_new = last_chunk && (pgl == npg - 1);
+        const int nsub = PAIR == 1 ? 1 : min(PAIR, npg - pgl);         // tiles of the stage
+        const bool has_new = last_chunk && (pgl + PAIR >= npg);        // the last of them is the request's
         if (has_new) {
+          uint8_t* tile = stage + (nsub - 1) * GEO::TILE_BYTES;
           // append: slot n_old of this page receives k_t, v_t; patch the staged copy too
-          const int s = n_old - tok0;
+          const int s = n_old - tok0 - (nsub - 1) * GP_PAGE;
           const int page = sd[GEO::SLOT_PAGES + npg - 1];
           constexpr int CH = D / 8;
           uint4 k_new = make_uint4(0, 0, 0, 0);
@@ -721,38 +730,39 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           }
           __syncwarp();
         }
-        const uint32_t kt = smem_u32(tile);
-        const uint32_t vt = kt + GP_PAGE * GEO::ROW_BYTES;
-
-        // S = Q K^T for the 16 tokens of the page
-        float s_acc[2][4];
+        // S = Q K^T for the 16 tokens of each page
+        float s_acc[PAIR][2][4];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) s_acc[i][0] = s_acc[i][1] = s_acc[i][2] = s_acc[i][3] = 0.f;
-        {
+        for (int i = 0; i < PAIR * 8; ++i) (&s_acc[0][0][0])[i] = 0.f;
+#pragma unroll
+        for (int sub = 0; sub < PAIR; ++sub) {
+          if (sub && sub >= nsub) break;
           const int token = (lane & 7) + ((lane >> 4) << 3);
           const int csel = (lane >> 3) & 1;
-          const uint32_t rowaddr = kt + token * GEO::ROW_BYTES;
+          const uint32_t rowaddr = smem_u32(stage) + sub * GEO::TILE_BYTES + token * GEO::ROW_BYTES;
 #pragma unroll
           for (int kk = 0; kk < GEO::KSTEPS; ++kk) {
             uint32_t b00, b01, b10, b11;
             ldsm_x4(rowaddr + ((((2 * kk + csel) ^ (token & 7))) << 4), b00, b01, b10, b11);
-            mma_bf16(s_acc[0], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b00, b01);
-            mma_bf16(s_acc[1], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b10, b11);
+            mma_bf16(s_acc[sub][0], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b00, b01);
+            mma_bf16(s_acc[sub][1], qa[kk][0], ql[kk][0], qa[kk][1], ql[kk][1], b10, b11);
           }
         }
         // online softmax in the log2 domain
-        float sv[2][2];
-        const int n_valid = has_new ? (n_new - tok0) : GP_PAGE;
+        float sv[PAIR][2][2];
+        const int n_valid = has_new ? (n_new - tok0) : nsub * GP_PAGE;
         float mx = -INFINITY;
+#pragma unroll
+        for (int sub = 0; sub < PAIR; ++sub)
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            float x = s_acc[nt][j];
-            if (ROPE) x += s_acc[nt][j + 2];
+            float x = s_acc[sub][nt][j];
+            if (ROPE) x += s_acc[sub][nt][j + 2];
             x *= sc;
-            if (nt * 8 + qc + j >= n_valid) x = -INFINITY;
-            sv[nt][j] = x;
+            if (sub * GP_PAGE + nt * 8 + qc + j >= n_valid) x = -INFINITY;
+            sv[sub][nt][j] = x;
             mx = fmaxf(mx, x);
           }
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
@@ -767,20 +777,22 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           }
         }
         m_run = m_new;
-        uint32_t pa[4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const float p0 = exp2f(sv[nt][0] - m_new), p1 = exp2f(sv[nt][1] - m_new);
-          l_run += p0 + p1;
-          const uint32_t hi = pack_bf16(p0, p1);
-          pa[nt * 2] = hi;
-          pa[nt * 2 + 1] = pack_bf16(p0 - bf16_lo_f(hi), p1 - bf16_hi_f(hi));
-        }
-        // O += P V
-        {
+        for (int sub = 0; sub < PAIR; ++sub) {
+          if (sub && sub >= nsub) break;
+          uint32_t pa[4];
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            const float p0 = exp2f(sv[sub][nt][0] - m_new), p1 = exp2f(sv[sub][nt][1] - m_new);
+            l_run += p0 + p1;
+            const uint32_t hi = pack_bf16(p0, p1);
+            pa[nt * 2] = hi;
+            pa[nt * 2 + 1] = pack_bf16(p0 - bf16_lo_f(hi), p1 - bf16_hi_f(hi));
+          }
+          // O += P V
           const int token = (lane & 7) + (((lane >> 3) & 1) << 3);
           const int csel = lane >> 4;
-          const uint32_t rowaddr = vt + token * GEO::ROW_BYTES;
+          const uint32_t rowaddr = smem_u32(stage) + sub * GEO::TILE_BYTES + GP_PAGE * GEO::ROW_BYTES + token * GEO::ROW_BYTES;
 #pragma unroll
           for (int jd = 0; jd < GEO::DTILES; jd += 2) {
             uint32_t v0, v1, v2, v3;
@@ -796,8 +808,12 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             qt_here = true;
           }
           const long long zoff = ((long long)(unsigned)sd[10]) | ((long long)sd[11] << 32);
-          summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 0);
-          if (WIDE) summary_logits<D>(p, tile, qt, G, lh, zoff, tok0, 1);
+#pragma unroll 1
+          for (int sub = 0; sub < PAIR; ++sub) {
+            if (sub && (sub >= nsub || pg0 + pgl + sub >= Pr - 1)) break;
+            summary_logits<D>(p, stage + sub * GEO::TILE_BYTES, qt, G, lh, zoff, tok0 + sub * GP_PAGE, 0);
+            if (WIDE) summary_logits<D>(p, stage + sub * GEO::TILE_BYTES, qt, G, lh, zoff, tok0 + sub * GP_PAGE, 1);
+          }
         }
         __syncwarp();
         if (!top_up(it)) { ok = false; break; }            // the stage is free: fetch the next tile into it
