@@ -83,7 +83,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
   if (n_bnd > 0) {
     top0 = p.async ? __ldcg(p.free_top) : __ldcg(p.free_peek);
     for (int e = tid; e < n_bnd; e += blockDim.x) {
-      const int4 inf = p.bnd_info[2 * e];
+      const int4 inf = p.bnd_info[2 * e], inf2 = p.bnd_info[2 * e + 1];
       int4 acc = __ldcg(reinterpret_cast<const int4*>(p.bnd_acc) + e);
       if (from_sums) { acc.x = __ldcg(p.shard_sums + 2 * e); acc.y = __ldcg(p.shard_sums + 2 * e + 1); }
       s_free[e] = p.async ? (e < top0 ? __ldcg(p.free_stack + top0 - 1 - e) : 0) : __ldcg(p.free_peek + 1 + e);
@@ -119,6 +119,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
       // pages and slots as the step left them (full); the allocator below changes what the decision changes.  In
       // the asynchronous mode the plan of the step in between leaves these two words of a held request alone.
       p.P[r] = Pr; p.n[r] = Pr * GP_PAGE;
+      p.cmp_off[e] = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
       s_want[e] = want; s_ksh[e] = acc.z; s_P[e] = Pr; s_req[e] = r; s_bi[e] = inf.x;
     }
   }
@@ -1192,10 +1193,9 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     }
     __syncthreads();
     if (n_part > 1) {
-      // where a unit's evicted slots lie, found by its parts: in the place of its scores, which are done with
-      const int4 inf2 = p.bnd_info[2 * e_bnd + 1];
-      const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
-      int* found = reinterpret_cast<int*>(p.scores + (size_t)lh * p.max_boundary_tokens + off);        // [ne][2] (a unit has ne candidates at least)
+      // where a unit's evicted slots lie, found by its parts: in the place of its scores, which are done with (from cmp_off: with
+      // early planning the next step's plan may be writing its own boundary records by now)
+      int* found = reinterpret_cast<int*>(p.scores + (size_t)lh * p.max_boundary_tokens + __ldcg(p.cmp_off + e_bnd));        // [ne][2] (a unit has ne candidates at least)
       if (part < n_part - 1) {
         for (int t = tid; t < ne; t += CT)
           if (C.ev_slot[t] >= 0) { found[2 * t] = C.ev_slot[t]; found[2 * t + 1] = C.ev_page[t]; }
@@ -1219,6 +1219,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       for (int t = tid; t < ne; t += CT)
         if (C.ev_slot[t] < 0) {
           const int2 f = __ldcg(reinterpret_cast<const int2*>(found) + t);
+          if (f.x < 0 || f.x >= n_src || f.y < 0 || f.y >= p.n_pages) { atomicOr(p.err, GP_E_BOUNDS); continue; }     // that slot stays as it is
           C.ev_slot[t] = f.x; C.ev_page[t] = f.y;
         }
       __syncthreads();

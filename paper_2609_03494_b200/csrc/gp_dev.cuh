@@ -129,6 +129,7 @@ struct GpDev {
   int* bnd_acc;                          // [M][4] per boundary request: sum of K^S, sum of K^L, shared pages of C, 0
   int* free_peek;                        // [M+1] free_top at plan time, then the top entries of the free list, top first
   int4* cmp_info;                        // [M+1] compressing requests: {request, P, index in bnd_info, first compaction part}
+  long long* cmp_off;                    // [M] per boundary request its place in the scores: bnd_info's, kept for the compaction, beside which the next plan may write that
   double* zbuf;                          // [L*H_kv][2][z_stride][G] boundary units, per view (short, long): exp(summary logit - its page's max)
   long long z_stride;                    // max_boundary_tokens rounded up to a multiple of the page size
   double* zstat;                         // [L*H_kv][max_boundary_tokens / b][2][G][2] per-page softmax partials (max, sum)

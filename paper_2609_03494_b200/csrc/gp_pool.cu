@@ -71,7 +71,7 @@ namespace {
 
 struct Layout {
   size_t kv, tok, rank, refcount, free_stack, words, page_table, shadow, reqi, pos, summ, Kx, Hx, delta, rc,
-      merge_cnt, bnd_info, bnd_acc, free_peek, cmp_info, zbuf, zstat, sum_par, inv_freq, tickets, rope_f,
+      merge_cnt, bnd_info, bnd_acc, free_peek, cmp_info, cmp_off, zbuf, zstat, sum_par, inv_freq, tickets, rope_f,
       unit_ready, shard_sums, bnd_info2, bnd_acc2, zbuf2, zstat2, rc2, rope_cs2, rope_f2,
       evict, evict2, cflags, rope_cs, partials, scores, counters, dbg,
       st_ids, st_q, st_k, st_v, st_out, st_act, st2_ids, st2_q, st2_k, st2_v, total;
@@ -164,6 +164,7 @@ Layout make_layout(const gp_config& c) {
   L.shard_sums = take((size_t)M * 2 * 4);
   L.free_peek = take((M + 1) * 4);
   L.cmp_info = take((M + 1) * 16);
+  L.cmp_off = take(M * 8);
   L.zbuf = take(LH * (Tb + b) * 2 * G * 8);
   L.zstat = take(LH * (Tb / b + 1) * 2 * G * 2 * 8);
   L.evict = take(M * LH * blk * 4);
@@ -762,6 +763,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.units_total = cfg->n_layers * cfg->n_kv_heads * cfg->kv_shard_count;
   d.free_peek = reinterpret_cast<int*>(base + L.free_peek);
   d.cmp_info = reinterpret_cast<int4*>(base + L.cmp_info);
+  d.cmp_off = reinterpret_cast<long long*>(base + L.cmp_off);
   d.zbuf = reinterpret_cast<double*>(base + L.zbuf);
   d.zstat = reinterpret_cast<double*>(base + L.zstat);
   d.evict = reinterpret_cast<int*>(base + L.evict);

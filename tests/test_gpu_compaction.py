@@ -71,3 +71,68 @@ def test_rows_and_ids_stay_together_through_many_compactions(d):
         assert compressed >= 5 and B.gp_pool_status(pool.handle) == (B.GP_OK, 0)
     finally:
         pool.close()
+
+
+def _decode(lens, steps, forms, layers=2, hq=4, hkv=2, d=64, page=16, tau=10.0, **config):
+    """`steps` decode steps of requests with prompts of `lens` tokens on a pool with a page to spare for each, once per form (early
+    planning, compaction switch, overlap_slots; a host wait after every step only where there is no early planning): outputs, actions,
+    and every request's state, ids and rows."""
+    import torch
+    n_req, cap = len(lens), max(lens) // page + 3
+    rng = np.random.default_rng(41)
+    bits = lambda *shape: W.f32_to_bf16_bits(rng.standard_normal(shape).astype(np.float32))
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).cuda()
+    prompts = [(dev(bits(layers, n, hkv, d)), dev(bits(layers, n, hkv, d)), n) for n in lens]
+    ins = [tuple(dev(bits(layers, n_req, h, d)) for h in (hq, hkv, hkv)) for _ in range(steps)]
+    ids = torch.arange(n_req, dtype=torch.int32, device="cuda")
+    results = []
+    for early, switch, overlap in forms:
+        pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(n // page + 2 for n in lens), max_pages_per_req=cap, page_size=page,
+                                    k_loc=page // 4, max_requests=max(4, n_req), overlap_slots=overlap, tau=tau, **config))
+        try:
+            for k, v, n in prompts:
+                assert pool.request_add(-1, 0, k, v, n, 0)[0] == B.GP_OK
+            B.gp_set_early_plan(pool.handle, early)
+            B.gp_test_withhold(pool.handle, switch, 0)
+            outs = torch.zeros((steps, layers, n_req, hq, d), dtype=torch.float32, device="cuda")
+            acts = torch.zeros((steps, n_req), dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            for t in range(steps):
+                pool.decode_step(ids, *ins[t], outs[t], acts[t])
+                if not early:
+                    torch.cuda.synchronize()
+            torch.cuda.synchronize()
+            assert B.gp_pool_status(pool.handle) == (B.GP_OK, 0)
+            state = [B.gp_debug_request(pool.handle, r, cap)[:3] for r in range(n_req)]
+            kept = [a for r in range(n_req) for l in range(layers) for h in range(hkv)
+                    for a in (B.gp_debug_retained(pool.handle, r, l, h, state[r][1]), *B.gp_debug_kv(pool.handle, r, l, h, state[r][1], d))]
+            results.append((outs.cpu().numpy(), acts.cpu().numpy(), state, kept))
+        finally:
+            pool.close()
+    return results
+
+
+def _assert_equal(results):
+    (o1, a1, s1, k1) = results[0]
+    for o2, a2, s2, k2 in results[1:]:
+        assert np.array_equal(a1, a2) and s1 == s2 and np.array_equal(o1, o2)
+        assert len(k1) == len(k2) and all(np.array_equal(x, y) for x, y in zip(k1, k2))
+
+
+def test_parts_beside_an_early_plan():
+    """With early planning the plan of a step runs beside the compaction of the step before and writes its own boundary records there.
+    Three requests of unequal length compress at every step, other ones from step to step (the records' places in the scratch differ),
+    no host wait lies between the steps: parts of 64 slots give what whole units without early planning give, bit for bit."""
+    lens = [16 * (4 + (7 * i) % 45) - 1 - i // 3 for i in range(48)]
+    results = _decode(lens, 40, [(False, 16, -1), (True, 32, -2), (True, 32, -1), (True, 16, -2), (False, 32, -2)])
+    compress = np.isin(results[0][1], (B.GP_ACT_COMPRESS, B.GP_ACT_COMPRESS_FALLBACK))
+    assert (compress.sum(axis=1) >= 3).all()
+    _assert_equal(results)
+
+
+def test_parts_of_long_units_beside_an_early_plan():
+    """The parts as they are (units of up to three, each of several passes of its thread block), early planning on and off."""
+    lens = [16 * m - 1 - i % 2 for i, m in enumerate((257, 300, 513, 520, 770, 40))]
+    results = _decode(lens, 20, [(False, 16, -1), (True, 0, -2), (True, 0, -1)], layers=1)
+    assert np.isin(results[0][1], (B.GP_ACT_COMPRESS, B.GP_ACT_COMPRESS_FALLBACK)).sum() >= 12
+    _assert_equal(results)
