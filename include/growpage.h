@@ -387,15 +387,17 @@ int gp_set_profiling(gp_pool* pool, int32_t enable);
 
 /* Early planning (off by default).  The first kernel of gp_decode_step is launched as a programmatic
  * dependent of whatever kernel precedes it on the stream.  With the option off it waits for that
- * kernel to end before it reads anything: always safe.  With it on, it reads dev_req_ids and plans
- * the step before that wait, beside the compaction of the step before, and waits only before it looks
+ * kernel to end before it reads anything of the caller's: always safe.  (The pool's own counters it reads
+ * before, in every synchronous step: they are final once the step before has taken its decisions, and
+ * behind a gp_release or a gp_step_abort the kernel is launched the plain way.)  With it on, it reads
+ * dev_req_ids and plans the step before that wait, beside the compaction of the step before, and waits only before it looks
  * at the free list.  That is correct only if dev_req_ids is complete in memory by the time the preceding
  * kernel on the stream lets its dependents be scheduled: true when it was produced by copies or by
  * kernels that do not signal programmatic launch completion (or when nothing was enqueued since the
  * step before); not true when a kernel enqueued just before the step writes the ids and signals completion
  * ahead of its stores.  (Queries, keys and values are read by the step's second kernel: nothing is asked of
  * them.)  gp_decode_step_host always plans early (its inputs arrive by copies).  The layer-by-layer
- * calls are not affected; the step after a gp_step_abort waits whatever the option says. */
+ * calls are not affected; the step after a gp_step_abort or a gp_release waits whatever the option says. */
 int gp_set_early_plan(gp_pool* pool, int32_t enable);
 
 /* Synchronises, then returns the accumulated device time in milliseconds and the launch count of

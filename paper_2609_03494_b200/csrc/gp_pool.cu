@@ -34,7 +34,7 @@ struct gp_pool {
   int num_sms, attn_grid, sel_grid, compact_grid;
   int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
-  int abandoned;                                    // a step was abandoned since the last plan: its kernels may still run
+  int plain_plan;                                   // a request was released or a step abandoned since the last plan, whose counters or items its kernels may still change
   std::vector<uint8_t> step_layer_seen;             // layers gp_attn_layer has run in the open step
   cudaStream_t layer_stream;                        // stream of the last of them
   // error bits set by the kernels (GP_E_*): one int of page-locked host memory that the device addresses directly,
@@ -688,7 +688,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   pool->profiling = 0;
   pool->early_plan = 0;
   pool->first_plain = 0;
-  pool->step_open = 0; pool->step_n_req = 0; pool->step_layers_done = 0; pool->abandoned = 0;
+  pool->step_open = 0; pool->step_n_req = 0; pool->step_layers_done = 0; pool->plain_plan = 0;
   pool->step_layer_seen.assign(cfg->n_layers, 0);
   pool->h_err = nullptr;
   pool->launch_count = 0;
@@ -894,15 +894,17 @@ int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, co
 
 static const GpNorm kNoNorm = {nullptr, nullptr, 0.0};
 
-// CTA 0 plans; the others fill the table of cosines and sines (a thread per entry).  Behind an abandoned step the launch is a
-// plain one, without early planning: that step's kernels let their dependents go at their top and no decision waited for them,
-// so that a plan beside them would take the items they still draw and the counters they draw from.
+// CTA 0 plans; the others fill the table of cosines and sines (a thread per entry).  The plan reads the requests' counters before
+// its wait, so what writes them has to be done when it starts.  Behind the kernels of a step it is; behind a release or an abandoned
+// step the launch is a plain one, without early planning: only the wait would show the plan what a release has written, and an abandoned
+// step's kernels let their dependents go at their top and no decision waited for them, so that a plan beside them would take the items
+// they still draw and the counters they draw from.  (An admission is waited for on the host.)
 static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_t* actions, bool early, cudaStream_t s, bool pdl,
                         bool by_layer = false, const GpDev* dev = nullptr, int attn_grid = 0) {
   const GpDev& d = dev ? *dev : pool->dev;
   const int threads = n_req <= GP_PLAN_SMALL ? GP_PLAN_SMALL : GP_PLAN_THREADS;
   const int table = d.rope_theta != 0.0 ? (n_req * (d.d / 2) + threads - 1) / threads : 0;
-  if (pool->abandoned) { early = false; pdl = false; pool->abandoned = 0; }
+  if (pool->plain_plan) { early = false; pdl = false; pool->plain_plan = 0; }
   gp_launch(gp_plan_kernel, 1 + table, threads, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
             by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff));
 }
@@ -1112,7 +1114,7 @@ int gp_step_abort(gp_pool* pool) {
   // Nothing of an open step is committed before gp_step_end: the requests' counters are untouched, rows appended
   // by the layers that ran lie beyond the occupied slots, and the summaries went to the buffer not in use.
   pool->step_open = 0;
-  pool->abandoned = 1;
+  pool->plain_plan = 1;
   return GP_OK;
 }
 
@@ -1340,6 +1342,7 @@ int gp_release(gp_pool* pool, int32_t req, void* stream) {
   if (flush_chain(pool, static_cast<cudaStream_t>(stream)) != GP_OK) return GP_ERR_CUDA;
   gp_release_kernel<<<1, ADMIT_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(pool->dev, req);
   pool->launch_count++;
+  pool->plain_plan = 1;
   pool->live[req] = 0;
   GP_CUDA(cudaGetLastError());
   return GP_OK;

@@ -185,6 +185,40 @@ def test_early_planned_steps_behind_abandoned_ones_are_undisturbed():
     assert all(np.array_equal(x, y) for x, y in zip(k1 + m1, k2 + m2)) and np.array_equal(o1, o2)
 
 
+@pytest.mark.parametrize("overlap,early", [(-2, False), (-2, True), (-1, False), (-1, True)])
+def test_a_request_released_right_before_a_step_is_invalid_in_it(overlap, early):
+    """The plan reads the requests' counters ahead of its wait for the kernel before it, but not ahead of a release: no host wait lies
+    between steps and releases, every step still names all requests."""
+    import torch
+    n_req, hq, hkv, d = 24, 8, 2, 64
+    rng = np.random.default_rng(43)
+    pool = B.Pool(B.make_config(1, hq, hkv, d, n_pages=16 * n_req, max_pages_per_req=16, max_requests=n_req, overlap_slots=overlap, tau=10.0))
+    try:
+        for i in range(n_req):
+            n = 47 + 3 * i
+            assert pool.request_add(-1, 0, _bits(rng, 1, n, hkv, d), _bits(rng, 1, n, hkv, d), n, 0)[0] == B.GP_OK
+        B.gp_set_early_plan(pool.handle, early)
+        q, k, v = (_dev(torch, _bits(rng, 1, n_req, h, d)) for h in (hq, hkv, hkv))
+        ids = torch.arange(n_req, dtype=torch.int32, device="cuda")
+        out = torch.zeros((1, n_req, hq, d), dtype=torch.float32, device="cuda")
+        acts = torch.zeros((n_req, n_req), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        order = [int(x) for x in rng.permutation(n_req)]
+        for t in range(n_req):
+            pool.release(order[t])
+            pool.decode_step(ids, q, k, v, out, acts[t])
+        torch.cuda.synchronize()
+        got = acts.cpu().numpy()
+        for t in range(n_req):
+            dead = np.isin(np.arange(n_req), order[:t + 1])
+            assert np.array_equal(got[t] == B.GP_ACT_INVALID, dead), t
+        assert B.gp_pool_status(pool.handle) == (B.GP_OK, 0)
+        n_free, ref, _ = B.gp_debug_pool(pool.handle, 16 * n_req)
+        assert n_free == 16 * n_req and not ref.any()
+    finally:
+        pool.close()
+
+
 # ----------------------------------------------------------------------------------------------------------------
 # bounded waits that run out: the kernel gives up, says so, and ends; nothing hangs, nothing faults
 # ----------------------------------------------------------------------------------------------------------------
