@@ -1056,9 +1056,10 @@ __device__ __forceinline__ int warp_pack(int n, int* out, F flag) {
 // rows, stores), three thread blocks to an SM.  Every row behind the first evicted slot moved down (in 64-slot chunks that waited for one
 // another where units were few): 467 us at 36 layers x 256 requests, now 73; 53, now 12, at 36 x 16; 187, now 26, at 64 x 32; the
 // one-layer step of 64 requests 74.8 us, now 70.1.
-// The first ticket of a CTA is its number, the others come from a counter.  A ticket is a unit, or, where a unit has more than
-// GP_PART_SLOTS slots, a part of one: a part tells where its evicted slots lie, and the unit's last part, which waits for that
-// word of the others (tickets are handed out in order, so those are running or done), moves the rows.
+// A ticket is a unit, or, where a unit has more than GP_PART_SLOTS slots, a part of one: a part tells where its evicted slots lie, and
+// the unit's last part, which waits for that word of the others, moves the rows.  Tickets come from a counter, in order, so that those
+// of a unit's other parts are with CTAs that run or have ended; only where every unit is one ticket, and none waits, a CTA's first is its
+// number, which saves a round trip.
 template <int D>
 __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, int serial) {
   constexpr int CH = D / 8;
@@ -1085,11 +1086,12 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
   const int part_slots = part_slots_of(p);
   int moved = 0;
 
+  const bool own_first = n_items == n_cmp * LH;          // (every unit is one ticket)
   int item = blockIdx.x;
-  for (bool first = true;; first = false) {
+  for (bool first = own_first;; first = false) {
     __syncthreads();
     if (!first) {
-      if (tid == 0) s_i[0] = gridDim.x + atomicAdd(&p.hdr[HDR_WORK_CMP], 1);
+      if (tid == 0) s_i[0] = (own_first ? (int)gridDim.x : 0) + atomicAdd(&p.hdr[HDR_WORK_CMP], 1);
       __syncthreads();
       item = s_i[0];
     }
