@@ -46,13 +46,15 @@ __device__ __forceinline__ unsigned long long to_fix(double a) {
   return (unsigned long long)__double2ll_rn(a * TWO62);
 }
 
-// slots per compaction ticket, and the tickets of a unit that keeps n_end slots: the last one has what lies behind them as well
-// (test support: see GP_WITHHOLD_CHUNK)
-__device__ __forceinline__ int part_slots_of(const GpDev& p) {
-  return (p.withhold & (GP_WITHHOLD_CHUNK | GP_TEST_COMPACT_BY_PART)) ? GP_PART_MIN : GP_PART_SLOTS;
+// Compaction tickets of a unit that keeps n_end slots, in parts of `most` slots at most (test support: see GP_WITHHOLD_CHUNK), and the
+// slots of each: equal shares in whole tiles.  The last one has what lies behind them as well.
+__device__ __forceinline__ int parts_of(const GpDev& p, int n_end, int most) {
+  if (p.withhold & GP_TEST_COMPACT_BY_UNIT) return 1;
+  if (p.withhold & (GP_WITHHOLD_CHUNK | GP_TEST_COMPACT_BY_PART)) most = GP_PART_MIN;
+  return (n_end + most - 1) / most;
 }
-__device__ __forceinline__ int parts_of(const GpDev& p, int n_end) {
-  return (p.withhold & GP_TEST_COMPACT_BY_UNIT) ? 1 : (n_end + part_slots_of(p) - 1) / part_slots_of(p);
+__device__ __forceinline__ int part_slots_of(int n_end, int n_part) {
+  return (n_end / GP_PAGE + n_part - 1) / n_part * GP_PAGE;
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -146,6 +148,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
     int n_cmp = 0, chunks = 0;
     unsigned long long grow = 0, comp = 0, fall = 0, stall = 0, cow = 0, scored = 0, shr = 0;
     const int sub = p.sub;
+    int copies = 0;                                      // tiles per (layer, KV head) that pass 2 may have copied
     for (int k = 0; k < n_bnd; ++k) {                    // pass 1: grants, ascending request id
       const int e = s_order[k];
       const int r = s_req[e], Pr = s_P[e], bi = s_bi[e];
@@ -166,8 +169,15 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
         report(bi, r, GP_ACT_STALLED);
         s_want[e] |= 4;
         ++stall;
+      } else {
+        copies += s_ksh[e];
       }
     }
+    // Units whose pages are shared are copied tile by tile, 8 KB each at d = 128.  Where they are too few for the grid (one has more than
+    // twice a thread block's even share of the tiles) they are cut into parts of a quarter of that share, of eight tiles at least.  Requests of
+    // 2048 tokens that share a prompt, us of the step in which all are copied, by units / cut (one layer, 8 KV heads): 2 requests
+    // 127 / 88, 4 148 / 106, 8 173 / 141, 16 227 / 214; cut all the same: 32 312 / 320, 4 layers x 16 494 / 519.
+    const float copy_share = (float)copies * p.copy_share;
     for (int k = 0; k < n_bnd; ++k) {                    // pass 2: copy-on-write targets
       const int e = s_order[k];
       if (s_want[e] & 6) continue;
@@ -182,7 +192,8 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
       cow += s_ksh[e];
       const bool shrink = (s_want[e] & 16) != 0;
       p.cmp_info[n_cmp] = make_int4(r, s_P[e], e | (shrink ? CMP_SHRINK : 0), chunks);
-      chunks += parts_of(p, (s_P[e] - (shrink ? 2 : 1) * sub) * GP_PAGE);
+      chunks += parts_of(p, (s_P[e] - (shrink ? 2 : 1) * sub) * GP_PAGE,
+                         s_ksh[e] > 2.f * copy_share && s_ksh[e] > 8 ? (int)fmaxf(8.f, 0.25f * copy_share) * GP_PAGE : GP_PART_SLOTS);
       ++n_cmp;
       if (s_want[e] & 1) { report(bi, r, GP_ACT_COMPRESS_FALLBACK); ++fall; }
       else if (shrink) { report(bi, r, GP_ACT_SHRINK); ++shr; }
@@ -1056,7 +1067,7 @@ __device__ __forceinline__ int warp_pack(int n, int* out, F flag) {
 // rows, stores), three thread blocks to an SM.  Every row behind the first evicted slot moved down (in 64-slot chunks that waited for one
 // another where units were few): 467 us at 36 layers x 256 requests, now 73; 53, now 12, at 36 x 16; 187, now 26, at 64 x 32; the
 // one-layer step of 64 requests 74.8 us, now 70.1.
-// A ticket is a unit, or, where a unit has more than GP_PART_SLOTS slots, a part of one: a part tells where its evicted slots lie, and
+// A ticket is a unit, or, where a unit has more than GP_PART_SLOTS slots or is copied with few others, a part of one: a part tells where its evicted slots lie, and
 // the unit's last part, which waits for that word of the others, moves the rows.  Tickets come from a counter, in order, so that those
 // of a unit's other parts are with CTAs that run or have ended; only where every unit is one ticket, and none waits, a CTA's first is its
 // number, which saves a round trip.
@@ -1083,7 +1094,6 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
   // on the device, so that a step replayed from a CUDA graph gets a stamp of its own
   const int stamp = p.async ? serial + 1 : p.hdr[HDR_STEP];
   for (int i = tid + CT; i <= n_cmp; i += CT) s_info[i] = p.cmp_info[i];
-  const int part_slots = part_slots_of(p);
   int moved = 0;
 
   const bool own_first = n_items == n_cmp * LH;          // (every unit is one ticket)
@@ -1111,7 +1121,8 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     const int e_bnd = inf.z & (CMP_SHRINK - 1);
     const int ne = shrink ? 2 * p.blk : p.blk;             // slots freed: one page of the method, two at a Shrink
     const int n_src = Pr * GP_PAGE, n_end = n_src - ne;    // the unit's slots, and those that stay in use
-    const int c0 = n_part == 1 ? 0 : part * part_slots, c1 = part == n_part - 1 ? n_src : c0 + part_slots;
+    const int part_slots = part_slots_of(n_end, n_part);
+    const int c0 = part * part_slots, c1 = part == n_part - 1 ? n_src : c0 + part_slots;
     // order indices of a page's slots, and its rows: the unit's place in a page
     const size_t tok_stride = (size_t)p.Hkv * GP_PAGE, tok_base = gp_tok_off(p, l, 0, h);
     const size_t page_stride = (size_t)p.Hkv * 2 * GP_PAGE * ROW_BYTES;
@@ -1136,7 +1147,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
           to[u] = pg < pg_end && pg < Pr - 1 ? shadow[pg] : -1;
           const uint4* src = reinterpret_cast<const uint4*>(unit_base + (size_t)(to[u] >= 0 ? table[pg] : 0) * page_stride);
 #pragma unroll
-          for (int e = 0; e < TB / CT; ++e) if (to[u] >= 0) val[u][e] = src[tid + e * CT];
+          for (int e = 0; e < TB / CT; ++e) if (to[u] >= 0) val[u][e] = __ldcg(src + tid + e * CT);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {

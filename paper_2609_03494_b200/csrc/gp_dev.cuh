@@ -78,6 +78,7 @@ struct GpDev {
   long long max_boundary_tokens;         // bound on the summed candidate tokens of one step's boundary requests
   unsigned spin_limit;                   // iterations after which a bounded wait gives up (GP_SPIN_LIMIT; tests shorten it)
   int withhold;                          // test support, GP_WITHHOLD_*: a hand-over inside a kernel that is made not to happen
+  float copy_share;                      // (layer, KV head) units per thread block of the compaction: see decide_and_allocate
   int async;                             // 1: the boundary chain of a step runs beside the next step (see gp_decode_step)
   double beta_s, beta_l, top_p, tau, rope_theta;
   int bchunk_pages;                      // pages per work item of a request at its capacity boundary

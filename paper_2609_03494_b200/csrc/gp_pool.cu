@@ -814,6 +814,8 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
     pool->chain_grid_ov = slots;
   }
   pool->dev.report_units = pool->dev_alt.report_units = pool->chain_grid_ov > 0;
+  const int cmp_ctas = cfg->async_boundary ? pool->chain_grid : pool->chain_grid_ov > 0 ? pool->chain_grid_ov : pool->compact_grid;
+  pool->dev.copy_share = pool->dev_alt.copy_share = (float)(cfg->n_layers * cfg->n_kv_heads) / (float)cmp_ctas;
   pool->dbg = base + L.dbg;
   if (cfg->host_staging) {
     pool->st_ids = reinterpret_cast<int*>(base + L.st_ids);

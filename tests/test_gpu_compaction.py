@@ -73,16 +73,17 @@ def test_rows_and_ids_stay_together_through_many_compactions(d):
         pool.close()
 
 
-def _decode(lens, steps, forms, layers=2, hq=4, hkv=2, d=64, page=16, tau=10.0, **config):
-    """`steps` decode steps of requests with prompts of `lens` tokens on a pool with a page to spare for each, once per form (early
-    planning, compaction switch, overlap_slots; a host wait after every step only where there is no early planning): outputs, actions,
-    and every request's state, ids and rows."""
+def _decode(lens, steps, forms, layers=2, hq=4, hkv=2, d=64, page=16, tau=10.0, shared=None, **config):
+    """`steps` decode steps of requests with prompts of `lens` tokens (the first `shared` pages of each those of request 0) on a pool
+    with a page to spare for each, once per form (early planning, compaction switch, overlap_slots; a host wait after every step only
+    where there is no early planning): outputs, actions, and every request's state, ids and rows."""
     import torch
     n_req, cap = len(lens), max(lens) // page + 3
+    shared = shared or [0] * n_req
     rng = np.random.default_rng(41)
     bits = lambda *shape: W.f32_to_bf16_bits(rng.standard_normal(shape).astype(np.float32))
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).cuda()
-    prompts = [(dev(bits(layers, n, hkv, d)), dev(bits(layers, n, hkv, d)), n) for n in lens]
+    prompts = [(m, dev(bits(layers, n - m * page, hkv, d)), dev(bits(layers, n - m * page, hkv, d)), n - m * page) for n, m in zip(lens, shared)]
     ins = [tuple(dev(bits(layers, n_req, h, d)) for h in (hq, hkv, hkv)) for _ in range(steps)]
     ids = torch.arange(n_req, dtype=torch.int32, device="cuda")
     results = []
@@ -90,8 +91,8 @@ def _decode(lens, steps, forms, layers=2, hq=4, hkv=2, d=64, page=16, tau=10.0, 
         pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(n // page + 2 for n in lens), max_pages_per_req=cap, page_size=page,
                                     k_loc=page // 4, max_requests=max(4, n_req), overlap_slots=overlap, tau=tau, **config))
         try:
-            for k, v, n in prompts:
-                assert pool.request_add(-1, 0, k, v, n, 0)[0] == B.GP_OK
+            for m, k, v, n in prompts:
+                assert pool.request_add(0 if m else -1, m, k, v, n, 0)[0] == B.GP_OK
             B.gp_set_early_plan(pool.handle, early)
             B.gp_test_withhold(pool.handle, switch, 0)
             outs = torch.zeros((steps, layers, n_req, hq, d), dtype=torch.float32, device="cuda")
@@ -135,4 +136,18 @@ def test_parts_of_long_units_beside_an_early_plan():
     lens = [16 * m - 1 - i % 2 for i, m in enumerate((257, 300, 513, 520, 770, 40))]
     results = _decode(lens, 20, [(False, 16, -1), (True, 0, -2), (True, 0, -1)], layers=1)
     assert np.isin(results[0][1], (B.GP_ACT_COMPRESS, B.GP_ACT_COMPRESS_FALLBACK)).sum() >= 12
+    _assert_equal(results)
+
+
+@pytest.mark.parametrize("d,page,over", [(128, 16, {}), (64, 16, {}), (64, 32, {}), (128, 16, dict(policy=B.GP_POLICY_SHRINK, min_capacity=64,
+                                                                                           shrink_below=0.05))])
+def test_copied_units_in_parts(d, page, over):
+    """Units that are copied on write are shared out by their tiles: requests that share all, some or few of their pages, that compress in
+    the same step or later ones, against whole units."""
+    shared = [0, 139, 80, 100, 9, 8, 1, 60, 0, 139]
+    lens = [page * m - x for m, x in ((140, 1), (140, 1), (90, 1), (200, 1), (10, 1), (9, 1), (30, 1), (70, 5), (30, 1), (141, 3))]
+    results = _decode(lens, page + 6, [(False, 16, -1), (False, 0, -2), (True, 0, -2), (True, 0, -1), (True, 32, -2)], d=d, page=page, shared=shared,
+                      **over)
+    done = np.isin(results[0][1], (B.GP_ACT_COMPRESS, B.GP_ACT_COMPRESS_FALLBACK, B.GP_ACT_SHRINK))
+    assert done.any(axis=0).all() and (done[0].sum() >= 7 if page == 16 else True)
     _assert_equal(results)
