@@ -58,9 +58,17 @@ struct Geo {
   static constexpr int ROW_BYTES = D * 2;
   static constexpr int TILE_BYTES = 2 * GP_PAGE * ROW_BYTES;
   // Tiles a consumer warp takes at a time: two of 4 KB at d = 64, where one cost nearly the instructions (softmax, its shuffles, the ring) of
-  // one of 8 KB (64 layers x 32 requests of 200 to 1800 tokens, groups of 4: 774 us one by one, 5.6 TB/s; now 676, 6.4 TB/s)
+  // one of 8 KB (64 layers x 32 requests of 200 to 1800 tokens, groups of 4: 772 us one by one, 5.6 TB/s; now 690, 6.3 TB/s)
   static constexpr int PAIR = 128 / D;
   static constexpr int STAGE_BYTES = PAIR * TILE_BYTES;                // 8 KB
+  // The weights are carried as two bf16 terms, 2^-17 of each, where two tiles share a running maximum as three: the weight at a new maximum
+  // is one and carries no rounding, and tile by tile there are more of those (error of the outputs against 64 bits, 48 requests of 64 to 240
+  // tokens in groups of 1 to 8: tile by tile 1.61e-6 to 1.66e-6, in pairs with two terms 1.71e-6 to 1.78e-6, now 1.6e-7, groups of eight
+  // 1.22e-6).  For groups of up to four the third stands in rows of the product that no head has: lanes 16 to 31 repeat the heads of lanes
+  // 0 to 15.  Groups of eight take another product, for the first tile of a pair only (for both: 6.5 % of a step).  us of this kernel at
+  // 64 layers x 32 requests of 200 to 1800 tokens, none / two of them at a boundary: groups of four one by one 772 / 877, in pairs
+  // 673 / 775, with the third term 690 / 803; groups of eight 821 / 1029, 741 / 1044, 757 / 1086.
+  static constexpr bool THREE = PAIR > 1;
   static constexpr int KSTEPS = D / 16;
   static constexpr int DTILES = D / 8;
   static constexpr int SLOT_DESC = 384;                                // 96 ints: descriptor (32), then up to 64 page ids
@@ -82,7 +90,7 @@ __host__ __device__ constexpr Lay make_lay(int G) {
   L.off_qt = L.off_slots + NI * GEO::SLOT_BYTES;
   const int nrows = 2 * G < 8 ? 8 : 2 * G;
   L.off_comb = L.off_qt + nrows * (D + QT_PAD) * 8;
-  L.comb_warp = (16 + G * D) * 4;
+  L.comb_warp = (16 + (GEO::THREE && G < 8 ? 2 : 1) * G * D) * 4;     // maxima and sums, then rows (and the third terms' part of them)
   L.off_bars = L.off_comb + L.ncomb * NCW * L.comb_warp;
   L.off_misc = L.off_bars + (4 * NI + 2 + 4) * 8;
   L.total = L.off_misc + 128 + SMEM_ALIGN;   // abort flag and code; room for the rounding
@@ -289,6 +297,8 @@ __device__ __forceinline__ bool summary_rows(const GpDev& p, const GpNorm& nm, u
   }
   return true;
 }
+
+__device__ __forceinline__ float upper_half(float x, uint32_t mask) { return __uint_as_float(__float_as_uint(x) & mask); }
 
 // bf16 -> double by its bits, scaled by 2^-896 (an 8-bit exponent read as an 11-bit one): exact for every finite number, and
 // cheaper than the conversion unit.  The q~ buffer holds the summaries times 2^880, the logits are scaled by the remaining 2^16:
@@ -554,7 +564,11 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
     // ================================= consumers ==========================================
     const int cw = warp - 4;
     const float sc = 1.4426950408889634f * rsqrtf((float)D);
+    constexpr bool REPEAT = GEO::THREE && !WIDE;
     const int row = lane >> 2;
+    const bool third = REPEAT && row >= 4;                 // this lane has the third terms of head row - 4
+    const int head = third ? row - 4 : row;
+    const uint32_t keep = third ? 0u : 0xffffffffu, cut = third || WIDE ? 0xffff0000u : 0u;
     const int qc = (lane & 3) * 2;
     uint32_t qt_uses = 0, my_tiles = 0;
     // Each consumer warp fetches its own tiles (tile j of an item belongs to warp j mod 4) into its private
@@ -623,8 +637,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       uint32_t qa[GEO::KSTEPS][2];
       uint32_t ql[GEO::KSTEPS][2];
       {
-        const bool valid = row < G;
-        const uint8_t* qrow = slot + GEO::SLOT_DESC + (valid ? row : 0) * GEO::ROW_BYTES;
+        const bool valid = head < G;
+        const uint8_t* qrow = slot + GEO::SLOT_DESC + (valid ? head : 0) * GEO::ROW_BYTES;
 #pragma unroll
         for (int kk = 0; kk < GEO::KSTEPS; ++kk)
 #pragma unroll
@@ -780,14 +794,24 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
 #pragma unroll
         for (int sub = 0; sub < PAIR; ++sub) {
           if (sub && sub >= nsub) break;
-          uint32_t pa[4];
+          const bool three = REPEAT || (GEO::THREE && sub == 0);
+          uint32_t pa[4], pc[2];
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt) {
             const float p0 = exp2f(sv[sub][nt][0] - m_new), p1 = exp2f(sv[sub][nt][1] - m_new);
             l_run += p0 + p1;
             const uint32_t hi = pack_bf16(p0, p1);
-            pa[nt * 2] = hi;
-            pa[nt * 2 + 1] = pack_bf16(p0 - bf16_lo_f(hi), p1 - bf16_hi_f(hi));
+            const float r0 = p0 - bf16_lo_f(hi), r1 = p1 - bf16_hi_f(hi);
+            if (!three) {
+              pa[nt * 2] = hi;
+              pa[nt * 2 + 1] = pack_bf16(r0, r1);
+            } else {
+              // the residual has 16 bits at most: the second term is the upper eight, cut off, the third the others
+              const float c0 = r0 - upper_half(r0, cut), c1 = r1 - upper_half(r1, cut);
+              pa[nt * 2] = REPEAT ? hi & keep : hi;
+              pa[nt * 2 + 1] = __byte_perm(__float_as_uint(REPEAT ? c0 : r0), __float_as_uint(REPEAT ? c1 : r1), 0x7632);
+              if (WIDE) pc[nt] = __byte_perm(__float_as_uint(c0), __float_as_uint(c1), 0x7632);
+            }
           }
           // O += P V
           const int token = (lane & 7) + (((lane >> 3) & 1) << 3);
@@ -799,6 +823,10 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
             ldsm_x4_t(rowaddr + (((jd + csel) ^ (token & 7)) << 4), v0, v1, v2, v3);
             mma_bf16(o[jd], pa[0], pa[1], pa[2], pa[3], v0, v1);
             mma_bf16(o[jd + 1], pa[0], pa[1], pa[2], pa[3], v2, v3);
+            if (WIDE && three) {
+              mma_bf16(o[jd], pc[0], 0u, pc[1], 0u, v0, v1);
+              mma_bf16(o[jd + 1], pc[0], 0u, pc[1], 0u, v2, v3);
+            }
           }
         }
         // Boundary unit: fp64 logits of the calibrated summaries against the 16 keys of a candidate page
@@ -835,11 +863,12 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const int cb = it % NCOMB;
       if (!wait_bar(&comb_empty[cb], ((it / NCOMB) & 1u) ^ 1u, s_misc, 6, lim)) break;
       float* my_comb = comb + (cb * NCW + cw) * comb_w;
-      if (row < G) {
-        if ((lane & 3) == 0) { my_comb[row] = m_run; my_comb[8 + row] = l_run; }
+      if (head < G) {
+        if ((lane & 3) == 0 && !third) { my_comb[row] = m_run; my_comb[8 + row] = l_run; }
+        float* my_row = my_comb + 16 + (head + (third ? G : 0)) * D + qc;
 #pragma unroll
         for (int jd = 0; jd < GEO::DTILES; ++jd) {
-          *reinterpret_cast<float2*>(&my_comb[16 + row * D + jd * 8 + qc]) =
+          *reinterpret_cast<float2*>(my_row + jd * 8) =
               make_float2(o[jd][0] + o[jd][2], o[jd][1] + o[jd][3]);
         }
       }
@@ -892,7 +921,11 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           const float ww = __shfl_sync(0xffffffffu, wgt, g * 4 + w);
 #pragma unroll
           for (int e = 0; e < PER2; ++e) {
-            const float2 x = *reinterpret_cast<const float2*>(cbuf + w * comb_w + 16 + g * D + 2 * lane + 64 * e);
+            float2 x = *reinterpret_cast<const float2*>(cbuf + w * comb_w + 16 + g * D + 2 * lane + 64 * e);
+            if (GEO::THREE && !WIDE) {
+              const float2 y = *reinterpret_cast<const float2*>(cbuf + w * comb_w + 16 + (g + G) * D + 2 * lane + 64 * e);
+              x.x += y.x; x.y += y.y;
+            }
             acc[e].x += ww * x.x; acc[e].y += ww * x.y;
           }
         }
