@@ -41,20 +41,17 @@ constexpr int SEL_NW = SEL_T / 32;
 constexpr int SEL_CAP = 5120;        // candidate tokens whose scores (both views) are kept in shared memory, at most
 constexpr int CT = 256;              // threads of the compaction kernel
 constexpr int CMP_SHRINK = 1 << 30;       // flag on a compressing request's boundary index: the action is a Shrink
+constexpr int CMP_LOG = 16;               // ... and from this bit on log2 of the slots of a ticket
+static_assert(GP_MAX_REQ <= 1 << CMP_LOG, "a boundary index fits below");
 
 __device__ __forceinline__ unsigned long long to_fix(double a) {
   return (unsigned long long)__double2ll_rn(a * TWO62);
 }
 
-// Compaction tickets of a unit that keeps n_end slots, in parts of `most` slots at most (test support: see GP_WITHHOLD_CHUNK), and the
-// slots of each: equal shares in whole tiles.  The last one has what lies behind them as well.
-__device__ __forceinline__ int parts_of(const GpDev& p, int n_end, int most) {
-  if (p.withhold & GP_TEST_COMPACT_BY_UNIT) return 1;
-  if (p.withhold & (GP_WITHHOLD_CHUNK | GP_TEST_COMPACT_BY_PART)) most = GP_PART_MIN;
-  return (n_end + most - 1) / most;
-}
-__device__ __forceinline__ int part_slots_of(int n_end, int n_part) {
-  return (n_end / GP_PAGE + n_part - 1) / n_part * GP_PAGE;
+// log2 of the slots of a compaction ticket (test support: see GP_WITHHOLD_CHUNK).  A unit's last ticket has what lies behind its new end too.
+__device__ __forceinline__ int part_log_of(const GpDev& p, int want) {
+  if (p.withhold & GP_TEST_COMPACT_BY_UNIT) return GP_PART_LOG_UNIT;
+  return (p.withhold & (GP_WITHHOLD_CHUNK | GP_TEST_COMPACT_BY_PART)) ? GP_PART_LOG_MIN : want;
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -148,7 +145,6 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
     int n_cmp = 0, chunks = 0;
     unsigned long long grow = 0, comp = 0, fall = 0, stall = 0, cow = 0, scored = 0, shr = 0;
     const int sub = p.sub;
-    int copies = 0;                                      // tiles per (layer, KV head) that pass 2 may have copied
     for (int k = 0; k < n_bnd; ++k) {                    // pass 1: grants, ascending request id
       const int e = s_order[k];
       const int r = s_req[e], Pr = s_P[e], bi = s_bi[e];
@@ -169,15 +165,13 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
         report(bi, r, GP_ACT_STALLED);
         s_want[e] |= 4;
         ++stall;
-      } else {
-        copies += s_ksh[e];
       }
     }
+    int copies = -1;                                     // tiles per (layer, KV head) that this pass may have copied
     // Units whose pages are shared are copied tile by tile, 8 KB each at d = 128.  Where they are too few for the grid (one has more than
-    // twice a thread block's even share of the tiles) they are cut into parts of a quarter of that share, of eight tiles at least.  Requests of
-    // 2048 tokens that share a prompt, us of the step in which all are copied, by units / cut (one layer, 8 KV heads): 2 requests
-    // 127 / 88, 4 148 / 106, 8 173 / 141, 16 227 / 214; cut all the same: 32 312 / 320, 4 layers x 16 494 / 519.
-    const float copy_share = (float)copies * p.copy_share;
+    // twice a thread block's even share of the tiles) they are cut into parts of about a quarter of that share, of eight tiles at least.
+    // Requests of 2048 tokens that share a prompt, us of the step in which all are copied, by units / cut (one layer, 8 KV heads): 2 requests
+    // 127 / 88, 4 148 / 106, 8 173 / 141, 16 227 / 211; cut all the same: 32 312 / 320, 4 layers x 16 494 / 519.
     for (int k = 0; k < n_bnd; ++k) {                    // pass 2: copy-on-write targets
       const int e = s_order[k];
       if (s_want[e] & 6) continue;
@@ -191,9 +185,18 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
       top -= s_ksh[e];
       cow += s_ksh[e];
       const bool shrink = (s_want[e] & 16) != 0;
-      p.cmp_info[n_cmp] = make_int4(r, s_P[e], e | (shrink ? CMP_SHRINK : 0), chunks);
-      chunks += parts_of(p, (s_P[e] - (shrink ? 2 : 1) * sub) * GP_PAGE,
-                         s_ksh[e] > 2.f * copy_share && s_ksh[e] > 8 ? (int)fmaxf(8.f, 0.25f * copy_share) * GP_PAGE : GP_PART_SLOTS);
+      int log = GP_PART_LOG;
+      if (s_ksh[e] > 8) {
+        if (copies < 0) {
+          copies = 0;
+          for (int f = 0; f < n_bnd; ++f) copies += (s_want[f] & 6) ? 0 : s_ksh[f];
+        }
+        const float share = (float)copies * p.copy_share;
+        if ((float)s_ksh[e] > 2.f * share) log = min(log, max(7, 33 - __clz((int)(1.5f * share))));
+      }
+      log = part_log_of(p, log);
+      p.cmp_info[n_cmp] = make_int4(r, s_P[e], e | log << CMP_LOG | (shrink ? CMP_SHRINK : 0), chunks);
+      chunks += ((s_P[e] - (shrink ? 2 : 1) * sub) * GP_PAGE + (1 << log) - 1) >> log;
       ++n_cmp;
       if (s_want[e] & 1) { report(bi, r, GP_ACT_COMPRESS_FALLBACK); ++fall; }
       else if (shrink) { report(bi, r, GP_ACT_SHRINK); ++shr; }
@@ -1067,10 +1070,10 @@ __device__ __forceinline__ int warp_pack(int n, int* out, F flag) {
 // rows, stores), three thread blocks to an SM.  Every row behind the first evicted slot moved down (in 64-slot chunks that waited for one
 // another where units were few): 467 us at 36 layers x 256 requests, now 73; 53, now 12, at 36 x 16; 187, now 26, at 64 x 32; the
 // one-layer step of 64 requests 74.8 us, now 70.1.
-// A ticket is a unit, or, where a unit has more than GP_PART_SLOTS slots or is copied with few others, a part of one: a part tells where its evicted slots lie, and
-// the unit's last part, which waits for that word of the others, moves the rows.  Tickets come from a counter, in order, so that those
-// of a unit's other parts are with CTAs that run or have ended; only where every unit is one ticket, and none waits, a CTA's first is its
-// number, which saves a round trip.
+// A ticket is a unit, or, where a unit has more than 4096 slots or is copied with few others, a part of one: a part tells where its
+// evicted slots lie, and the unit's last part, which waits for that word of the others, moves the rows.  Tickets come from a counter, in
+// order, so that those of a unit's other parts are with CTAs that run or have ended; only where every unit is one ticket, and none waits,
+// a CTA's first is its number, which saves a round trip.
 template <int D>
 __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, int serial) {
   constexpr int CH = D / 8;
@@ -1111,18 +1114,18 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (LH * s_info[mid].w <= item) lo = mid; else hi = mid; }
     const int n_part = s_info[lo + 1].w - s_info[lo].w;
     const int rem = item - LH * s_info[lo].w;
-    const int lh = rem / n_part, part = rem % n_part;
+    int lh = rem, part = 0;
+    if (n_part > 1) { lh = rem / n_part; part = rem - lh * n_part; }
     const int4 inf = s_info[lo];
     const int l = lh / p.Hkv, h = lh % p.Hkv;
     const int Pr = inf.y;
     const int* table = p.page_table + (size_t)inf.x * p.cap;
     const int* shadow = p.shadow + (size_t)inf.x * p.cap;
     const bool shrink = (inf.z & CMP_SHRINK) != 0;
-    const int e_bnd = inf.z & (CMP_SHRINK - 1);
+    const int e_bnd = inf.z & ((1 << CMP_LOG) - 1), log = (inf.z & (CMP_SHRINK - 1)) >> CMP_LOG;
     const int ne = shrink ? 2 * p.blk : p.blk;             // slots freed: one page of the method, two at a Shrink
     const int n_src = Pr * GP_PAGE, n_end = n_src - ne;    // the unit's slots, and those that stay in use
-    const int part_slots = part_slots_of(n_end, n_part);
-    const int c0 = part * part_slots, c1 = part == n_part - 1 ? n_src : c0 + part_slots;
+    const int c0 = part << log, c1 = part == n_part - 1 ? n_src : c0 + (1 << log);
     // order indices of a page's slots, and its rows: the unit's place in a page
     const size_t tok_stride = (size_t)p.Hkv * GP_PAGE, tok_base = gp_tok_off(p, l, 0, h);
     const size_t page_stride = (size_t)p.Hkv * 2 * GP_PAGE * ROW_BYTES;

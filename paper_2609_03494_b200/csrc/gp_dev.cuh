@@ -28,8 +28,9 @@
 #define GP_MAX_TILES_PER_REQ 61773   // 16-token tiles a request may hold: the selection keeps a bit per candidate in shared memory
 #define GP_SPIN_LIMIT (1u << 21)
 #define GP_MAX_REQ 1024        // upper limit of max_requests (shared-memory arrays are sized by it)
-#define GP_PART_SLOTS 4096     // slots per compaction ticket: units beyond that are shared out (a unit of 20 000 slots in one block: 15 us of loads)
-#define GP_PART_MIN 64         // ... in tests
+#define GP_PART_LOG 12         // 4096 slots per compaction ticket: units beyond that are shared out (a unit of 20 000 slots in one block: 15 us of loads)
+#define GP_PART_LOG_MIN 6      // ... 64 in tests
+#define GP_PART_LOG_UNIT 20    // ... and no bound (GP_MAX_TILES_PER_REQ tiles)
 #define GP_COST_BINS 160       // cost classes of attention work items: pages, from the middle on those of requests at a boundary
 #define GP_DESC_INTS 16        // ints per attention work descriptor
 #define GP_ATTN_CONSUMERS 4    // consumer warps of an attention thread block: each reports once per item it worked on
@@ -54,11 +55,11 @@ enum {
 // hand-overs a test can withhold (gp_test_withhold): the bounded wait for it then runs out
 enum {
   GP_WITHHOLD_ITEM = 1,     // attention kernel, first CTA: its second work item is never published to the consumers
-  GP_WITHHOLD_CHUNK = 2,    // compaction, in parts of GP_PART_MIN slots: the first part of a unit never says where its evicted slots lie
+  GP_WITHHOLD_CHUNK = 2,    // compaction, in parts of 64 slots: the first part of a unit never says where its evicted slots lie
   GP_WITHHOLD_DECIDED = 4,  // boundary kernel: the deciding CTA never tells the others
   GP_WITHHOLD_READY = 8,    // attention kernel: the consumer warps never report a boundary unit's logits complete
   GP_TEST_COMPACT_BY_UNIT = 16,   // (not withheld hand-overs) the compaction claims whole units whatever their size,
-  GP_TEST_COMPACT_BY_PART = 32,   // ... parts of GP_PART_MIN slots
+  GP_TEST_COMPACT_BY_PART = 32,   // ... parts of 64 slots
 };
 
 // error bits

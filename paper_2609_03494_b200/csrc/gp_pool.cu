@@ -169,7 +169,7 @@ Layout make_layout(const gp_config& c) {
   L.zstat = take(LH * (Tb / b + 1) * 2 * G * 2 * 8);
   L.evict = take(M * LH * blk * 4);
   L.evict2 = take(c.policy == GP_POLICY_SHRINK ? M * LH * 2 * blk * 4 : 16);
-  L.cflags = take(LH * ((Tb + M * b) / GP_PART_MIN + 2 * M + 1) * 4);
+  L.cflags = take(LH * ((Tb + M * b) / (1 << GP_PART_LOG_MIN) + 2 * M + 1) * 4);
   L.inv_freq = take(d / 2 * 8);
   L.tickets = take((size_t)c.n_layers * 2 * 4);
   L.rope_f = take(M * (d / 2) * 2 * 4);
