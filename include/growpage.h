@@ -349,11 +349,11 @@ int gp_debug_request(gp_pool* pool, int32_t req, int32_t* P, int32_t* n, int64_t
  * NULL); slots that are not live read 0. */
 int gp_debug_state(gp_pool* pool, int32_t* P, int32_t* n);
 
-/* Original token index of every occupied slot of one (layer, KV head) stream, in slot order:
- * host int32 [n].  This is the retained-index set of Sec. 3.3. */
+/* Original token index of every occupied slot of one (layer, KV head) stream, in the order of the
+ * tokens (ascending; where a row lies in its pages is not part of it): host int32 [n].  This is the retained-index set of Sec. 3.3. */
 int gp_debug_retained(gp_pool* pool, int32_t req, int32_t layer, int32_t kv_head, int32_t* token_ids);
 
-/* K and V rows of the occupied slots of one (layer, KV head) stream in slot order:
+/* K and V rows of the occupied slots of one (layer, KV head) stream in the same order:
  * host bf16 [n][d] each (either may be NULL). */
 int gp_debug_kv(gp_pool* pool, int32_t req, int32_t layer, int32_t kv_head, void* k_rows, void* v_rows);
 
@@ -371,7 +371,8 @@ int gp_debug_entropy(gp_pool* pool, int32_t req, double* H_S, double* H_L);
 /* Free pages, per-page reference counts (host int32 [n_pages], may be NULL) and event counters:
  * [0] grow [1] compress [2] fallback-compress [3] stalled [4] copy-on-write pages
  * [5] decode steps [6] tokens decoded [7] internal error bits (0 when healthy)
- * [8] (layer, head, token) rows rewritten by compaction [9] candidate tokens scored at boundaries
+ * [8] retained (layer, head, token) rows whose place in the order of the tokens a compaction changed, or
+ * that it copied (of the former it moves a page per unit at most) [9] candidate tokens scored at boundaries
  * [10] Shrink events (not counted under [1]) [11] reserved. */
 int gp_debug_pool(gp_pool* pool, int64_t* n_free, int32_t* refcounts, int64_t counters[12]);
 

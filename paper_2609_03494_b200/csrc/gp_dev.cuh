@@ -67,7 +67,7 @@ enum {
   GP_E_SPIN = 1,        // a bounded wait gave up
   GP_E_FREELIST = 2,    // free-list accounting went negative or overflowed
   GP_E_BOUNDS = 4,      // an index failed a bounds check and the access was skipped
-  GP_E_SPIN_CMP = 8,    // the compaction kernel's bounded wait on the previous chunk gave up
+  GP_E_SPIN_CMP = 8,    // the bounded wait for a unit's other compaction parts, or for the step's decisions, gave up
   GP_E_SPIN_SEL = 16,   // a selection job's bounded wait for its unit's summary logits gave up
 };
 
@@ -136,8 +136,8 @@ struct GpDev {
   long long z_stride;                    // max_boundary_tokens rounded up to a multiple of the page size
   double* zstat;                         // [L*H_kv][max_boundary_tokens / b][2][G][2] per-page softmax partials (max, sum)
   int* sum_par;                          // [M] which of the two summary buffers is current
-  int* evict;                            // [M][L*H_kv][page_size] slots a compression evicts, ascending
-  int* evict2;                           // [M][L*H_kv][2 page_size] slots a Shrink evicts, ascending (Shrink policy only)
+  int* evict;                            // [M][L*H_kv][page_size] places in the order of the tokens that a compression evicts, ascending
+  int* evict2;                           // [M][L*H_kv][2 page_size] ... that a Shrink evicts (Shrink policy only)
   int* cflags;                           // compaction part flags, stamped with the step number
   int* tickets;                          // [L][2] next attention work item to draw, per list: of the whole step (0) or of a layer's launch
   double* inv_freq;                      // [d/2] rope_theta^(-2j/d)
