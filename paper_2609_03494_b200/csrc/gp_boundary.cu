@@ -1336,8 +1336,8 @@ gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_
   // Synchronous mode (same_step): the chain belongs to the step whose attention kernel runs beside this grid.
   // A selection job then waits until the consumer warps of that kernel have reported the unit's summary logits
   // complete (the items of requests at their boundary are a list of their own there, which a part of its grid draws
-  // from first), the decisions are reported through `actions` as usual, and the next kernel on the stream may only be scheduled once the attention kernel has
-  // ended (its early part reads counters that kernel advances).
+  // from first), the decisions are reported through `actions` as usual, and the next kernel on the stream may only be
+  // scheduled once the attention kernel has ended (its early part reads counters that kernel advances).
   const bool same_step = !p.async;
   if (!same_step) gp_pdl_launch_dependents();
   if (has_chain) {
