@@ -413,8 +413,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   // its stream, and that one waited for the plan before it let this one be scheduled.  Then only the caller's tensors depend on the
   // kernel before this one: descriptor, page ids, the first tiles and the old summaries are asked for while that kernel drains, and
   // the producer waits before it asks for the first rows.  Whatever is written follows those rows.  (36 layers x 16 requests of 400 to 1000
-  // tokens, layer by layer: 864 us per step with every launch waiting at its top, now 760.  In the whole step's kernel the rows share
-  // the descriptor's barrier: two barriers there cost 1 to 2 %.)
+  // tokens, layer by layer: 864 us per step with every launch waiting at its top, now 760; with an ordinary kernel of 3 us before each
+  // layer 999, now 925.  In the whole step's kernel the rows share the descriptor's barrier: two barriers there cost 1 to 2 %.)
   constexpr bool LAYER = MODE != WHOLE_STEP, NORM = MODE == ONE_LAYER_NORM;
   using GEO = Geo<D>;
   extern __shared__ uint8_t smem_raw[];

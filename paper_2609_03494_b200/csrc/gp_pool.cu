@@ -14,6 +14,7 @@
 #define GP_PLAN_THREADS 1024       // threads of the plan kernel for batches of up to GP_MAX_REQ requests (a thread each) ...
 #define GP_PLAN_SMALL 256          // ... and for batches of up to this many: its time is block barriers, which 8 warps pass faster than 32
 #define PLAN_STATES 512            // requests of a pool whose counters the plan kernel reads ahead (8 KB: it starts beside the boundary kernel)
+enum { LAUNCH_RUNS = 1, LAUNCH_CAPTURED = 2 };     // a launch now, or one into the graph that its stream is captured into
 #define GP_NEVER (-(1 << 30))      // bstep of a request that has not reached a boundary
 
 struct gp_pool {
@@ -34,7 +35,8 @@ struct gp_pool {
   int num_sms, attn_grid, sel_grid, compact_grid;
   int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
-  int plain_plan;                                   // a request was released or a step abandoned since the last plan, whose counters or items its kernels may still change
+  int plain_plan;                                   // a request was released or a step abandoned since the last plan: the next launch
+                                                    // of one that runs (LAUNCH_RUNS) or is captured (LAUNCH_CAPTURED) waits for it
   std::vector<uint8_t> step_layer_seen;             // layers gp_attn_layer has run in the open step
   cudaStream_t layer_stream;                        // stream of the last of them
   // error bits set by the kernels (GP_E_*): one int of page-locked host memory that the device addresses directly,
@@ -848,6 +850,12 @@ int gp_pool_destroy(gp_pool* pool) {
   return GP_OK;
 }
 
+static int launch_kind(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) (void)cudaGetLastError();      // (the legacy stream beside a capture: runs)
+  return st == cudaStreamCaptureStatusNone ? LAUNCH_RUNS : LAUNCH_CAPTURED;
+}
+
 int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, const void* k_tail, const void* v_tail,
                    int32_t n_tail, int32_t initial_pages, void* stream, int32_t* out_req) {
   if (!pool || !out_req || n_tail < 0 || n_shared_pages < 0 || initial_pages < 0) return GP_ERR_INVALID;
@@ -906,7 +914,10 @@ static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_
   const GpDev& d = dev ? *dev : pool->dev;
   const int threads = n_req <= GP_PLAN_SMALL ? GP_PLAN_SMALL : GP_PLAN_THREADS;
   const int table = d.rope_theta != 0.0 ? (n_req * (d.d / 2) + threads - 1) / threads : 0;
-  if (pool->plain_plan) { early = false; pdl = false; pool->plain_plan = 0; }
+  if (pool->plain_plan) {
+    const int mine = launch_kind(s);
+    if (pool->plain_plan & mine) { early = false; pdl = false; pool->plain_plan &= ~mine; }
+  }
   gp_launch(gp_plan_kernel, 1 + table, threads, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
             by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff));
 }
@@ -1116,7 +1127,7 @@ int gp_step_abort(gp_pool* pool) {
   // Nothing of an open step is committed before gp_step_end: the requests' counters are untouched, rows appended
   // by the layers that ran lie beyond the occupied slots, and the summaries went to the buffer not in use.
   pool->step_open = 0;
-  pool->plain_plan = 1;
+  pool->plain_plan = LAUNCH_RUNS | LAUNCH_CAPTURED;
   return GP_OK;
 }
 
@@ -1344,7 +1355,7 @@ int gp_release(gp_pool* pool, int32_t req, void* stream) {
   if (flush_chain(pool, static_cast<cudaStream_t>(stream)) != GP_OK) return GP_ERR_CUDA;
   gp_release_kernel<<<1, ADMIT_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(pool->dev, req);
   pool->launch_count++;
-  pool->plain_plan = 1;
+  pool->plain_plan |= launch_kind(static_cast<cudaStream_t>(stream));
   pool->live[req] = 0;
   GP_CUDA(cudaGetLastError());
   return GP_OK;

@@ -204,8 +204,14 @@ def test_a_request_released_right_before_a_step_is_invalid_in_it(overlap, early)
         acts = torch.zeros((n_req, n_req), dtype=torch.int32, device="cuda")
         torch.cuda.synchronize()
         order = [int(x) for x in rng.permutation(n_req)]
+        graph, side, captured = torch.cuda.CUDAGraph(), torch.cuda.Stream(), torch.zeros_like(acts[0])
         for t in range(n_req):
             pool.release(order[t])
+            if t == n_req // 2:                              # a step that is only captured does not stand between release and step
+                with torch.cuda.stream(side):
+                    graph.capture_begin(capture_error_mode="thread_local")
+                    pool.decode_step(ids, q, k, v, out, captured)
+                    graph.capture_end()
             pool.decode_step(ids, q, k, v, out, acts[t])
         torch.cuda.synchronize()
         got = acts.cpu().numpy()
