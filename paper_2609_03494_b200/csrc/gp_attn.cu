@@ -51,6 +51,7 @@ constexpr int NSUM = 2;                    // summary warps
 constexpr int MERGE_FAN = 8;               // partial outputs merged at a time
 constexpr double QT_SCALE = 0x1p880;       // of the q~ buffer: see bf16_lo_scaled
 constexpr double Z_SCALE = 0x1p16;         // of the logits made from it
+constexpr int SLOT_UNIT = 20;              // of an item's slot: offset of the unit's tile of page 0 (two words)
 constexpr int QT_PAD = 8;                  // doubles of padding per q~ row: rows alternate bank halves
 
 template <int D>
@@ -456,10 +457,16 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   // the descriptor of the item of this CTA's own number, which its first one nearly always is, is fetched before the numbers of items
   // are known (same round trip): a slot past them holds stale but readable data that is then not used
   int hFirst = 0;
-  if (warp == 0 && lane < GP_DESC_INTS && (int)(blockIdx.x / lh_n) < p.max_rc) hFirst = p.rcx[(size_t)(blockIdx.x / lh_n) * GP_DESC_INTS + lane];
+  // What runs once before the first tile is paid in instruction fetch: the numbers of items in 32 bits (their 64-bit quotients were calls of a
+  // hundred instructions), a unit's layer and head worked out by the producer alone (us a pass with the tiles' addresses as they are: tiny, 16
+  // steps, 286 / 279; 36 x 16 layer by layer, 4 steps, 3040 / 3000; 1 x 64, 16 steps, 1085 / 1074).
+  const unsigned units = (unsigned)lh_n;
+  unsigned rc = blockIdx.x / units;            // the item's descriptor
+  if (warp == 0 && lane < GP_DESC_INTS && (int)rc < p.max_rc) hFirst = p.rcx[(size_t)rc * GP_DESC_INTS + lane];
   const int n_rc = __ldcg(p.hdr + HDR_N_RC), n_brc = __ldcg(p.hdr + HDR_N_BRC);
   const int LH = p.L * p.Hkv;
-  const long long total_b = (long long)n_brc * lh_n, total = (long long)n_rc * lh_n;
+  // (32 bits: every item has a partial output of 264 bytes or more in the pool)
+  const int total_b = n_brc * lh_n, total = n_rc * lh_n;
   const int q_bytes = G * GEO::ROW_BYTES;
 
   if (warp < 4) {
@@ -480,14 +487,17 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
     // left goes to whoever is free.  (Dealt out statically by an estimate of their cost, the CTAs of a one-layer step ended
     // between 26 and 38 us; drawn as far ahead as a ring of eight slots allows, they hoarded.)  Which CTA takes an item does
     // not change its result.
-    const long long total_p = total - total_b, cta = blockIdx.x, grid = gridDim.x;
-    const long long b_ctas = total_b <= grid / 2 ? total_b : grid / 3;      // blocks that draw boundary items first
-    const long long first_p = min(total_p, grid - b_ctas), first_b = min(total_b, grid - first_p);
+    const int total_p = total - total_b, cta = blockIdx.x, grid = gridDim.x;
+    const int b_ctas = total_b <= grid / 2 ? total_b : grid / 3;      // blocks that draw boundary items first
+    const int first_p = min(total_p, grid - b_ctas), first_b = min(total_b, grid - first_p);
     // an item's number: of the first list, then of the second
-    long long item = cta < b_ctas ? cta : cta - b_ctas < first_p ? total_b + cta - b_ctas : cta - first_p < first_b ? cta - first_p : total;
+    int item = cta < b_ctas ? cta : cta - b_ctas < first_p ? total_b + cta - b_ctas : cta - first_p < first_b ? cta - first_p : total;
     bool left[2] = {true, true};               // items of the lists this CTA still asks for
     int hdr = hFirst;                          // descriptor header, word `lane` (lanes 0..15)
-    if (item != cta && item < total && lane < GP_DESC_INTS) hdr = p.rcx[(size_t)(item / lh_n) * GP_DESC_INTS + lane];
+    if (item != cta && item < total) {
+      rc = (unsigned)item / units;
+      if (lane < GP_DESC_INTS) hdr = p.rcx[(size_t)rc * GP_DESC_INTS + lane];
+    }
     for (uint32_t n = 0;; ++n) {
       const int sl = n % NI;
       if (!wait_bar(&slot_empty[sl], ((n / NI) & 1u) ^ 1u, s_misc, 1, lim)) break;
@@ -504,8 +514,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
         }
         break;
       }
-      const int lh = lh0 + (int)(item % lh_n);
-      const int l = lh / p.Hkv, h = lh % p.Hkv;
+      const int lh = lh0 + item - (int)(rc * units);
+      const int l = (int)((unsigned)lh / (unsigned)p.Hkv), h = lh - l * p.Hkv;
       const int bi = __shfl_sync(0xffffffffu, hdr, 0);
       const int r = __shfl_sync(0xffffffffu, hdr, 1), pg0 = __shfl_sync(0xffffffffu, hdr, 2);
       const int npg = __shfl_sync(0xffffffffu, hdr, 3);
@@ -517,7 +527,9 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       if (lane < 14) sd[lane] = hdr;
       if (lane == 14) sd[14] = lh;
       if (lane == 15) sd[15] = hdr;            // index among the step's boundary requests
-      if (lane == 16) sd[16] = (int)(item & (NCW - 1));       // the consumer warp that takes the item's first tile
+      if (lane == 16) sd[16] = item & (NCW - 1);              // the consumer warp that takes the item's first tile
+      if (lane == 17) sd[17] = l;
+      if (lane == 18) sd[18] = h;
       __syncwarp();
       auto ask_rows = [&]() {
         const bool has_new = (chunk == nchunks - 1);
@@ -533,6 +545,8 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
         }
       };
       if (lane == 0 && !rows_later) ask_rows();
+      if (lane == 0)                                         // the unit's place in a page, in bytes from the first layer's first page
+        *reinterpret_cast<unsigned long long*>(sd + SLOT_UNIT) = gp_tile_off(p, l, 0, h) * sizeof(__nv_bfloat16);
       sd[GEO::SLOT_PAGES + lane] = pg;
       sd[GEO::SLOT_PAGES + 32 + lane] = pg2;
       __syncwarp();
@@ -553,12 +567,15 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
         if (item < total || !left[list]) continue;
         int t = 0;
         if (lane == 0) t = atomicAdd(p.tickets + 2 * (lh0 / p.Hkv) + list, 1);
-        const long long at = (list ? first_p : first_b) + __shfl_sync(0xffffffffu, t, 0);
+        const int at = (list ? first_p : first_b) + __shfl_sync(0xffffffffu, t, 0);
         left[list] = at < (list ? total_p : total_b);
         if (left[list]) item = list ? total_b + at : at;
       }
       hdr = 0;
-      if (item < total && lane < GP_DESC_INTS) hdr = p.rcx[(size_t)(item / lh_n) * GP_DESC_INTS + lane];
+      if (item < total) {
+        rc = (unsigned)item / units;
+        if (lane < GP_DESC_INTS) hdr = p.rcx[(size_t)rc * GP_DESC_INTS + lane];
+      }
     }
   } else if (warp >= 4) {
     // ================================= consumers ==========================================
@@ -579,7 +596,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
     const uint64_t kv_policy = l2_policy_evict_first();    // the K/V stream is read once per step: first out of the L2
     constexpr int PAIR = GEO::PAIR;
     uint32_t my_fetch = 0, f_it = 0;
-    int f_pgl = 0, f_npg = 0, f_lh = 0;
+    int f_pgl = 0, f_npg = 0;
     bool f_have = false, f_done = false;
     auto top_up = [&](uint32_t it_now) -> bool {           // false: a wait gave up
       while (!f_done && my_fetch - my_tiles < (uint32_t)NSW) {
@@ -595,7 +612,6 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           }
           f_npg = fsd[3];
           if (f_npg < 0) { f_done = true; break; }
-          f_lh = fsd[14];
           f_pgl = (cw + fsd[16]) % NCW;                   // in units of PAIR tiles; the first goes to another warp from item to item
           f_have = true;
         }
@@ -607,7 +623,13 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           const int page = fsd[GEO::SLOT_PAGES + f_pgl * PAIR + sub];
           // 16-byte asynchronous copies through the load/store path, 512 contiguous bytes per warp instruction:
           // the bulk-copy engine takes several hundred cycles to accept an 8 KB copy, which paced the kernel
-          const uint8_t* src = reinterpret_cast<const uint8_t*>(p.kv + gp_tile_off(p, f_lh / p.Hkv, page, f_lh % p.Hkv)) + lane * 16;
+          // A fetch is a third of what a tile costs a consumer warp (cycles, one request alone: fetch 530, S 290, softmax 300, weights and
+          // P V 310, the rest 250), so the unit's place is in the slot: with the unit's layer and head taken apart here by divisions, per
+          // fetch, it was that; now 390, and no register more is held through the loop and the logits (kept in registers it cost
+          // groups of eight 5 % of a step in spills).  us of this kernel before / now: 64 layers x 32 requests, groups of eight, none and two at a
+          // boundary 1345 / 1328 and 1741 / 1659; 36 x 256, 16 at a boundary 3941 / 3763; 36 x 16, two 285 / 280.
+          const uint8_t* src = reinterpret_cast<const uint8_t*>(p.kv) + *reinterpret_cast<const unsigned long long*>(fsd + SLOT_UNIT) +
+                               (uint64_t)(uint32_t)page * ((uint32_t)p.Hkv * GEO::TILE_BYTES) + lane * 16;
           const uint32_t dst = smem_u32(smem + fst * GEO::STAGE_BYTES + sub * GEO::TILE_BYTES) + lane * 16;
 #pragma unroll
           for (int c = 0; c < GEO::TILE_BYTES / 512; ++c) cp_async16_hint(dst + c * 512, src + c * 512, kv_policy);
@@ -628,7 +650,6 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       if (npg < 0) break;
       const int bi = sd[0], pg0 = sd[2], chunk = sd[4], nchunks = sd[5], n_old = sd[6];
       const int flags = sd[8], Pr = sd[9], lh = sd[14];
-      const int l = lh / p.Hkv, h = lh % p.Hkv;
       const int n_new = n_old + 1;
       const bool need_qt = (flags & 1) && (pg0 < Pr - 1);
 
@@ -691,7 +712,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           uint8_t* tile = stage + (nsub - 1) * GEO::TILE_BYTES;
           // append: slot n_old of this page receives k_t, v_t; patch the staged copy too
           const int s = n_old - tok0 - (nsub - 1) * GP_PAGE;
-          const int page = sd[GEO::SLOT_PAGES + npg - 1];
+          const int page = sd[GEO::SLOT_PAGES + npg - 1], l = sd[17], h = sd[18];
           constexpr int CH = D / 8;
           uint4 k_new = make_uint4(0, 0, 0, 0);
           if (NORM) {
@@ -891,7 +912,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const int npg = sd[3];
       if (npg < 0) break;
       const int bi = sd[0], chunk = sd[4], nchunks = sd[5], rc_i = sd[13], lh = sd[14];
-      const int l = lh / p.Hkv, h = lh % p.Hkv;
+      const int l = sd[17], h = sd[18];
       const int cb = it % NCOMB;
       if (!wait_bar(&comb_full[cb], (it / NCOMB) & 1u, s_misc, 8, lim)) break;
       const float* cbuf = comb + (size_t)cb * NCW * comb_w;
@@ -980,7 +1001,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       const bool need_qt = (flags & 1) && sd[2] < sd[9] - 1;
       if (NORM || owner || need_qt) {
         if (need_qt && !wait_bar(qt_empty, (qt_uses & 1u) ^ 1u, s_misc, 10, lim)) break;
-        const int l = lh / p.Hkv, h = lh % p.Hkv;
+        const int l = sd[17], h = sd[18];
         auto rows_there = [&]() { return !LAYER || wait_bar(&slot_rows[sl], (it / NI) & 1u, s_misc, 13, lim); };
         if (!summary_rows<D, ROPE, NORM>(p, nm, slot + GEO::SLOT_DESC, rows_there, &slot_norm[sl], w, G, l, h, r, bi, par, (flags & 2) != 0, owner,
                                          need_qt ? qt : nullptr)) break;
