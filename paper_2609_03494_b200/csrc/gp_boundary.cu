@@ -30,6 +30,12 @@
 // scores differ, until the bin with the crossing point holds at most 32 scores, which one warp sorts.  The top-p mass
 // is accumulated in 2^62 fixed point with integer atomics, so the result does not depend on the order in which
 // threads add.
+//
+// Size of the code: a step of a few units runs these functions once per thread block, and what they then cost is the fetch of their
+// instructions.  So loops whose trips are not the point are kept from being unrolled (`unroll 1`; the compiler unrolled the loop over the two
+// supports, and the decisions' loops four to eight times): gp_chain_kernel<128, 4> 258 -> 170 KB, the compaction 62 -> 52, the decisions
+// 26 -> 17.  us a pass before / now: one layer x 64 requests, 16 steps, 1067 / 1039; four requests, 16 steps, 267 / 259; 256 requests copied
+// on write in one of 24 steps 14 315 / 13 979; 36 layers x 16, 16 steps, 4912 / 4897.
 #include "../../include/growpage.h"
 #include "gp_dev.cuh"
 
@@ -81,6 +87,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
   int top0 = 0;
   if (n_bnd > 0) {
     top0 = p.async ? __ldcg(p.free_top) : __ldcg(p.free_peek);
+#pragma unroll 1
     for (int e = tid; e < n_bnd; e += blockDim.x) {
       const int4 inf = p.bnd_info[2 * e], inf2 = p.bnd_info[2 * e + 1];
       int4 acc = __ldcg(reinterpret_cast<const int4*>(p.bnd_acc) + e);
@@ -97,6 +104,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
           // the same mean with H / ln |C| in the place of K / |C|, summed unit by unit in (layer, head) order
           const double* hx = p.Hx + (size_t)r * LH * 2;
           double accd = 0.0;
+#pragma unroll 1
           for (int u2 = 0; u2 < LH; ++u2) accd += __ldcg(hx + 2 * u2) - __ldcg(hx + 2 * u2 + 1);
           delta = nC > 1 ? accd / ((double)LH * log((double)nC)) : 0.0;
         }
@@ -130,8 +138,10 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
   }
   if (n_bnd == 0) return;
   __syncthreads();
+#pragma unroll 1
   for (int e = tid; e < n_bnd; e += blockDim.x) {
     int rank = 0;
+#pragma unroll 2
     for (int f = 0; f < n_bnd; ++f) rank += (s_req[f] < s_req[e]);
     s_order[rank] = e;
   }
@@ -145,12 +155,14 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
     int n_cmp = 0, chunks = 0;
     unsigned long long grow = 0, comp = 0, fall = 0, stall = 0, cow = 0, scored = 0, shr = 0;
     const int sub = p.sub;
+#pragma unroll 1
     for (int k = 0; k < n_bnd; ++k) {                    // pass 1: grants, ascending request id
       const int e = s_order[k];
       const int r = s_req[e], Pr = s_P[e], bi = s_bi[e];
       scored += (unsigned long long)(Pr - sub) * GP_PAGE;
       if ((s_want[e] & 1) && Pr + sub <= p.cap && top >= sub) {
         // one page of the method: `sub` tiles from the top of the free list
+#pragma unroll 1
         for (int t = 0; t < sub; ++t) {
           const int page = (sub == 1 && !p.async) ? s_free[top0 - top] : p.free_stack[top - 1];
           --top;
@@ -172,6 +184,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
     // twice a thread block's even share of the tiles) they are cut into parts of about a quarter of that share, of eight tiles at least.
     // Requests of 2048 tokens that share a prompt, us of the step in which all are copied, by units / cut (one layer, 8 KV heads): 2 requests
     // 127 / 88, 4 148 / 106, 8 173 / 141, 16 227 / 211; cut all the same: 32 312 / 320, 4 layers x 16 494 / 519.
+#pragma unroll 1
     for (int k = 0; k < n_bnd; ++k) {                    // pass 2: copy-on-write targets
       const int e = s_order[k];
       if (s_want[e] & 6) continue;
@@ -189,6 +202,7 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
       if (s_ksh[e] > 8) {
         if (copies < 0) {
           copies = 0;
+#pragma unroll 1
           for (int f = 0; f < n_bnd; ++f) copies += (s_want[f] & 6) ? 0 : s_ksh[f];
         }
         const float share = (float)copies * p.copy_share;
@@ -224,12 +238,14 @@ __device__ void decide_and_allocate(const GpDev& p, const int* req_ids, int n_re
     atomicAdd(cn + 9, scored);
   }
   __syncthreads();
+#pragma unroll 1
   for (int e = warp; e < n_bnd; e += nwarp) {             // fill in the targets, in table order
     if (!(s_want[e] & 8) || s_ksh[e] == 0) continue;
     const int r = s_req[e], Pr = s_P[e], base = s_base[e];
     const int* table = p.page_table + (size_t)r * p.cap;
     int* shadow = p.shadow + (size_t)r * p.cap;
     int running = 0;
+#pragma unroll 1
     for (int j0 = 0; j0 < Pr - p.sub; j0 += 32) {
       const int j = j0 + lane;
       const bool sh = j < Pr - p.sub && p.refcount[table[j]] > 1;
@@ -277,6 +293,7 @@ __device__ __forceinline__ void column_reduce(double v, int ncols, double* red, 
   __syncthreads();
   if (threadIdx.x < ncols) {
     double r = red[threadIdx.x];
+#pragma unroll 1
     for (int w = 1; w < SEL_T / 32; ++w) r = IS_MAX ? fmax(r, red[w * 16 + threadIdx.x]) : r + red[w * 16 + threadIdx.x];
     result[threadIdx.x] = r;
   }
@@ -399,6 +416,7 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
       if (t < FT) m.F[t * NC + myc] = f;
     }
   }
+#pragma unroll 1
   for (int tb = t0 + KEEP * TSTEP; tb < ntile; tb += 4 * TSTEP) {
     double2 ms[4];
 #pragma unroll
@@ -418,9 +436,11 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
   }
   column_reduce<false>(acc, NC, m.red, m.sZ);
   const double rz = 1.0 / ((double)GG * m.sZ[myc]);        // group mean and normaliser in one factor
+#pragma unroll 1
   for (int t = t0; t < min(ntile, FT); t += TSTEP) m.F[t * NC + myc] *= rz;       // (the thread that wrote the entry)
   __syncthreads();
   unsigned lo_w[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi_w[3] = {0u, 0u, 0u};
+#pragma unroll 1
   for (int tb = 0; tb < ntile; tb += FT) {               // a set of pages whose factors are in shared memory
     const int k_begin = tb * GP_PAGE, k_end = min(n, k_begin + FT * GP_PAGE);
     if (tb) {
@@ -428,10 +448,12 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
       load_order(k_begin);
       load_pages(k_begin + U * SEL_T);
       __syncthreads();
+#pragma unroll 1
       for (int t = tb + t0; t < min(ntile, tb + FT); t += TSTEP)
         m.F[(t - tb) * NC + myc] = exp(__ldcg(zs + ((size_t)t * NC + myc) * 2) - mc) * rz;
       __syncthreads();
     }
+#pragma unroll 1
     for (int k0 = k_begin; k0 < k_end; k0 += U * SEL_T) {
       if (k0 != k_begin) { load(k0, k_end); load_order(k0); load_pages(k0 + U * SEL_T); }
 #pragma unroll
@@ -471,6 +493,7 @@ __device__ __forceinline__ void unit_softmax(const SelSmem& S, const double* __r
 __device__ __forceinline__ void mark_local(const double* aS, const double* aL, int n, int blk, int kq, unsigned* loc, int w, int nw) {
   const int lane = threadIdx.x & 31;
   if (blk == GP_PAGE) {                                   // two blocks to a warp: every score against its block's others
+#pragma unroll 1
     for (int b0 = w * 32; b0 < n; b0 += nw * 32) {
       const int i = b0 + lane;
       const unsigned long long key = i < n ? max(key_of(aS[i]), key_of(aL[i])) : 0ull;
@@ -498,6 +521,7 @@ __device__ __forceinline__ void mark_local(const double* aS, const double* aL, i
   }
   // A warp to a block of 32 to 256: descends the bits of the kq-th largest score, counting with ballots; it may stop
   // where exactly kq scores lie at or above the candidate.
+#pragma unroll 1
   for (int b0 = w * blk; b0 < n; b0 += nw * blk) {
     const int per = blk / 32, have = min(blk, n - b0);
     unsigned long long key[8];
@@ -520,6 +544,7 @@ __device__ __forceinline__ void mark_local(const double* aS, const double* aL, i
 #pragma unroll
       for (int j = 0; j < 8; ++j) top = max(top, (unsigned)(key[j] >> 32));
       top = __reduce_max_sync(0xffffffffu, top);
+#pragma unroll 1
       for (int bit = top ? 63 - __clz((int)top) : 31; bit >= 0 && !exact; --bit) {
         const unsigned long long t = thr | (1ull << bit);
         const int c = count(t);
@@ -588,6 +613,7 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
     // four at a time: their loads, then their adds, in flight together
     const unsigned mask = (1u << width) - 1u;
     if (run && task != 2) {
+#pragma unroll 1
       for (int i0 = gt; i0 < n; i0 += 4 * T) {
         unsigned long long f[4]; bool on[4]; int b[4]; unsigned old[4];
 #pragma unroll
@@ -611,6 +637,7 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
         }
       }
     } else if (run) {
+#pragma unroll 1
       for (int i0 = gt; i0 < n; i0 += 4 * T) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -661,6 +688,7 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
         // rounding kept the total below p: everything.  (Task 2 has more than `ne` eligible candidates by the quota's size.)
         K = n; run = false;
         if (task == 2) {                                     // (scores that are not numbers: some list within bounds, and the error bit)
+#pragma unroll 1
           for (int t = gt; t < ne; t += T) m.ev[t] = t;
           if (gt == 0) atomicOr(p.err, GP_E_BOUNDS);
         }
@@ -672,6 +700,7 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
         else if (in_bin <= 32) run = false;
         else if (shift == 0) { ties = true; run = false; }              // copies of one value
         else { width = min(8, shift); shift -= width; }
+#pragma unroll 1
         for (int i = gt; i < BIN_STRIDE; i += T) { bcnt[i] = 0; blo[i] = 0; bhi[i] = 0; }
       }
     }
@@ -741,12 +770,14 @@ __device__ __forceinline__ void unit_select(const GpDev& p, const SelSmem& S, co
       if (lane < (int)in_bin && rank < ne - (int)before) m.ev[before + rank] = slot;
     } else if (ties && lane == 0) {                        // rare: older (lower) slots win ties
       int at = (int)before;
+#pragma unroll 1
       for (int i = n - 1; i >= 0 && at < ne; --i)
         if (key2(i) == prefix && eligible(i)) m.ev[at++] = i;
     }
   }
   if (!(tasks & 4)) return;
   __syncthreads();
+#pragma unroll 1
   for (int t = tid; t < ne; t += SEL_T) {                    // the evicted slots in ascending order, by rank
     const int slot = m.ev[t];
     int rank = 0;
@@ -794,6 +825,7 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
   const UnitOrder ord = {p.page_table + (size_t)r * p.cap, p.rank + gp_tok_off(p, lh / p.Hkv, 0, lh % p.Hkv), (size_t)p.Hkv * GP_PAGE};
   const bool one_support = p.sub == 1;
   const bool entropy = p.metric == GP_METRIC_ENTROPY;
+#pragma unroll 1
   for (int pass = 0; pass < (one_support ? 1 : 2); ++pass) {
     const int ntile = pass == 0 ? nt_d : nt_e, n = ntile * GP_PAGE;
     int tasks = want & (one_support ? 7 : pass == 0 ? 3 : 4);
@@ -810,6 +842,7 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
         if (!((tasks >> view) & 1)) continue;
         const double* a = view ? aL : aS;
         double hsum = 0.0;
+#pragma unroll 1
         for (int i = tid; i < n; i += SEL_T) { const double v = a[i]; if (v > 0.0) hsum -= v * log(v); }
 #pragma unroll
         for (int o2 = 16; o2 > 0; o2 >>= 1) hsum += __shfl_xor_sync(0xffffffffu, hsum, o2);
@@ -817,6 +850,7 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
         __syncthreads();
         if (tid == 0) {
           double tot = 0.0;
+#pragma unroll 1
           for (int w = 0; w < SEL_NW; ++w) tot += m.red[w];
           Kout[view] = 0;
           Hout[view] = tot;
@@ -1053,6 +1087,7 @@ template <typename F>
 __device__ __forceinline__ int warp_pack(int n, int* out, F flag) {
   const int lane = threadIdx.x & 31;
   int at = 0;
+#pragma unroll 1
   for (int i0 = 0; i0 < n; i0 += 32) {
     const bool f = i0 + lane < n && flag(i0 + lane);
     const unsigned m = __ballot_sync(0xffffffffu, f);
@@ -1096,6 +1131,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
   // asynchronous mode, where the two scratch sets count on their own; otherwise the counter the plan kernel keeps
   // on the device, so that a step replayed from a CUDA graph gets a stamp of its own
   const int stamp = p.async ? serial + 1 : p.hdr[HDR_STEP];
+#pragma unroll 1
   for (int i = tid + CT; i <= n_cmp; i += CT) s_info[i] = p.cmp_info[i];
   int moved = 0;
 
@@ -1111,6 +1147,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     if (item >= n_items) break;
     // ticket -> (compressing request, layer/head, part); the parts of a unit are consecutive
     int lo = 0, hi = n_cmp;
+#pragma unroll 1
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (LH * s_info[mid].w <= item) lo = mid; else hi = mid; }
     const int n_part = s_info[lo + 1].w - s_info[lo].w;
     const int rem = item - LH * s_info[lo].w;
@@ -1131,6 +1168,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     const size_t page_stride = (size_t)p.Hkv * 2 * GP_PAGE * ROW_BYTES;
     uint8_t* const unit_base = reinterpret_cast<uint8_t*>(p.kv + gp_tile_off(p, l, 0, h));
 
+#pragma unroll 1
     for (int t = tid; t < ne; t += CT) {
       ev[t] = shrink ? p.evict2[((size_t)e_bnd * LH + lh) * 2 * p.blk + t] : p.evict[((size_t)e_bnd * LH + lh) * p.blk + t];
       C.ev_slot[t] = -1;
@@ -1141,6 +1179,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       constexpr int TB = 2 * GP_PAGE * ROW_BYTES / 16;     // 16-byte pieces of a tile
       constexpr int U = 4;                                 // tiles in flight
       const int pg_end = min(c1, n_end) / GP_PAGE;
+#pragma unroll 1
       for (int pg0 = c0 / GP_PAGE; pg0 < pg_end; pg0 += U) {
         uint4 val[U][TB / CT];
         int to[U];
@@ -1163,6 +1202,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     // the slots' new order indices, a slot per thread, SU of them in flight
     constexpr int SU = 4;
     bool listed = false;
+#pragma unroll 1
     for (int i0 = c0; i0 < c1; i0 += SU * CT) {
       int from[SU], to[SU], rk[SU];
 #pragma unroll
@@ -1188,6 +1228,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
           for (int e = 0; e < GP_PAGE; ++e) { const int x = ev[e]; below += x < rk[u]; gone |= x == rk[u]; }
         } else {
           int hi2 = ne;
+#pragma unroll 1
           while (below < hi2) { const int mid = (below + hi2) >> 1; if (ev[mid] < rk[u]) below = mid + 1; else hi2 = mid; }
           gone = below < ne && ev[below] == rk[u];
         }
@@ -1213,6 +1254,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       // early planning the next step's plan may be writing its own boundary records by now)
       int* found = reinterpret_cast<int*>(p.scores + (size_t)lh * p.max_boundary_tokens + __ldcg(p.cmp_off + e_bnd));        // [ne][2] (a unit has ne candidates at least)
       if (part < n_part - 1) {
+#pragma unroll 1
         for (int t = tid; t < ne; t += CT)
           if (C.ev_slot[t] >= 0) { found[2 * t] = C.ev_slot[t]; found[2 * t + 1] = C.ev_page[t]; }
         __threadfence();
@@ -1223,6 +1265,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       }
       if (tid == 0) s_i[4] = 1;
       __syncthreads();
+#pragma unroll 1
       for (int back = 1 + tid; back <= part; back += CT) {
         volatile int* prev = reinterpret_cast<volatile int*>(p.cflags + item - back);
         unsigned it = 0;
@@ -1232,6 +1275,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       __threadfence();
       __syncthreads();
       if (!s_i[4]) continue;                               // nothing is known of those slots: no row moves
+#pragma unroll 1
       for (int t = tid; t < ne; t += CT)
         if (C.ev_slot[t] < 0) {
           const int2 f = __ldcg(reinterpret_cast<const int2*>(found) + t);
@@ -1251,6 +1295,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
     }
     __syncthreads();
     const int n_mv = min(s_i[1], s_i[5]);
+#pragma unroll 1
     for (int k = tid; k < n_mv; k += CT) {
       const int hole = C.hole[k], mv = C.mover[k], ds = C.ev_slot[hole];
       const size_t at = tok_base + (size_t)C.ev_page[hole] * tok_stride + ds % GP_PAGE;
@@ -1258,6 +1303,7 @@ __device__ __forceinline__ void compact_body(const GpDev& p, const CmpSmem& C, i
       p.tok[at] = __ldcg(p.tok + tok_base + (size_t)C.mv_page[mv] * tok_stride + (n_end + mv) % GP_PAGE);
     }
     constexpr int MU = 2;
+#pragma unroll 1
     for (int q0 = tid; q0 < n_mv * PPS; q0 += MU * CT) {
       uint4 val[MU];
 #pragma unroll
