@@ -131,10 +131,12 @@ template <int D>
 __device__ __forceinline__ void merge_unit(float* first, size_t stride, int n, int G, float* __restrict__ orow, bool into) {
   constexpr int PER2 = D / 64;                           // float2 pieces of a row per lane
   const int lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int g0 = 0; g0 < G; g0 += 4) {                    // four heads at a time
     const int g = g0 + (lane & 3);                       // lane: head g0 + lane % 4, partials lane / 4, + 8, ...
     const float* ml = first + (g < G ? g : 0) * (D + 2) + D;
     float M = -INFINITY, ls = 0.f;
+#pragma unroll 1
     for (int c = lane >> 2; c < n; c += 8) {
       const float2 v = __ldcg(reinterpret_cast<const float2*>(ml + c * stride));
       const float Mn = fmaxf(M, v.x);
@@ -153,6 +155,7 @@ __device__ __forceinline__ void merge_unit(float* first, size_t stride, int n, i
     for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int e = 0; e < PER2; ++e) acc[q][e] = make_float2(0.f, 0.f);
+#pragma unroll 1
     for (int c0 = 0; c0 < n; c0 += 2) {                  // two partials' values in flight
       float2 vv[2][4][PER2];
       float mv[2][4];
@@ -231,6 +234,7 @@ __device__ __forceinline__ bool summary_rows(const GpDev& p, const GpNorm& nm, u
     if (lane == 0) mbar_arrive(norm_bar);
   }
   if (!owner && !qt) return true;
+#pragma unroll 1
   for (int g0 = w; g0 < G; g0 += 2 * NSUM) {
     if (g0 != w) load_old(g0);
     double ss[2][2], sq[2];                                // sums of squares: new summaries, query
@@ -860,8 +864,9 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
 #pragma unroll 1
           for (int sub = 0; sub < PAIR; ++sub) {
             if (sub && (sub >= nsub || pg0 + pgl + sub >= Pr - 1)) break;
-            summary_logits<D>(p, stage + sub * GEO::TILE_BYTES, qt, G, lh, zoff, tok0 + sub * GP_PAGE, 0);
-            if (WIDE) summary_logits<D>(p, stage + sub * GEO::TILE_BYTES, qt, G, lh, zoff, tok0 + sub * GP_PAGE, 1);
+#pragma unroll
+            for (int nt = 0; nt < (WIDE ? 2 : 1); ++nt)
+              summary_logits<D>(p, stage + sub * GEO::TILE_BYTES, qt, G, lh, zoff, tok0 + sub * GP_PAGE, nt);
           }
         }
         __syncwarp();
@@ -976,13 +981,19 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
           return last != 0;
         };
         int* cnt = p.merge_cnt + ((size_t)rc_i - chunk) * LH + (size_t)lh * nchunks;       // the unit's: one per chunk
-        if (last_of(cnt + c_grp, in_grp)) {
-          if (n_grp == 1) {
-            merge_unit<D>(unit, PSTRIDE, nchunks, G, out + out_row0, false);
-          } else {
-            if (in_grp > 1) merge_unit<D>(unit + (size_t)c_grp * PSTRIDE, PSTRIDE, in_grp, G, nullptr, true);
-            if (last_of(cnt + 1, n_grp)) merge_unit<D>(unit, (size_t)MERGE_FAN * PSTRIDE, n_grp, G, out + out_row0, false);
-          }
+        const bool tree = n_grp > 1;
+        bool go = last_of(cnt + c_grp, in_grp), into = tree;
+#pragma unroll 1
+        while (go) {
+          // One call of the merge: three copies, unrolled, were 37 KB of the kernel's 130, and these kernels' few units wait for instructions
+          // (gp_attn_kernel<128, true, WHOLE_STEP, false> 102 KB now; us a pass: four requests, 16 steps, 259 / 256; one layer x 64, 16 steps,
+          // 1039 / 1026; long contexts, 16 steps, 5080 / 5039).  Its first rows asked for before the maxima: spills at 80 registers, 4 % of a layer.
+          const bool groups = tree && !into;
+          const int n = groups ? n_grp : tree ? in_grp : nchunks;
+          if (!into || n > 1)
+            merge_unit<D>(unit + (into ? (size_t)c_grp * PSTRIDE : 0), groups ? (size_t)MERGE_FAN * PSTRIDE : PSTRIDE, n, G, out + out_row0, into);
+          go = into && last_of(cnt + 1, n_grp);
+          into = false;
         }
       }
     }
@@ -996,7 +1007,7 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
       uint8_t* slot = smem + L.off_slots + sl * GEO::SLOT_BYTES;
       const int* sd = reinterpret_cast<const int*>(slot);
       if (sd[3] < 0) break;
-      const int bi = sd[0], r = sd[1], flags = sd[8], par = sd[12], lh = sd[14];
+      const int bi = sd[0], r = sd[1], flags = sd[8], par = sd[12];
       const bool owner = sd[4] == 0;                       // this item writes the unit's new summaries
       const bool need_qt = (flags & 1) && sd[2] < sd[9] - 1;
       if (NORM || owner || need_qt) {
