@@ -258,6 +258,8 @@ __device__ __forceinline__ void plan_scan(PlanScan& S, int a, int b, long long w
 // What bounds it: two dependent round trips (request ids; descriptors out) and six block barriers between them.  (With the counters read
 // behind the ids, three scans and a scan of the cost bins of 45 dependent steps: 12.3 us between events for 64 requests, now 10.2;
 // 16 steps of four requests 317 us, now 280.)
+// Loops that one request in a few hundred makes longer than a trip are not unrolled: instruction fetch (26 KB of them, now 20; us a step, two requests
+// 17.9 / 17.5, 16 with rotary embeddings 30.4 / 30.0, 20 in groups of one 32.9 / 32.6, 64 62.9 / 62.9).
 __global__ void __launch_bounds__(GP_PLAN_THREADS)
 gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions, int early,
                int cp_norm, int cp_bnd, int launch_units, int launch_grid, int serial) {
@@ -292,8 +294,13 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   };
   const bool preloaded = !p.async && p.M <= PLAN_STATES;
   if (blockIdx.x == 0) {
-    if (preloaded) for (int t = i; t < p.M; t += blockDim.x) s_state[t] = load_state(t);
+    if (preloaded) {
+#pragma unroll 1
+      for (int t = i; t < p.M; t += blockDim.x) s_state[t] = load_state(t);
+    }
+#pragma unroll 1
     for (int t = i; t < p.M; t += blockDim.x) s_first[t] = 0x7fffffff;
+#pragma unroll 1
     for (int t = i; t < GP_COST_BINS; t += blockDim.x) s_bin[t] = 0;
     if (i == 0) s_pages = 0;
     __syncthreads();
@@ -328,6 +335,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   if (inrange) st = preloaded ? s_state[r] : load_state(r);
   // the attention kernel draws its items from these (the one of the step before, the last to draw, has ended: that step's
   // decisions waited for it, or, where it was abandoned before it had any, this launch did)
+#pragma unroll 1
   for (int idx = threadIdx.x; idx < 2 * p.L; idx += blockDim.x) p.tickets[idx] = 0;
   __syncthreads();
   int chunks = 0, pages = 0, act = GP_ACT_NONE;
@@ -413,6 +421,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
       within += ((e.x >> 16) == key ? (e.x & 0xffff) : 0) + ((e.y >> 16) == key ? (e.y & 0xffff) : 0) +
                 ((e.z >> 16) == key ? (e.z & 0xffff) : 0) + ((e.w >> 16) == key ? (e.w & 0xffff) : 0);
     }
+#pragma unroll 1
     for (; j < i; ++j) { const int e = s_first[j]; within += (e >> 16) == key ? (e & 0xffff) : 0; }
   }
   __syncthreads();
@@ -428,6 +437,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     }
     // descriptors of this request's chunks: four 16-byte stores each
     const int flags = isb | (st.w & 2);
+#pragma unroll 1
     for (int c = 0; c < chunks; ++c) {
       const int pg0 = c * cp;
       int4* d = reinterpret_cast<int4*>(p.rcx + (size_t)(sorted0 + c) * GP_DESC_INTS);
@@ -438,8 +448,10 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     }
   }
   // the attention kernel counts, per unit of a boundary request, the work items its consumer warps have finished
-  if (p.report_units)
+  if (p.report_units) {
+#pragma unroll 1
     for (int idx = threadIdx.x; idx < n_bnd * p.L * p.Hkv; idx += blockDim.x) p.unit_ready[idx] = 0;
+  }
   if (threadIdx.x == 0) {
     p.hdr[HDR_N_RC] = n_rc;
     p.hdr[HDR_N_BRC] = s_binbase[GP_COST_BINS / 2] + s_bin[GP_COST_BINS / 2];
