@@ -272,7 +272,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // early: the caller's request ids may be read before the wait for the preceding kernel (see below)
   __shared__ PlanScan s_scan[2];
   __shared__ __align__(16) int s_first[GP_MAX_REQ];      // lowest batch index naming a request; then cost classes and items
-  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS], s_pages;
+  __shared__ int s_bin[GP_COST_BINS], s_binbase[GP_COST_BINS], s_pages, s_bpages;
   // .x slots in use, .y pages, .z position, .w: 1 live, 2 has decoded, 4 summary buffer in use, 8 sits this step out
   __shared__ int4 s_state[PLAN_STATES];
   const int i = threadIdx.x;
@@ -302,7 +302,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     for (int t = i; t < p.M; t += blockDim.x) s_first[t] = 0x7fffffff;
 #pragma unroll 1
     for (int t = i; t < GP_COST_BINS; t += blockDim.x) s_bin[t] = 0;
-    if (i == 0) s_pages = 0;
+    if (i == 0) s_pages = s_bpages = 0;
     __syncthreads();
   }
   if (!early) gp_pdl_wait();
@@ -363,7 +363,14 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     // with fine items, 64 requests of 44 pages and more 3 us faster with large ones.
     const int warp_pages = __reduce_add_sync(0xffffffffu, pages);
     if ((i & 31) == 0 && warp_pages) atomicAdd(&s_pages, warp_pages);
+    if (isb) atomicAdd(&s_bpages, pages);
     __syncthreads();
+    // Boundary requests in large items as well where that leaves two of them per CTA: each item works out its q~ anew, which its consumer warps wait for
+    // (groups of eight: 24 000 cycles an item, 3000 a tile in items of 32).  us of the attention kernel, items of 32 / 64: 64 layers x 32 requests, groups of
+    // eight, two at a boundary 1636 / 1573, four 1843 / 1782; 36 x 256, 16 at a boundary 3884 / 3866, 22 4046 / 3972.  With few of them the items are
+    // too long for the selection behind them: one layer x 64, four at a boundary 46 / 57; 36 x 4, one, 77.4 / 77.9 us a step.
+    // (Not where the items, cut the smaller way, might not fit the scratch: who is refused below stays who was.)
+    if ((long long)s_bpages * launch_units >= 2LL * cp_norm * launch_grid && s_pages / cp_bnd + n_req <= p.max_rc) cp_bnd = cp_norm;
     if ((long long)s_pages * launch_units < (long long)cp_norm * launch_grid) { cp_norm = GP_FINE_CHUNK; cp_bnd = GP_FINE_BCHUNK; }
   }
   if (pages > 0) {
