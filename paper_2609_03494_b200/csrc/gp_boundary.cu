@@ -316,8 +316,13 @@ struct SelMisc {
   int s_i[8];
   int ev[2 * GP_MAX_BLK];
   unsigned bins[3][3][BIN_STRIDE];                // per task: members, mass (low, high word)
-  double F[SEL_F];
+  double gM[16], gR[16];                          // a unit shared out over a cluster: the maxima and factors of the whole unit ...
+  unsigned grng[3][2];                            // ... and the range of its scores' high words
+  unsigned shared_out[GP_MAX_REQ / 32];           // a bit per boundary request: its units are shared out
+  int n_shared, ticket;
+  alignas(16) double F[SEL_F];                    // page factors; of a unit shared out, after that, the cluster's bins
 };
+static_assert(SEL_F * sizeof(double) >= (3 * 4 + 2 * 8) * BIN_STRIDE, "the cluster's bins fit");
 struct SelSmem {
   SelMisc* m;
   unsigned* loc;                     // [cap * 16 / 32 + 2] block-local picks, one bit per candidate
@@ -872,6 +877,393 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
   }
 }
 
+// ------------------------------------------------------------------------------------------------------
+// a unit of many candidates, shared out over the thread blocks of a cluster
+// ------------------------------------------------------------------------------------------------------
+// One thread block walks 20 000 candidates of a group of eight in 380 us (logits of two views and eight heads, 128 bytes each, and then every
+// level of the descent over scores that do not fit its shared memory), while most of the chip has no unit at all.  Here the CLUSTER blocks of
+// a cluster share one: each takes a part of the pages for the softmax (its normalisers are merged over the cluster), the scores go to the
+// pool's scratch in the order of the tokens, and each takes a part of that order into its shared memory for the descents, whose bins are added
+// up over the cluster at every level.  Counts and fixed-point masses are integers, so the result is that of one block over the same scores.
+// What bounds it: the logits' bytes, then a chain of a dozen cluster barriers.  Two requests of 20 000, us a step: one layer, groups of eight
+// 101.6 / 79.7, of four 76.3 / 65.0; four layers 184.9 / 161.2 and 147.1 / 138.3.
+constexpr int CLUSTER = 8;
+constexpr int SPLIT_FROM = 2 * SEL_CAP;     // candidates above which a unit is shared out: see split_unit
+__device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the same place in the shared memory of another block of the cluster
+template <typename T>
+__device__ __forceinline__ T* of_block(T* ptr, unsigned rank) {
+  T* q;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(ptr), "r"(rank));
+  return q;
+}
+
+// Scores of the pages [t_lo, t_hi) into aS, aL (global, in the order of the tokens), normalised over all of the unit's.  Ends with a
+// barrier of the cluster, behind which all scores and the blocks' ranges of high words are there.
+template <int GG>
+__device__ __forceinline__ void split_softmax(const SelSmem& S, const double* __restrict__ x, size_t view_stride, const double* __restrict__ zs,
+                                              double* aS, double* aL, int t_lo, int t_hi, int n, const UnitOrder& ord) {
+  constexpr int NC = 2 * GG, U = GG >= 4 ? 2 : 4, FT = SEL_F / NC, TSTEP = SEL_T / NC;
+  SelMisc& m = *S.m;
+  const int tid = threadIdx.x, myc = tid % NC, t0 = tid / NC;
+  double mx = -INFINITY;
+#pragma unroll 4
+  for (int t = t_lo + t0; t < t_hi; t += TSTEP) mx = fmax(mx, __ldcg(zs + ((size_t)t * NC + myc) * 2));
+  column_reduce<true>(mx, NC, m.red, m.sM);
+  double acc = 0.0;
+#pragma unroll 2
+  for (int t = t_lo + t0; t < t_hi; t += TSTEP) {
+    const double2 ms = __ldcg(reinterpret_cast<const double2*>(zs + ((size_t)t * NC + myc) * 2));
+    acc += ms.y * exp(ms.x - m.sM[myc]);
+  }
+  column_reduce<false>(acc, NC, m.red, m.sZ);
+  // the places of this block's candidates in the order, ahead of their scores (in the place the scores take later)
+  int* const at = reinterpret_cast<int*>(S.sS);
+#pragma unroll 8
+  for (int i = tid; i < (t_hi - t_lo) * GP_PAGE; i += SEL_T)
+    at[i] = min(max(__ldcg(ord.rank + (size_t)__ldg(ord.table + t_lo + i / GP_PAGE) * ord.page_stride + i % GP_PAGE), 0), n - 1);  // (in bounds whatever a wait that gave up left behind)
+  cluster_sync();
+  if (tid < NC) {
+    double M = -INFINITY, Z = 0.0;
+#pragma unroll
+    for (int r = 0; r < CLUSTER; ++r) M = fmax(M, of_block(m.sM, r)[tid]);
+#pragma unroll 1
+    for (int r = 0; r < CLUSTER; ++r) {
+      const double zr = of_block(m.sZ, r)[tid], mr = of_block(m.sM, r)[tid];
+      Z += zr == 0.0 ? 0.0 : zr * exp(mr - M);            // (a block without pages: 0; what is no number stays none)
+    }
+    m.gM[tid] = M; m.gR[tid] = 1.0 / ((double)GG * Z);
+  }
+  unsigned lo_w[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi_w[3] = {0u, 0u, 0u};
+#pragma unroll 1
+  for (int tb = t_lo; tb < t_hi; tb += FT) {
+    const int te = min(t_hi, tb + FT), k_end = te * GP_PAGE;
+    __syncthreads();
+#pragma unroll 2
+    for (int t = tb + t0; t < te; t += TSTEP) m.F[(t - tb) * NC + myc] = exp(__ldcg(zs + ((size_t)t * NC + myc) * 2) - m.gM[myc]) * m.gR[myc];
+    __syncthreads();
+#pragma unroll 1
+    for (int k0 = tb * GP_PAGE; k0 < k_end; k0 += U * SEL_T) {
+      double xv[U][2][GG];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tok = k0 + tid + u * SEL_T;
+        if (tok < k_end) {
+          ld_early_row<GG>(x + (size_t)tok * GG, xv[u][0]);
+          ld_early_row<GG>(x + view_stride + (size_t)tok * GG, xv[u][1]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tok = k0 + tid + u * SEL_T;
+        if (tok < k_end) {
+          const double* f = m.F + (tok / GP_PAGE - tb) * NC;
+          double a[2];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            a[q] = xv[u][q][0] * f[q * GG];
+#pragma unroll
+            for (int g = 1; g < GG; ++g) a[q] += xv[u][q][g] * f[q * GG + g];
+          }
+          const int i = at[tok - t_lo * GP_PAGE];
+          __stcg(aS + i, a[0]); __stcg(aL + i, a[1]);
+          const unsigned w0 = (unsigned)__double2hiint(a[0]), w1 = (unsigned)__double2hiint(a[1]), w2 = max(w0, w1);
+          lo_w[0] = min(lo_w[0], w0); lo_w[1] = min(lo_w[1], w1); lo_w[2] = min(lo_w[2], w2);
+          hi_w[0] = max(hi_w[0], w0); hi_w[1] = max(hi_w[1], w1); hi_w[2] = max(hi_w[2], w2);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const unsigned a = __reduce_min_sync(0xffffffffu, lo_w[q]), b = __reduce_max_sync(0xffffffffu, hi_w[q]);
+    if ((tid & 31) == 0) { atomicMin(&m.rng[q][0], a); atomicMax(&m.rng[q][1], b); }
+  }
+  cluster_sync();
+}
+
+// The tasks of unit_select over this block's part of the order, candidates [i_lo, i_lo + nl) of the unit's n, in S.sS and S.sL.  All blocks
+// of the cluster take the same decisions from the same sums; lists are gathered in the first one, which writes the results.
+__device__ __forceinline__ void split_select(const GpDev& p, const SelSmem& S, const double* gS, const double* gL, int i_lo, int nl, int per, int n,
+                                             int tasks, int ne, int kq, int* Kout, int* acc, int* evout) {
+  SelMisc& m = *S.m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned me = cluster_rank();
+  const int task = warp < 2 ? 0 : (warp < 4 ? 1 : 2), T = task == 2 ? 128 : 64, gt = task == 2 ? tid - 128 : tid & 63;
+  const double* a = task == 1 ? S.sL : S.sS;
+  const bool lead = gt < 32, mine = (tasks >> task) & 1;
+  bool run = mine;
+  unsigned* bcnt = m.bins[task][0]; unsigned* blo = m.bins[task][1]; unsigned* bhi = m.bins[task][2];
+  unsigned* const ccnt = reinterpret_cast<unsigned*>(m.F);                                     // [3][BIN_STRIDE] members, the cluster's
+  unsigned long long* const cmass = reinterpret_cast<unsigned long long*>(ccnt + 3 * BIN_STRIDE + (3 * BIN_STRIDE & 1));      // [2][BIN_STRIDE]
+#pragma unroll 1
+  for (int i = tid; i < 3 * 3 * BIN_STRIDE; i += SEL_T) (&m.bins[0][0][0])[i] = 0;
+  if (tid < 4) m.cnt[tid] = 0;
+  if (tid < 3) {
+    unsigned lo = 0xffffffffu, hi = 0u;
+#pragma unroll 1
+    for (int r = 0; r < CLUSTER; ++r) { lo = min(lo, of_block(&m.rng[tid][0], r)[0]); hi = max(hi, of_block(&m.rng[tid][0], r)[1]); }
+    m.grng[tid][0] = lo; m.grng[tid][1] = hi;
+  }
+  __syncthreads();
+  if (tasks & 4) {
+    if (kq > 0) mark_local(S.sS, S.sL, nl, p.blk, kq, S.loc, warp, SEL_NW);
+    else for (int i = tid; i < (nl + 31) / 32; i += SEL_T) S.loc[i] = 0;
+  }
+  auto key2 = [&](int i) { return max(key_of(S.sS[i]), key_of(S.sL[i])); };
+  auto eligible = [&](int i) { return !((S.loc[i >> 5] >> (i & 31)) & 1u); };
+  const unsigned h0 = m.grng[task][0], h1 = m.grng[task][1];
+  int shift = h0 == h1 ? 24 : max(0, 32 + (31 - __clz((int)(h0 ^ h1))) - 7);
+  int width = 8;
+  unsigned long long prefix = ((unsigned long long)h1 << 32) >> (shift + 8);
+  unsigned before = 0, in_bin = 0;
+  unsigned long long mass = 0;
+  int K = -1;
+  bool ties = false, whole = false;
+  __syncthreads();
+  for (;;) {
+    const unsigned mask = (1u << width) - 1u;
+    if (run) {
+#pragma unroll 1
+      for (int i0 = gt; i0 < nl; i0 += 4 * T) {            // four at a time: their loads, then their adds, in flight together
+        unsigned long long f[4]; bool on[4]; int b[4]; unsigned old[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int i = i0 + e * T, j = i < nl ? i : gt;
+          const double v = a[j];
+          const unsigned long long k = (task != 2 ? key_of(v) : key2(j)) >> shift;
+          on[e] = i < nl && (k >> width) == prefix && (task != 2 || eligible(j));
+          b[e] = BIDX((int)((unsigned)k & mask));
+          f[e] = to_fix(v);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          old[e] = 0u;
+          if (on[e]) { atomicAdd(&bcnt[b[e]], 1u); if (task != 2) old[e] = atomicAdd(&blo[b[e]], (unsigned)f[e]); }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {                      // the carry travels with the high word's add
+          const unsigned up = (unsigned)(f[e] >> 32) + (old[e] + (unsigned)f[e] < old[e] ? 1u : 0u);
+          if (on[e] && task != 2 && up) atomicAdd(&bhi[b[e]], up);
+        }
+      }
+    }
+    cluster_sync();
+    {                                                      // the cluster's bins, a bin of each task per thread
+      const int b = BIDX(tid);
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        unsigned c = 0; unsigned long long s = 0;
+#pragma unroll
+        for (int r = 0; r < CLUSTER; ++r) {
+          const unsigned* q = of_block(&m.bins[t][0][b], r);
+          c += q[0];
+          if (t < 2) s += ((unsigned long long)q[2 * BIN_STRIDE] << 32) + q[BIN_STRIDE];
+        }
+        ccnt[t * BIN_STRIDE + b] = c;
+        if (t < 2) cmass[t * BIN_STRIDE + b] = s;
+      }
+    }
+    cluster_sync();                                        // (every block has read every block's: they may be cleared)
+    if (run && lead) {                                     // lane owns bins [8 lane, 8 lane + 8)
+      unsigned c8[8]; unsigned long long m8[8];
+      unsigned c = 0; unsigned long long s = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int b = lane * 9 + j;                        // BIDX(8 lane + j)
+        c8[j] = ccnt[task * BIN_STRIDE + b];
+        m8[j] = task != 2 ? cmass[task * BIN_STRIDE + b] : 0ull;
+        c += c8[j]; s += m8[j];
+      }
+      unsigned ic = c; unsigned long long is = s;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned td = __shfl_down_sync(0xffffffffu, ic, o), tu = __shfl_up_sync(0xffffffffu, ic, o);
+        const unsigned long long ts = __shfl_down_sync(0xffffffffu, is, o);
+        if (task != 2) { if (lane + o < 32) { ic += td; is += ts; } }         // largest scores first
+        else if (lane >= o) ic += tu;                                          // lowest scores first
+      }
+      unsigned rc = before + ic - c; unsigned long long rs = mass + is - s;
+      bool hit = false;
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        const int j = task != 2 ? 7 - jj : jj;
+        const bool here = task != 2 ? rs < p.p_fix && rs + m8[j] >= p.p_fix : rc < (unsigned)ne && rc + c8[j] >= (unsigned)ne;
+        if (here) { m.res[task][0] = lane * 8 + j; m.res[task][1] = rc; m.res[task][2] = (long long)rs; m.res[task][3] = c8[j]; hit = true; }
+        rc += c8[j]; rs += m8[j];
+      }
+      if (!__any_sync(0xffffffffu, hit) && lane == 0) m.res[task][0] = -1;
+    }
+    __syncthreads();
+    if (run) {
+      const int bin = (int)m.res[task][0];
+      if (bin < 0) {
+        K = n; run = false;                                // rounding kept the total below p: everything
+        if (task == 2 && me == 0) {                        // (scores that are not numbers: some list within bounds, and the error bit)
+          for (int t = gt; t < ne; t += T) m.ev[t] = t;
+          if (gt == 0) atomicOr(p.err, GP_E_BOUNDS);
+        }
+      } else {
+        before = (unsigned)m.res[task][1]; mass = (unsigned long long)m.res[task][2]; in_bin = (unsigned)m.res[task][3];
+        prefix = (prefix << width) | (unsigned long long)bin;
+        if (task != 2 && in_bin == 1) { K = (int)before + 1; run = false; }
+        else if (task == 2 && before + in_bin == (unsigned)ne) { whole = true; run = false; }       // the bin goes as a whole
+        else if (in_bin <= 32) run = false;
+        else if (shift == 0) { ties = true; run = false; }              // copies of one value
+        else { width = min(8, shift); shift -= width; }
+        for (int i = gt; i < BIN_STRIDE; i += T) { bcnt[i] = 0; blo[i] = 0; bhi[i] = 0; }
+      }
+    }
+    if (!__syncthreads_or(run)) break;                     // (the same in every block of the cluster)
+  }
+  // ---- the members of the crossing bin and the evicted candidates, gathered in the first block ------------------------
+  SelMisc* const m0 = of_block(S.m, 0);
+  const bool listed = mine && K < 0 && !ties && !whole;
+  if (mine && K < 0) {
+#pragma unroll 4
+    for (int i = gt; i < nl; i += T) {
+      if (task != 2) {
+        const double v = a[i];
+        if (listed && (key_of(v) >> shift) == prefix) {
+          const int at = atomicAdd(&m0->cnt[1 + task], 1);
+          if (at < 32) { m0->list[task][at] = key_of(v); m0->list_fix[task][at] = to_fix(v); }
+        }
+      } else {
+        const unsigned long long full = key2(i), k = full >> shift;
+        if (k <= prefix && eligible(i)) {
+          if (k < prefix || whole) { const int at = atomicAdd(&m0->cnt[0], 1); if (at < ne) m0->ev[at] = i_lo + i; }
+          else if (listed) { const int at = atomicAdd(&m0->cnt[3], 1); if (at < 32) { m0->list[2][at] = full; m0->list_slot[at] = i_lo + i; } }
+        }
+      }
+    }
+  }
+  const bool evict_ties = __syncthreads_or(task == 2 && ties);
+  cluster_sync();
+  if (me == 0) {
+    if (mine && lead) {
+      if (task != 2) {
+        if (listed) {
+          const unsigned long long v = m.list[task][lane];
+          int rank = 0;
+          unsigned long long inc = 0;
+#pragma unroll 1
+          for (int j = 0; j < (int)in_bin; ++j) {
+            const unsigned long long t = m.list[task][j];
+            const bool first = t > v || (t == v && j <= lane);
+            rank += first;
+            inc += first ? m.list_fix[task][j] : 0ull;
+          }
+          K = (int)before + (int)__reduce_min_sync(0xffffffffu, lane < (int)in_bin && mass + inc >= p.p_fix ? (unsigned)rank : in_bin);
+        } else if (ties) {
+          const unsigned long long f = to_fix(__longlong_as_double((long long)prefix));
+          unsigned long long j = f ? (p.p_fix - mass + f - 1) / f : 1ull;
+          if (j < 1) j = 1;
+          if (j > in_bin) j = in_bin;
+          K = (int)before + (int)j;
+        }
+        if (lane == 0) { Kout[task] = K; atomicAdd(acc + task, K); }
+      } else if (listed) {                                 // the lowest scores of the bin, later slots first among equals
+        const unsigned long long v = m.list[2][lane];
+        const int slot = m.list_slot[lane];
+        int rank = 0;
+#pragma unroll 1
+        for (int j = 0; j < (int)in_bin; ++j) {
+          const unsigned long long t = m.list[2][j];
+          rank += t < v || (t == v && m.list_slot[j] > slot);
+        }
+        if (lane < (int)in_bin && rank < ne - (int)before) m.ev[before + rank] = slot;
+      } else if (ties && lane == 0) {                      // rare: older (lower) slots win ties
+        int at = (int)before;
+        for (int i = n - 1; i >= 0 && at < ne; --i) {
+          const unsigned r = (unsigned)(i / per);
+          const int j = i - (int)r * per;
+          if (max(key_of(__ldcg(gS + i)), key_of(__ldcg(gL + i))) == prefix && !((of_block(S.loc, r)[j >> 5] >> (j & 31)) & 1u)) m.ev[at++] = i;
+        }
+      }
+    }
+    if (tasks & 4) {
+      __syncthreads();
+#pragma unroll 1
+      for (int t = tid; t < ne; t += SEL_T) {              // the evicted places in ascending order, by rank
+        const int slot = m.ev[t];
+        int rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < ne; ++j) rank += (m.ev[j] < slot);
+        evout[rank] = slot;
+      }
+    }
+  }
+  if (evict_ties) cluster_sync();                          // (the first block has read the others' bits)
+}
+
+// candidates a block of the cluster holds for the descents: whole blocks of Eq. 10, whole words of the bitmap
+__device__ __forceinline__ int split_part(const GpDev& p, int n) {
+  const int align = p.blk > 32 ? p.blk : 32;
+  return ((n + CLUSTER - 1) / CLUSTER + align - 1) / align * align;
+}
+// Whether the unit of a request with `Pr` pages is shared out, `units` of them in the step and `clusters` of the grid.  The line: up to 10 240
+// candidates the scores of a job fit one block's shared memory, and three blocks by themselves take no longer than the cluster's chain of
+// barriers (two requests of 7000, one layer, groups of four / eight, us a step, by themselves 36.6 / 49.9, shared 36.4 / 45.5; of 4500 33.1 / 43.2 and
+// 34.3 / 42.6; four layers of 7000 64.3 / 67.5), of 12 000 57.5 / 52.1 and 79.2 / 66.4; and a cluster takes its units one after the other, so that with
+// three for each (12 layers of 12 000: 220 / 227, of 20 000 344 / 344) nothing is left of it.
+__device__ __forceinline__ bool split_unit(const GpDev& p, const SelSmem& S, int Pr, long long units, int clusters) {
+  const long long rounds = (units + clusters - 1) / clusters;
+  const int n = (Pr - 1) * GP_PAGE;
+  return rounds <= 2 && n > SPLIT_FROM * rounds && split_part(p, n) <= S.n_cap && ((n / GP_PAGE + CLUSTER - 1) / CLUSTER + 1) * GP_PAGE <= 2 * S.n_cap &&
+         p.metric != GP_METRIC_ENTROPY && p.policy != GP_POLICY_SHRINK;
+}
+
+// the k-th of the n boundary requests whose bit is `set` (or not)
+__device__ __forceinline__ int nth_request(const unsigned* bits, int n, int k, bool set) {
+#pragma unroll 1
+  for (int w = 0; w * 32 < n; ++w) {
+    unsigned v = set ? bits[w] : ~bits[w];
+    if (n - w * 32 < 32) v &= (1u << (n - w * 32)) - 1u;
+    const int c = __popc(v);
+    if (k < c) {
+#pragma unroll 1
+      for (; k > 0; --k) v &= v - 1u;
+      return w * 32 + __ffs((int)v) - 1;
+    }
+    k -= c;
+  }
+  return 0;                                                // (there are as many)
+}
+
+template <int GG>
+__device__ __forceinline__ void sel_split(const GpDev& p, const SelSmem& S, int bidx, int lh, const int4 inf, const int4 inf2) {
+  SelMisc& m = *S.m;
+  const int LH = p.L * p.Hkv, r = inf.y, Pr = inf.z, me = (int)cluster_rank();
+  const long long off = (long long)(unsigned)inf2.x | ((long long)inf2.y << 32);
+  int* Kout = p.Kx + ((size_t)r * LH + lh) * 2;
+  const size_t view_stride = (size_t)p.z_stride * GG;
+  const double* z = p.zbuf + (size_t)lh * 2 * view_stride + (size_t)off * GG;
+  const double* zs = p.zstat + ((size_t)lh * (p.max_boundary_tokens / GP_PAGE) + off / GP_PAGE) * 2 * GG * 2;
+  double* aS = p.scores + (size_t)lh * p.max_boundary_tokens + off;
+  double* aL = aS + (size_t)LH * p.max_boundary_tokens;
+  const UnitOrder ord = {p.page_table + (size_t)r * p.cap, p.rank + gp_tok_off(p, lh / p.Hkv, 0, lh % p.Hkv), (size_t)p.Hkv * GP_PAGE};
+  const bool one_support = p.sub == 1;
+#pragma unroll 1
+  for (int pass = 0; pass < (one_support ? 1 : 2); ++pass) {          // the two supports: see sel_unit
+    const int ntile = pass == 0 ? Pr - p.sub : Pr - 1, n = ntile * GP_PAGE;
+    const int tasks = one_support ? 7 : pass == 0 ? 3 : 4;
+    __syncthreads();
+    if (threadIdx.x < 3) { m.rng[threadIdx.x][0] = 0xffffffffu; m.rng[threadIdx.x][1] = 0u; }
+    const int tpb = (ntile + CLUSTER - 1) / CLUSTER, t_lo = min(ntile, me * tpb), t_hi = min(ntile, t_lo + tpb);
+    split_softmax<GG>(S, z, view_stride, zs, aS, aL, t_lo, t_hi, n, ord);
+    const int per = split_part(p, n), i_lo = min(n, me * per), nl = min(n, i_lo + per) - i_lo;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nl; i += SEL_T) { S.sS[i] = __ldcg(aS + i_lo + i); S.sL[i] = __ldcg(aL + i_lo + i); }
+    const int nblk = (n + p.blk - 1) / p.blk;
+    split_select(p, S, aS, aL, i_lo, nl, per, n, tasks, p.blk, min(p.k_loc, (n - p.blk) / nblk), Kout, p.bnd_acc + 4 * bidx,
+                 p.evict + ((size_t)bidx * LH + lh) * p.blk);
+  }
+}
+
 // Rarely taken tails of the selection kernel's last thread block, kept out of line so that they do not weigh on the
 // register allocation of the jobs.
 // Layer-by-layer step: the requests' counters move on at the end of the step (a whole-step launch does it where
@@ -1368,7 +1760,8 @@ gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_i
 // kernel to end.  The grid therefore ends after both, and the plan of step t + 2, its programmatic dependent, finds the
 // pages and counters of the requests that sat step t + 1 out in their final state.  `p`: the view of step t (its
 // scratch set, the copy of the counters its decisions go to).
-template <int D, int GG>
+// LONG: launched in clusters, which share out units of many candidates (split_unit).
+template <int D, int GG, bool LONG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_chain, const int* __restrict__ req_ids,
                 int* __restrict__ actions, int* __restrict__ actions_copy) {
@@ -1392,29 +1785,98 @@ gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_
     const int n_bnd = __ldcg(p.hdr + HDR_N_BND);
     const int NJ = jobs_per_unit((long long)n_bnd * LH, gridDim.x);
     const long long items = (long long)n_bnd * LH * NJ;
-    for (long long item = blockIdx.x; item < items + n_bnd; item += gridDim.x) {
-      if (item >= items) { count_shared(p, (int)(item - items)); continue; }
-      const int u = (int)(item / NJ), bidx = u / LH, lh = u % LH;
-      const int4 inf = p.bnd_info[2 * bidx];
-      const int4 inf2 = p.bnd_info[2 * bidx + 1];
-      if (same_step && inf.z > p.sub) {
-        // every work item of the request reports once per consumer warp for this unit (bounded wait; the
-        // attention kernel's thread blocks were all resident before this grid could be scheduled)
+    const long long units = (long long)n_bnd * LH;
+    const int clusters = LONG ? (int)gridDim.x / CLUSTER : 0;
+    // every work item of the request reports once per consumer warp for this unit (bounded wait; the
+    // attention kernel's thread blocks were all resident before this grid could be scheduled)
+    auto unit_there = [&](int bidx, int lh, int reports) {
+      __syncthreads();
+      if (tid == 0) {
+        const volatile int* rdy = p.unit_ready + (size_t)bidx * LH + lh;
+        unsigned it = 0;
+        while (*rdy < reports && it < p.spin_limit) { ++it; __nanosleep(200); }
+        if (it >= p.spin_limit) atomicOr(p.err, GP_E_SPIN_SEL);
+        __threadfence();
+      }
+      __syncthreads();
+    };
+    bool last = false;                                     // this block finished the step's last job
+    if (LONG && n_bnd > 0) {
+      // Jobs are drawn from counters, not numbered by block, and counted as they are done: a cluster finds its place only where eight slots of
+      // one GPC are free, and a block of more shared memory than an attention block left may not fit beside another until that one is gone, so no job may
+      // be tied to a block that is not there yet (a grid that the occupancy query calls resident waited for its own decision that way).
+      SelMisc& m = *S.m;
+      if (tid < 32) {
+        int cnt = 0;
+        for (int b0 = 0; b0 < n_bnd; b0 += 32) {
+          const unsigned bits = __ballot_sync(0xffffffffu, b0 + tid < n_bnd && split_unit(p, S, __ldcg(&p.bnd_info[2 * min(b0 + tid, n_bnd - 1)].z), units, clusters));
+          if (tid == 0) m.shared_out[b0 / 32] = bits;
+          cnt += __popc(bits);
+        }
+        if (tid == 0) m.n_shared = cnt;
+      }
+      __syncthreads();
+      const int n_sh = m.n_shared, sh_units = n_sh * LH;
+      const int nj = jobs_per_unit((long long)(n_bnd - n_sh) * LH, gridDim.x), others = (n_bnd - n_sh) * LH * nj;
+      auto done = [&]() {                                  // a job is; whether it was the last of all
         __syncthreads();
         if (tid == 0) {
-          const volatile int* rdy = p.unit_ready + (size_t)bidx * LH + lh;
-          unsigned it = 0;
-          while (*rdy < inf2.z && it < p.spin_limit) { ++it; __nanosleep(200); }
-          if (it >= p.spin_limit) atomicOr(p.err, GP_E_SPIN_SEL);
           __threadfence();
+          const int total = sh_units + others + n_bnd;
+          s_i[2] = atomicAdd(&p.hdr[HDR_DONE_SEL], 1) == total - 1;
+          if (s_i[2]) p.hdr[HDR_DONE_SEL] = 0;
         }
         __syncthreads();
+        last |= s_i[2] != 0;
+      };
+      if (n_sh > 0) {
+#pragma unroll 1
+        for (;;) {
+          if (cluster_rank() == 0 && tid == 0) {
+            const int t = atomicAdd(&p.hdr[HDR_WORK_SPLIT], 1);
+#pragma unroll 1
+            for (int r = 0; r < CLUSTER; ++r) *of_block(&m.ticket, r) = t;
+          }
+          cluster_sync();
+          const int u = m.ticket;
+          if (u >= sh_units) break;
+          const int bidx = nth_request(m.shared_out, n_bnd, u / LH, true), lh = u % LH;
+          const int4 inf = p.bnd_info[2 * bidx], inf2 = p.bnd_info[2 * bidx + 1];
+          unit_there(bidx, lh, inf2.z);
+          sel_split<GG>(p, S, bidx, lh, inf, inf2);
+          if (cluster_rank() == 0) done();
+        }
       }
-      sel_unit<GG>(p, S, bidx, lh, inf, inf2, NJ == 1 ? 7 : 1 << (int)(item % NJ));
+#pragma unroll 1
+      for (;;) {
+        __syncthreads();
+        if (tid == 0) m.ticket = atomicAdd(&p.hdr[HDR_WORK_SEL], 1);
+        __syncthreads();
+        const int item = m.ticket;
+        if (item >= others + n_bnd) break;
+        if (item >= others) {
+          count_shared(p, item - others);
+        } else {
+          const int u = item / nj, bidx = nth_request(m.shared_out, n_bnd, u / LH, false), lh = u % LH;
+          const int4 inf = p.bnd_info[2 * bidx], inf2 = p.bnd_info[2 * bidx + 1];
+          if (inf.z > p.sub) unit_there(bidx, lh, inf2.z);
+          sel_unit<GG>(p, S, bidx, lh, inf, inf2, nj == 1 ? 7 : 1 << (item - u * nj));
+        }
+        done();
+      }
+    }
+#pragma unroll 1
+    for (int item = blockIdx.x; !LONG && item < (int)items + n_bnd; item += gridDim.x) {
+      if (item >= (int)items) { count_shared(p, item - (int)items); continue; }
+      const int u = item / NJ, bidx = u / LH, lh = u % LH;
+      const int4 inf = p.bnd_info[2 * bidx];
+      const int4 inf2 = p.bnd_info[2 * bidx + 1];
+      if (same_step && inf.z > p.sub) unit_there(bidx, lh, inf2.z);
+      sel_unit<GG>(p, S, bidx, lh, inf, inf2, NJ == 1 ? 7 : 1 << (item - u * NJ));
     }
     // ---- the last CTA to finish its jobs takes the decisions and tells the others ------------------------------
     const int stamp = same_step ? p.hdr[HDR_STEP] : serial + 1;
-    if (last_of_the_jobs(p, items + n_bnd, s_i)) {
+    if (LONG && n_bnd > 0 ? last : last_of_the_jobs(p, items + n_bnd, s_i)) {
       __threadfence();
       decide_and_allocate(p, req_ids, n_req, n_bnd, same_step ? actions : nullptr, reinterpret_cast<int*>(S.loc), serial);
       __syncthreads();
@@ -1466,10 +1928,13 @@ static SelKernel sel_kernel_of(const GpDev& p) {
   return p.G == 1 ? gp_bsel_kernel<1> : p.G == 2 ? gp_bsel_kernel<2> : p.G == 4 ? gp_bsel_kernel<4> : gp_bsel_kernel<8>;
 }
 typedef void (*ChainKernel)(const GpDev, int, int, int, const int*, int*, int*);
-template <int D> static ChainKernel chain_kernel_d(const GpDev& p) {
-  return p.G == 1 ? gp_chain_kernel<D, 1> : p.G == 2 ? gp_chain_kernel<D, 2> : p.G == 4 ? gp_chain_kernel<D, 4> : gp_chain_kernel<D, 8>;
+template <int D, bool LONG> static ChainKernel chain_kernel_d(const GpDev& p) {
+  return p.G == 1 ? gp_chain_kernel<D, 1, LONG> : p.G == 2 ? gp_chain_kernel<D, 2, LONG> : p.G == 4 ? gp_chain_kernel<D, 4, LONG> : gp_chain_kernel<D, 8, LONG>;
 }
-static ChainKernel chain_kernel_of(const GpDev& p) { return p.d == 128 ? chain_kernel_d<128>(p) : chain_kernel_d<64>(p); }
+static ChainKernel chain_kernel_of(const GpDev& p, bool clusters) {
+  if (clusters) return p.d == 128 ? chain_kernel_d<128, true>(p) : chain_kernel_d<64, true>(p);
+  return p.d == 128 ? chain_kernel_d<128, false>(p) : chain_kernel_d<64, false>(p);
+}
 
 // shared memory of the selection for a per-request page cap
 static size_t gp_sel_smem(const GpDev& p) {
@@ -1482,7 +1947,7 @@ static_assert(CMP_SMEM_BYTES <= sizeof(SelMisc) + DECIDE_SMEM, "the compaction's
 
 // one-time setup for a pool: opts the selection kernels into their shared memory and sizes the grids to at most one
 // resident wave, so that no CTA waits for another to leave before it can start
-void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain) {
+void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain, int* grid_long) {
   const size_t sel_sm = gp_sel_smem(p);
   auto blocks = [&](auto kern, int threads, size_t smem, int most) {
     if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1491,14 +1956,32 @@ void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_com
     return num_sms * (occ > most ? most : occ > 0 ? occ : 1);
   };
   *grid_sel = blocks(sel_kernel_of(p), SEL_T, sel_sm, 32);
-  *grid_chain = blocks(chain_kernel_of(p), SEL_T, sel_sm, 2);
+  *grid_chain = blocks(chain_kernel_of(p, false), SEL_T, sel_sm, 2);
+  // in clusters, where a request of this pool can have a unit that they share out: as many as are resident at once
+  *grid_long = 0;
+  if ((long long)p.cap * GP_PAGE > SPLIT_FROM && p.metric != GP_METRIC_ENTROPY && p.policy != GP_POLICY_SHRINK) {
+    const ChainKernel kern = chain_kernel_of(p, true);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CLUSTER; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(num_sms * 2 / CLUSTER * CLUSTER)); cfg.blockDim = dim3(SEL_T); cfg.dynamicSmemBytes = sel_sm;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_sm) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
+      *grid_long = (n * CLUSTER < num_sms * 2 ? n : num_sms * 2 / CLUSTER) * CLUSTER;
+    else
+      (void)cudaGetLastError();
+  }
   *grid_compact = blocks(compact_kernel_of(p), CT, 0, 32);
 }
 
 // the boundary chain of the step whose view is `p` (asynchronous mode: none when !has_chain)
 void gp_launch_chain(const GpDev& p, int n_req, int serial, int has_chain, int grid, cudaStream_t s, bool pdl, const int* req_ids,
-                     int* actions, int* actions_copy) {
-  gp_launch(chain_kernel_of(p), grid, SEL_T, gp_sel_smem(p), s, pdl, p, n_req, serial, has_chain, req_ids, actions, actions_copy);
+                     int* actions, int* actions_copy, bool clusters) {
+  gp_launch_clusters(clusters ? CLUSTER : 1, chain_kernel_of(p, clusters), grid, SEL_T, gp_sel_smem(p), s, pdl, p, n_req, serial, has_chain, req_ids,
+                     actions, actions_copy);
 }
 
 void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_sel, cudaStream_t s, bool pdl,

@@ -49,6 +49,8 @@ enum {
   HDR_N_CITEM,       // compaction work items (parts x layers x heads)
   HDR_N_COW,         // copy-on-write targets allotted this step
   HDR_N_BRC,         // (request, chunk) work items of requests at their boundary: the first of the list
+  HDR_WORK_SPLIT,    // boundary work in clusters: units shared out over a cluster that have been drawn (cleared by the plan)
+  HDR_WORK_SEL,      // ... and its other jobs
   HDR_COUNT = 16
 };
 
@@ -270,27 +272,39 @@ __device__ __forceinline__ void gp_pdl_wait() { asm volatile("griddepcontrol.wai
 __device__ __forceinline__ void gp_pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t gp_launch(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl,
-                             Args&&... args) {
+inline cudaError_t gp_launch_clusters(int cluster, void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl,
+                                      Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
   cfg.dynamicSmemBytes = smem; cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at; cfg.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t gp_launch(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl,
+                             Args&&... args) {
+  return gp_launch_clusters(1, kern, grid, block, smem, s, pdl, static_cast<Args&&>(args)...);
 }
 #endif
 
 void gp_attention_setup(const GpDev& p);
 void gp_launch_chain(const GpDev& p, int n_req, int serial, int has_chain, int grid, cudaStream_t s, bool pdl,
-                     const int* req_ids = nullptr, int* actions = nullptr, int* actions_copy = nullptr);
+                     const int* req_ids = nullptr, int* actions = nullptr, int* actions_copy = nullptr, bool clusters = false);
 void gp_launch_select_only(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_sel, cudaStream_t s, bool pdl,
                            int serial);
 void gp_launch_decide_compact(const GpDev& p, const int* req_ids, int n_req, int* actions, int grid_compact, cudaStream_t s,
                               int serial);
-void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain);
+void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_compact, int* grid_chain, int* grid_long);
 #define GP_MAX_DYN_SMEM (227 * 1024)   // opt-in shared memory per CTA on sm_100
 // boundary chain: probabilities + working sets + selection + decision, then compaction.
 // `ev`, when not null, is recorded between the two kernels.  `pdl`: launch with programmatic stream serialization.

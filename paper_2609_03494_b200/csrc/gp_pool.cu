@@ -34,6 +34,8 @@ struct gp_pool {
   std::vector<uint8_t> live;      // host mirror of the slot free list
   int num_sms, attn_grid, sel_grid, compact_grid;
   int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
+  int chain_grid_long;                              // ... in clusters that share out units of many candidates (0: no request can have them)
+  bool chain_clusters;                              // the path is launched that way
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
   int plain_plan;                                   // a request was released or a step abandoned since the last plan: the next launch
                                                     // of one that runs (LAUNCH_RUNS) or is captured (LAUNCH_CAPTURED) waits for it
@@ -337,6 +339,7 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
   // decisions waited for it, or, where it was abandoned before it had any, this launch did)
 #pragma unroll 1
   for (int idx = threadIdx.x; idx < 2 * p.L; idx += blockDim.x) p.tickets[idx] = 0;
+  if (i == 0) p.hdr[HDR_WORK_SPLIT] = p.hdr[HDR_WORK_SEL] = 0;           // (the boundary work before drew from these until it let this kernel be scheduled)
   __syncthreads();
   int chunks = 0, pages = 0, act = GP_ACT_NONE;
   const int n_old = st.x, Pr = st.y, pos = st.z;
@@ -798,7 +801,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   d.scores = reinterpret_cast<double*>(base + L.scores);
   d.counters = reinterpret_cast<long long*>(base + L.counters);
   gp_attention_setup(d);
-  gp_boundary_setup(d, pool->num_sms, &pool->sel_grid, &pool->compact_grid, &pool->chain_grid_max);
+  gp_boundary_setup(d, pool->num_sms, &pool->sel_grid, &pool->compact_grid, &pool->chain_grid_max, &pool->chain_grid_long);
   pool->dev_alt = d;
   pool->chain_pending = 0;
   pool->last_stream = nullptr;
@@ -820,6 +823,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   }
   pool->attn_grid_ov = pool->attn_grid;
   pool->chain_grid_ov = 0;
+  pool->chain_clusters = false;
   // How the boundary work of a step is launched where the caller leaves it open.  One kernel behind the attention kernel saves a kernel
   // boundary and starts its jobs while the attention kernel drains (us per step, four kernels / one, layers x requests, 8 KV heads:
   // 1 x 64 73.5 / 65.7; 8 x 16 91 / 87; 36 x 4 84 / 83; 36 x 16 314 / 310); from about ten thousand units on the two kernels'
@@ -828,7 +832,8 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   int slots = cfg->overlap_slots;
   if (slots == 0) slots = units <= 8192 ? -2 : -1;
   if (!cfg->async_boundary && slots == -2) {
-    pool->chain_grid_ov = pool->chain_grid_max;    // the whole grid, behind the attention kernel's
+    pool->chain_clusters = pool->chain_grid_long > 0;
+    pool->chain_grid_ov = pool->chain_clusters ? pool->chain_grid_long : pool->chain_grid_max;    // the whole grid, behind the attention kernel's
   } else if (!cfg->async_boundary && slots > 0) {
     if (slots > pool->attn_grid / 2) slots = pool->attn_grid / 2;
     pool->attn_grid_ov = pool->attn_grid - slots;
@@ -971,7 +976,7 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
       if (prof) cudaEventRecord(pool->ev[1], s);
       gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0, false, false, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
-      gp_launch_chain(d, n_req, serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy);
+      gp_launch_chain(d, n_req, serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy, pool->chain_clusters);
       if (prof) { cudaEventRecord(pool->ev[3], s); cudaEventRecord(pool->ev[4], s); }    // the last interval stays empty
       pool->launch_count += 3;
     } else {

@@ -1,0 +1,58 @@
+"""Boundary units of many candidates, shared out over the thread blocks of a cluster: around the size where that begins, at counts that
+leave the last blocks a short part or none, for every group size, head dimension and page size, and where all scores are equal."""
+import numpy as np
+import pytest
+
+from paper_2609_03494_b200 import binding as B
+from paper_2609_03494_b200 import workload as W
+from tests import lockstep as LS
+
+pytestmark = pytest.mark.gpu
+
+
+# A request of P pages of b tokens has P b - 16 candidates; units are shared out above 10 240.  Eight blocks take whole pages each for the softmax
+# and whole blocks of Eq. 10, and words of 32 candidates, for the descents.
+@pytest.mark.parametrize("hq,hkv,d,page,prompt,rope", [
+    (4, 2, 64, 16, 10237, 0.0), (4, 2, 64, 16, 10256, 0.0), (2, 2, 128, 16, 10269, 1e6), (8, 1, 128, 16, 10493, 0.0), (8, 1, 64, 16, 11192, 1e6),
+    (8, 2, 128, 64, 10363, 0.0), (8, 2, 64, 128, 11262, 0.0), (8, 2, 64, 256, 10492, 0.0), (8, 1, 64, 256, 12282, 1e6)])
+def test_shared_units_against_the_oracle(hq, hkv, d, page, prompt, rope):
+    P = prompt // page + 1
+    s = W.Shape(1, hq, hkv, d, page_size=page)
+    reqs = [W.RequestSpec(i, n, P * page - prompt + 3 + i, 0.05, share_group=-1) for i, n in enumerate((prompt, prompt - 5))]
+    wl = W.Workload("shared", 11, s, reqs, n_resident=2, initial_pages=0, max_pages_per_req=P + 1, n_pages=2 * P, k_loc=page // 4)
+    st = LS.run_lockstep(wl, tau=-1.0, rope_theta=rope, check_pool_every=16)
+    assert st.decisions["sel"] > 0 and st.near_ties == {"ws": 0, "sel": 0, "act": 0}
+
+
+@pytest.mark.parametrize("page,P", [(16, 643), (16, 675), (64, 163), (256, 43)])
+def test_equal_scores_of_shared_units_go_by_slot(page, P):
+    """Keys of zero make every score equal: the working sets are ceil(0.99 n), every block keeps its first k_loc slots and the
+    last `page` of the other candidates go."""
+    import torch
+    rng = np.random.default_rng(3)
+    L, hq, hkv, d, k_loc = 1, 8, 2, 64, page // 4
+    n = P * page - 1
+    pool = B.Pool(B.make_config(L, hq, hkv, d, n_pages=P, max_pages_per_req=P, max_requests=4, k_loc=k_loc, tau=1.0, page_size=page))
+    try:
+        zero = np.zeros((L, n, hkv, d), dtype=np.uint16)
+        vals = W.f32_to_bf16_bits(rng.standard_normal((L, n, hkv, d)).astype(np.float32))
+        assert pool.request_add(-1, 0, zero, vals, n, 0)[0] == B.GP_OK
+        dev = lambda a: torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).cuda()
+        q = W.f32_to_bf16_bits(rng.standard_normal((L, 1, hq, d)).astype(np.float32))
+        out = torch.zeros((L, 1, hq, d), dtype=torch.float32, device="cuda")
+        act = torch.zeros(1, dtype=torch.int32, device="cuda")
+        pool.decode_step(torch.zeros(1, dtype=torch.int32, device="cuda"), dev(q), dev(zero[:, :1]), dev(vals[:, :1]), out, act)
+        assert act.tolist() == [B.GP_ACT_COMPRESS]
+        n_d, n_e = (P - 1) * page, P * page - 16
+        ks, kl, _ = B.gp_debug_boundary(pool.handle, 0, L, hkv)
+        # 0.99 n is not a whole number at these sizes, so rounding of the n equal weights cannot move the count
+        assert (ks == -(-99 * n_d // 100)).all() and (kl == ks).all()
+        quota = min(k_loc, (n_e - page) // -(-n_e // page))
+        slots_left = np.arange(n_e)
+        rest = slots_left[slots_left % page >= quota]
+        want = np.setdiff1d(np.arange(P * page), rest[len(rest) - page:])
+        for h in range(hkv):
+            assert np.array_equal(B.gp_debug_retained(pool.handle, 0, 0, h, want.size), want)
+        assert B.gp_debug_pool(pool.handle)[2][7] == 0
+    finally:
+        pool.close()
