@@ -92,6 +92,7 @@ inline size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 // with 16 requests, layer by layer, 1030 us per step that way, 1252 with the large items; a layer is one launch now, 900 us).
 constexpr int GP_CHUNK = 64, GP_BCHUNK = 32;
 constexpr int GP_FINE_CHUNK = 32, GP_FINE_BCHUNK = 8;
+constexpr int GP_WIDE_BCHUNK = 16;       // few boundary tiles of groups of eight (see the plan kernel)
 int chunk_pages_setting() { return GP_CHUNK; }
 int bchunk_pages_setting() { return GP_BCHUNK; }
 
@@ -372,6 +373,11 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     // (groups of eight: 24 000 cycles an item, 3000 a tile in items of 32).  us of the attention kernel, items of 32 / 64: 64 layers x 32 requests, groups of
     // eight, two at a boundary 1636 / 1573, four 1843 / 1782; 36 x 256, 16 at a boundary 3884 / 3866, 22 4046 / 3972.  With few of them the items are
     // too long for the selection behind them: one layer x 64, four at a boundary 46 / 57; 36 x 4, one, 77.4 / 77.9 us a step.
+    // In small items for groups of eight, whose boundary tiles take a consumer warp 15 000 cycles each, where there are few of them: what the step then waits
+    // for is the longest (64 requests of 128 to 1400 tokens on one layer 84.4 / 79.8 us a step; 20 on eight layers 153.4 / 154.8 if it were not for
+    // the bound; groups of four 62.9 / 64.3).
+    if (p.G == 8 && cp_bnd > GP_WIDE_BCHUNK && (long long)s_bpages * launch_units < 8LL * launch_grid && s_pages / GP_WIDE_BCHUNK + n_req <= p.max_rc)
+      cp_bnd = GP_WIDE_BCHUNK;
     // (Not where the items, cut the smaller way, might not fit the scratch: who is refused below stays who was.)
     if ((long long)s_bpages * launch_units >= 2LL * cp_norm * launch_grid && s_pages / cp_bnd + n_req <= p.max_rc) cp_bnd = cp_norm;
     if ((long long)s_pages * launch_units < (long long)cp_norm * launch_grid) { cp_norm = GP_FINE_CHUNK; cp_bnd = GP_FINE_BCHUNK; }
