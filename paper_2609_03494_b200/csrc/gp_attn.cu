@@ -31,10 +31,7 @@
 //               them all, in the order of the chunks.
 //               Consumers hand over through a double buffer and go straight on to the next item.
 //
-// The two warp groups re-split the register file (setmaxnreg): the service warps keep 80 registers per
-// thread, the consumers, which hold the output accumulators, get 176 (at 160 their loop spills: 13.8 ms against 12.0 on
-// pages of 256).  At this split the kernel still spills: 60 bytes a thread at d = 64, 128 to 184 at d = 128.  All of it at d = 64 and
-// most at d = 128 is the merge of split outputs (a service warp, once per split unit); without it 24 to 72 bytes are left.
+// The two warp groups re-split the register file (setmaxnreg; 256 registers for a thread of each as launched): see SERVICE_REGS.
 // All waits are bounded; a wait that gives up sets an error bit (with a code for which wait it was) and an
 // abort flag that drains the CTA.  No wait of an item depends on a later item being published.
 #include "gp_dev.cuh"
@@ -45,8 +42,6 @@ constexpr int NI = 4;                      // item slots per CTA
 constexpr int NSW = 2;                     // tile stages per consumer warp (at most 3: see the wait in the tile loop)
 constexpr int NCW = 4;                     // consumer warps
 constexpr int NTHREADS = 256;              // warp group 0: producer, summaries, merger, summaries; warp group 1: consumers
-constexpr int REGS_SERVICE = 80;           // registers per thread after the split (setmaxnreg): 128 x (80 + 176) as launched
-constexpr int REGS_CONSUMER = 176;
 constexpr int NSUM = 2;                    // summary warps
 constexpr int MERGE_FAN = 8;               // partial outputs merged at a time
 constexpr double QT_SCALE = 0x1p880;       // of the q~ buffer: see bf16_lo_scaled
@@ -421,6 +416,12 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   // tokens, layer by layer: 864 us per step with every launch waiting at its top, now 760; with an ordinary kernel of 3 us before each
   // layer 999, now 925.  In the whole step's kernel the rows share the descriptor's barrier: two barriers there cost 1 to 2 %.)
   constexpr bool LAYER = MODE != WHOLE_STEP, NORM = MODE == ONE_LAYER_NORM;
+  // Registers of a service thread; the consumers, which hold the output accumulators, get the rest of 256.  At 80 it is the merge and the summaries that
+  // spill (140 to 180 bytes a thread at d = 128), at 88 48 to 64, at 96 0 to 16, at 104 the consumers again.  us of a step at 72 / 80 / 88 / 96 / 104:
+  // one layer x 64 requests 63.1 / 62.7 / 62.4 / 62.3 / 64.7, 150 of 100 to 500 tokens 65.0 / 64.4 / 63.5 / 63.1 / 67.3, d = 64 52.0 / 51.1 / 51.0 / 51.2 / 51.1;
+  // a layer by itself (4 steps x 36) 3089 / 3025 / 2964 / 3005 / 3311 (groups of eight, us a layer, 28.9 at 80, 27.5 at 88); groups of eight on 8 layers x 20 154.9 / 152.4 / 157 / 148.5 / 160.9, and with
+  // rotary embeddings (64 layers x 32, no request / two at a boundary) 1340 / 1312 / 1305 / 1303 and 1590 / 1565 / 1598 / 1623.
+  constexpr int SERVICE_REGS = D == 64 || LAYER ? 88 : WIDE && ROPE ? 80 : 96;
   using GEO = Geo<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + (-smem_u32(smem_raw) & (SMEM_ALIGN - 1u));
@@ -474,9 +475,9 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   const int q_bytes = G * GEO::ROW_BYTES;
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SERVICE_REGS));
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_CONSUMER));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(256 - SERVICE_REGS));
   }
   if (warp == 0) {
     // ================================= producer ===========================================
