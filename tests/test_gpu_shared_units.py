@@ -56,3 +56,56 @@ def test_equal_scores_of_shared_units_go_by_slot(page, P):
         assert B.gp_debug_pool(pool.handle)[2][7] == 0
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("how", ["early plan", "graph", "four kernels"])
+def test_shared_units_whatever_way_the_steps_are_launched(how):
+    """Every plan clears the counters the boundary work draws its jobs from: also one that starts beside the compaction, and one that is
+    replayed.  The kernel that takes such units on one thread block each gives the same."""
+    import torch
+    L, hq, hkv, d, steps = 2, 4, 2, 64, 36
+    lens = (10300, 10270, 300)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    rand = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    prompts = [(rand(L, n, hkv, d), rand(L, n, hkv, d)) for n in lens]
+    qs, ks, vs = rand(steps, L, 3, hq, d), rand(steps, L, 3, hkv, d), rand(steps, L, 3, hkv, d)
+    pages = sum(n // 16 + 1 for n in lens)
+
+    def run(how):
+        pool = B.Pool(B.make_config(L, hq, hkv, d, n_pages=pages + 1, max_pages_per_req=max(lens) // 16 + 3, max_requests=4, tau=-1.0,
+                                    overlap_slots=-1 if how == "four kernels" else 0))
+        try:
+            for (k, v), n in zip(prompts, lens):
+                assert pool.request_add(-1, 0, k, v, n, 0)[0] == B.GP_OK
+            B.gp_set_early_plan(pool.handle, how == "early plan")
+            ids = torch.arange(3, dtype=torch.int32, device="cuda")
+            out = torch.zeros((L, 3, hq, d), dtype=torch.float32, device="cuda")
+            act = torch.zeros(3, dtype=torch.int32, device="cuda")
+            q, k, v = qs[0].clone(), ks[0].clone(), vs[0].clone()
+            outs, acts, graph = [], [], None
+            if how == "graph":
+                side = torch.cuda.Stream()
+                side.wait_stream(torch.cuda.current_stream())
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=side):
+                    pool.decode_step(ids, q, k, v, out, act)
+            torch.cuda.synchronize()
+            for t in range(steps):
+                if graph is not None:
+                    q.copy_(qs[t]); k.copy_(ks[t]); v.copy_(vs[t])
+                    graph.replay()
+                else:
+                    pool.decode_step(ids, qs[t], ks[t], vs[t], out, act)
+                outs.append(out.clone()); acts.append(act.clone())
+            torch.cuda.synchronize()
+            n = B.gp_debug_state(pool.handle, 4)[1]
+            kept = [B.gp_debug_retained(pool.handle, r, l, h, int(n[r])) for r in range(3) for l in range(L) for h in range(hkv)]
+            assert B.gp_pool_status(pool.handle) == (B.GP_OK, 0)
+            return torch.stack(outs).cpu().numpy(), torch.stack(acts).cpu().numpy(), kept
+        finally:
+            pool.close()
+
+    want, got = run("plain"), run(how)
+    assert (want[1][:, :2] != 0).sum() >= 4                            # both long requests at boundaries, growing and compressing
+    assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
+    assert all(np.array_equal(a, b) for a, b in zip(want[2], got[2]))
