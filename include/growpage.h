@@ -373,7 +373,7 @@ int gp_debug_entropy(gp_pool* pool, int32_t req, double* H_S, double* H_L);
  * [5] decode steps [6] tokens decoded [7] internal error bits (0 when healthy)
  * [8] retained (layer, head, token) rows whose place in the order of the tokens a compaction changed, or
  * that it copied (of the former it moves a page per unit at most) [9] candidate tokens scored at boundaries
- * [10] Shrink events (not counted under [1]) [11] reserved. */
+ * [10] Shrink events (not counted under [1]) [11] boundary units shared out over a cluster of thread blocks. */
 int gp_debug_pool(gp_pool* pool, int64_t* n_free, int32_t* refcounts, int64_t counters[12]);
 
 /* ---- measurement ----------------------------------------------------------------------------- */

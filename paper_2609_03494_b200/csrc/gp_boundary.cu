@@ -1830,6 +1830,7 @@ gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_
         last |= s_i[2] != 0;
       };
       if (n_sh > 0) {
+        cluster_sync();                                    // every block of the cluster has started: another's shared memory may be written from here on
 #pragma unroll 1
         for (;;) {
           if (cluster_rank() == 0 && tid == 0) {
@@ -1844,7 +1845,10 @@ gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_
           const int4 inf = p.bnd_info[2 * bidx], inf2 = p.bnd_info[2 * bidx + 1];
           unit_there(bidx, lh, inf2.z);
           sel_split<GG>(p, S, bidx, lh, inf, inf2);
-          if (cluster_rank() == 0) done();
+          if (cluster_rank() == 0) {
+            if (tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(p.counters + 11), 1ull);
+            done();
+          }
         }
       }
 #pragma unroll 1

@@ -109,3 +109,56 @@ def test_shared_units_whatever_way_the_steps_are_launched(how):
     assert (want[1][:, :2] != 0).sum() >= 4                            # both long requests at boundaries, growing and compressing
     assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
     assert all(np.array_equal(a, b) for a, b in zip(want[2], got[2]))
+
+
+def _decode(layers, hq, hkv, d, lens, steps, page=16, k_loc=4, tau=-1.0, four=False, edit=None, spin_limit=0, withhold=0):
+    """Decodes `steps` tokens of requests of these lengths in a pool with one page to spare.  Everything a step decides, and how many units were
+    shared out (`four`: the kernels that never do)."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(4)
+    rand = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    pages = [n // page + 1 for n in lens]
+    pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(pages) + 1, max_pages_per_req=max(pages) + 2, max_requests=len(lens), k_loc=k_loc,
+                                tau=tau, page_size=page, overlap_slots=-1 if four else 0))
+    try:
+        for i, n in enumerate(lens):
+            k, v = rand(layers, n, hkv, d), rand(layers, n, hkv, d)
+            if edit:
+                edit(i, k, v)
+            assert pool.request_add(-1, 0, k, v, n, 0)[0] == B.GP_OK
+            del k, v
+        if spin_limit:
+            B.gp_test_withhold(pool.handle, withhold, spin_limit)
+        R = len(lens)
+        ids = torch.arange(R, dtype=torch.int32, device="cuda")
+        outs, acts = [], []
+        for _ in range(steps):
+            out = torch.zeros((layers, R, hq, d), dtype=torch.float32, device="cuda")
+            act = torch.zeros(R, dtype=torch.int32, device="cuda")
+            pool.decode_step(ids, rand(layers, R, hq, d), rand(layers, R, hkv, d), rand(layers, R, hkv, d), out, act)
+            outs.append(out); acts.append(act)
+        torch.cuda.synchronize()
+        n = B.gp_debug_state(pool.handle, R)[1]
+        return dict(out=torch.stack(outs).cpu().numpy(), act=torch.stack(acts).cpu().numpy(), status=B.gp_pool_status(pool.handle),
+                    sets=[B.gp_debug_boundary(pool.handle, r, layers, hkv)[:2] for r in range(R)],
+                    kept=[B.gp_debug_retained(pool.handle, r, l, h, int(n[r])) for r in range(R) for l in range(layers) for h in range(hkv)],
+                    state=[B.gp_debug_request(pool.handle, r, max(pages) + 2) for r in range(R)], shared=int(B.gp_debug_pool(pool.handle)[2][11]))
+    finally:
+        pool.close()
+
+
+def _same(a, b):
+    assert a["status"] == b["status"] and np.array_equal(a["act"], b["act"])
+    assert all(np.array_equal(x, y) for s, t in zip(a["sets"], b["sets"]) for x, y in zip(s, t))
+    assert len(a["kept"]) == len(b["kept"]) and all(np.array_equal(x, y) for x, y in zip(a["kept"], b["kept"]))
+    assert np.array_equal(a["out"], b["out"], equal_nan=True)
+
+
+@pytest.mark.parametrize("hq,d", [(8, 64), (64, 64), (16, 128)])
+def test_more_shared_units_than_clusters(hq, d):
+    """48 units on at most 37 clusters (two blocks on each of 148 SMs): some clusters draw a second one, in the place of the first.  Two units one after the
+    other are shared out from 20 480 candidates on.  The second step is a boundary that takes the spare page, the eighteenth one that evicts."""
+    got, want = (_decode(6, hq, 8, d, [1302 * 16 - 2], 20, four=four) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (2 * 48, 0) and got["status"] == (B.GP_OK, 0)
+    assert [t for t in range(20) if got["act"][t, 0]] == [1, 17]
+    _same(got, want)
