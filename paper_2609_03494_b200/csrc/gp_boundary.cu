@@ -888,7 +888,9 @@ __device__ __forceinline__ void sel_unit(const GpDev& p, const SelSmem& S, int b
 // What bounds it: the logits' bytes, then a chain of a dozen cluster barriers.  Two requests of 20 000, us a step: one layer, groups of eight
 // 101.6 / 79.7, of four 76.3 / 65.0; four layers 184.9 / 161.2 and 147.1 / 138.3.
 constexpr int CLUSTER = 8;
-constexpr int SPLIT_FROM = 2 * SEL_CAP;     // candidates above which a unit is shared out: see split_unit
+constexpr int SPLIT_ROUNDS = 2;             // units a cluster takes one after the other at most
+constexpr int SPLIT_FROM = GP_SHARED_FROM;  // candidates above which a unit is shared out: see split_unit
+static_assert(SPLIT_FROM == 2 * SEL_CAP, "up to there the scores of a job fit one thread block's shared memory");
 __device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ void cluster_sync() {
   __syncwarp();
@@ -1213,7 +1215,7 @@ __device__ __forceinline__ int split_part(const GpDev& p, int n) {
 __device__ __forceinline__ bool split_unit(const GpDev& p, const SelSmem& S, int Pr, long long units, int clusters) {
   const long long rounds = (units + clusters - 1) / clusters;
   const int n = (Pr - 1) * GP_PAGE;
-  return rounds <= 2 && n > SPLIT_FROM * rounds && split_part(p, n) <= S.n_cap && ((n / GP_PAGE + CLUSTER - 1) / CLUSTER + 1) * GP_PAGE <= 2 * S.n_cap &&
+  return rounds <= SPLIT_ROUNDS && n > SPLIT_FROM * rounds && split_part(p, n) <= S.n_cap && ((n / GP_PAGE + CLUSTER - 1) / CLUSTER + 1) * GP_PAGE <= 2 * S.n_cap &&
          p.metric != GP_METRIC_ENTROPY && p.policy != GP_POLICY_SHRINK;
 }
 
@@ -1977,6 +1979,8 @@ void gp_boundary_setup(const GpDev& p, int num_sms, int* grid_sel, int* grid_com
       *grid_long = (n * CLUSTER < num_sms * 2 ? n : num_sms * 2 / CLUSTER) * CLUSTER;
     else
       (void)cudaGetLastError();
+    // (one request alone must not have more units than the clusters may take; see split_unit)
+    if ((long long)p.L * p.Hkv > (long long)SPLIT_ROUNDS * (*grid_long / CLUSTER)) *grid_long = 0;
   }
   *grid_compact = blocks(compact_kernel_of(p), CT, 0, 32);
 }

@@ -28,6 +28,7 @@
 #define GP_MAX_TILES_PER_REQ 61773   // 16-token tiles a request may hold: the selection keeps a bit per candidate in shared memory
 #define GP_SPIN_LIMIT (1u << 21)
 #define GP_MAX_REQ 1024        // upper limit of max_requests (shared-memory arrays are sized by it)
+#define GP_SHARED_FROM 10240   // candidates above which a boundary unit may be shared out over a cluster of thread blocks
 #define GP_PART_LOG 12         // 4096 slots per compaction ticket: units beyond that are shared out (a unit of 20 000 slots in one block: 15 us of loads)
 #define GP_PART_LOG_MIN 6      // ... 64 in tests
 #define GP_PART_LOG_UNIT 20    // ... and no bound (GP_MAX_TILES_PER_REQ tiles)

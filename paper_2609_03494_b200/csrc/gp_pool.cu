@@ -35,7 +35,11 @@ struct gp_pool {
   int num_sms, attn_grid, sel_grid, compact_grid;
   int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
   int chain_grid_long;                              // ... in clusters that share out units of many candidates (0: no request can have them)
-  bool chain_clusters;                              // the path is launched that way
+  bool chain_clusters;                              // the path is launched that way where a request may be that long
+  // A live request holds at most as many tokens as it was admitted with and steps have been issued since, unless a captured step is replayed.
+  std::vector<long long> began;                     // of each: tokens admitted with, less the steps issued before
+  long long began_max;                              // ... the most of the live ones
+  bool captured;                                    // a step was captured
   int step_open, step_n_req, step_layers_done;      // per-layer entry points: a step begun and not yet ended
   int plain_plan;                                   // a request was released or a step abandoned since the last plan: the next launch
                                                     // of one that runs (LAUNCH_RUNS) or is captured (LAUNCH_CAPTURED) waits for it
@@ -715,6 +719,9 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   pool->blob = dev_blob;
   pool->bytes = bytes;
   pool->live.assign(cfg->max_requests, 0);
+  pool->began.assign(cfg->max_requests, 0);
+  pool->began_max = 0;
+  pool->captured = false;
   pool->profiling = 0;
   pool->early_plan = 0;
   pool->first_plain = 0;
@@ -839,7 +846,7 @@ int gp_pool_create(const gp_config* cfg, void* dev_blob, size_t bytes, int devic
   if (slots == 0) slots = units <= 8192 ? -2 : -1;
   if (!cfg->async_boundary && slots == -2) {
     pool->chain_clusters = pool->chain_grid_long > 0;
-    pool->chain_grid_ov = pool->chain_clusters ? pool->chain_grid_long : pool->chain_grid_max;    // the whole grid, behind the attention kernel's
+    pool->chain_grid_ov = pool->chain_grid_max;    // the whole grid, behind the attention kernel's
   } else if (!cfg->async_boundary && slots > 0) {
     if (slots > pool->attn_grid / 2) slots = pool->attn_grid / 2;
     pool->attn_grid_ov = pool->attn_grid - slots;
@@ -928,6 +935,8 @@ int gp_request_add(gp_pool* pool, int32_t share_from, int32_t n_shared_pages, co
   const int st = *h_status;
   if (st != GP_OK) return st;
   pool->live[slot] = 1;
+  pool->began[slot] = n_prompt - pool->serial;
+  if (pool->began[slot] > pool->began_max) pool->began_max = pool->began[slot];
   *out_req = slot;
   return GP_OK;
 }
@@ -948,6 +957,7 @@ static void launch_plan(gp_pool* pool, const int32_t* ids, int32_t n_req, int32_
     const int mine = launch_kind(s);
     if (pool->plain_plan & mine) { early = false; pdl = false; pool->plain_plan &= ~mine; }
   }
+  if (pool->chain_clusters && !pool->captured) pool->captured = launch_kind(s) == LAUNCH_CAPTURED;
   gp_launch(gp_plan_kernel, 1 + table, threads, 0, s, pdl, d, ids, n_req, actions, early ? 1 : 0, d.chunk_pages, d.bchunk_pages,
             by_layer ? d.Hkv : d.L * d.Hkv, attn_grid ? attn_grid : pool->attn_grid, (int)(pool->serial & 0x3fffffff));
 }
@@ -982,7 +992,13 @@ int gp_decode_step(gp_pool* pool, const int32_t* dev_req_ids, int32_t n_req, con
       if (prof) cudaEventRecord(pool->ev[1], s);
       gp_launch_attention(d, n_req, q, k, v, static_cast<float*>(out), pool->attn_grid_ov, s, pdl, 0, LH, 0, false, false, kNoNorm);
       if (prof) cudaEventRecord(pool->ev[2], s);
-      gp_launch_chain(d, n_req, serial, 1, pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy, pool->chain_clusters);
+      // In clusters where a request may be long enough for one to share out its units: blocks that find their places eight at a time and draw their
+      // jobs are slower where none is.  us a step with requests of up to 1400 tokens that might grow to 16 000, in clusters / not, layers x
+      // requests: 1 x 64 65.8 / 62.7, at d = 64 54.4 / 51.3; four short ones 17.4 / 16.7; 36 x 16 312.5 / 295.2.  Replays of a captured step are not
+      // counted, so from the first capture on every launch is one in clusters.  The results are those of the other form.
+      const bool clusters = pool->chain_clusters && (pool->captured || pool->began_max + pool->serial > GP_SHARED_FROM);
+      gp_launch_chain(d, n_req, serial, 1, clusters ? pool->chain_grid_long : pool->chain_grid_ov, s, pdl, dev_req_ids, dev_actions, pool->actions_copy,
+                      clusters);
       if (prof) { cudaEventRecord(pool->ev[3], s); cudaEventRecord(pool->ev[4], s); }    // the last interval stays empty
       pool->launch_count += 3;
     } else {
@@ -1387,6 +1403,11 @@ int gp_release(gp_pool* pool, int32_t req, void* stream) {
   pool->launch_count++;
   pool->plain_plan |= launch_kind(static_cast<cudaStream_t>(stream));
   pool->live[req] = 0;
+  if (pool->began[req] == pool->began_max) {
+    pool->began_max = -pool->serial;
+    for (int i = 0; i < pool->cfg.max_requests; ++i)
+      if (pool->live[i] && pool->began[i] > pool->began_max) pool->began_max = pool->began[i];
+  }
   GP_CUDA(cudaGetLastError());
   return GP_OK;
 }

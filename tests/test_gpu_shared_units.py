@@ -111,14 +111,14 @@ def test_shared_units_whatever_way_the_steps_are_launched(how):
     assert all(np.array_equal(a, b) for a, b in zip(want[2], got[2]))
 
 
-def _decode(layers, hq, hkv, d, lens, steps, page=16, k_loc=4, tau=-1.0, four=False, edit=None, spin_limit=0, withhold=0):
-    """Decodes `steps` tokens of requests of these lengths in a pool with one page to spare.  Everything a step decides, and how many units were
+def _decode(layers, hq, hkv, d, lens, steps, page=16, k_loc=4, tau=-1.0, spare=1, four=False, graph=False, edit=None, spin_limit=0, withhold=0):
+    """Decodes `steps` tokens of requests of these lengths in a pool with `spare` free pages, one step captured and replayed with `graph`.  Everything a step decides, and how many units were
     shared out (`four`: the kernels that never do)."""
     import torch
     g = torch.Generator(device="cuda").manual_seed(4)
     rand = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
     pages = [n // page + 1 for n in lens]
-    pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(pages) + 1, max_pages_per_req=max(pages) + 2, max_requests=len(lens), k_loc=k_loc,
+    pool = B.Pool(B.make_config(layers, hq, hkv, d, n_pages=sum(pages) + spare, max_pages_per_req=max(pages) + 3, max_requests=len(lens), k_loc=k_loc,
                                 tau=tau, page_size=page, overlap_slots=-1 if four else 0))
     try:
         for i, n in enumerate(lens):
@@ -131,18 +131,27 @@ def _decode(layers, hq, hkv, d, lens, steps, page=16, k_loc=4, tau=-1.0, four=Fa
             B.gp_test_withhold(pool.handle, withhold, spin_limit)
         R = len(lens)
         ids = torch.arange(R, dtype=torch.int32, device="cuda")
-        outs, acts = [], []
+        out = torch.zeros((layers, R, hq, d), dtype=torch.float32, device="cuda")
+        act = torch.zeros(R, dtype=torch.int32, device="cuda")
+        ins = [torch.empty((layers, R, heads, d), dtype=torch.bfloat16, device="cuda") for heads in (hq, hkv, hkv)]
+        outs, acts, step = [], [], lambda: pool.decode_step(ids, *ins, out, act)
+        if graph:
+            side, g_step = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.graph(g_step, stream=side):
+                step()
+            step = g_step.replay
         for _ in range(steps):
-            out = torch.zeros((layers, R, hq, d), dtype=torch.float32, device="cuda")
-            act = torch.zeros(R, dtype=torch.int32, device="cuda")
-            pool.decode_step(ids, rand(layers, R, hq, d), rand(layers, R, hkv, d), rand(layers, R, hkv, d), out, act)
-            outs.append(out); acts.append(act)
+            for t in ins:
+                t.copy_(rand(*t.shape))
+            step()
+            outs.append(out.clone()); acts.append(act.clone())
         torch.cuda.synchronize()
         n = B.gp_debug_state(pool.handle, R)[1]
         return dict(out=torch.stack(outs).cpu().numpy(), act=torch.stack(acts).cpu().numpy(), status=B.gp_pool_status(pool.handle),
                     sets=[B.gp_debug_boundary(pool.handle, r, layers, hkv)[:2] for r in range(R)],
                     kept=[B.gp_debug_retained(pool.handle, r, l, h, int(n[r])) for r in range(R) for l in range(layers) for h in range(hkv)],
-                    state=[B.gp_debug_request(pool.handle, r, max(pages) + 2) for r in range(R)], shared=int(B.gp_debug_pool(pool.handle)[2][11]))
+                    state=[B.gp_debug_request(pool.handle, r, max(pages) + 3) for r in range(R)], shared=int(B.gp_debug_pool(pool.handle)[2][11]))
     finally:
         pool.close()
 
@@ -161,4 +170,40 @@ def test_more_shared_units_than_clusters(hq, d):
     got, want = (_decode(6, hq, 8, d, [1302 * 16 - 2], 20, four=four) for four in (False, True))
     assert (got["shared"], want["shared"]) == (2 * 48, 0) and got["status"] == (B.GP_OK, 0)
     assert [t for t in range(20) if got["act"][t, 0]] == [1, 17]
+    _same(got, want)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_requests_that_grow_into_shared_units(graph):
+    """Admitted with fewer tokens than a unit that is shared out: the third boundary has 10 256 candidates, after 42 steps or as many replays of one."""
+    got, want = (_decode(2, 8, 2, 64, [10230, 200], 43, spare=40, four=four, graph=graph and not four) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (4, 0) and got["status"] == (B.GP_OK, 0)
+    _same(got, want)
+
+
+def test_shared_units_of_a_request_admitted_by_reference():
+    """The donor has gone when the request that took its prompt by reference reaches its boundary."""
+    import torch
+    L, hq, hkv, d = 2, 8, 2, 64
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rand = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    pool = B.Pool(B.make_config(L, hq, hkv, d, n_pages=645, max_pages_per_req=644, max_requests=4, tau=1.0))
+    try:
+        assert pool.request_add(-1, 0, rand(L, 10260, hkv, d), rand(L, 10260, hkv, d), 10260, 0) == (B.GP_OK, 0)
+        assert pool.request_add(0, 641, rand(L, 15, hkv, d), rand(L, 15, hkv, d), 15, 0) == (B.GP_OK, 1)
+        pool.release(0)
+        out = torch.zeros((L, 1, hq, d), dtype=torch.float32, device="cuda")
+        act = torch.zeros(1, dtype=torch.int32, device="cuda")
+        pool.decode_step(torch.ones(1, dtype=torch.int32, device="cuda"), rand(L, 1, hq, d), rand(L, 1, hkv, d), rand(L, 1, hkv, d), out, act)
+        assert act.tolist() == [B.GP_ACT_COMPRESS]
+        counters = B.gp_debug_pool(pool.handle)[2]
+        assert counters[11] == L * hkv and counters[7] == 0
+    finally:
+        pool.close()
+
+
+def test_a_request_with_more_units_than_clusters_may_take():
+    """80 units: more than twice the clusters of a B200, so that pool never launches them."""
+    got, want = (_decode(10, 8, 8, 64, [10271], 2, tau=1.0, four=four) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (0, 0) and got["status"] == (B.GP_OK, 0) and got["act"][0, 0] == B.GP_ACT_COMPRESS
     _same(got, want)
