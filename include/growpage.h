@@ -410,9 +410,11 @@ int64_t gp_launch_count(gp_pool* pool);
 
 /* ---- test support --------------------------------------------------------------------------------------------- */
 
-/* Every wait of one thread block for another inside the kernels is bounded: after a number of iterations it gives
+/* Every wait of one thread block for a word that another writes is bounded inside the kernels: after a number of iterations it gives
  * up, sets an error bit (gp_pool_status) and the kernel runs to its end, with wrong results for the work concerned
- * but without hanging and with the pool's page accounting intact.  This call lets a test see that happen without
+ * but without hanging and with the pool's page accounting intact.  (The eight thread blocks of a cluster that share a long request's boundary
+ * units out also meet at the cluster's hardware barrier, which has no limit: they run at the same time and, whatever a bounded wait
+ * left behind, all reach the same barriers.)  This call lets a test see that happen without
  * any fault: `what` names hand-overs that are then simply not made (1 the attention kernel's first thread block
  * never completes its second work item for its consumer warps; 2 the compaction claims parts of 64 slots, and the first
  * part of every unit never says where its evicted slots lie; 4 the deciding thread block of the boundary kernel never tells

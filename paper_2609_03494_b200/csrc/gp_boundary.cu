@@ -892,6 +892,10 @@ constexpr int SPLIT_ROUNDS = 2;             // units a cluster takes one after t
 constexpr int SPLIT_FROM = GP_SHARED_FROM;  // candidates above which a unit is shared out: see split_unit
 static_assert(SPLIT_FROM == 2 * SEL_CAP, "up to there the scores of a job fit one thread block's shared memory");
 __device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+// The wait of the cluster's barrier has no limit, unlike those for a word that another block writes.  It ends because the eight blocks run at the same
+// time and reach the same barriers: what any of them branches on in between are the plan's words, the ticket, and sums that each
+// takes over all eight blocks' shared memory behind a barrier, the same in every block whatever the scores are.  So a wait with a limit (unit_there) that
+// gives up in one block alone changes what is in the scores and not where the blocks go.
 __device__ __forceinline__ void cluster_sync() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1090,15 +1094,20 @@ __device__ __forceinline__ void split_select(const GpDev& p, const SelSmem& S, c
         else if (lane >= o) ic += tu;                                          // lowest scores first
       }
       unsigned rc = before + ic - c; unsigned long long rs = mass + is - s;
-      bool hit = false;
+      int bin = -1;
+      unsigned bin_rc = 0, bin_c = 0; unsigned long long bin_rs = 0;
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
         const int j = task != 2 ? 7 - jj : jj;
         const bool here = task != 2 ? rs < p.p_fix && rs + m8[j] >= p.p_fix : rc < (unsigned)ne && rc + c8[j] >= (unsigned)ne;
-        if (here) { m.res[task][0] = lane * 8 + j; m.res[task][1] = rc; m.res[task][2] = (long long)rs; m.res[task][3] = c8[j]; hit = true; }
+        if (here) { bin = lane * 8 + j; bin_rc = rc; bin_rs = rs; bin_c = c8[j]; }
         rc += c8[j]; rs += m8[j];
       }
-      if (!__any_sync(0xffffffffu, hit) && lane == 0) m.res[task][0] = -1;
+      // (sums of scores that a wait that gave up left behind can wrap, and more than one lane find a crossing: one of them, the same in every block)
+      const unsigned found = __ballot_sync(0xffffffffu, bin >= 0);
+      if (lane == (found ? __ffs((int)found) - 1 : 0)) {
+        m.res[task][0] = bin; m.res[task][1] = bin_rc; m.res[task][2] = (long long)bin_rs; m.res[task][3] = bin_c;
+      }
     }
     __syncthreads();
     if (run) {

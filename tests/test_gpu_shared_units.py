@@ -207,3 +207,70 @@ def test_a_request_with_more_units_than_clusters_may_take():
     got, want = (_decode(10, 8, 8, 64, [10271], 2, tau=1.0, four=four) for four in (False, True))
     assert (got["shared"], want["shared"]) == (0, 0) and got["status"] == (B.GP_OK, 0) and got["act"][0, 0] == B.GP_ACT_COMPRESS
     _same(got, want)
+
+
+@pytest.mark.parametrize("what,bit", [(4, 8), (8, 16)])
+def test_waits_of_shared_units_that_run_out_are_reported(what, bit):
+    """The decisions never told to the waiting blocks (4), the logits never reported complete (8): every block of a cluster gives up by itself, meets
+    the others at the cluster's barriers all the same, and the pool steps on."""
+    import torch
+    L, hq, hkv, d, lens = 1, 8, 2, 64, (642 * 16 - 1, 643 * 16 - 1, 303)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    rand = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    pages = [n // 16 + 1 for n in lens]
+    pool = B.Pool(B.make_config(L, hq, hkv, d, n_pages=sum(pages), max_pages_per_req=643, max_requests=4, tau=1.0))
+    try:
+        for n in lens:
+            assert pool.request_add(-1, 0, rand(L, n, hkv, d), rand(L, n, hkv, d), n, 0)[0] == B.GP_OK
+        ids = torch.arange(3, dtype=torch.int32, device="cuda")
+        out = torch.zeros((L, 3, hq, d), dtype=torch.float32, device="cuda")
+        act = torch.zeros(3, dtype=torch.int32, device="cuda")
+        step = lambda: pool.decode_step(ids, rand(L, 3, hq, d), rand(L, 3, hkv, d), rand(L, 3, hkv, d), out, act)
+        B.gp_test_withhold(pool.handle, what, 2000)
+        step()
+        assert act.tolist() == [B.GP_ACT_COMPRESS] * 3
+        status, bits = B.gp_pool_status(pool.handle)
+        assert status == B.GP_ERR_CUDA and (bits & bit), bits
+        n_free, ref, counters = B.gp_debug_pool(pool.handle, sum(pages))
+        assert counters[11] == 2 * L * hkv and n_free == 0 and ref.tolist() == [1] * sum(pages)
+        assert [B.gp_debug_request(pool.handle, r, 643)[:2] for r in range(3)] == [(P, (P - 1) * 16) for P in pages]
+        B.gp_test_withhold(pool.handle, 0, 0)
+        step()
+        assert act.tolist() == [B.GP_ACT_NONE] * 3 and bool(torch.isfinite(out).all())
+    finally:
+        pool.close()
+
+
+# 8 x 5120 places for scores: 40 960 candidates are the most that a cluster takes; of two units one after the other more than 20 480 each.  With pages
+# of b > 16 tokens the larger of the two candidate sets counts: all but the protected window, P b - 16, where `cand` is (P - 1) b.
+@pytest.mark.parametrize("hq,d,page,cand,k_loc,shared", [
+    (8, 64, 16, 20000, 4, 1), (4, 128, 16, 20000, 0, 1), (1, 64, 16, 40960, 4, 1), (8, 128, 16, 40960, 16, 1), (8, 64, 256, 159 * 256, 64, 1),
+    (2, 64, 128, 319 * 128, 0, 1), (8, 64, 16, 40976, 4, 0), (4, 64, 256, 160 * 256, 64, 0)])
+def test_shared_units_up_to_the_largest(hq, d, page, cand, k_loc, shared):
+    n = cand + page - 1
+    got, want = (_decode(1, hq, 1, d, [n], 2, page=page, k_loc=k_loc, tau=1.0, four=four) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (shared, 0) and got["status"] == (B.GP_OK, 0) and got["act"][0, 0] == B.GP_ACT_COMPRESS
+    _same(got, want)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+def test_shared_units_with_keys_that_are_no_numbers(value):
+    """One key element of one unit.  What the unit's scores then are, and the lists made from them, is what one thread block makes of them."""
+    def edit(i, k, v):
+        if i == 0:
+            k[0, 5000, 1, 7] = value
+    got, want = (_decode(1, 8, 2, 64, [642 * 16 - 1, 643 * 16 - 1], 2, tau=1.0, four=four, edit=edit) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (4, 0)
+    _same(got, want)
+
+
+@pytest.mark.parametrize("long_at_boundary", [True, False])
+def test_shared_units_among_many_requests(long_at_boundary):
+    """40 requests at their boundary, two of them long (the 35th and 38th), or only short ones beside long requests that are not at theirs.  One unit
+    each: more than the clusters, so that a unit is shared out above 20 480 candidates."""
+    lens = [47 + 16 * (i % 18) for i in range(40)]
+    lens[34], lens[37] = (1302 * 16 - 1, 1310 * 16 - 1) if long_at_boundary else (1302 * 16 + 3, 1310 * 16 + 4)
+    got, want = (_decode(1, 8, 1, 64, lens, 3, tau=1.0, four=four) for four in (False, True))
+    assert (got["shared"], want["shared"]) == (2 if long_at_boundary else 0, 0) and got["status"] == (B.GP_OK, 0)
+    assert (got["act"][0] == B.GP_ACT_COMPRESS).sum() == (40 if long_at_boundary else 38)
+    _same(got, want)
