@@ -417,10 +417,12 @@ gp_attn_kernel(const __grid_constant__ GpDev p, int n_req, const __nv_bfloat16* 
   // layer 999, now 925.  In the whole step's kernel the rows share the descriptor's barrier: two barriers there cost 1 to 2 %.)
   constexpr bool LAYER = MODE != WHOLE_STEP, NORM = MODE == ONE_LAYER_NORM;
   // Registers of a service thread; the consumers, which hold the output accumulators, get the rest of 256.  At 80 it is the merge and the summaries that
-  // spill (140 to 180 bytes a thread at d = 128), at 88 48 to 64, at 96 0 to 16, at 104 the consumers again.  us of a step at 72 / 80 / 88 / 96 / 104:
+  // spill at d = 128 (140 bytes a thread for whole steps of groups of eight with rotary embeddings), at 88 52 to 96 bytes in a layer's launches, at 96 0 to 16
+  // in a whole step's, at 104 the consumers again; nothing at d = 64.  us of a step at 72 / 80 / 88 / 96 / 104 for all launches:
   // one layer x 64 requests 63.1 / 62.7 / 62.4 / 62.3 / 64.7, 150 of 100 to 500 tokens 65.0 / 64.4 / 63.5 / 63.1 / 67.3, d = 64 52.0 / 51.1 / 51.0 / 51.2 / 51.1;
-  // a layer by itself (4 steps x 36) 3089 / 3025 / 2964 / 3005 / 3311 (groups of eight, us a layer, 28.9 at 80, 27.5 at 88); groups of eight on 8 layers x 20 154.9 / 152.4 / 157 / 148.5 / 160.9, and with
-  // rotary embeddings (64 layers x 32, no request / two at a boundary) 1340 / 1312 / 1305 / 1303 and 1590 / 1565 / 1598 / 1623.
+  // a layer by itself (4 steps x 36) 3089 / 3025 / 2964 / 3005 / 3311 (groups of eight, us a layer, 28.9 at 80, 27.5 at 88); groups of eight on 8 layers x 20
+  // 154.9 / 152.4 / 157 / 148.5 / 160.9.  Groups of eight with rotary embeddings at 72 / 80 / 88 / 96: 64 layers x 32 1630 / 1607 / 1611 / 1623,
+  // 8 x 20 158.5 / 156.0 / 155.8 / 157.1, one layer x 64 80.2 / 79.2 / 78.8 / 79.5, 4 x 4 of 2000 to 8000 tokens 104.0 / 103.8 / 104.2 / 105.1.
   constexpr int SERVICE_REGS = D == 64 || LAYER ? 88 : WIDE && ROPE ? 80 : 96;
   using GEO = Geo<D>;
   extern __shared__ uint8_t smem_raw[];

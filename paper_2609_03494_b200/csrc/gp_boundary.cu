@@ -33,8 +33,8 @@
 //
 // Size of the code: a step of a few units runs these functions once per thread block, and what they then cost is the fetch of their
 // instructions.  So loops whose trips are not the point are kept from being unrolled (`unroll 1`; the compiler unrolled the loop over the two
-// supports, and the decisions' loops four to eight times): gp_chain_kernel<128, 4> 258 -> 170 KB, the compaction 62 -> 52, the decisions
-// 26 -> 17.  us a pass before / now: one layer x 64 requests, 16 steps, 1067 / 1039; four requests, 16 steps, 267 / 259; 256 requests copied
+// supports, and the decisions' loops four to eight times): gp_chain_kernel<128, 4> 258 -> 170 KB (its form in clusters, which holds both ways of taking a unit,
+// 272), the compaction 62 -> 52, the decisions 26 -> 17.  us a pass before / now: one layer x 64 requests, 16 steps, 1067 / 1039; four requests, 16 steps, 267 / 259; 256 requests copied
 // on write in one of 24 steps 14 315 / 13 979; 36 layers x 16, 16 steps, 4912 / 4897.
 #include "../../include/growpage.h"
 #include "gp_dev.cuh"
@@ -1216,11 +1216,15 @@ __device__ __forceinline__ int split_part(const GpDev& p, int n) {
   const int align = p.blk > 32 ? p.blk : 32;
   return ((n + CLUSTER - 1) / CLUSTER + align - 1) / align * align;
 }
-// Whether the unit of a request with `Pr` pages is shared out, `units` of them in the step and `clusters` of the grid.  The line: up to 10 240
+// Whether the units of a boundary request with `Pr` pages are shared out, in a step with `units` of all its boundary requests, on a grid of `clusters`.  The line: up to 10 240
 // candidates the scores of a job fit one block's shared memory, and three blocks by themselves take no longer than the cluster's chain of
 // barriers (two requests of 7000, one layer, groups of four / eight, us a step, by themselves 36.6 / 49.9, shared 36.4 / 45.5; of 4500 33.1 / 43.2 and
 // 34.3 / 42.6; four layers of 7000 64.3 / 67.5), of 12 000 57.5 / 52.1 and 79.2 / 66.4; and a cluster takes its units one after the other, so that with
-// three for each (12 layers of 12 000: 220 / 227, of 20 000 344 / 344) nothing is left of it.
+// three for each (12 layers of 12 000: 220 / 227, of 20 000 344 / 344) nothing is left of it.  Two units one after the other have to be of more than 20 480.
+// The upper end: a block's part of the scores has to fit its shared memory, an eighth of 40 960 candidates (us of a step with
+// a boundary at 40 960 / 40 976 / 60 000, one layer of 8 KV heads, groups of four 196 / 374 / 532, of eight 286 / 601 / 871).  A unit above that, and every unit of the
+// entropy metric (a sum of logarithms in a fixed order), of Shrink (two eviction lists) and of the kernels launched one after the other, is one block's, or
+// three blocks'.
 __device__ __forceinline__ bool split_unit(const GpDev& p, const SelSmem& S, int Pr, long long units, int clusters) {
   const long long rounds = (units + clusters - 1) / clusters;
   const int n = (Pr - 1) * GP_PAGE;
@@ -1336,8 +1340,9 @@ __device__ __forceinline__ bool last_of_the_jobs(const GpDev& p, long long jobs,
 }
 
 // The selection as a kernel of its own.  Two thread blocks to an SM at 128 registers; three at 80 spill and are slower
-// (20 000 cycles per unit become 36 000).  Groups of eight spill at 128 as well (240 bytes a thread here, 192 in gp_chain_kernel: the
-// values of a token, eight per view, are loaded two tokens ahead), the smaller groups by 8 to 24 bytes.
+// (20 000 cycles per unit become 36 000).  Groups of eight spill at 128 as well (236 bytes a thread here, 268 in gp_chain_kernel, 244 in its form in clusters:
+// the values of a token, eight per view, are loaded two tokens ahead), the smaller groups by 8 to 16 here, not at all in gp_chain_kernel (12 for
+// groups of two in clusters).
 template <int GG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_bsel_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids, int n_req, int* __restrict__ actions,
@@ -1771,7 +1776,7 @@ gp_compact_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_i
 // kernel to end.  The grid therefore ends after both, and the plan of step t + 2, its programmatic dependent, finds the
 // pages and counters of the requests that sat step t + 1 out in their final state.  `p`: the view of step t (its
 // scratch set, the copy of the counters its decisions go to).
-// LONG: launched in clusters, which share out units of many candidates (split_unit).
+// LONG: launched in clusters, which share out units of many candidates (split_unit).  Synchronous mode only.
 template <int D, int GG, bool LONG>
 __global__ void __launch_bounds__(SEL_T, 2)
 gp_chain_kernel(const __grid_constant__ GpDev p, int n_req, int serial, int has_chain, const int* __restrict__ req_ids,

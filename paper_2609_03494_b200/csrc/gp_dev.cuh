@@ -45,7 +45,7 @@ enum {
   HDR_DONE_CMP,      // CTAs of the compaction kernel that have finished
   HDR_STEP,          // step serial number
   HDR_N_ACTIVE,      // requests actually stepped
-  HDR_DONE_SEL,      // CTAs of the selection kernel that have finished
+  HDR_DONE_SEL,      // CTAs of the selection that have finished their jobs; in clusters, jobs that are done
   HDR_WORK_CMP,      // ticket counter of the compaction kernel
   HDR_N_CITEM,       // compaction work items (parts x layers x heads)
   HDR_N_COW,         // copy-on-write targets allotted this step

@@ -34,7 +34,7 @@ struct gp_pool {
   std::vector<uint8_t> live;      // host mirror of the slot free list
   int num_sms, attn_grid, sel_grid, compact_grid;
   int chain_grid_max;                               // thread blocks of the one-kernel boundary path that are resident at once
-  int chain_grid_long;                              // ... in clusters that share out units of many candidates (0: no request can have them)
+  int chain_grid_long;                              // ... in clusters that share out units of many candidates (0: this pool never has such)
   bool chain_clusters;                              // the path is launched that way where a request may be that long
   // A live request holds at most as many tokens as it was admitted with and steps have been issued since, unless a captured step is replayed.
   std::vector<long long> began;                     // of each: tokens admitted with, less the steps issued before
@@ -90,7 +90,7 @@ struct Layout {
 inline size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Pages per attention work item: 64 (two page ids per producer lane), and half of that for requests at their
-// capacity boundary, whose pages also pay for the fp64 logits.  When an attention launch has less than one such
+// capacity boundary, whose pages also pay for the fp64 logits (the plan kernel has the two exceptions).  When an attention launch has less than one such
 // item of work per CTA (small batches, short sequences; a layer-by-layer launch, which covers one layer's heads
 // only), smaller items (32 and 8 pages) keep more CTAs busy (measured when a layer was three launches: the 36-layer shape
 // with 16 requests, layer by layer, 1030 us per step that way, 1252 with the large items; a layer is one launch now, 900 us).
@@ -379,7 +379,8 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     // too long for the selection behind them: one layer x 64, four at a boundary 46 / 57; 36 x 4, one, 77.4 / 77.9 us a step.
     // In small items for groups of eight, whose boundary tiles take a consumer warp 15 000 cycles each, where there are few of them: what the step then waits
     // for is the longest (64 requests of 128 to 1400 tokens on one layer 84.4 / 79.8 us a step; 20 on eight layers 153.4 / 154.8 if it were not for
-    // the bound; groups of four 62.9 / 64.3).
+    // the bound; groups of four 62.9 / 64.3).  At d = 64 as well, items of 32 / 16: 70.2 / 65.6, 32 of 500 to 9000 on two KV heads 112.7 / 103.3 (d = 128 125.2 / 114.1), 8 on
+    // four layers 78.9 / 77.3 (98.3 / 97.0); 120 requests on one layer 93.3 / 94.0, the most it costs.
     if (p.G == 8 && cp_bnd > GP_WIDE_BCHUNK && (long long)s_bpages * launch_units < 8LL * launch_grid && s_pages / GP_WIDE_BCHUNK + n_req <= p.max_rc)
       cp_bnd = GP_WIDE_BCHUNK;
     // (Not where the items, cut the smaller way, might not fit the scratch: who is refused below stays who was.)
@@ -387,8 +388,8 @@ gp_plan_kernel(const __grid_constant__ GpDev p, const int* __restrict__ req_ids,
     if ((long long)s_pages * launch_units < (long long)cp_norm * launch_grid) { cp_norm = GP_FINE_CHUNK; cp_bnd = GP_FINE_BCHUNK; }
   }
   if (pages > 0) {
-    // a page of a boundary request also pays for the fp64 summary logits: its items are half as large
-    // (measured best: 16, 24, 40 and 48 pages against 64 for the others were all slower)
+    // a page of a boundary request also pays for the fp64 summary logits: its items are smaller, by the rules above (32 in general: 16, 24, 40 and 48
+    // pages against 64 for the others, whatever the step, were all slower)
     cp = isb ? cp_bnd : cp_norm;
     chunks = (pages + cp - 1) / cp;
     cp = (pages + chunks - 1) / chunks;              // equal sizes: chunks of cp pages, the last one shorter
@@ -1403,7 +1404,7 @@ int gp_release(gp_pool* pool, int32_t req, void* stream) {
   pool->launch_count++;
   pool->plain_plan |= launch_kind(static_cast<cudaStream_t>(stream));
   pool->live[req] = 0;
-  if (pool->began[req] == pool->began_max) {
+  if (pool->chain_clusters && pool->began[req] == pool->began_max) {
     pool->began_max = -pool->serial;
     for (int i = 0; i < pool->cfg.max_requests; ++i)
       if (pool->live[i] && pool->began[i] > pool->began_max) pool->began_max = pool->began[i];
